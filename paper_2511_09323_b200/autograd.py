@@ -1,4 +1,5 @@
-"""`torch.autograd` front end of the MoC FFN operator: marshalling only, every step runs in the CUDA library.
+"""`torch.autograd` front end of the MoC FFN operator: marshalling only (the autograd node is in `csrc/torch_front.cpp`), every
+step runs in the CUDA library.
 
 `moc_ffn(x, w_gate, w_up, w_down, k)` is the layer of Section 3.2 (Eq. (Moc-1), the Top-K mask, Eq. (MoC-2)) with the
 backward of Section 4 (Eqs. (bp-1)..(bp-5)); between forward and backward only the compact Top-K activations are kept alive
@@ -16,36 +17,6 @@ import torch
 from . import binding as B
 
 
-class _MoCFFNFunction(torch.autograd.Function):
-    @staticmethod
-    def forward(ctx, x, w_gate, w_up, w_down, k, d_ff, grouped, recompute_up, post_silu=False):
-        shape = x.shape
-        x2 = x.reshape(-1, shape[-1]).contiguous()
-        save = any(ctx.needs_input_grad[:4])
-        out, idx, tg, tu = B.moc_ffn_forward(x2, w_gate, w_up, w_down, None if k is None else int(k), d_ff=d_ff,
-                                             save=save, grouped=bool(grouped), post_silu=bool(post_silu))
-        if save:
-            # recompute_up: the up values are dropped here and formed again in backward from x, w_up and the indices
-            ctx.save_for_backward(x2, w_gate, w_up, w_down, idx, tg, *(() if recompute_up else (tu,)))
-            ctx.d_ff = d_ff
-            ctx.grouped = bool(grouped)
-            ctx.x_shape = shape
-        return out.reshape(shape)
-
-    @staticmethod
-    def backward(ctx, grad_out):
-        x2, w_gate, w_up, w_down, idx, tg, *rest = ctx.saved_tensors
-        names = ("x", "w_gate", "w_up", "w_down")
-        want = tuple(n for n, need in zip(names, ctx.needs_input_grad[:4]) if need)
-        go = grad_out.reshape(-1, grad_out.shape[-1]).contiguous()
-        tu = rest[0] if rest else B.moc_ffn_recompute_up(x2, w_up, idx, d_ff=ctx.d_ff)
-        res = B.moc_ffn_backward(x2, w_gate, w_up, w_down, idx, tg, tu, go, d_ff=ctx.d_ff, want=want,
-                                 grouped=ctx.grouped)
-        gx = res["grad_x"]
-        return (None if gx is None else gx.reshape(ctx.x_shape), res["grad_w_gate"], res["grad_w_up"],
-                res["grad_w_down"], None, None, None, None, None)
-
-
 def moc_ffn(x: torch.Tensor, w_gate: torch.Tensor, w_up: torch.Tensor, w_down: torch.Tensor, k: int | None,
             d_ff: int | None = None, grouped: bool = False, recompute_up: bool = False,
             post_silu: bool = False) -> torch.Tensor:
@@ -56,7 +27,7 @@ def moc_ffn(x: torch.Tensor, w_gate: torch.Tensor, w_up: torch.Tensor, w_down: t
     the indices and the gate values between forward and backward (k * (2 + e) instead of k * (2 + 2 e) bytes per token)
     and pays one more up projection in backward.  post_silu=True ranks the channels by SiLU(gate value) instead of the
     gate value (the paper's ablation of the Top-K position, Section 6.5; exact but slow kernels)."""
-    return _MoCFFNFunction.apply(x, w_gate, w_up, w_down, k, d_ff, grouped, recompute_up, post_silu)
+    return (B._front or B.front()).ffn(x, w_gate, w_up, w_down, k, d_ff, B._flags(grouped, post_silu), recompute_up)
 
 
 class MoCFFN(torch.nn.Module):

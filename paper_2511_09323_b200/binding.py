@@ -1,7 +1,9 @@
 """ctypes binding of the MoC FFN C ABI (``include/moc_ffn.h``).
 
 Argument marshalling only: every step of the operator runs in the CUDA library.  PyTorch is
-used for device memory and streams.  There is no fallback: if ``libmoc_ffn.so`` has not been
+used for device memory and streams.  The calls of a model's inner loop (forward, decode and the
+autograd node) hand their arguments to ``_front.so`` (``csrc/torch_front.cpp``), which does the same
+marshalling in C++.  There is no fallback: if ``libmoc_ffn.so`` or ``_front.so`` has not been
 built (``python -m paper_2511_09323_b200.build``) or cannot be loaded, the first call raises.
 """
 from __future__ import annotations
@@ -134,6 +136,23 @@ def load() -> ctypes.CDLL:
     return _lib
 
 
+_front = None
+
+
+def front():
+    """The host side of forward, decode and the autograd node in C++ (``csrc/torch_front.cpp``); raises if it is missing."""
+    global _front
+    if _front is None:
+        load()
+        try:
+            from . import _front as module
+        except ImportError as exc:
+            raise RuntimeError(f"_front.so cannot be loaded ({exc}): build it with `python -m paper_2511_09323_b200.build`") from exc
+        module.set_error(MocError)
+        _front = module
+    return _front
+
+
 def status_string(status: int) -> str:
     return load().moc_status_string(int(status)).decode()
 
@@ -184,6 +203,10 @@ def alloc_workspace(desc: MocFfnDesc, op: int, device=None) -> torch.Tensor:
     return torch.empty(max(n, 16), dtype=torch.uint8, device=device or torch.device("cuda"))
 
 
+def _flags(grouped, post_silu):
+    return (MOC_FLAG_SELECT_2_OF_8 if grouped else 0) | (MOC_FLAG_SELECT_POST_SILU if post_silu else 0)
+
+
 def _grouped_k(k, d_ff):
     """k of the 2-of-8 mask (d_ff / 4); a caller may pass it or leave it None."""
     if d_ff % 8:
@@ -198,31 +221,9 @@ def moc_ffn_forward(x, w_gate, w_up, w_down, k, d_ff=None, save=True, out=None, 
     """Returns (out, topk_idx, topk_gate, topk_up); the last three are None when save=False.
     grouped=True: the 2-of-8 mask (MOC_FLAG_SELECT_2_OF_8) instead of the row Top-K; k is then d_ff / 4.
     post_silu=True: the Top-K on SiLU(g) instead of g (MOC_FLAG_SELECT_POST_SILU, the ablation variant)."""
-    _check_dev(x, w_gate, w_up, w_down, out, workspace)
-    T, d = x.shape
-    F_ld = w_gate.shape[0]
-    if grouped:
-        k = _grouped_k(k, F_ld if d_ff is None else d_ff)
-    desc = make_desc(T, d, F_ld if d_ff is None else d_ff, k, x.dtype, d_ff_ld=F_ld,
-                     flags=(MOC_FLAG_SELECT_2_OF_8 if grouped else 0) | (MOC_FLAG_SELECT_POST_SILU if post_silu else 0))
-    if out is None:
-        out = torch.empty_like(x)
-    if save:
-        if saved is None:
-            saved = (torch.empty((T, k), dtype=torch.int16, device=x.device),
-                     torch.empty((T, k), dtype=x.dtype, device=x.device),
-                     torch.empty((T, k), dtype=x.dtype, device=x.device))
-        idx, tg, tu = saved
-    else:
-        idx = tg = tu = None
-    if workspace is None:
-        workspace = alloc_workspace(desc, MOC_OP_FORWARD, x.device)
-    rc = load().moc_ffn_forward(ctypes.byref(desc), _ptr(x), _ptr(w_gate), _ptr(w_up), _ptr(w_down), _ptr(out),
-                                _ptr(idx), _ptr(tg), _ptr(tu), _ptr(workspace), workspace.numel(),
-                                _stream_ptr(stream))
-    if rc != MOC_OK:
-        raise MocError(rc, "moc_ffn_forward")
-    return out, idx, tg, tu
+    idx, tg, tu = saved if save and saved is not None else (None, None, None)
+    return (_front or front()).forward(x, w_gate, w_up, w_down, k, d_ff, _flags(grouped, post_silu), save, out, idx, tg, tu,
+                                       workspace, stream)
 
 
 def moc_ffn_backward(x, w_gate, w_up, w_down, topk_idx, topk_gate, topk_up, grad_out, d_ff=None,
@@ -288,46 +289,14 @@ def moc_ffn_recompute_up(x, w_up, topk_idx, d_ff=None, out=None, workspace=None,
 
 def moc_ffn_decode(x, w_gate, w_up, w_down, k, d_ff=None, out=None, workspace=None, stream=None, grouped=False,
                    post_silu=False):
-    _check_dev(x, w_gate, w_up, w_down, out, workspace)
-    T, d = x.shape
-    F_ld = w_gate.shape[0]
-    if grouped:
-        k = _grouped_k(k, F_ld if d_ff is None else d_ff)
-    desc = make_desc(T, d, F_ld if d_ff is None else d_ff, k, x.dtype, d_ff_ld=F_ld,
-                     flags=(MOC_FLAG_SELECT_2_OF_8 if grouped else 0) | (MOC_FLAG_SELECT_POST_SILU if post_silu else 0))
-    if out is None:
-        out = torch.empty_like(x)
-    if workspace is None:
-        workspace = alloc_workspace(desc, MOC_OP_DECODE, x.device)
-    rc = load().moc_ffn_decode(ctypes.byref(desc), _ptr(x), _ptr(w_gate), _ptr(w_up), _ptr(w_down), _ptr(out),
-                               _ptr(workspace), workspace.numel(), _stream_ptr(stream))
-    if rc != MOC_OK:
-        raise MocError(rc, "moc_ffn_decode")
-    return out
+    return (_front or front()).decode(x, w_gate, w_up, w_down, k, d_ff, _flags(grouped, post_silu), out, workspace, stream)
 
 
 def moc_ffn_decode_block(h, rms_weight, rms_eps, w_gate, w_up, w_down, k, d_ff=None, out=None, workspace=None,
                          stream=None, grouped=False):
     """out = h + MoC_FFN(RMSNorm(h; rms_weight, rms_eps)) for up to 256 bf16 tokens; `out` may be `h`."""
-    _check_dev(h, rms_weight, w_gate, w_up, w_down, out, workspace)
-    T, d = h.shape
-    if rms_weight.dtype != h.dtype or tuple(rms_weight.shape) != (d,):
-        raise TypeError("rms_weight must be a [d_model] tensor of the activations' dtype")
-    F_ld = w_gate.shape[0]
-    if grouped:
-        k = _grouped_k(k, F_ld if d_ff is None else d_ff)
-    desc = make_desc(T, d, F_ld if d_ff is None else d_ff, k, h.dtype, d_ff_ld=F_ld,
-                     flags=MOC_FLAG_SELECT_2_OF_8 if grouped else 0)
-    if out is None:
-        out = torch.empty_like(h)
-    if workspace is None:
-        workspace = alloc_workspace(desc, MOC_OP_DECODE_BLOCK, h.device)
-    rc = load().moc_ffn_decode_block(ctypes.byref(desc), _ptr(h), _ptr(rms_weight), float(rms_eps), _ptr(w_gate),
-                                     _ptr(w_up), _ptr(w_down), _ptr(out), _ptr(workspace), workspace.numel(),
-                                     _stream_ptr(stream))
-    if rc != MOC_OK:
-        raise MocError(rc, "moc_ffn_decode_block")
-    return out
+    return (_front or front()).decode_block(h, rms_weight, rms_eps, w_gate, w_up, w_down, k, d_ff, _flags(grouped, False), out,
+                                            workspace, stream)
 
 
 def moc_ffn_decode_static(x, w_gate, w_up, w_down, k, out, d_ff=None, stream=None, grouped=False, post_silu=False):

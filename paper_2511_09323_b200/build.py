@@ -8,6 +8,8 @@ import sys
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libmoc_ffn.so")
+FRONT_SOURCE = "torch_front.cpp"
+FRONT = os.path.join(HERE, "_front.so")   # the PyTorch entry points' host side, linked against LIB
 SOURCES = ["api.cu"]
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -23,6 +25,36 @@ def _nvcc() -> str:
     return "nvcc"
 
 
+def _front_is_current() -> bool:
+    if not os.path.exists(FRONT):
+        return False
+    have = os.path.getmtime(FRONT)
+    include = os.path.join(os.path.dirname(HERE), "include")
+    sources = [os.path.join(CSRC, FRONT_SOURCE)] + [os.path.join(include, n) for n in os.listdir(include)]
+    return all(have >= os.path.getmtime(p) for p in sources)
+
+
+def build_front() -> str:
+    """Compile csrc/torch_front.cpp into _front.so, a CPython module that calls libmoc_ffn.so; returns its path."""
+    import sysconfig
+
+    import torch
+    from torch.utils import cpp_extension
+    tmp = FRONT + ".tmp.%d" % os.getpid()
+    libs = cpp_extension.library_paths(device_type="cuda")
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", "-Wall",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"]
+    cmd += ["-isystem" + p for p in cpp_extension.include_paths(device_type="cuda") + [sysconfig.get_paths()["include"]]]
+    cmd += [os.path.join(CSRC, FRONT_SOURCE), "-o", tmp, "-L" + HERE, "-l:" + os.path.basename(LIB), "-Wl,-rpath,$ORIGIN"]
+    cmd += ["-L" + p for p in libs] + ["-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
+    proc = subprocess.run(cmd, capture_output=True, text=True)
+    if proc.returncode != 0:
+        sys.stderr.write(proc.stdout + proc.stderr)
+        raise RuntimeError("building _front.so failed")
+    os.replace(tmp, FRONT)
+    return FRONT
+
+
 def _newest_source_mtime() -> float:
     newest = 0.0
     for root in (CSRC, os.path.join(os.path.dirname(HERE), "include")):
@@ -33,9 +65,16 @@ def _newest_source_mtime() -> float:
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile csrc/*.cu into libmoc_ffn.so next to this file; returns its path."""
-    if not force and os.path.exists(LIB) and os.path.getmtime(LIB) >= _newest_source_mtime():
-        return LIB
+    """Compile csrc/*.cu into libmoc_ffn.so and csrc/torch_front.cpp into _front.so, next to this file; returns the
+    library's path."""
+    if force or not os.path.exists(LIB) or os.path.getmtime(LIB) < _newest_source_mtime():
+        _build_library(verbose)
+    if force or not _front_is_current():
+        build_front()
+    return LIB
+
+
+def _build_library(verbose: bool) -> None:
     tmp = LIB + ".tmp.%d" % os.getpid()
     extra = os.environ.get("MOC_FFN_NVCC_FLAGS", "").split()   # e.g. -DMOC_TIMELINE for a development build
     cmd = [_nvcc()] + NVCC_FLAGS + extra + (["-Xptxas", "-v"] if verbose else []) + \
@@ -47,7 +86,6 @@ def build(force: bool = False, verbose: bool = False) -> str:
     if verbose:
         sys.stderr.write(proc.stdout + proc.stderr)
     os.replace(tmp, LIB)
-    return LIB
 
 
 if __name__ == "__main__":

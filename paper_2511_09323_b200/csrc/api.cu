@@ -533,8 +533,6 @@ int sparse_gemm_pair(int64_t M, int N, int K, int segments, const __nv_bfloat16 
                      const uint32_t *const meta[2], const SparseOperandLayout &L, const __nv_bfloat16 *const b[2],
                      int ldb, __nv_bfloat16 *c, int ldc, bool accumulate, int kid, int *status, cudaStream_t st) {
     using namespace tcsp;
-    using tc::EncodeTiledFn;
-    using tc::encode_fn;
     SpPairParams p;
     memset(&p, 0, sizeof(p));
     for (int sgm = 0; sgm < segments; ++sgm) {
@@ -543,16 +541,14 @@ int sparse_gemm_pair(int64_t M, int N, int K, int segments, const __nv_bfloat16 
             !tc::make_map(&p.b_map[sgm], b[sgm], K, N, ldb, 64, 64))
             return MOC_ERR_CUDA;
         // the metadata as a matrix of 32-bit words, 4 per row: one stage of one 128-row block is a box of 4 x 128
-        EncodeTiledFn fn = encode_fn();
-        if (!fn) return MOC_ERR_CUDA;
         const int64_t blocks = (M + 127) / 128;
         cuuint64_t dims[2] = {4, (cuuint64_t)(blocks * L.k_stages * 128)};
         cuuint64_t strides[1] = {16};
         cuuint32_t box[2] = {4, 128};
         cuuint32_t estr[2] = {1, 1};
-        if (fn(&p.e_map[sgm], CU_TENSOR_MAP_DATA_TYPE_UINT32, 2, const_cast<uint32_t *>(meta[sgm]), dims, strides, box, estr,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
-               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        if (!tc::encode_tiled(&p.e_map[sgm], CU_TENSOR_MAP_DATA_TYPE_UINT32, 2, const_cast<uint32_t *>(meta[sgm]), dims, strides,
+                              box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                              CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE))
             return MOC_ERR_CUDA;
     }
     p.segments = segments;

@@ -38,19 +38,32 @@ inline EncodeTiledFn encode_fn() {
     return fn;
 }
 
+// One tensor map; false when the driver refuses it.  Encoding is a driver call and needs a current context, which a host
+// thread has only after its first runtime call: where this call comes first (an autograd thread's), the device's
+// primary context is made current and the call repeated.
+template <typename... Args>
+inline bool encode_tiled(Args... args) {
+    const EncodeTiledFn fn = encode_fn();
+    if (!fn) return false;
+    CUresult r = fn(args...);
+    if (r == CUDA_ERROR_INVALID_CONTEXT) {
+        int dev = 0;
+        if (cudaGetDevice(&dev) == cudaSuccess && cudaSetDevice(dev) == cudaSuccess) r = fn(args...);
+    }
+    return r == CUDA_SUCCESS;
+}
+
 // bf16 matrix [rows, cols] row-major with leading dimension ld (elements); box = box_cols x box_rows.
 // Out-of-range parts of a box read as zero.
 inline bool make_map(CUtensorMap *m, const void *ptr, int64_t rows, int64_t cols, int64_t ld, int box_cols,
                      int box_rows) {
-    EncodeTiledFn fn = encode_fn();
-    if (!fn) return false;
     cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
     cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
     cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows};
     cuuint32_t estr[2] = {1, 1};
-    return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(ptr), dims, strides, box, estr,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    return encode_tiled(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(ptr), dims, strides, box, estr,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
 }
 // K-major operand: tensor [mn, k], k contiguous; a tile is `tile_mn` rows of 64 k-elements
 inline bool map_k_major(CUtensorMap *m, const void *ptr, int64_t mn, int64_t k, int64_t ld, int tile_mn) {
@@ -93,17 +106,16 @@ inline void init_params(Params &p) {
 // Output [rows, cols] with leading dimension ld as 32-row boxes of 128 bytes.  False when the tensor-map rules
 // (16-byte aligned base and row pitch) do not hold.
 inline bool make_out_map(CUtensorMap *m, void *ptr, int64_t rows, int64_t cols, int64_t ld, bool f32) {
-    EncodeTiledFn fn = encode_fn();
     const size_t esz = f32 ? 4 : 2;
-    if (!fn || (reinterpret_cast<uintptr_t>(ptr) & 15u) || ((size_t)ld * esz) % 16 != 0 || rows <= 0 || cols <= 0)
+    if ((reinterpret_cast<uintptr_t>(ptr) & 15u) || ((size_t)ld * esz) % 16 != 0 || rows <= 0 || cols <= 0)
         return false;
     cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
     cuuint64_t strides[1] = {(cuuint64_t)ld * esz};
     cuuint32_t box[2] = {(cuuint32_t)(128 / esz), 32};
     cuuint32_t estr[2] = {1, 1};
-    return fn(m, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, ptr, dims, strides, box,
-              estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    return encode_tiled(m, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, ptr, dims, strides, box,
+                        estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
 }
 
 template <bool A_MN, bool B_MN, int EPI>

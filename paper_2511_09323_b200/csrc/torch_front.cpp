@@ -1,0 +1,316 @@
+// The host side of the PyTorch entry points: argument checks, output and workspace tensors and the autograd node, in
+// C++ so that a call costs the GPU's launches and little else.  No arithmetic: every step of the operator is a call of
+// the C ABI (include/moc_ffn.h), which this module links against.
+//
+// What bounds it: a small call is over on the GPU in some tens of microseconds, and the same work written in Python
+// (tensor checks, ctypes marshalling, a Python autograd.Function, whose backward has to take the interpreter lock on
+// the autograd thread) took longer than that: 256 fp32 tokens of a 128 x 512 layer, forward and backward, 191 us of which
+// the GPU worked for 62; now 99.  The host's part of a one-token decode call: 15.5 us, now 6.1.  binding.py and autograd.py keep the public signatures and pass their
+// arguments on by position; one call here crosses the language border once, through the vectorcall convention.
+#include <Python.h>
+
+#include <ATen/ATen.h>
+#include <c10/cuda/CUDAGuard.h>
+#include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Exceptions.h>
+#include <torch/csrc/autograd/custom_function.h>
+#include <torch/csrc/autograd/python_variable.h>
+
+#include "../../include/moc_ffn.h"
+
+namespace {
+
+using at::Tensor;
+
+PyObject *g_moc_error = nullptr;  // binding.MocError(status, where)
+
+// Raises binding.MocError as a C++ exception that the interpreter, or the autograd engine's thread, turns back into it.
+[[noreturn]] void raise_moc(int status, const char *where) {
+    pybind11::gil_scoped_acquire gil;
+    PyObject *args = Py_BuildValue("(is)", status, where);
+    PyObject *exc = args ? PyObject_CallObject(g_moc_error, args) : nullptr;
+    Py_XDECREF(args);
+    if (exc) {
+        PyErr_SetObject(reinterpret_cast<PyObject *>(Py_TYPE(exc)), exc);
+        Py_DECREF(exc);
+    }
+    python_error err;
+    err.persist();
+    throw err;
+}
+
+void check_dev(const Tensor &t) {
+    if (!t.defined()) return;
+    TORCH_CHECK_VALUE(t.is_cuda(), "expected CUDA tensors");
+    TORCH_CHECK_VALUE(t.is_contiguous(), "expected contiguous tensors");
+}
+
+template <typename... Ts>
+void check_all(const Ts &...ts) {
+    (check_dev(ts), ...);
+}
+
+int dtype_code(const Tensor &t) {
+    if (t.scalar_type() == at::kFloat) return MOC_F32;
+    if (t.scalar_type() == at::kBFloat16) return MOC_BF16;
+    TORCH_CHECK_TYPE(false, "unsupported storage dtype torch.", c10::toString(t.scalar_type()));
+}
+
+// d_ff < 0: all rows of the weights are channels; k < 0: not given (the 2-of-8 mask implies it)
+moc_ffn_desc make_desc(const Tensor &x, const Tensor &w, int64_t k, int64_t d_ff, uint32_t flags) {
+    TORCH_CHECK_VALUE(x.dim() == 2, "expected a [tokens, d_model] tensor");
+    moc_ffn_desc d{};
+    const int64_t rows = w.size(0);
+    if (d_ff < 0) d_ff = rows;
+    if (flags & MOC_FLAG_SELECT_2_OF_8) {
+        TORCH_CHECK_VALUE(d_ff % 8 == 0, "the 2-of-8 mask needs d_ff to be a multiple of 8");
+        TORCH_CHECK_VALUE(k < 0 || k == d_ff / 4, "the 2-of-8 mask keeps d_ff / 4 channels");
+        k = d_ff / 4;
+    }
+    d.tokens = x.size(0);
+    d.d_model = (int32_t)x.size(1);
+    d.d_ff = (int32_t)d_ff;
+    d.d_ff_ld = (int32_t)rows;
+    d.k = (int32_t)k;
+    d.dtype = dtype_code(x);
+    d.flags = flags;
+    return d;
+}
+
+Tensor workspace_for(const moc_ffn_desc &d, int op, const Tensor &like) {
+    const size_t n = std::max<size_t>(moc_ffn_workspace_bytes(&d, op), 16);
+    return at::empty({(int64_t)n}, like.options().dtype(at::kByte));
+}
+
+const void *in(const Tensor &t) { return t.defined() ? t.const_data_ptr() : nullptr; }
+void *outp(const Tensor &t) { return t.defined() ? t.data_ptr() : nullptr; }
+
+// the stream a call goes to: the caller's, or the current one of the current device
+void *stream_of(PyObject *stream) {
+    if (stream == Py_None) return c10::cuda::getCurrentCUDAStream().stream();
+    PyObject *v = PyObject_GetAttrString(stream, "cuda_stream");
+    if (!v) throw python_error();
+    void *p = PyLong_AsVoidPtr(v);
+    Py_DECREF(v);
+    if (!p && PyErr_Occurred()) throw python_error();
+    return p;
+}
+
+// ---- the autograd node ----------------------------------------------------------------------------------------
+// Between forward and backward only the compact Top-K activations live (Section 4, Table 1, column "MoC+GCP"), plus x.
+// recompute_up drops the up values as well; backward forms them again from x, w_up and the indices.
+struct MocFfnNode : public torch::autograd::Function<MocFfnNode> {
+    static Tensor forward(torch::autograd::AutogradContext *ctx, const Tensor &x, const Tensor &w_gate, const Tensor &w_up,
+                          const Tensor &w_down, int64_t k, int64_t d_ff, int64_t flags, bool recompute_up) {
+        const bool save = x.requires_grad() || w_gate.requires_grad() || w_up.requires_grad() || w_down.requires_grad();
+        const Tensor x2 = x.dim() == 2 && x.is_contiguous() ? x : x.reshape({-1, x.size(-1)}).contiguous();
+        check_all(x2, w_gate, w_up, w_down);
+        const moc_ffn_desc d = make_desc(x2, w_gate, k, d_ff, (uint32_t)flags);
+        Tensor out = at::empty_like(x2), idx, tg, tu;
+        if (save) {
+            idx = at::empty({d.tokens, d.k}, x2.options().dtype(at::kShort));
+            tg = at::empty({d.tokens, d.k}, x2.options());
+            tu = at::empty({d.tokens, d.k}, x2.options());
+        }
+        const Tensor ws = workspace_for(d, MOC_OP_FORWARD, x2);
+        const int rc = moc_ffn_forward(&d, in(x2), in(w_gate), in(w_up), in(w_down), outp(out), static_cast<int16_t *>(outp(idx)),
+                                       outp(tg), outp(tu), outp(ws), (size_t)ws.numel(), c10::cuda::getCurrentCUDAStream().stream());
+        if (rc != MOC_OK) raise_moc(rc, "moc_ffn_forward");
+        if (save) {
+            ctx->save_for_backward(recompute_up ? torch::autograd::variable_list{x2, w_gate, w_up, w_down, idx, tg}
+                                                : torch::autograd::variable_list{x2, w_gate, w_up, w_down, idx, tg, tu});
+            ctx->saved_data["d_ff"] = d_ff;
+            // the Top-K after the activation changes the choice of channels only: backward takes the mask as saved
+            ctx->saved_data["flags"] = flags & (int64_t)MOC_FLAG_SELECT_2_OF_8;
+            ctx->saved_data["shape"] = x.sizes();
+        }
+        return x.dim() == 2 ? out : out.reshape(x.sizes());
+    }
+
+    static torch::autograd::variable_list backward(torch::autograd::AutogradContext *ctx, torch::autograd::variable_list grads) {
+        const auto saved = ctx->get_saved_variables();
+        const Tensor &x = saved[0], &w_gate = saved[1], &w_up = saved[2], &w_down = saved[3], &idx = saved[4], &tg = saved[5];
+        const int64_t d_ff = ctx->saved_data["d_ff"].toInt();
+        const uint32_t flags = (uint32_t)ctx->saved_data["flags"].toInt();
+        torch::autograd::variable_list res(8);
+        if (!grads[0].defined()) return res;
+        const Tensor &g0 = grads[0];
+        const Tensor go = g0.dim() == 2 && g0.is_contiguous() ? g0 : g0.reshape({-1, g0.size(-1)}).contiguous();
+        check_dev(go);
+        moc_ffn_desc d = make_desc(x, w_gate, idx.size(1), d_ff, flags);
+        void *stream = c10::cuda::getCurrentCUDAStream().stream();
+        const Tensor ws = workspace_for(d, MOC_OP_BACKWARD, x);
+        Tensor tu;
+        if (saved.size() > 6) {
+            tu = saved[6];
+        } else {
+            tu = at::empty(tg.sizes(), tg.options());
+            moc_ffn_desc plain = d;
+            plain.flags = 0;
+            const int rc = moc_ffn_recompute_up(&plain, in(x), in(w_up), static_cast<const int16_t *>(in(idx)), outp(tu), outp(ws),
+                                                (size_t)ws.numel(), stream);
+            if (rc != MOC_OK) raise_moc(rc, "moc_ffn_recompute_up");
+        }
+        const Tensor *like[4] = {&x, &w_gate, &w_up, &w_down};
+        for (int i = 0; i < 4; ++i)
+            if (ctx->needs_input_grad(i)) res[i] = at::empty_like(*like[i]);
+        const int rc = moc_ffn_backward(&d, in(x), in(w_gate), in(w_up), in(w_down), static_cast<const int16_t *>(in(idx)), in(tg),
+                                        in(tu), in(go), outp(res[0]), outp(res[1]), outp(res[2]), outp(res[3]), outp(ws),
+                                        (size_t)ws.numel(), stream);
+        if (rc != MOC_OK) raise_moc(rc, "moc_ffn_backward");
+        if (res[0].defined()) {
+            const auto shape = ctx->saved_data["shape"].toIntVector();
+            if (shape.size() != 2) res[0] = res[0].reshape(shape);
+        }
+        return res;
+    }
+};
+
+// ---- Python ---------------------------------------------------------------------------------------------------
+Tensor tensor_arg(PyObject *o, const char *name, bool optional) {
+    if (optional && o == Py_None) return Tensor();
+    if (!THPVariable_Check(o)) {
+        PyErr_Format(PyExc_TypeError, "%s must be a torch.Tensor, not %s", name, Py_TYPE(o)->tp_name);
+        throw python_error();
+    }
+    return THPVariable_Unpack(o);
+}
+// a whole number, or -1 for None
+int64_t int_arg(PyObject *o) {
+    if (o == Py_None) return -1;
+    const long long v = PyLong_AsLongLong(o);
+    if (v != -1 || !PyErr_Occurred()) return v;
+    // (numbers that int() takes, as before: numpy integers, 0-d tensors, floats)
+    PyErr_Clear();
+    PyObject *n = PyNumber_Long(o);
+    if (!n) throw python_error();
+    const long long w = PyLong_AsLongLong(n);
+    Py_DECREF(n);
+    if (w == -1 && PyErr_Occurred()) throw python_error();
+    return w;
+}
+bool bool_arg(PyObject *o) {
+    const int v = PyObject_IsTrue(o);
+    if (v < 0) throw python_error();
+    return v != 0;
+}
+void need_args(Py_ssize_t have, Py_ssize_t want) {
+    if (have != want) {
+        PyErr_Format(PyExc_TypeError, "expected %zd arguments, got %zd", want, have);
+        throw python_error();
+    }
+}
+
+// ffn(x, w_gate, w_up, w_down, k, d_ff, flags, recompute_up) -> out, differentiable
+PyObject *py_ffn(PyObject *, PyObject *const *a, Py_ssize_t n) {
+    HANDLE_TH_ERRORS
+    need_args(n, 8);
+    const Tensor x = tensor_arg(a[0], "x", false), wg = tensor_arg(a[1], "w_gate", false), wu = tensor_arg(a[2], "w_up", false),
+                 wd = tensor_arg(a[3], "w_down", false);
+    const int64_t k = int_arg(a[4]), d_ff = int_arg(a[5]), flags = int_arg(a[6]);
+    const bool recompute = bool_arg(a[7]);
+    Tensor out;
+    {
+        pybind11::gil_scoped_release no_gil;
+        out = MocFfnNode::apply(x, wg, wu, wd, k, d_ff, flags, recompute);
+    }
+    return THPVariable_Wrap(out);
+    END_HANDLE_TH_ERRORS
+}
+
+// forward(x, w_gate, w_up, w_down, k, d_ff, flags, save, out, idx, gate, up, workspace, stream) -> (out, idx, gate, up)
+PyObject *py_forward(PyObject *, PyObject *const *a, Py_ssize_t n) {
+    HANDLE_TH_ERRORS
+    need_args(n, 14);
+    const Tensor x = tensor_arg(a[0], "x", false), wg = tensor_arg(a[1], "w_gate", false), wu = tensor_arg(a[2], "w_up", false),
+                 wd = tensor_arg(a[3], "w_down", false);
+    Tensor out = tensor_arg(a[8], "out", true), idx = tensor_arg(a[9], "topk_idx", true), tg = tensor_arg(a[10], "topk_gate", true),
+           tu = tensor_arg(a[11], "topk_up", true), ws = tensor_arg(a[12], "workspace", true);
+    check_all(x, wg, wu, wd, out, ws);
+    const moc_ffn_desc d = make_desc(x, wg, int_arg(a[4]), int_arg(a[5]), (uint32_t)int_arg(a[6]));
+    if (!out.defined()) out = at::empty_like(x);
+    if (bool_arg(a[7])) {
+        if (!idx.defined()) {
+            idx = at::empty({d.tokens, d.k}, x.options().dtype(at::kShort));
+            tg = at::empty({d.tokens, d.k}, x.options());
+            tu = at::empty({d.tokens, d.k}, x.options());
+        }
+    } else {
+        idx = tg = tu = Tensor();
+    }
+    if (!ws.defined()) ws = workspace_for(d, MOC_OP_FORWARD, x);
+    void *stream = stream_of(a[13]);
+    int rc;
+    {
+        pybind11::gil_scoped_release no_gil;
+        rc = moc_ffn_forward(&d, in(x), in(wg), in(wu), in(wd), outp(out), static_cast<int16_t *>(outp(idx)), outp(tg), outp(tu),
+                             outp(ws), (size_t)ws.numel(), stream);
+    }
+    if (rc != MOC_OK) raise_moc(rc, "moc_ffn_forward");
+    PyObject *t = PyTuple_New(4);
+    if (!t) throw python_error();
+    const Tensor *r[4] = {&out, &idx, &tg, &tu};
+    for (int i = 0; i < 4; ++i) PyTuple_SET_ITEM(t, i, THPVariable_Wrap(*r[i]));  // (an undefined tensor wraps to None)
+    return t;
+    END_HANDLE_TH_ERRORS
+}
+
+// decode(x, w_gate, w_up, w_down, k, d_ff, flags, out, workspace, stream) -> out
+// decode_block: the same with rms_weight, rms_eps behind x
+template <bool BLOCK>
+PyObject *py_decode(PyObject *, PyObject *const *a, Py_ssize_t n) {
+    HANDLE_TH_ERRORS
+    need_args(n, BLOCK ? 12 : 10);
+    const Tensor x = tensor_arg(a[0], "x", false);
+    Tensor rms;
+    double eps = 0.0;
+    if (BLOCK) {
+        rms = tensor_arg(a[1], "rms_weight", false);
+        eps = PyFloat_AsDouble(a[2]);
+        if (eps == -1.0 && PyErr_Occurred()) throw python_error();
+        a += 2;
+    }
+    const Tensor wg = tensor_arg(a[1], "w_gate", false), wu = tensor_arg(a[2], "w_up", false), wd = tensor_arg(a[3], "w_down", false);
+    Tensor out = tensor_arg(a[7], "out", true), ws = tensor_arg(a[8], "workspace", true);
+    check_all(x, rms, wg, wu, wd, out, ws);
+    if (BLOCK)
+        TORCH_CHECK_TYPE(rms.scalar_type() == x.scalar_type() && rms.dim() == 1 && x.dim() == 2 && rms.size(0) == x.size(1),
+                         "rms_weight must be a [d_model] tensor of the activations' dtype");
+    const moc_ffn_desc d = make_desc(x, wg, int_arg(a[4]), int_arg(a[5]), (uint32_t)int_arg(a[6]));
+    if (!out.defined()) out = at::empty_like(x);
+    if (!ws.defined()) ws = workspace_for(d, BLOCK ? MOC_OP_DECODE_BLOCK : MOC_OP_DECODE, x);
+    void *stream = stream_of(a[9]);
+    int rc;
+    {
+        pybind11::gil_scoped_release no_gil;
+        rc = BLOCK ? moc_ffn_decode_block(&d, in(x), in(rms), (float)eps, in(wg), in(wu), in(wd), outp(out), outp(ws),
+                                          (size_t)ws.numel(), stream)
+                   : moc_ffn_decode(&d, in(x), in(wg), in(wu), in(wd), outp(out), outp(ws), (size_t)ws.numel(), stream);
+    }
+    if (rc != MOC_OK) raise_moc(rc, BLOCK ? "moc_ffn_decode_block" : "moc_ffn_decode");
+    return THPVariable_Wrap(out);
+    END_HANDLE_TH_ERRORS
+}
+
+// set_error(class): the exception raised for a negative moc_status
+PyObject *py_set_error(PyObject *, PyObject *cls) {
+    Py_INCREF(cls);
+    Py_XDECREF(g_moc_error);
+    g_moc_error = cls;
+    Py_RETURN_NONE;
+}
+
+#define MOC_FAST(f) reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(f))
+PyMethodDef kMethods[] = {
+    {"ffn", MOC_FAST(py_ffn), METH_FASTCALL, nullptr},
+    {"forward", MOC_FAST(py_forward), METH_FASTCALL, nullptr},
+    {"decode", MOC_FAST(py_decode<false>), METH_FASTCALL, nullptr},
+    {"decode_block", MOC_FAST(py_decode<true>), METH_FASTCALL, nullptr},
+    {"set_error", py_set_error, METH_O, nullptr},
+    {nullptr, nullptr, 0, nullptr},
+};
+PyModuleDef kModule = {PyModuleDef_HEAD_INIT, "_front", nullptr, -1, kMethods, nullptr, nullptr, nullptr, nullptr};
+
+}  // namespace
+
+PyMODINIT_FUNC PyInit__front() { return PyModule_Create(&kModule); }
