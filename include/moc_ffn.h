@@ -263,15 +263,16 @@ MOC_API int moc_topk_select(int64_t rows, int32_t n, int32_t n_ld, int32_t k, co
 /*
  * The row Top-K selector of the tensor-core plan (the one moc_ffn_forward runs on training-sized bf16 batches) alone,
  * on caller-supplied fp32 gate rows, so that the mask definition of Section 3.2 can be checked bit-exactly on it too.
- * Which kernel form runs depends on the row length and k exactly as in moc_ffn_forward: teams of two or four warps per
- * row with the row staged in shared memory, the same with one buffer for the gate and the up row (long rows), or one
- * CTA per row (rows too long for a team's slice); `*variant` (host, may be NULL) receives which:
- * 0 CTA per row, 1 teams of two, 2 teams of four, 3 teams of four with a shared buffer.
+ * Which kernel form runs depends on the row length and k exactly as in moc_ffn_forward: teams of one to eight warps per
+ * row with the row in registers, teams of four with one shared-memory buffer for the gate and the up row (long rows), or
+ * one CTA per row (rows too long for a team's slice); `*variant` (host, may be NULL) receives which:
+ * 0 CTA per row, 1 teams of one or two warps and 2 teams of four or eight (the row in registers), 3 teams of four with the
+ * row in shared memory.
  *   gate     [rows, n_ld] fp32, device; n_ld a multiple of 8 with n <= n_ld <= n rounded up to 128
  *   idx_out  [rows, k] int16, device, ascending
  *   bracket  host pointer to {center, half width} of the threshold bracket the launch starts from (what the previous
- *            launch of a forward pass would have left in the workspace), or NULL for the state of a first call; the
- *            bracket is a hint only: any value, however wrong, must give the same exact result
+ *            launch of a forward pass would have left in the workspace; the forms with the row in registers use none), or
+ *            NULL for the state of a first call; the bracket is a hint only: any value, however wrong, must give the same exact result
  *   workspace  moc_topk_select_tc_workspace_bytes(rows, n, n_ld, k) bytes (0 = shape not served by this selector:
  *            (n + k) * 4 bytes must fit 170 KiB)
  */

@@ -16,6 +16,7 @@
 #include "gather_kernels.cuh"
 #include "grouped_select.cuh"
 #include "moc_common.cuh"
+#include "row_select.cuh"
 #include "small_batch.cuh"
 #include "small_batch_fused.cuh"
 #include "tc_gemm.cuh"
@@ -380,16 +381,13 @@ bool use_tc_forward(const moc_ffn_desc &d) { return use_tc_plan(d) && !(d.flags 
 inline int ceil_div(int64_t a, int64_t b) { return (int)((a + b - 1) / b); }
 
 // ---- the row Top-K selector of the tensor-core plan: which kernel form serves a row of F channels with K kept ----
-// A team of warps per token while at least two tokens' rows fit an SM's shared memory (each team stages its token's
-// rows in its own slice: as many teams per SM as fit, in one or two CTAs; rows too long for that with separate gate
-// and up buffers let the two rows share one buffer), else one CTA per token.  Teams of four warps for long rows (few
-// tokens fit an SM there), pairs otherwise (measured: LLaMA-1B width 0.59 -> 0.50 ms and LLaMA-7B width 0.56 -> 0.41 ms
-// with four; 2048 channels 0.080 -> 0.124 ms, so short rows keep pairs).
+// Rows of up to 14336 channels: a team of W warps per token with the row in registers, 16 to 64 values per lane
+// (row_select.cuh).  Longer rows: teams of four with the row in shared memory, gate and up row sharing one buffer, while
+// two such tokens fit an SM (up to some 17000 channels); else one CTA per token.
 struct TcSelect {
+    enum Kind { kRegisters, kSharedRow, kCtaPerRow } kind;
     int nv;             // 128-channel groups of a row
-    int team;           // warps per token (2 or 4)
-    bool team_select;   // false: one CTA per token (select_mask_rows_kernel)
-    bool shared_u;      // gate and up row share one buffer
+    int team, vpl;      // warps per token; values per lane (kRegisters)
     int tokens_per_cta, ctas_per_sm;
     size_t smem;        // dynamic shared memory of the launch
     int variant;        // MOC_SELECT_VARIANT_* (what a test hook reports)
@@ -397,35 +395,48 @@ struct TcSelect {
 
 enum {
     MOC_SELECT_VARIANT_CTA_PER_ROW = 0,   // select_mask_rows_kernel
-    MOC_SELECT_VARIANT_TEAM2 = 1,         // teams of two warps, separate gate / up buffers
-    MOC_SELECT_VARIANT_TEAM4 = 2,         // teams of four warps, separate buffers
-    MOC_SELECT_VARIANT_TEAM4_SHARED = 3,  // teams of four, one buffer for both rows
+    MOC_SELECT_VARIANT_TEAM2 = 1,         // one or two warps per row, the row in registers
+    MOC_SELECT_VARIANT_TEAM4 = 2,         // four or eight warps per row, the row in registers
+    MOC_SELECT_VARIANT_TEAM4_SHARED = 3,  // teams of four, one shared-memory buffer for both rows
 };
+
+// (warps per token, values per lane), each for up to 32 * W * VPL channels.  The fewest warps that leave a lane at most 64
+// values: every warp of a team repeats the scan of the histogram and the ranking (16384 rows of 2048 channels: 71 us with
+// one or two warps, 119 us with four).
+#define MOC_ROW_SELECT_FORMS(DO) DO(1, 16) DO(1, 32) DO(2, 32) DO(2, 48) DO(4, 32) DO(4, 44) DO(4, 64) DO(8, 44) DO(8, 56)
 
 TcSelect tc_select_config(int F, int K) {
     using namespace tc;
     TcSelect c{};
     c.nv = ceil_div(F, 128);
-    c.team = c.nv >= 40 ? 4 : 2;
-    const auto units_fit = [&](bool shared) {  // tokens in flight per SM
-        return (int)std::min<size_t>(
-            (size_t)220 * 1024 / (pair_select_words(c.nv, K, shared, c.team) * sizeof(uint32_t)), 16);
-    };
-    const bool parks = pair_select_parks_gates(c.nv, K, c.team);
-    const int min_units = 2;  // at least two tokens in flight per SM
-    // (rows short enough for teams of two always fit with separate buffers: the shared form exists for teams of four)
-    c.shared_u = c.team == 4 && units_fit(false) < min_units && parks && units_fit(true) >= min_units;
-    const size_t team_bytes = pair_select_words(c.nv, K, c.shared_u, c.team) * sizeof(uint32_t);
-    const int per_sm = units_fit(c.shared_u);
-    const int units_per_cta = kPairSelMaxWarps / c.team;
-    c.team_select = per_sm >= min_units;
-    if (c.team_select) {
+#define MOC_DO_PICK(W, VPL)                      \
+    if (c.team == 0 && F <= 32 * W * VPL) {      \
+        c.team = W;                              \
+        c.vpl = VPL;                             \
+        c.ctas_per_sm = rs::ctas_per_sm(W, VPL); \
+    }
+    MOC_ROW_SELECT_FORMS(MOC_DO_PICK)
+#undef MOC_DO_PICK
+    if (c.team) {
+        c.kind = TcSelect::kRegisters;
+        c.tokens_per_cta = 1;
+        c.smem = rs::layout(c.team, c.nv * 128, K).total;  // (rows may be padded up to whole groups)
+        c.ctas_per_sm = std::max(1, std::min(c.ctas_per_sm, (int)((size_t)kMaxDynSmem / (c.smem + 1024))));
+        c.variant = c.team <= 2 ? MOC_SELECT_VARIANT_TEAM2 : MOC_SELECT_VARIANT_TEAM4;
+        return c;
+    }
+    const size_t team_bytes = team_select_words(c.nv, K) * sizeof(uint32_t);
+    const int per_sm = (int)std::min<size_t>((size_t)220 * 1024 / team_bytes, 16);  // tokens in flight per SM
+    if (per_sm >= 2 && team_select_parks_gates(c.nv, K)) {
+        c.kind = TcSelect::kSharedRow;
+        c.team = 4;
+        const int units_per_cta = kTeamSelMaxWarps / 4;
         c.ctas_per_sm = per_sm > units_per_cta ? 2 : 1;
         c.tokens_per_cta = std::min(per_sm / c.ctas_per_sm, units_per_cta);
         c.smem = (size_t)c.tokens_per_cta * team_bytes;
-        c.variant = c.team == 4 ? (c.shared_u ? MOC_SELECT_VARIANT_TEAM4_SHARED : MOC_SELECT_VARIANT_TEAM4)
-                                : MOC_SELECT_VARIANT_TEAM2;
+        c.variant = MOC_SELECT_VARIANT_TEAM4_SHARED;
     } else {
+        c.kind = TcSelect::kCtaPerRow;
         c.ctas_per_sm = 6;
         c.tokens_per_cta = 1;
         c.smem = ((size_t)F + K) * sizeof(uint32_t);
@@ -434,57 +445,47 @@ TcSelect tc_select_config(int F, int K) {
     return c;
 }
 
-// the usual row lengths get their loops unrolled (the template's first parameter)
-#define MOC_TC_SELECT_DISPATCH(c, DO)                                                   \
-    do {                                                                                \
-        if ((c).team == 4) {                                                            \
-            if ((c).shared_u) DO((tc::select_mask_rows_pair_kernel<0, true, 4>), 128);  \
-            else if ((c).nv == 43) DO((tc::select_mask_rows_pair_kernel<43, false, 4>), 128); \
-            else DO((tc::select_mask_rows_pair_kernel<0, false, 4>), 128);              \
-        } else {                                                                        \
-            if ((c).nv == 8) DO((tc::select_mask_rows_pair_kernel<8, false, 2>), 64);   \
-            else if ((c).nv == 16) DO((tc::select_mask_rows_pair_kernel<16, false, 2>), 64); \
-            else if ((c).nv == 32) DO((tc::select_mask_rows_pair_kernel<32, false, 2>), 64); \
-            else DO((tc::select_mask_rows_pair_kernel<0, false, 2>), 64);               \
-        }                                                                               \
-    } while (0)
-
 int tc_select_prepare(const TcSelect &c, int F, int K) {
-    int rc = MOC_OK;
-    if (c.team_select) {
-#define MOC_DO_SET(KERN, TPT) rc = set_smem(KERN, c.smem, 2048)
-        MOC_TC_SELECT_DISPATCH(c, MOC_DO_SET);
+    if (c.kind == TcSelect::kRegisters) {
+#define MOC_DO_SET(W, VPL) \
+    if (c.team == W && c.vpl == VPL) return set_smem(rs::select_rows_reg_kernel<W, VPL>, c.smem, 1024);
+        MOC_ROW_SELECT_FORMS(MOC_DO_SET)
 #undef MOC_DO_SET
-    } else {
-        rc = set_smem(tc::select_mask_rows_kernel, c.smem);
     }
+    if (c.kind == TcSelect::kSharedRow) return set_smem(tc::select_mask_rows_team_kernel, c.smem, 2048);
+    const int rc = set_smem(tc::select_mask_rows_kernel, c.smem);
     if (rc != MOC_OK) return rc;
     return set_smem(tc::select_hint_kernel, (size_t)F * sizeof(uint32_t));
 }
 
-// Team selector: every launch works with one bracket kept in the workspace ({center, width, tag} at hint[0..2]); it
-// gathers the statistics of its thresholds (hint[4..6], CTA counter at hint[8]) and its last CTA rewrites the bracket
-// for the next launch.  The bracket is only a hint: a stale or garbage one costs time (rows take the general exact
-// path), never correctness; the statistics and the counter reset themselves at the end of every launch.
-// CTA-per-token selector: hint[0..1] is the guess select_hint_kernel left.
+// Team selector with the row in shared memory: every launch works with one bracket kept in the workspace ({center, width,
+// tag} at hint[0..2]); it gathers the statistics of its thresholds (hint[4..6], CTA counter at hint[8]) and its last CTA
+// rewrites the bracket for the next launch.  The bracket is only a hint: a stale or garbage one costs time (rows take the
+// general exact path), never correctness; the statistics and the counter reset themselves at the end of every launch.
+// CTA-per-token selector: hint[0..1] is the guess select_hint_kernel left.  The register form needs no hint.
 void tc_select_launch(const TcSelect &c, const float *G, int ldg, __nv_bfloat16 *U, int ldu, int64_t n, int F, int K,
                       int16_t *o_idx, __nv_bfloat16 *o_g, __nv_bfloat16 *o_u, float *hint, int *status, cudaStream_t st) {
     using namespace tc;
-    if (c.team_select) {
+    const unsigned grid = (unsigned)std::min<int64_t>((n + c.tokens_per_cta - 1) / c.tokens_per_cta,
+                                                      (int64_t)sm_count() * c.ctas_per_sm);
+    if (c.kind == TcSelect::kRegisters) {
+#define MOC_DO_LAUNCH(W, VPL)                                                                                                   \
+    if (c.team == W && c.vpl == VPL)                                                                                            \
+        MOC_LAUNCH(KID_TC_SELECT_MASK, st,                                                                                      \
+                   (rs::select_rows_reg_kernel<W, VPL><<<grid, 32 * W, c.smem, st>>>(G, ldg, U, ldu, n, F, K,                   \
+                                                                                     rs::normal_quantile(F, K), o_idx, o_g, o_u, \
+                                                                                     status)));
+        MOC_ROW_SELECT_FORMS(MOC_DO_LAUNCH)
+#undef MOC_DO_LAUNCH
+    } else if (c.kind == TcSelect::kSharedRow) {
         SelectMeta meta{};
         meta.bracket = hint;
         meta.acc = hint + 4;
         meta.done = reinterpret_cast<unsigned int *>(hint + 8);
-        const unsigned grid = (unsigned)std::min<int64_t>((n + c.tokens_per_cta - 1) / c.tokens_per_cta,
-                                                          (int64_t)sm_count() * c.ctas_per_sm);
-#define MOC_DO_LAUNCH(KERN, TPT)                                                                     \
-    MOC_LAUNCH(KID_TC_SELECT_MASK, st,                                                               \
-               (KERN<<<grid, c.tokens_per_cta * TPT, c.smem, st>>>(G, ldg, U, ldu, n, F, c.nv, K, o_idx, o_g, o_u, \
-                                                                    meta, status)))
-        MOC_TC_SELECT_DISPATCH(c, MOC_DO_LAUNCH);
-#undef MOC_DO_LAUNCH
+        MOC_LAUNCH(KID_TC_SELECT_MASK, st,
+                   (select_mask_rows_team_kernel<<<grid, c.tokens_per_cta * 128, c.smem, st>>>(G, ldg, U, ldu, n, F, c.nv, K, o_idx,
+                                                                                               o_g, o_u, meta, status)));
     } else {
-        const unsigned grid = (unsigned)std::min<int64_t>(n, (int64_t)sm_count() * 6);
         MOC_LAUNCH(KID_TC_SELECT_MASK, st,
                    (select_mask_rows_kernel<<<grid, kSelectThreads, c.smem, st>>>(G, ldg, U, ldu, n, F, K, o_idx, o_g,
                                                                                    o_u, hint)));
@@ -738,7 +739,7 @@ int forward_tc(const moc_ffn_desc &d, const __nv_bfloat16 *x, const __nv_bfloat1
         p.c[1] = U + t0 * L.ldf;
         MOC_LAUNCH(KID_TC_GATE_UP_GEMM, st, (rc = launch_gemm<false, false, EPI_GATE_UP>(p, st)));
         if (rc != MOC_OK) return rc;
-        if (t0 == 0 && !sel.team_select) {
+        if (t0 == 0 && sel.kind == TcSelect::kCtaPerRow) {
             MOC_LAUNCH(KID_TC_SELECT_HINT, st,
                        (select_hint_kernel<<<1, kSelectThreads, (size_t)F * sizeof(uint32_t), st>>>(G, F, K, hint)));
             if ((rc = launch_ok()) != MOC_OK) return rc;
@@ -1978,7 +1979,7 @@ int moc_topk_select_tc(int64_t rows, int32_t n, int32_t n_ld, int32_t k, const f
     if (cudaMemsetAsync(hint, 0, 256, st) != cudaSuccess) return MOC_ERR_CUDA;
     if (bracket) {
         set_hint_kernel<<<1, 1, 0, st>>>(hint, bracket[0], bracket[1], tc::kBracketTag);
-    } else if (!sel.team_select) {
+    } else if (sel.kind == TcSelect::kCtaPerRow) {
         // as in the forward pass: the CTA-per-row form starts from the exact threshold of the first row
         tc::select_hint_kernel<<<1, kSelectThreads, (size_t)n * sizeof(uint32_t), st>>>(gate, n, k, hint);
     }

@@ -75,7 +75,7 @@ struct Vec8<float> {
 __device__ __forceinline__ float sigmoid_f(float g) {
     // evaluated from exp(-|g|) so that large |g| neither overflows nor produces NaN
     float e = expf(-fabsf(g));
-    float r = 1.0f / (1.0f + e);
+    float r = __frcp_rn(1.0f + e);  // (the correctly rounded 1 / (1 + e), as the division gives it)
     return g >= 0.0f ? r : e * r;
 }
 __device__ __forceinline__ float silu_f(float g) { return g * sigmoid_f(g); }

@@ -203,9 +203,9 @@ __global__ void __launch_bounds__(kSelectThreads) select_hint_kernel(const float
 }
 
 // ------------------------------------------------------------------------------------------------
-// Forward selector for rows that fit a slice of shared memory: a TEAM of two or four warps per token, no block
-// barriers (the warps of a team meet at a named barrier of their own).  nv = number of 128-channel groups of a row.
-// Same outputs as the CTA-per-token kernel below.
+// Forward selector for rows too long for registers (row_select.cuh) that still fit a slice of shared memory: a TEAM of
+// four warps per token, no block barriers (the warps of a team meet at a named barrier of their own).  nv = number of
+// 128-channel groups of a row.  Same outputs as the CTA-per-token kernel below.
 //
 // Every team owns a slice of shared memory into which its first thread bulk-copies the token's gate row (fp32)
 // and up row (bf16); the team works on those copies, turns the up row into the masked Z' row in place and
@@ -315,40 +315,33 @@ __device__ __noinline__ uint32_t warp_select_row_general(const float *g, int F, 
 
 // ------------------------------------------------------------------------------------------------
 // The kernel.  Warp w of a team of W takes the 128-channel groups w, w + W, ... in steps 1 and 3 and every W-th
-// batch of kept channels in step 4; the warps meet at the team's named barrier between the steps.  The shared
-// memory of an SM bounds the tokens in flight, so W warps per token make it feed W times as many warps (measured
-// against one warp per token: 2048 channels 0.086 -> 0.080 ms with pairs; 5504 channels 0.85 -> 0.50 ms and 11008
-// channels 0.68 -> 0.41 ms with teams of four).
-// shared_u: the up row is copied into the gate row's buffer once the gate values are no longer needed there
-// (less shared memory per token, so longer rows still fit; no prefetch of the next gate row).  It is a template
-// parameter: as a run-time flag it slowed the common path by a quarter.
-__host__ __device__ constexpr size_t pair_select_words(int nv, int K, bool shared_u, int W = 2) {
-    return (size_t)nv * 128 + (shared_u ? 0 : (size_t)nv * 64) + (size_t)W * warp_select_cand_words(nv) +
-           warp_select_bitmap_words(nv) + (size_t)((K + 3) & ~3) + 40 /* exchange */ + 4 /* two mbarriers */;
+// batch of kept channels in step 4; the warps meet at the team's named barrier between the steps.  The up row is copied
+// into the gate row's buffer once the gate values are no longer needed there, so that two tokens' rows fit an SM.
+constexpr int kTeamWarps = 4;
+__host__ __device__ constexpr size_t team_select_words(int nv, int K) {
+    return (size_t)nv * 128 + (size_t)kTeamWarps * warp_select_cand_words(nv) + warp_select_bitmap_words(nv) +
+           (size_t)((K + 3) & ~3) + 40 /* exchange */ + 4 /* two mbarriers */;
 }
-__host__ __device__ constexpr bool pair_select_parks_gates(int nv, int K, int W = 2) {
-    return K <= W * warp_select_cand_words(nv) + warp_select_bitmap_words(nv);
+__host__ __device__ constexpr bool team_select_parks_gates(int nv, int K) {
+    return K <= kTeamWarps * warp_select_cand_words(nv) + warp_select_bitmap_words(nv);
 }
-constexpr int kPairSelMaxWarps = 12;  // warps per CTA, at most (six pairs or three teams of four; two CTAs per SM)
+constexpr int kTeamSelMaxWarps = 12;  // warps per CTA, at most (three teams of four; two CTAs per SM)
 
-template <int NV, bool shared_u, int W>
-__global__ void __launch_bounds__(kPairSelMaxWarps * 32, 2) select_mask_rows_pair_kernel(
-    const float *__restrict__ G, int ldg, __nv_bfloat16 *__restrict__ U, int ldu, int64_t rows, int F, int nv_runtime, int K,
+__global__ void __launch_bounds__(kTeamSelMaxWarps * 32, 2) select_mask_rows_team_kernel(
+    const float *__restrict__ G, int ldg, __nv_bfloat16 *__restrict__ U, int ldu, int64_t rows, int F, int nv, int K,
     int16_t *__restrict__ idx_out, __nv_bfloat16 *__restrict__ g_out, __nv_bfloat16 *__restrict__ u_out,
     SelectMeta meta, int *status) {
     extern __shared__ __align__(128) uint32_t warp_sel_smem[];
-    static_assert(W == 2 || W == 4, "teams of two or four warps");
-    constexpr int TT = 32 * W;  // threads of a team
-    __shared__ float s_stat[kPairSelMaxWarps / 2][3];
+    constexpr int W = kTeamWarps, TT = 32 * W;  // threads of a team
+    __shared__ float s_stat[kTeamSelMaxWarps / W][3];
     __shared__ int s_abort;
-    const int nv = NV > 0 ? NV : nv_runtime;
     const int slots = warp_select_slots(nv), cw = warp_select_cand_words(nv);
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, ppc = blockDim.x / TT;  // teams per CTA
     const int pair = wib / W, w = wib % W, pl = (w << 5) | lane;                       // pl: thread index within the team
-    uint32_t *base = warp_sel_smem + (size_t)pair * pair_select_words(nv, K, shared_u, W);
+    uint32_t *base = warp_sel_smem + (size_t)pair * team_select_words(nv, K);
     float *sg = reinterpret_cast<float *>(base);
-    __nv_bfloat16 *su = reinterpret_cast<__nv_bfloat16 *>(shared_u ? base : base + nv * 128);
-    uint32_t *cand0 = base + nv * 128 + (shared_u ? 0 : nv * 64);  // [W warps][slot][lane] parked values
+    __nv_bfloat16 *su = reinterpret_cast<__nv_bfloat16 *>(base);
+    uint32_t *cand0 = base + nv * 128;  // [W warps][slot][lane] parked values
     uint32_t *cand = cand0 + w * cw;
     uint32_t *bitmap = cand0 + W * cw;
     uint32_t *kept = bitmap + warp_select_bitmap_words(nv);
@@ -356,7 +349,6 @@ __global__ void __launch_bounds__(kPairSelMaxWarps * 32, 2) select_mask_rows_pai
     uint64_t *bar_mem = reinterpret_cast<uint64_t *>(xch + 40);  // (xch[32..35]: the warps' wait verdicts)
     const uint32_t bar_g = smem_u32(bar_mem), bar_u = smem_u32(bar_mem + 1);
     float *gkept = reinterpret_cast<float *>(cand0);
-    const bool early_gate = pair_select_parks_gates(nv, K, W);
     auto pair_sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(pair + 1), "n"(TT) : "memory"); };
     const int64_t gp = (int64_t)blockIdx.x * ppc + pair, np = (int64_t)gridDim.x * ppc;
     const float b_center = meta.bracket[0], b_width = meta.bracket[1];
@@ -378,10 +370,6 @@ __global__ void __launch_bounds__(kPairSelMaxWarps * 32, 2) select_mask_rows_pai
     uint32_t phase = 0;
     int xp = 0;  // parity of the exchange slot in use
     bool dead = false;
-    if (pl == 0 && gp < rows && !shared_u) {
-        mbar_expect_tx(bar_g, g_bytes);
-        bulk_copy_g2s(smem_u32(sg), G + gp * (int64_t)ldg, g_bytes, bar_g);
-    }
     // the warps of a team take every branch below together: all conditions come from values they share
 
     for (int64_t r = gp; r < rows && !dead; r += np) {
@@ -389,13 +377,8 @@ __global__ void __launch_bounds__(kPairSelMaxWarps * 32, 2) select_mask_rows_pai
         if (pl == 0) {
             bulk_store_wait_read<0>();
             fence_async_smem();
-            if (shared_u) {
-                mbar_expect_tx(bar_g, g_bytes);
-                bulk_copy_g2s(smem_u32(sg), G + r * (int64_t)ldg, g_bytes, bar_g);
-            } else {
-                mbar_expect_tx(bar_u, u_bytes);
-                bulk_copy_g2s(smem_u32(su), u, u_bytes, bar_u);
-            }
+            mbar_expect_tx(bar_g, g_bytes);
+            bulk_copy_g2s(smem_u32(sg), G + r * (int64_t)ldg, g_bytes, bar_g);
         }
         // a wait that gave up ends the team: the warps exchange their verdicts so that all of them leave together
         // (another team's time-out can make one warp's wait return early and not its partner's)
@@ -585,23 +568,12 @@ __global__ void __launch_bounds__(kPairSelMaxWarps * 32, 2) select_mask_rows_pai
             pair_sync();
         }
         // ---- 4. values of the kept channels, entries pl, pl + 64, ...
-        auto request_next_gate = [&]() {
-            if (pl == 0 && r + np < rows) {
-                fence_async_smem();
-                mbar_expect_tx(bar_g, g_bytes);
-                bulk_copy_g2s(smem_u32(sg), G + (r + np) * (int64_t)ldg, g_bytes, bar_g);
-            }
-        };
-        if (early_gate) {
-            for (int i = pl; i < K; i += TT) gkept[i] = sg[kept[i]];
-            pair_sync();
-            if (!shared_u) {
-                request_next_gate();
-            } else if (pl == 0) {
-                fence_async_smem();
-                mbar_expect_tx(bar_u, u_bytes);
-                bulk_copy_g2s(smem_u32(su), u, u_bytes, bar_u);
-            }
+        for (int i = pl; i < K; i += TT) gkept[i] = sg[kept[i]];
+        pair_sync();
+        if (pl == 0) {
+            fence_async_smem();
+            mbar_expect_tx(bar_u, u_bytes);
+            bulk_copy_g2s(smem_u32(su), u, u_bytes, bar_u);
         }
         if (!team_agrees(__all_sync(0xffffffffu, mbar_wait(bar_u, phase, &s_abort, status)))) {
             dead = true;
@@ -610,7 +582,7 @@ __global__ void __launch_bounds__(kPairSelMaxWarps * 32, 2) select_mask_rows_pai
         phase ^= 1u;
         for (int i = pl; i < K; i += TT) {
             const uint32_t j = kept[i];
-            const float gval = early_gate ? gkept[i] : sg[j];
+            const float gval = gkept[i];
             const __nv_bfloat16 ub = su[j];
             const __nv_bfloat16 zb = __float2bfloat16_rn(silu_f(gval) * __bfloat162float(ub));
             kept[i] = j | ((uint32_t)(*reinterpret_cast<const uint16_t *>(&zb)) << 16);
@@ -621,7 +593,6 @@ __global__ void __launch_bounds__(kPairSelMaxWarps * 32, 2) select_mask_rows_pai
             }
         }
         pair_sync();
-        if (!early_gate) request_next_gate();
         // ---- up row -> masked Z' row, in shared memory, then one bulk store
         uint4 *row16 = reinterpret_cast<uint4 *>(su);
         for (int i = pl; i < (ldu >> 3); i += TT) row16[i] = make_uint4(0, 0, 0, 0);
