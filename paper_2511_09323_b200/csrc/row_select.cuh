@@ -9,8 +9,9 @@
 // What bounds it: 8 bytes per channel have to move (G, U in, Z' out), and the instructions of the search have to stay
 // below what the SM issues meanwhile.  A row is therefore read once, into registers, and walked three times in straight
 // lines of predicated instructions (as branches, which is what plain code compiles to, each walk costs twice as much):
-//   1. histogram: every value is mapped to one of 256 equal bins of a window around the expected threshold (multiply-add
-//      with saturation, so that what lies outside falls into the end bins) and counted with one shared-memory atomic;
+//   1. histogram: every value is mapped to one of 256 equal bins (512 for teams of eight) of a window around the expected
+//      threshold (multiply-add with saturation, so that what lies outside falls into the end bins) and counted with one
+//      shared-memory atomic;
 //   2. every warp scans the counts: bin b of the K-th largest value.  Everything from (just below) bin b on is a candidate
 //      set of K + a few values: counted per group of 128 channels, one packed prefix sum over the lanes;
 //   3. the candidate set goes to shared memory in ascending channel order, {value, channel} each.
@@ -32,7 +33,10 @@
 namespace moc {
 namespace rs {
 
-constexpr int kBins = 256;
+constexpr int kMaxBins = 512;
+// Bins of the histogram: some 7 values in the threshold's bin (2048 channels: 3, 5504: 7, 11008: 7).  More would go over
+// what one lane each can rank for a row in a few hundred, and a row searched over the whole range takes 30 us.
+constexpr int bins(int W) { return W >= 8 ? 512 : 256; }
 constexpr uint32_t kMaxRanked = 32;     // candidates ranked by one lane each
 constexpr float kWindowMad = 0.95f;     // half width of the window in mean absolute deviations (0.76 sigma of normal values)
 
@@ -62,7 +66,7 @@ __host__ __device__ inline Layout layout(int W, int ldu, int K) {
     L.kept = o;  // {gate value, channel} in ascending channel order
     o += (((uint32_t)K + kMaxRanked) * 8u + 15u) & ~15u;
     L.hist = o;
-    o += kBins * 4u;
+    o += kMaxBins * 4u;
     L.xch = o;  // number of ranked entries, pad[3] | ranked entries {value, list index} | two words per warp
     o += (4u + 2u * kMaxRanked + 2u * (uint32_t)W) * 4u;
     L.bar = (o + 7u) & ~7u;
@@ -78,12 +82,13 @@ __device__ __forceinline__ void keep_if_ge(float x, float tau, int ch, uint32_t 
         : "memory");
     at += x >= tau ? 8u : 0u;
 }
-// four times the bin of a value: non-decreasing in x, NaN and everything below the window in bin 0, above it in bin 255
+// four times the bin of a value: non-decreasing in x, NaN and everything below the window in bin 0, above it in the last
+template <int BINS>
 __device__ __forceinline__ uint32_t bin4(float x, float scale, float offset) {
+    constexpr int bits = BINS == 512 ? 9 : 8;
     const float q = __saturatef(fmaf(x, scale, offset));
-    return (__float_as_uint(fmaf(q, 0.998046875f, 1.0f)) >> 13) & 0x3fcu;
+    return (__float_as_uint(fmaf(q, 1.0f - 0.5f / BINS, 1.0f)) >> (23 - bits - 2)) & (4u * BINS - 4u);
 }
-constexpr float kBinsPerUnit = 255.5f;  // bins per unit of q
 
 // where the want-th largest of the counted values lies
 struct BinRank {
@@ -92,13 +97,21 @@ struct BinRank {
     uint32_t above;  // values in higher bins
     uint32_t count;  // values in the bin
 };
+template <int BINS>
 __device__ __forceinline__ BinRank scan_bins(const uint32_t *hist, uint32_t want) {
+    constexpr int N = BINS / 32;  // bins of a lane
     const int lane = threadIdx.x & 31;
-    const uint4 a = reinterpret_cast<const uint4 *>(hist)[2 * lane], b = reinterpret_cast<const uint4 *>(hist)[2 * lane + 1];
-    const uint32_t h[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-    uint32_t tot = 0;
+    uint32_t h[N], tot = 0;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) tot += h[i];
+    for (int i = 0; i < N / 4; ++i) {
+        const uint4 q = reinterpret_cast<const uint4 *>(hist)[N / 4 * lane + i];
+        h[4 * i] = q.x;
+        h[4 * i + 1] = q.y;
+        h[4 * i + 2] = q.z;
+        h[4 * i + 3] = q.w;
+    }
+#pragma unroll
+    for (int i = 0; i < N; ++i) tot += h[i];
     uint32_t suf = tot;  // values in this lane's bins and those of higher lanes
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -110,9 +123,9 @@ __device__ __forceinline__ BinRank scan_bins(const uint32_t *hist, uint32_t want
     uint32_t gt = suf - tot, bin = 0, above = 0, cnt = 0;
     const bool here = gt < want && want <= suf;
 #pragma unroll
-    for (int i = 7; i >= 0; --i) {
+    for (int i = N - 1; i >= 0; --i) {
         if (gt < want && want <= gt + h[i]) {
-            bin = (uint32_t)(lane * 8 + i);
+            bin = (uint32_t)(lane * N + i);
             above = gt;
             cnt = h[i];
         }
@@ -139,15 +152,16 @@ __device__ __noinline__ void search_whole_range(const float *g, int F, int K, ui
     uint32_t base = 0u, want = (uint32_t)K;
     for (int shift = 24; shift >= 0; shift -= 8) {
         sync();
-        for (int i = tid; i < kBins; i += TT) hist[i] = 0u;
+        for (int i = tid; i < 256; i += TT) hist[i] = 0u;
         sync();
         const uint32_t limit = shift == 24 ? 0xffffffffu : (1u << (shift + 8)) - 1u;
+#pragma unroll 8
         for (int c = tid; c < F; c += TT) {
-            const uint32_t d = gate_key(g[c]) - base;
+            const uint32_t d = gate_key(__ldg(g + c)) - base;
             if (d <= limit) atomicAdd(&hist[d >> shift], 1u);
         }
         sync();
-        const BinRank k = scan_bins(hist, want);
+        const BinRank k = scan_bins<256>(hist, want);
         base += k.bin << shift;
         want -= k.above;
     }
@@ -156,9 +170,10 @@ __device__ __noinline__ void search_whole_range(const float *g, int F, int K, ui
     // group of its W-th of the row: first it counts, then it writes behind what the warps before it count.
     const int groups = (F + 31) >> 5, g0 = groups * w / W, g1 = groups * (w + 1) / W;
     uint32_t n_gt = 0, n_eq = 0;
+#pragma unroll 4
     for (int v = g0; v < g1; ++v) {
         const int c = v * 32 + lane;
-        const uint32_t key = c < F ? gate_key(g[c]) : 0u;
+        const uint32_t key = c < F ? gate_key(__ldg(g + c)) : 0u;
         n_gt += (uint32_t)__popc(__ballot_sync(0xffffffffu, c < F && key > base));
         n_eq += (uint32_t)__popc(__ballot_sync(0xffffffffu, c < F && key == base));
     }
@@ -173,9 +188,10 @@ __device__ __noinline__ void search_whole_range(const float *g, int F, int K, ui
         eq += xw[W + i];
     }
     const uint32_t lt = (1u << lane) - 1u;
+#pragma unroll 4
     for (int v = g0; v < g1; ++v) {
         const int c = v * 32 + lane;
-        const float x = c < F ? g[c] : 0.f;
+        const float x = c < F ? __ldg(g + c) : 0.f;
         const uint32_t key = c < F ? gate_key(x) : 0u;
         const bool is_gt = c < F && key > base, is_eq = c < F && key == base;
         const uint32_t bg = __ballot_sync(0xffffffffu, is_gt), be = __ballot_sync(0xffffffffu, is_eq);
@@ -185,7 +201,7 @@ __device__ __noinline__ void search_whole_range(const float *g, int F, int K, ui
         eq += (uint32_t)__popc(be);
     }
     sync();
-    for (int i = tid; i < kBins; i += TT) hist[i] = 0u;
+    for (int i = tid; i < bins(W); i += TT) hist[i] = 0u;
     sync();
 }
 
@@ -196,6 +212,7 @@ __global__ void __launch_bounds__(32 * W, ctas_per_sm(W, VPL)) select_rows_reg_k
     using namespace tc;
     extern __shared__ __align__(16) uint8_t smem[];
     constexpr int TT = 32 * W;         // threads of the team (= of the CTA)
+    constexpr int BINS = bins(W);
     constexpr int GPW = VPL / 4;       // 128-channel groups per warp: lane l of a group holds channels 4 l .. 4 l + 3
     constexpr int NP = (GPW + 3) / 4;  // words of packed per-group counts
     const Layout L = layout(W, ldu, K);
@@ -218,7 +235,7 @@ __global__ void __launch_bounds__(32 * W, ctas_per_sm(W, VPL)) select_rows_reg_k
     };
     const uint32_t u_bytes = (uint32_t)ldu * 2u;
     auto clear_hist = [&]() {
-        for (int i = tid; i < kBins / 4; i += TT) reinterpret_cast<uint4 *>(hist)[i] = make_uint4(0, 0, 0, 0);
+        for (int i = tid; i < BINS / 4; i += TT) reinterpret_cast<uint4 *>(hist)[i] = make_uint4(0, 0, 0, 0);
     };
     float x[VPL];
     // the sample: a quad per lane, spread over the row (every warp of the team reads the same 128 values)
@@ -275,7 +292,8 @@ __global__ void __launch_bounds__(32 * W, ctas_per_sm(W, VPL)) select_rows_reg_k
         const float mean = warp_sum(sample.x + sample.y + sample.z + sample.w) * (1.0f / 128.0f);
         const float mad = warp_sum(fabsf(sample.x - mean) + fabsf(sample.y - mean) + fabsf(sample.z - mean) + fabsf(sample.w - mean)) *
                           (1.0f / 128.0f);
-        const bool window = sampled && mad > 1e-30f && mad < 1e30f && fabsf(mean) < 1e5f * mad;
+        // (with the mean within 128 deviations, the roundings of the bins' edges stay below a hundredth of a bin)
+        const bool window = sampled && mad > 1e-30f && mad < 1e30f && fabsf(mean) < 128.f * mad;
         const float lo = fmaf(mad, 1.2533f * quantile - kWindowMad, mean);  // sigma of normal values = 1.2533 mad
         const float scale = window ? 0.5f / (kWindowMad * mad) : 0.f, offset = -lo * scale;
         // ---- 1. histogram
@@ -285,11 +303,11 @@ __global__ void __launch_bounds__(32 * W, ctas_per_sm(W, VPL)) select_rows_reg_k
         if (window) {
 #pragma unroll
             for (int i = 0; i < VPL; ++i)
-                asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(hist_at + bin4(x[i], scale, offset)) : "memory");
+                asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(hist_at + bin4<BINS>(x[i], scale, offset)) : "memory");
             sync();
-            b = scan_bins(hist, (uint32_t)K);
-            fast = b.bin >= 1u && b.bin <= 254u && b.count <= kMaxRanked - 4u;
-            const float width = 2.f * kWindowMad * mad * (1.f / kBinsPerUnit);
+            b = scan_bins<BINS>(hist, (uint32_t)K);
+            fast = b.bin >= 1u && b.bin < BINS - 1u && b.count <= kMaxRanked - 4u;
+            const float width = 2.f * kWindowMad * mad / (BINS - 0.5f);
             from = fmaf((float)b.bin - 0.05f, width, lo);   // a little below and above the bin: rounding decides into which
             below = fmaf((float)b.bin + 1.05f, width, lo);  // bin a value at its edge falls
         }
