@@ -721,7 +721,7 @@ int forward_tc(const moc_ffn_desc &d, const __nv_bfloat16 *x, const __nv_bfloat1
     }
     Params p;
     init_params(p);
-    if (!map_k_major(&p.b_map[0], wg, F, dm, dm, b_box_rows()) || !map_k_major(&p.b_map[1], wu, F, dm, dm, b_box_rows()))
+    if (!map_b_k_major(p, 0, wg, F, dm, dm) || !map_b_k_major(p, 1, wu, F, dm, dm))
         return MOC_ERR_CUDA;
     p.status = status;
     p.num_problems = 2;
@@ -786,7 +786,7 @@ int backward_tc(const moc_ffn_desc &d, const __nv_bfloat16 *x, const __nv_bfloat
     {
         Params p;
         init_params(p);
-        if (!map_k_major(&p.a_map[0], dout, T, dm, dm, BM) || !map_k_major(&p.b_map[0], wd, F, dm, dm, b_box_rows()))
+        if (!map_k_major(&p.a_map[0], dout, T, dm, dm, BM) || !map_b_k_major(p, 0, wd, F, dm, dm))
             return MOC_ERR_CUDA;
         p.k_blocks = ceil_div(dm, BK);
         p.M = (int)T;
@@ -848,8 +848,6 @@ int backward_tc(const moc_ffn_desc &d, const __nv_bfloat16 *x, const __nv_bfloat
         p.m_tiles = ceil_div(d.d_ff_ld, BM);
         p.n_tiles = ceil_div(dm, BN);
         p.accumulate = (d.flags & MOC_FLAG_ACCUMULATE_WGRAD) ? 1 : 0;
-        // long contraction, few tiles: the finer tile granularity of single CTAs fills the last wave better
-        p.single_cta = 1;
         static const bool problem_major = [] {
             const char *e = getenv("MOC_FFN_WGRAD_ORDER");  // "m": the m-block-major order (comparisons)
             return !(e && strcmp(e, "m") == 0);
@@ -1861,7 +1859,7 @@ int moc_ffn_recompute_up(const moc_ffn_desc *desc, const void *x, const void *w_
         B16 *U = reinterpret_cast<B16 *>(static_cast<char *>(workspace) + L.off_z);
         Params p;
         init_params(p);
-        if (!map_k_major(&p.a_map[0], x, T, dm, dm, BM) || !map_k_major(&p.b_map[0], w_up, F, dm, dm, b_box_rows()))
+        if (!map_k_major(&p.a_map[0], x, T, dm, dm, BM) || !map_b_k_major(p, 0, w_up, F, dm, dm))
             return MOC_ERR_CUDA;
         p.k_blocks = ceil_div(dm, BK);
         p.M = (int)T;
@@ -2074,7 +2072,7 @@ int moc_tc_gemm_bf16(int64_t m, int64_t n, int64_t k, const void *a, int a_mn_ma
     Params p;
     init_params(p);
     const bool ok_a = a_mn_major ? map_mn_major(&p.a_map[0], a, k, m, lda) : map_k_major(&p.a_map[0], a, m, k, lda, BM);
-    const bool ok_b = b_mn_major ? map_mn_major(&p.b_map[0], b, k, n, ldb) : map_k_major(&p.b_map[0], b, n, k, ldb, b_box_rows());
+    const bool ok_b = b_mn_major ? map_mn_major(&p.b_map[0], b, k, n, ldb) : map_b_k_major(p, 0, b, n, k, ldb);
     if (!ok_a || !ok_b) return MOC_ERR_CUDA;
     p.k_blocks = ceil_div(k, BK);
     p.M = (int)m;

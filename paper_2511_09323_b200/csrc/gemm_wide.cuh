@@ -1,0 +1,502 @@
+// The dense bf16 GEMM of the tensor-core plan: CTA pairs on tiles of 256 rows and up to 512 columns.
+//
+// What bounds it: a pair's MMA (cta_group::2, M = 256) works 2 cycles per column and 64-element contraction block; the two
+// CTAs' operands have to arrive from L2 meanwhile.  On 256 x 256 tiles those are 32 KiB per CTA and block of 512 cycles,
+// 64 bytes a cycle, and the SMs together get some 58 (measured with the MMAs left out: 550 to 615 cycles a block; the kernel
+// of such tiles that this one replaced needed 700, 65536 x 2048 x 11008 in 2.13 ms; now 1.90).  Twice the columns per tile share the rows' half of that: 48 KiB per 1024 cycles.  The tile then fills
+// tensor memory (two accumulators of 256 columns), so nothing is left to work in while the epilogue drains it; instead the
+// two accumulators run a few blocks apart: the first is ahead at both ends of the contraction, so that its epilogue overlaps
+// the second's last blocks and its next tile starts while the second is being drained.
+//
+// The tiles need not have one width.  With few tiles, or a last wave that few of them fill, the remaining rows (or columns)
+// are cut into narrower ones, in steps of 64 columns, so that all pairs finish together: plan_tiles() below chooses.
+//
+// Roles: warp 0 TMA loads, warp 1 MMAs (leading CTA) and the TMEM allocation, warps 2..9 epilogue, two per TMEM lane quarter.
+// Barriers as in the pair kernel of tc_gemm.cuh.
+#pragma once
+
+#include <algorithm>
+#include <mutex>
+#include <unordered_map>
+
+#include "tc_gemm.cuh"
+
+namespace moc {
+namespace tc {
+
+constexpr int WIDE_N = 512, WIDE_STEP = 64, WIDE_SKEW = 2;
+constexpr int WIDE_THREADS = 320, WIDE_EPI_WARPS = 8, WIDE_STAGES_MAX = 6;
+constexpr uint32_t WIDE_B_BYTES = (BN / 2) * BK * 2;  // one accumulator's half of B in a stage, at most
+constexpr uint32_t WIDE_RING_BYTES = 192 * 1024;      // 4 stages of A | B | B, or 6 of A | B where no tile is wider than 256
+constexpr size_t WIDE_SMEM_BYTES = 1024 + WIDE_RING_BYTES + BAR_REGION_BYTES + WIDE_EPI_WARPS * EPI_BOX_BYTES;
+
+// How the output is cut.  Rows: 256-row blocks of all problems.  The first `t1` tiles are 512 columns wide, the others w2.
+//   by_columns == 0: rows one after the other, their tiles from left to right; the first `split` rows have wide tiles
+//   by_columns == 1: column by column, all rows in turn (few rows and a large B: B is read once); the first `split` columns
+//                    have wide tiles
+struct TilePlan {
+    int rows, by_columns, split, nt1, w2, nt2, t1, total;
+};
+
+struct WideParams {
+    Params g;
+    CUtensorMap b_rem[3];  // K-major B: boxes for the accumulator of fewer than 256 columns of the narrower tiles
+    TilePlan t;
+    int m_blocks;          // 256-row blocks of one problem
+    int stages;
+    uint32_t stage_bytes;
+};
+
+// one tile
+struct WideTile {
+    int m_blk, prob, n0;
+    int s0, s1;           // columns of the two accumulators (multiples of 64; s1 may be 0)
+    uint32_t box0, box1;  // K-major B: rows of the boxes loaded for them (the box of a clipped tile keeps its height)
+};
+__device__ __forceinline__ WideTile wide_tile(const WideParams &p, int tile) {
+    WideTile t;
+    int row, w;
+    const bool first = tile < p.t.t1;
+    const int i = first ? tile : tile - p.t.t1;
+    w = first ? WIDE_N : p.t.w2;
+    if (p.t.by_columns) {
+        const int c = i / p.t.rows;
+        row = i - c * p.t.rows;
+        t.n0 = (first ? 0 : p.t.split) + c * w;
+    } else {
+        const int nt = first ? p.t.nt1 : p.t.nt2, r = i / nt;
+        row = r + (first ? 0 : p.t.split);
+        t.n0 = (i - r * nt) * w;
+    }
+    if (p.g.problem_major) {
+        t.prob = row / p.m_blocks;
+        t.m_blk = row - t.prob * p.m_blocks;
+    } else {
+        t.m_blk = row / p.g.num_problems;
+        t.prob = row - t.m_blk * p.g.num_problems;
+    }
+    const int valid = min(w, (p.g.N - t.n0 + WIDE_STEP - 1) / WIDE_STEP * WIDE_STEP);
+    t.s0 = min(valid, BN);
+    t.s1 = valid - t.s0;
+    const int full0 = min(w, BN);
+    t.box0 = (uint32_t)full0 / 2;
+    t.box1 = (uint32_t)(w - full0) / 2;
+    return t;
+}
+
+// One warp's share of an accumulator of `cols` columns: every other 128-byte chunk (`half` says which) of its 32 rows.
+template <int EPI>
+__device__ __forceinline__ void wide_epilogue(const Params &p, int prob, int row0, int n0, int cols, int half, uint32_t taddr,
+                                              uint32_t box) {
+    const int lane = threadIdx.x & 31, row = row0 + lane;
+    const bool f32_out = EPI == EPI_F32 || (EPI == EPI_GATE_UP && prob == 0);
+    cols = min(cols, p.N - n0);
+    if (row0 >= p.M) return;
+    if (p.direct_store != 0 || (EPI == EPI_BF16 && p.accumulate)) {
+        // every thread stores its own row (outputs a tensor map cannot describe, accumulation)
+#pragma unroll 1
+        for (int c0 = 32 * half; c0 < cols; c0 += 64) {
+            uint32_t r[32];
+            __syncwarp();
+            tmem_ld32(taddr + (uint32_t)c0, r);
+            tmem_ld_wait();
+            const int valid = cols - c0;
+            if (row >= p.M) continue;
+            if (f32_out) {
+                store_row_f32(static_cast<float *>(p.c[prob]) + (int64_t)row * p.ldc[prob] + n0 + c0, r, valid);
+            } else {
+                __nv_bfloat16 *dst = static_cast<__nv_bfloat16 *>(p.c[prob]) + (int64_t)row * p.ldc[prob] + n0 + c0;
+                float v[32];
+#pragma unroll
+                for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+                if (EPI == EPI_BF16 && p.accumulate) {
+#pragma unroll
+                    for (int i = 0; i < 32; ++i)
+                        if (i < valid) v[i] += __bfloat162float(dst[i]);
+                }
+                store_row_bf16(dst, v, valid);
+            }
+        }
+        return;
+    }
+    // A chunk of 32 rows x 128 bytes goes through the warp's box in shared memory (16-byte pieces XOR-swizzled, free of bank
+    // conflicts both ways) and leaves as ordinary 16-byte stores, eight lanes to a row.  (Bulk tensor stores queue behind the
+    // loads in flight: some 3000 cycles until such a store has read its box, which the accumulator waits for.)
+    const uint32_t sw = (uint32_t)(lane & 7), my_row = box + (uint32_t)lane * 128u;
+    const int step = f32_out ? 32 : 64, esz = f32_out ? 4 : 2, per_piece = 16 / esz;
+    const int r_sub = lane >> 3, piece = lane & 7;
+    uint8_t *const out0 = static_cast<uint8_t *>(p.c[prob]) + ((int64_t)(row0 + r_sub) * p.ldc[prob] + n0 + piece * per_piece) * esz;
+    const int64_t pitch4 = (int64_t)p.ldc[prob] * esz * 4;
+    const int rows_left = p.M - row0 - r_sub;
+#pragma unroll 1
+    for (int c0 = step * half; c0 < cols; c0 += 2 * step) {
+        uint32_t r[32];
+        __syncwarp();
+        tmem_ld32(taddr + (uint32_t)c0, r);
+        if (f32_out) {
+            tmem_ld_wait();
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                st_shared_v4(my_row + (((uint32_t)i ^ sw) << 4), r[4 * i], r[4 * i + 1], r[4 * i + 2], r[4 * i + 3]);
+        } else {
+            uint32_t q[32];
+            tmem_ld32(taddr + (uint32_t)c0 + 32u, q);
+            tmem_ld_wait();
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                st_shared_v4(my_row + (((uint32_t)i ^ sw) << 4), pack_bf16(__uint_as_float(r[8 * i]), __uint_as_float(r[8 * i + 1])),
+                             pack_bf16(__uint_as_float(r[8 * i + 2]), __uint_as_float(r[8 * i + 3])),
+                             pack_bf16(__uint_as_float(r[8 * i + 4]), __uint_as_float(r[8 * i + 5])),
+                             pack_bf16(__uint_as_float(r[8 * i + 6]), __uint_as_float(r[8 * i + 7])));
+                st_shared_v4(my_row + (((uint32_t)(i + 4) ^ sw) << 4), pack_bf16(__uint_as_float(q[8 * i]), __uint_as_float(q[8 * i + 1])),
+                             pack_bf16(__uint_as_float(q[8 * i + 2]), __uint_as_float(q[8 * i + 3])),
+                             pack_bf16(__uint_as_float(q[8 * i + 4]), __uint_as_float(q[8 * i + 5])),
+                             pack_bf16(__uint_as_float(q[8 * i + 6]), __uint_as_float(q[8 * i + 7])));
+            }
+        }
+        __syncwarp();
+        const int left = cols - c0 - piece * per_piece;  // columns from this lane's piece on
+        uint8_t *dst = out0 + (int64_t)c0 * esz;
+#pragma unroll
+        for (int i = 0; i < 8; ++i, dst += pitch4) {
+            const uint32_t rr = (uint32_t)(4 * i + r_sub);
+            const uint4 v = ld_shared_v4(box + rr * 128u + (((uint32_t)piece ^ (rr & 7u)) << 4));
+            if (4 * i >= rows_left) continue;
+            if (left >= per_piece) {
+                *reinterpret_cast<uint4 *>(dst) = v;
+            } else if (left > 0) {
+                const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    if (e >= left) break;
+                    if (f32_out) {
+                        if (e < 4) reinterpret_cast<uint32_t *>(dst)[e] = w[e];
+                    } else {
+                        reinterpret_cast<uint16_t *>(dst)[e] = (uint16_t)(w[e >> 1] >> (16 * (e & 1)));
+                    }
+                }
+            }
+        }
+    }
+}
+
+template <bool A_MN, bool B_MN, int EPI>
+__global__ void __launch_bounds__(WIDE_THREADS, 1) gemm_wide_kernel(const __grid_constant__ WideParams p) {
+    extern __shared__ uint8_t smem_raw[];
+    const uint32_t raw = smem_u32(smem_raw);
+    const uint32_t base = (raw + 1023u) & ~1023u;  // 128-byte swizzle atoms need 1024-byte alignment
+    uint8_t *smem = smem_raw + (base - raw);
+    const uint32_t bar_base = base + WIDE_RING_BYTES;
+    const uint32_t epi_base = bar_base + BAR_REGION_BYTES;
+    auto full_bar = [&](int s) { return bar_base + 8u * s; };
+    auto empty_bar = [&](int s) { return bar_base + 8u * (WIDE_STAGES_MAX + s); };
+    auto tfull_bar = [&](uint32_t a) { return bar_base + 8u * (2 * WIDE_STAGES_MAX + a); };
+    auto tempty_bar = [&](uint32_t a) { return bar_base + 8u * (2 * WIDE_STAGES_MAX + ACC_STAGES + a); };
+    volatile uint32_t *tmem_holder =
+        reinterpret_cast<volatile uint32_t *>(smem + WIDE_RING_BYTES + 8 * (2 * WIDE_STAGES_MAX + 2 * ACC_STAGES));
+    volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_holder + 1);
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t rank = cluster_ctarank();  // 0: the pair's leading CTA
+    const int pair = blockIdx.x >> 1, num_pairs = gridDim.x >> 1;
+    const int kb_total = p.g.k_blocks * p.g.k_segments;
+    int *const status = p.g.status;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < p.stages; ++s) {
+            mbar_init(full_bar(s), 1);
+            mbar_init(empty_bar(s), 1);
+        }
+        for (uint32_t a = 0; a < ACC_STAGES; ++a) {
+            mbar_init(tfull_bar(a), 1);
+            mbar_init(tempty_bar(a), 2 * WIDE_EPI_WARPS);  // one arrival per epilogue warp of the pair
+        }
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    if (warp == 1) {
+        tmem_alloc_pair(smem_u32(const_cast<uint32_t *>(tmem_holder)), TMEM_COLS);
+        tmem_relinquish_pair();
+    }
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync_all();  // the partner's barriers exist before anything signals them
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_holder;
+
+    if (warp == 0) {
+        // ------------------------------------------------------------------ TMA producer (one per CTA).  One thread's
+        // instructions per block have to stay well below a block's MMAs: everything that a tile fixes is worked out ahead.
+        if (lane == 0) {
+            for (int i = 0; i < 3; ++i) {
+                prefetch_tmap(&p.g.a_map[i]);
+                prefetch_tmap(&p.g.b_map[i]);
+            }
+            const uint32_t lead_bars = map_to_cta(bar_base, 0), ring_end = base + (uint32_t)p.stages * p.stage_bytes;
+            uint32_t sa = base, bar = 0, phase = 0;  // stage: its A operand, its barriers' offset
+            bool ok = true;
+            for (int tile = pair; tile < p.t.total && ok; tile += num_pairs) {
+                const WideTile t = wide_tile(p, tile);
+                const int m0 = t.m_blk * (2 * BM) + (int)rank * BM;  // this CTA's rows of A
+                const int h0 = t.s0 / 2, h1 = t.s1 / 2;              // its share of the accumulators' columns of B
+                const int nb0 = t.n0 + (int)rank * h0, nb1 = t.n0 + BN + (int)rank * h1;
+                const bool two0 = h0 > 64, any1 = h1 > 0, two1 = h1 > 64;  // MN-major B: boxes of 64 columns
+                const uint32_t b_bytes = B_MN ? (uint32_t)(1 + (two0 ? 1 : 0) + (any1 ? 1 : 0) + (two1 ? 1 : 0)) * 8192u
+                                              : (t.box0 + (any1 ? t.box1 : 0u)) * (uint32_t)(BK * 2);
+                const uint32_t tx = 2 * (A_STAGE_BYTES + b_bytes);
+                for (int seg = 0; seg < p.g.k_segments && ok; ++seg) {
+                    const CUtensorMap *am = &p.g.a_map[p.g.a_idx[t.prob][seg]];
+                    const int bi = p.g.b_idx[t.prob][seg];
+                    const CUtensorMap *bm0 = !B_MN && t.box0 < BN / 2 ? &p.b_rem[bi] : &p.g.b_map[bi];
+                    const CUtensorMap *bm1 = !B_MN && t.box1 < BN / 2 ? &p.b_rem[bi] : &p.g.b_map[bi];
+                    const int k_end = p.g.k_blocks * BK;
+                    for (int kk = 0; kk < k_end; kk += BK) {
+                        if (!mbar_wait(bar_base + bar + 8u * WIDE_STAGES_MAX, phase ^ 1u, abort_flag, status)) {
+                            ok = false;
+                            break;
+                        }
+                        const uint32_t full = lead_bars + bar, sb = sa + A_STAGE_BYTES;
+                        if (rank == 0) mbar_expect_tx(bar_base + bar, tx);
+                        if (A_MN) {
+                            tma_load_2d_pair(sa, am, full, m0, kk);
+                            tma_load_2d_pair(sa + 64 * BK * 2, am, full, m0 + 64, kk);
+                        } else {
+                            tma_load_2d_pair(sa, am, full, kk, m0);
+                        }
+                        if (B_MN) {
+                            tma_load_2d_pair(sb, bm0, full, nb0, kk);
+                            if (two0) tma_load_2d_pair(sb + 64 * BK * 2, bm0, full, nb0 + 64, kk);
+                            if (any1) tma_load_2d_pair(sb + WIDE_B_BYTES, bm1, full, nb1, kk);
+                            if (two1) tma_load_2d_pair(sb + WIDE_B_BYTES + 64 * BK * 2, bm1, full, nb1 + 64, kk);
+                        } else {
+                            tma_load_2d_pair(sb, bm0, full, kk, nb0);
+                            if (any1) tma_load_2d_pair(sb + WIDE_B_BYTES, bm1, full, kk, nb1);
+                        }
+                        bar += 8u;
+                        sa += p.stage_bytes;
+                        if (sa == ring_end) {
+                            sa = base;
+                            bar = 0;
+                            phase ^= 1u;
+                        }
+                    }
+                }
+            }
+        }
+    } else if (warp == 1) {
+        // ------------------------------------------------------------------ MMA issuer (leading CTA only)
+        if (lane == 0 && rank == 0) {
+            // one instruction consumes 16 contraction elements: 32 bytes along a K-major row, or 16 rows of 128 bytes in
+            // an MN-major box (descriptor addresses are in units of 16 bytes)
+            constexpr uint32_t a_step = A_MN ? 128u : 2u, b_step = B_MN ? 128u : 2u;
+            constexpr uint32_t idesc0 = make_idesc<A_MN, B_MN, 2 * BM>() & ~(0x3fu << 17);
+            const uint64_t a_desc = make_smem_desc(base, A_MN ? BK * 128 : 16, 1024);
+            const uint64_t b_desc = make_smem_desc(base + A_STAGE_BYTES, B_MN ? BK * 128 : 16, 1024);
+            const uint32_t hi = (uint32_t)(a_desc >> 32), a_lo = (uint32_t)a_desc, b_lo = (uint32_t)b_desc;
+            // a stage: its barriers' offset, its operands' offset in the descriptors' units, the barriers' phase
+            struct Cursor {
+                uint32_t bar, off, phase;
+            } at = {0, 0, 0};
+            const uint32_t off_step = p.stage_bytes >> 4, off_end = (uint32_t)p.stages * off_step;
+            auto next = [&](Cursor &c) {
+                c.bar += 8u;
+                c.off += off_step;
+                if (c.off == off_end) {
+                    c.bar = c.off = 0;
+                    c.phase ^= 1u;
+                }
+            };
+            auto arrived = [&](const Cursor &c) {
+                if (!mbar_wait(bar_base + c.bar, c.phase, abort_flag, status)) return false;
+                tc_fence_after();
+                return true;
+            };
+            auto release = [&](const Cursor &c) { umma_commit_pair(bar_base + c.bar + 8u * WIDE_STAGES_MAX); };  // in both CTAs
+            auto mma = [&](const Cursor &c, uint32_t j, uint32_t d, uint32_t idesc, bool first) {
+                const uint32_t a = a_lo + c.off, b = b_lo + c.off + j * (WIDE_B_BYTES >> 4);
+                umma_bf16_pair_lohi(d, a, b, hi, idesc, first ? 0u : 1u);
+#pragma unroll
+                for (uint32_t k = 1; k < BK / 16; ++k) umma_bf16_pair_lohi(d, a + k * a_step, b + k * b_step, hi, idesc, 1u);
+            };
+            uint32_t used = 0;  // accumulators handed out so far: they alternate
+            bool ok = true;
+            for (int tile = pair; tile < p.t.total && ok; tile += num_pairs) {
+                const WideTile t = wide_tile(p, tile);
+                const uint32_t r0 = used & 1u, r1 = r0 ^ 1u;
+                const uint32_t id0 = idesc0 | ((uint32_t)(t.s0 >> 3) << 17), id1 = idesc0 | ((uint32_t)(t.s1 >> 3) << 17);
+                const uint32_t d0 = tmem_base + r0 * BN, d1 = tmem_base + r1 * BN;
+                if (!mbar_wait(tempty_bar(r0), ((used >> 1) & 1u) ^ 1u, abort_flag, status)) break;
+                tc_fence_after();
+                if (t.s1 == 0) {
+                    for (int kb = 0; kb < kb_total && ok; ++kb) {
+                        if (!(ok = arrived(at))) break;
+                        mma(at, 0, d0, id0, kb == 0);
+                        release(at);
+                        next(at);
+                    }
+                    if (!ok) break;
+                    umma_commit_pair(tfull_bar(r0));  // accumulator complete, in both CTAs
+                    ++used;
+                    continue;
+                }
+                const int skew = min(WIDE_SKEW, kb_total / 2);
+                // `skew` blocks of one accumulator, then the same blocks of the other; the stages go back with the second
+                auto first_pass = [&](bool begin) {
+                    Cursor c = at;
+                    for (int i = 0; i < skew && ok; ++i) {
+                        if (!(ok = arrived(c))) break;
+                        mma(c, 0, d0, id0, begin && i == 0);
+                        next(c);
+                    }
+                };
+                auto second_pass = [&](bool begin) {
+                    for (int i = 0; i < skew; ++i) {
+                        mma(at, 1, d1, id1, begin && i == 0);
+                        release(at);
+                        next(at);
+                    }
+                };
+                first_pass(true);
+                if (!ok || !(ok = mbar_wait(tempty_bar(r1), (((used + 1) >> 1) & 1u) ^ 1u, abort_flag, status))) break;
+                tc_fence_after();
+                if (skew > 0) second_pass(true);
+                for (int kb = skew; kb < kb_total - skew; ++kb) {
+                    if (!(ok = arrived(at))) break;
+                    mma(at, 0, d0, id0, kb == 0);
+                    mma(at, 1, d1, id1, kb == 0);
+                    release(at);
+                    next(at);
+                }
+                if (!ok) break;
+                first_pass(false);
+                if (!ok) break;
+                umma_commit_pair(tfull_bar(r0));
+                second_pass(false);
+                umma_commit_pair(tfull_bar(r1));
+                used += 2;
+            }
+        }
+    } else {
+        // ------------------------------------------------------------------ epilogue (warps 2..9 of each CTA)
+        const int quarter = warp & 3, half = (warp - 2) >> 2;
+        uint32_t used = 0;
+        bool ok = true;
+        for (int tile = pair; tile < p.t.total && ok; tile += num_pairs) {
+            const WideTile t = wide_tile(p, tile);
+#pragma unroll 1
+            for (int j = 0; j < (t.s1 ? 2 : 1); ++j, ++used) {
+                const uint32_t r = used & 1u;
+                ok = __all_sync(0xffffffffu, mbar_wait(tfull_bar(r), (used >> 1) & 1u, abort_flag, status));
+                if (!ok) break;
+                tc_fence_after();
+                wide_epilogue<EPI>(p.g, t.prob, t.m_blk * (2 * BM) + (int)rank * BM + quarter * 32, t.n0 + j * BN, j ? t.s1 : t.s0, half,
+                                   tmem_base + ((uint32_t)(quarter * 32) << 16) + r * BN, epi_base + (uint32_t)(warp - 2) * EPI_BOX_BYTES);
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive_cluster(map_to_cta(tempty_bar(r), 0));
+            }
+        }
+    }
+
+    // ---------------------------------------------------------------------- teardown
+    __syncwarp();
+    if (*abort_flag) {
+        const long long t0 = clock64();
+        while (clock64() - t0 < 2000000LL) __nanosleep(1000);
+    }
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync_all();  // neither CTA leaves while the partner may still read its shared memory or signal it
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc_pair(tmem_base, TMEM_COLS);
+    }
+}
+
+// SM cycles a pair needs for one contraction block of a tile of w columns: its MMAs, or the loads at what an SM gets from L2
+inline double wide_block_cycles(int w) { return std::max(2.06 * w, (16384.0 + 64.0 * w) / 58.0); }
+
+// Cycles in which the epilogue moves an accumulator of 256 columns (bf16, fp32 outputs).
+constexpr int WIDE_DRAIN_BF16 = 2000, WIDE_DRAIN_F32 = 3500;
+
+// Tiles of `rows` x N for `pairs` CTA pairs: wide ones for as many whole waves as there are (or one fewer), the rest in the
+// one width that finishes first; or that width throughout.  (Measured at d_model 2048, d_ff 5504: down projection of 1111
+// tokens, 40 tiles of 256 columns for 74 pairs, 36.8 us; 55 of 192.)  Remembered per problem size.
+// drain: cycles in which the epilogue moves an accumulator of 256 columns.  Of a tile with two accumulators the part of it
+// that the skew does not cover is lost; with one, the other is worked in meanwhile.
+inline TilePlan plan_tiles(int rows, int N, int kb, int pairs, bool by_columns, int drain) {
+    struct Key {
+        int rows, n, kb, pairs, by_columns, drain;
+        bool operator==(const Key &o) const {
+            return rows == o.rows && n == o.n && kb == o.kb && pairs == o.pairs && by_columns == o.by_columns && drain == o.drain;
+        }
+    };
+    struct Hash {
+        size_t operator()(const Key &k) const {
+            uint64_t h = 0x9e3779b97f4a7c15ull;
+            for (const int v : {k.rows, k.n, k.kb, k.pairs, k.by_columns, k.drain}) h = (h ^ (uint64_t)(uint32_t)v) * 0xff51afd7ed558ccdull;
+            return (size_t)(h ^ (h >> 32));
+        }
+    };
+    static std::mutex mu;
+    static std::unordered_map<Key, TilePlan, Hash> known;
+    const Key key{rows, N, kb, pairs, by_columns ? 1 : 0, drain};
+    {
+        std::lock_guard<std::mutex> lock(mu);
+        auto it = known.find(key);
+        if (it != known.end()) return it->second;
+    }
+    const auto tile_cycles = [&](int w) {
+        const double mma = kb * wide_block_cycles(w) + 350.0;
+        return w > BN ? mma + std::max(0, drain - WIDE_SKEW * 512) : std::max(mma, drain * w / 256.0);
+    };
+    const auto up = [](int64_t a, int64_t b) { return (int)((a + b - 1) / b); };
+    const int nt1 = up(N, WIDE_N);
+    TilePlan best{};
+    double best_cycles = 0.0;
+    const auto consider = [&](int split, int w2) {
+        TilePlan t{};
+        t.rows = rows;
+        t.by_columns = by_columns ? 1 : 0;
+        t.split = split;
+        t.nt1 = nt1;
+        t.w2 = w2;
+        if (by_columns) {
+            t.t1 = split / WIDE_N * rows;
+            t.nt2 = split < N ? up(N - split, w2) : 0;
+            t.total = t.t1 + t.nt2 * rows;
+        } else {
+            t.t1 = split * nt1;
+            t.nt2 = up(N, w2);
+            t.total = t.t1 + (rows - split) * t.nt2;
+        }
+        // tiles go round the pairs in turn: pair j has every pairs-th one from j on
+        double worst = 0.0;
+        for (int j = 0; j < pairs; ++j) {
+            const int n1 = t.t1 > j ? (t.t1 - 1 - j) / pairs + 1 : 0, n = t.total > j ? (t.total - 1 - j) / pairs + 1 : 0;
+            worst = std::max(worst, n1 * tile_cycles(WIDE_N) + (n - n1) * tile_cycles(w2));
+        }
+        if (best.total == 0 || worst < best_cycles) {
+            best = t;
+            best_cycles = worst;
+        }
+    };
+    const int units = by_columns ? N / WIDE_N : rows;              // what is split off as wide: columns' tiles or rows
+    const int per_unit = by_columns ? rows : nt1;                  // tiles of one
+    const int waves = (int)((int64_t)units * per_unit / pairs);
+    for (int w2 = WIDE_N; w2 >= WIDE_STEP; w2 -= WIDE_STEP) {
+        consider(0, w2);
+        for (int f = waves; f >= std::max(1, waves - 1); --f) {
+            const int u = std::min<int64_t>(units, (int64_t)f * pairs / per_unit);
+            for (int v = u; v >= std::max(1, u - 1); --v) consider(by_columns ? v * WIDE_N : v, w2);
+        }
+    }
+    std::lock_guard<std::mutex> lock(mu);
+    if (known.size() > 512) known.clear();
+    known[key] = best;
+    return best;
+}
+
+}  // namespace tc
+}  // namespace moc

@@ -1,11 +1,11 @@
 // bf16 tensor-core GEMM for sm_100a: tcgen05.mma with TMEM accumulators, TMA-fed operands.
 //
-// One persistent CTA per SM (192 threads): warp 0 issues TMA loads, warp 1 issues tcgen05.mma and
-// owns the TMEM allocation, warps 2..5 run the epilogue (TMEM -> swizzled shared-memory boxes -> bulk
-// tensor stores).  Two forms: gemm_kernel, one CTA per 128 x 256 output tile (K step 64, four 48 KiB
-// shared-memory stages), and gemm_pair_kernel, clusters of two CTAs sharing one cta_group::2 MMA on a
-// 256 x 256 tile (six 32 KiB stages per CTA).  Both keep two accumulator stages in TMEM (2 x 256
-// columns) so that the epilogue of tile i overlaps the main loop of tile i+1.
+// What the GEMM kernels share, and two of them.  gemm_wide.cuh holds the one that the plan's contractions run on.
+// Persistent CTAs: warp 0 issues TMA loads, warp 1 issues tcgen05.mma and owns the TMEM allocation, the other warps run
+// the epilogue.  gemm_kernel: one CTA per 128 x 256 output tile (K step 64, four 48 KiB shared-memory stages), for devices
+// or processes without CTA pairs.  gemm_pair_kernel: clusters of two CTAs sharing one cta_group::2 MMA on 256 rows x 128
+// channels of W_gate and W_up, with the MoC 2:8 mask in its epilogue (six 32 KiB stages per CTA).  Both keep two
+// accumulator stages in TMEM (2 x 256 columns) so that the epilogue of tile i overlaps the main loop of tile i+1.
 //
 // Operands may be K-major (rows of 64 contraction elements = one 128-byte swizzle row) or MN-major
 // (the tensor's contiguous dimension is M or N; loaded as 64-wide boxes of 64 contraction rows).
@@ -33,7 +33,7 @@ namespace tc {
 constexpr int BM = 128, BN = 256, BK = 64, STAGES = 4, ACC_STAGES = 2;
 constexpr int THREADS = 192;
 // the fused 2-of-8 epilogue is arithmetic-heavy: two epilogue warps per TMEM lane quarter there
-constexpr int pair_threads(int epi) { return epi == 3 ? 320 : THREADS; }
+constexpr int PAIR_THREADS = 320;
 constexpr uint32_t A_STAGE_BYTES = BM * BK * 2, B_STAGE_BYTES = BN * BK * 2;
 constexpr uint32_t STAGE_BYTES = A_STAGE_BYTES + B_STAGE_BYTES;
 constexpr uint32_t TMEM_COLS = ACC_STAGES * BN;  // 512
@@ -70,7 +70,6 @@ struct Params {
     int ldc[3];
     CUtensorMap c_map[3];  // per problem: [M, N] with 32-row boxes of 128 bytes (32 fp32 or 64 bf16 columns)
     int direct_store;      // 1: the output cannot be described by a tensor map; threads store their rows
-    int single_cta;        // 1: one CTA per tile even where CTA pairs are available (set by the caller)
     // Tile order.  0: (m block, problem, n block) -- tiles of one m block are adjacent, right when the problems share A
     // (gate | up).  1: (problem, m block, n block) -- a wave of CTAs works on ONE problem, right when the problems have
     // different operands on both sides (the three weight gradients: a wave then streams one B matrix instead of two).
@@ -86,6 +85,11 @@ struct Params {
     uint32_t *zmeta;
     int zmeta_stages;
     int *status;
+    // host only: the K-major B operands behind b_map (rows, contraction length, leading dimension), for boxes of other heights
+    struct BOperand {
+        const void *ptr;
+        int64_t n, k, ld;
+    } b_op[3];
 };
 
 // ---------------------------------------------------------------------------------------------- PTX
@@ -169,6 +173,11 @@ __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.a
 __device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
     asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
+__device__ __forceinline__ uint4 ld_shared_v4(uint32_t addr) {
+    uint4 v;
+    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
+    return v;
+}
 __device__ __forceinline__ void prefetch_tmap(const CUtensorMap *map) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
 }
@@ -236,13 +245,15 @@ __device__ __forceinline__ void tmem_relinquish_pair() {
 __device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t cols) {
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(cols) : "memory");
 }
-__device__ __forceinline__ void umma_bf16_pair(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                               uint32_t accumulate) {
+// The descriptors are given by their low words (address and leading-dimension fields) and the high word both
+// share: the issuing thread advances an operand with one addition.
+__device__ __forceinline__ void umma_bf16_pair_lohi(uint32_t tmem_d, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t idesc,
+                                                    uint32_t accumulate) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\tmov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
+        "setp.ne.b32 p, %5, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %4, p;\n\t}"
+        ::"r"(tmem_d), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate)
         : "memory");
 }
 // arrives (once the MMAs issued so far have completed) on the barrier at this shared-memory offset in both CTAs
@@ -785,11 +796,10 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const __grid_constant_
 
 
 // ---------------------------------------------------------------------------------------------- pair kernel
-// The same GEMM with the CTAs working in pairs (clusters of two, `cta_group::2`): a pair owns a 256 x 256 output
-// tile; each CTA stages its own 128 rows of A and HALF of the B tile (128 of the 256 columns), and one
-// `tcgen05.mma.cta_group::2` issued by the pair's leading CTA multiplies both A halves with both B halves, each
-// CTA's TMEM receiving its 128 rows.  Per CTA and k-block that is 32 KiB of operands instead of 48 KiB: a third
-// less traffic from L2 and a six-deep ring in the same shared memory.
+// EPI_GATE_UP_2OF8 with the CTAs working in pairs (clusters of two, `cta_group::2`): a pair owns 256 rows x 128 channels;
+// each CTA stages its own 128 rows of A and the channels' rows of one weight matrix (the first W_gate, the second W_up),
+// and one `tcgen05.mma.cta_group::2` issued by the pair's leading CTA multiplies both A halves with both B halves, each
+// CTA's TMEM receiving its 128 rows.
 //   full[s]   (leader's)  : counts the bytes both CTAs' loads bring in for stage s
 //   empty[s]  (each CTA's): the leader's commit arrives on it in both CTAs when the MMAs have read stage s
 //   tfull[a]  (each CTA's): ... when accumulator a is complete
@@ -798,8 +808,7 @@ constexpr int PAIR_STAGES = 6;
 constexpr uint32_t PAIR_B_STAGE_BYTES = (BN / 2) * BK * 2, PAIR_STAGE_BYTES = A_STAGE_BYTES + PAIR_B_STAGE_BYTES;
 static_assert(PAIR_STAGES * PAIR_STAGE_BYTES == STAGES * STAGE_BYTES, "both kernels use the same shared-memory layout");
 
-template <bool A_MN, bool B_MN, int EPI>
-__global__ void __launch_bounds__(pair_threads(EPI), 1) gemm_pair_kernel(const __grid_constant__ Params p) {
+__global__ void __launch_bounds__(PAIR_THREADS, 1) gemm_pair_kernel(const __grid_constant__ Params p) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;  // 128-byte swizzle atoms need 1024-byte alignment
@@ -818,8 +827,8 @@ __global__ void __launch_bounds__(pair_threads(EPI), 1) gemm_pair_kernel(const _
     const uint32_t rank = cluster_ctarank();  // 0: the pair's leading CTA
     const int pair = blockIdx.x >> 1, num_pairs = gridDim.x >> 1;
     const int m_pairs = (p.m_tiles + 1) >> 1;  // 256-row blocks
-    const int total_tiles = m_pairs * p.n_tiles * p.num_problems;
-    const int kb_total = p.k_blocks * p.k_segments;
+    const int total_tiles = m_pairs * p.n_tiles;
+    const int kb_total = p.k_blocks;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < PAIR_STAGES; ++s) {
@@ -828,7 +837,7 @@ __global__ void __launch_bounds__(pair_threads(EPI), 1) gemm_pair_kernel(const _
         }
         for (int a = 0; a < ACC_STAGES; ++a) {
             mbar_init(tfull_bar(a), 1);
-            mbar_init(tempty_bar(a), 2 * (pair_threads(EPI) / 32 - 2));  // one arrival per epilogue warp of the pair
+            mbar_init(tempty_bar(a), 2 * (PAIR_THREADS / 32 - 2));  // one arrival per epilogue warp of the pair
         }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -844,55 +853,36 @@ __global__ void __launch_bounds__(pair_threads(EPI), 1) gemm_pair_kernel(const _
     tc_fence_after();
     const uint32_t tmem_base = *tmem_holder;
 
-    auto decode_tile = [&](int tile, int &m_blk, int &prob, int &n_blk) {
-        const int per_m = p.num_problems * p.n_tiles;
-        m_blk = tile / per_m;
-        const int r = tile - m_blk * per_m;
-        prob = r / p.n_tiles;
-        n_blk = r - prob * p.n_tiles;
+    auto decode_tile = [&](int tile, int &m_blk, int &n_blk) {
+        m_blk = tile / p.n_tiles;
+        n_blk = tile - m_blk * p.n_tiles;
     };
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer (one per CTA)
         if (lane == 0) {
-            for (int i = 0; i < 3; ++i) {
-                prefetch_tmap(&p.a_map[i]);
-                prefetch_tmap(&p.b_map[i]);
-            }
+            const CUtensorMap *const am = &p.a_map[0], *const bm = &p.b_map[rank];
+            prefetch_tmap(am);
+            prefetch_tmap(bm);
+            const uint32_t lead_bars = map_to_cta(bar_base, 0);
             int stage = 0;
             uint32_t phase = 0;
             bool ok = true;
             for (int tile = pair; tile < total_tiles && ok; tile += num_pairs) {
-                int m_blk, prob, n_blk;
-                decode_tile(tile, m_blk, prob, n_blk);
+                int m_blk, n_blk;
+                decode_tile(tile, m_blk, n_blk);
                 const int m0 = m_blk * (2 * BM) + (int)rank * BM;          // this CTA's rows of A
-                // this CTA's half of the B tile (EPI_GATE_UP_2OF8: the same channels of its own weight matrix)
-                const int nb0 = EPI == EPI_GATE_UP_2OF8 ? n_blk * (BN / 2) : n_blk * BN + (int)rank * (BN / 2);
+                const int nb0 = n_blk * (BN / 2);                          // the channels, of its own weight matrix
                 for (int kb = 0; kb < kb_total; ++kb) {
                     if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, p.status)) {
                         ok = false;
                         break;
                     }
-                    const int seg = kb / p.k_blocks, kk = (kb - seg * p.k_blocks) * BK;
-                    const CUtensorMap *am = &p.a_map[p.a_idx[prob][seg]];
-                    const CUtensorMap *bm = &p.b_map[EPI == EPI_GATE_UP_2OF8 ? (int)rank : p.b_idx[prob][seg]];
                     const uint32_t sa = base + stage * PAIR_STAGE_BYTES, sb = sa + A_STAGE_BYTES;
-                    const uint32_t lead_full = map_to_cta(full_bar(stage), 0);
+                    const uint32_t lead_full = lead_bars + 8u * (uint32_t)stage;
                     if (rank == 0) mbar_expect_tx(full_bar(stage), 2 * PAIR_STAGE_BYTES);
-                    if (A_MN) {
-#pragma unroll
-                        for (int i = 0; i < BM / 64; ++i)
-                            tma_load_2d_pair(sa + i * (64 * BK * 2), am, lead_full, m0 + i * 64, kk);
-                    } else {
-                        tma_load_2d_pair(sa, am, lead_full, kk, m0);
-                    }
-                    if (B_MN) {
-#pragma unroll
-                        for (int i = 0; i < BN / 128; ++i)
-                            tma_load_2d_pair(sb + i * (64 * BK * 2), bm, lead_full, nb0 + i * 64, kk);
-                    } else {
-                        tma_load_2d_pair(sb, bm, lead_full, kk, nb0);
-                    }
+                    tma_load_2d_pair(sa, am, lead_full, kb * BK, m0);
+                    tma_load_2d_pair(sb, bm, lead_full, kb * BK, nb0);
                     if (++stage == PAIR_STAGES) {
                         stage = 0;
                         phase ^= 1u;
@@ -903,7 +893,9 @@ __global__ void __launch_bounds__(pair_threads(EPI), 1) gemm_pair_kernel(const _
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer (leading CTA only)
         if (lane == 0 && rank == 0) {
-            constexpr uint32_t idesc = make_idesc<A_MN, B_MN, 2 * BM>();
+            constexpr uint32_t idesc = make_idesc<false, false, 2 * BM>();
+            const uint64_t a_desc = make_smem_desc(base, 16, 1024), b_desc = make_smem_desc(base + A_STAGE_BYTES, 16, 1024);
+            const uint32_t hi = (uint32_t)(a_desc >> 32), a_lo0 = (uint32_t)a_desc, b_lo0 = (uint32_t)b_desc;
             int stage = 0, acc = 0;
             uint32_t phase = 0, acc_phase = 0;
             bool ok = true;
@@ -917,15 +909,10 @@ __global__ void __launch_bounds__(pair_threads(EPI), 1) gemm_pair_kernel(const _
                         break;
                     }
                     tc_fence_after();
-                    const uint32_t sa = base + stage * PAIR_STAGE_BYTES, sb = sa + A_STAGE_BYTES;
+                    const uint32_t off = (uint32_t)stage * (PAIR_STAGE_BYTES >> 4), a_lo = a_lo0 + off, b_lo = b_lo0 + off;
 #pragma unroll
-                    for (int k = 0; k < BK / 16; ++k) {
-                        const uint64_t ad = A_MN ? make_smem_desc(sa + k * 2048, BK * 128, 1024)
-                                                 : make_smem_desc(sa + k * 32, 16, 1024);
-                        const uint64_t bd = B_MN ? make_smem_desc(sb + k * 2048, BK * 128, 1024)
-                                                 : make_smem_desc(sb + k * 32, 16, 1024);
-                        umma_bf16_pair(tmem_d, ad, bd, idesc, (kb | k) != 0 ? 1u : 0u);
-                    }
+                    for (uint32_t k = 0; k < BK / 16; ++k)
+                        umma_bf16_pair_lohi(tmem_d, a_lo + 2u * k, b_lo + 2u * k, hi, idesc, kb != 0 || k != 0 ? 1u : 0u);
                     umma_commit_pair(empty_bar(stage));  // frees the stage in both CTAs
                     if (++stage == PAIR_STAGES) {
                         stage = 0;
@@ -943,21 +930,16 @@ __global__ void __launch_bounds__(pair_threads(EPI), 1) gemm_pair_kernel(const _
     } else {
         // ------------------------------------------------------------------ epilogue (warps 2..5 of each CTA)
         const int quarter = warp & 3;
-        int acc = 0, ebuf = 0;
+        int acc = 0;
         uint32_t acc_phase = 0;
         for (int tile = pair; tile < total_tiles; tile += num_pairs) {
-            int m_blk, prob, n_blk;
-            decode_tile(tile, m_blk, prob, n_blk);
+            int m_blk, n_blk;
+            decode_tile(tile, m_blk, n_blk);
             if (!__all_sync(0xffffffffu, mbar_wait(tfull_bar(acc), acc_phase, abort_flag, p.status))) break;
             tc_fence_after();
-            if (EPI == EPI_GATE_UP_2OF8)
-                epilogue_tile_2of8(p, m_blk * (2 * BM) + (int)rank * BM + quarter * 32, n_blk * (BN / 2), (warp - 2) >> 2,
-                                   tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)acc * BN,
-                                   epi_base + (uint32_t)(warp - 2) * EPI_BOX_BYTES);
-            else
-                epilogue_tile<EPI>(p, prob, m_blk * (2 * BM) + (int)rank * BM + quarter * 32, n_blk * BN,
-                                   tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)acc * BN,
-                                   epi_base + (uint32_t)quarter * EPI_BUFS * EPI_BOX_BYTES, ebuf);
+            epilogue_tile_2of8(p, m_blk * (2 * BM) + (int)rank * BM + quarter * 32, n_blk * (BN / 2), (warp - 2) >> 2,
+                               tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)acc * BN,
+                               epi_base + (uint32_t)(warp - 2) * EPI_BOX_BYTES);
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive_cluster(map_to_cta(tempty_bar(acc), 0));

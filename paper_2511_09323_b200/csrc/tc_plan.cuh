@@ -14,6 +14,7 @@
 #include <cstring>
 #include <cuda_runtime.h>
 
+#include "gemm_wide.cuh"
 #include "moc_common.cuh"
 #include "tc_gemm.cuh"
 #include "topk_select.cuh"
@@ -74,7 +75,7 @@ inline bool map_mn_major(CUtensorMap *m, const void *ptr, int64_t k, int64_t mn,
     return make_map(m, ptr, k, mn, ld, 64, BK);
 }
 
-// CTA pairs (clusters of two, one MMA across both) are the default; MOC_FFN_GEMM=single in the environment selects
+// CTA pairs (clusters of two, one MMA across both; gemm_wide.cuh) are the default; MOC_FFN_GEMM=single in the environment selects
 // the one-CTA kernel (kept for comparison and for devices that refuse the cluster launch).
 inline bool pair_mode() {
     static int mode = -1;
@@ -84,8 +85,13 @@ inline bool pair_mode() {
     }
     return mode == 1;
 }
-// rows of a K-major B box: a CTA of a pair stages half of the 256 B rows of a tile
+// rows of a K-major B box: a CTA of a pair stages half of the 256 B rows of an accumulator
 inline int b_box_rows() { return pair_mode() ? BN / 2 : BN; }
+// K-major B operand i of a launch
+inline bool map_b_k_major(Params &p, int i, const void *ptr, int64_t n, int64_t k, int64_t ld) {
+    p.b_op[i] = {ptr, n, k, ld};
+    return map_k_major(&p.b_map[i], ptr, n, k, ld, b_box_rows());
+}
 
 inline int sm_count() {
     static int n = 0;
@@ -103,12 +109,15 @@ inline void init_params(Params &p) {
     p.k_segments = 1;
 }
 
+// every row of an output begins on a 16-byte boundary
+inline bool aligned_rows(const void *ptr, int64_t ld, bool f32) {
+    return (reinterpret_cast<uintptr_t>(ptr) & 15u) == 0 && ((size_t)ld * (f32 ? 4 : 2)) % 16 == 0;
+}
 // Output [rows, cols] with leading dimension ld as 32-row boxes of 128 bytes.  False when the tensor-map rules
 // (16-byte aligned base and row pitch) do not hold.
 inline bool make_out_map(CUtensorMap *m, void *ptr, int64_t rows, int64_t cols, int64_t ld, bool f32) {
     const size_t esz = f32 ? 4 : 2;
-    if ((reinterpret_cast<uintptr_t>(ptr) & 15u) || ((size_t)ld * esz) % 16 != 0 || rows <= 0 || cols <= 0)
-        return false;
+    if (!aligned_rows(ptr, ld, f32) || rows <= 0 || cols <= 0) return false;
     cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
     cuuint64_t strides[1] = {(cuuint64_t)ld * esz};
     cuuint32_t box[2] = {(cuuint32_t)(128 / esz), 32};
@@ -118,54 +127,97 @@ inline bool make_out_map(CUtensorMap *m, void *ptr, int64_t rows, int64_t cols, 
                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
 }
 
+// one launch of CTA pairs
+template <typename Kernel, typename Prm>
+inline int launch_pairs(Kernel kern, const Prm &p, int pairs, int threads, size_t smem, cudaStream_t st) {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.gridDim = dim3(2 * (unsigned)pairs);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, p) == cudaSuccess ? MOC_OK : MOC_ERR_CUDA;
+}
+// pairs that can be resident at once (0: none, or an error)
+template <typename Kernel>
+inline int resident_pairs(Kernel kern, int threads, size_t smem, int &cached) {
+    if (cached) return cached;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.gridDim = dim3(2 * (unsigned)sm_count());
+    cfg.dynamicSmemBytes = smem;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n <= 0) return 0;
+    return cached = n;
+}
+
 template <bool A_MN, bool B_MN, int EPI>
 inline int launch_gemm(const Params &p_in, cudaStream_t st) {
     Params p = p_in;
+    if (p.M <= 0 || p.N <= 0) return MOC_OK;
     p.direct_store = 0;
+    const bool wide = EPI != EPI_GATE_UP_2OF8 && pair_mode();
     for (int i = 0; i < p.num_problems && !p.direct_store; ++i) {
         const bool f32 = EPI == EPI_F32 || (EPI == EPI_GATE_UP && i == 0);
-        if (!make_out_map(&p.c_map[i], p.c[i], p.M, p.N, p.ldc[i], f32)) p.direct_store = 1;
+        if (wide ? !aligned_rows(p.c[i], p.ldc[i], f32) : !make_out_map(&p.c_map[i], p.c[i], p.M, p.N, p.ldc[i], f32)) p.direct_store = 1;
     }
-    if (pair_mode() && !(p.single_cta && A_MN && B_MN)) {  // K-major B boxes are sized for the mode: no choice there
-        auto kern = gemm_pair_kernel<A_MN, B_MN, EPI>;
-        cudaLaunchConfig_t cfg = {};
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = 2;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        cfg.blockDim = dim3(pair_threads(EPI));
-        cfg.dynamicSmemBytes = SMEM_BYTES;
-        cfg.stream = st;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        static int max_pairs = 0;  // pairs that can be resident at once
-        if (!max_pairs) {
+    if constexpr (EPI == EPI_GATE_UP_2OF8) {
+        static int max_pairs = 0;
+        if (!resident_pairs(gemm_pair_kernel, PAIR_THREADS, SMEM_BYTES, max_pairs)) return MOC_ERR_CUDA;
+        return launch_pairs(gemm_pair_kernel, p, std::min(((p.m_tiles + 1) / 2) * p.n_tiles, max_pairs), PAIR_THREADS, SMEM_BYTES, st);
+    } else if (pair_mode()) {
+        static int max_pairs = 0;
+        const auto kern = gemm_wide_kernel<A_MN, B_MN, EPI>;
+        if (!resident_pairs(kern, WIDE_THREADS, WIDE_SMEM_BYTES, max_pairs)) return MOC_ERR_CUDA;
+        WideParams w;
+        memset(&w, 0, sizeof(w));
+        w.g = p;
+        w.m_blocks = (p.m_tiles + 1) / 2;
+        // Few rows and a B that does not stay in L2: all rows of a column of tiles in turn, so that B is read once (2048
+        // tokens, gate and up projection of the 4096 x 11008 layer: 301 us row by row).
+        const int kb = p.k_blocks * p.k_segments;
+        int n_b = 1, n_a = 1;
+        for (int i = 1; i < p.num_problems; ++i) {
+            n_b += p.b_idx[i][0] != p.b_idx[0][0] ? 1 : 0;
+            n_a += p.a_idx[i][0] != p.a_idx[0][0] ? 1 : 0;
+        }
+        const double block_bytes = (double)kb * BK * 2, b_bytes = block_bytes * p.N * n_b, a_bytes = block_bytes * p.M * n_a;
+        const bool by_columns = b_bytes > 64e6 && a_bytes < 0.5 * b_bytes;
+        w.t = plan_tiles(w.m_blocks * p.num_problems, p.N, kb, max_pairs, by_columns, EPI == EPI_BF16 ? WIDE_DRAIN_BF16 : WIDE_DRAIN_F32);
+        const int widest = w.t.t1 ? WIDE_N : w.t.w2;
+        w.stage_bytes = A_STAGE_BYTES + (widest > BN ? 2 : 1) * WIDE_B_BYTES;
+        w.stages = (int)(WIDE_RING_BYTES / w.stage_bytes);
+        const int rem = w.t.w2 > BN ? w.t.w2 - BN : w.t.w2;  // columns of the narrower tiles' smaller accumulator
+        if (!B_MN && rem < BN && w.t.total > w.t.t1)
+            for (int i = 0; i < 3; ++i)
+                if (p.b_op[i].ptr && !map_k_major(&w.b_rem[i], p.b_op[i].ptr, p.b_op[i].n, p.b_op[i].k, p.b_op[i].ld, rem / 2)) return MOC_ERR_CUDA;
+        return launch_pairs(kern, w, std::min(w.t.total, max_pairs), WIDE_THREADS, WIDE_SMEM_BYTES, st);
+    } else {
+        const auto kern = gemm_kernel<A_MN, B_MN, EPI>;
+        static bool configured = false;
+        if (!configured) {
             if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES) != cudaSuccess)
                 return MOC_ERR_CUDA;
-            cfg.gridDim = dim3(2 * (unsigned)sm_count());
-            int n = 0;
-            if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n <= 0) return MOC_ERR_CUDA;
-            max_pairs = n;
+            configured = true;
         }
-        const int tiles = ((p.m_tiles + 1) / 2) * p.n_tiles * p.num_problems;
-        const int pairs = tiles < max_pairs ? tiles : max_pairs;
-        if (pairs <= 0) return MOC_OK;
-        cfg.gridDim = dim3(2 * (unsigned)pairs);
-        return cudaLaunchKernelEx(&cfg, kern, p) == cudaSuccess ? MOC_OK : MOC_ERR_CUDA;
+        const int tiles = p.m_tiles * p.n_tiles * p.num_problems;
+        kern<<<std::min(tiles, sm_count()), THREADS, SMEM_BYTES, st>>>(p);
+        return cudaGetLastError() == cudaSuccess ? MOC_OK : MOC_ERR_CUDA;
     }
-    auto kern = gemm_kernel<A_MN, B_MN, EPI>;
-    static bool configured = false;
-    if (!configured) {
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES) != cudaSuccess)
-            return MOC_ERR_CUDA;
-        configured = true;
-    }
-    const int tiles = p.m_tiles * p.n_tiles * p.num_problems;
-    const int grid = tiles < sm_count() ? tiles : sm_count();
-    if (grid <= 0) return MOC_OK;
-    kern<<<grid, THREADS, SMEM_BYTES, st>>>(p);
-    return cudaGetLastError() == cudaSuccess ? MOC_OK : MOC_ERR_CUDA;
 }
 
 // ------------------------------------------------------------------------------------------------
