@@ -816,168 +816,6 @@ __global__ void __launch_bounds__(256) backward_sample_rows_kernel(
 }
 
 // ------------------------------------------------------------------------------------------------
-// The same step with ONE WARP per token and the rows staged in the warp's slice of shared memory: the dZ
-// row arrives by a bulk copy (the next token's row is already in flight while this one is worked on), the
-// three masked rows are built in shared memory and leave as bulk stores.  Global traffic is fully
-// coalesced and the scattered accesses stay on chip.  Used when the four rows of a token fit a slice.
-__host__ __device__ constexpr size_t sample_warp_words(int ld, int K) {
-    return (size_t)2 * ld /* four bf16 rows */ + (size_t)2 * ((K + 1) & ~1) /* entries */ +
-           (size_t)3 * ((K + 7) & ~7) /* saved idx, g, u of two tokens */ + 4 /* two mbarriers */ + 4 /* verdicts */;
-}
-constexpr int kSampleMaxWarps = 10;
-
-// W warps work on a token (W = 1 or 2: with two, the token's rows occupy the slice for about half as long and the
-// same shared memory feeds twice the warps); they meet at a named barrier of their own between the phases.
-template <int W>
-__global__ void __launch_bounds__(kSampleMaxWarps * 32) backward_sample_rows_warp_kernel(
-    const int16_t *__restrict__ idx, const __nv_bfloat16 *__restrict__ gval, const __nv_bfloat16 *__restrict__ uval,
-    int64_t T, int K, int F, int ld, __nv_bfloat16 *__restrict__ dz_z, __nv_bfloat16 *__restrict__ du,
-    __nv_bfloat16 *__restrict__ dg, int *__restrict__ status) {
-    extern __shared__ __align__(128) uint32_t sample_warp_smem[];
-    __shared__ int s_abort;
-    constexpr int TT = 32 * W;  // threads of a team
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, wpc = blockDim.x / TT;  // teams per CTA
-    const int team = wib / W, pl = ((wib % W) << 5) | lane;                            // pl: thread index within the team
-    auto team_sync = [&]() {
-        if (W == 1) __syncwarp();
-        else asm volatile("bar.sync %0, %1;" ::"r"(team + 1), "n"(TT) : "memory");
-    };
-    uint32_t *base = sample_warp_smem + (size_t)team * sample_warp_words(ld, K);
-    const int row_words = ld >> 1;  // ld is a multiple of 8: rows are multiples of 16 bytes
-    __nv_bfloat16 *zbuf0 = reinterpret_cast<__nv_bfloat16 *>(base);  // two dZ rows, used alternately
-    __nv_bfloat16 *ubuf = reinterpret_cast<__nv_bfloat16 *>(base + 2 * row_words);
-    __nv_bfloat16 *gbuf = reinterpret_cast<__nv_bfloat16 *>(base + 3 * row_words);
-    uint32_t *entry = base + 4 * row_words;  // K x {j | z << 16, dU | dG << 16}
-    // saved idx | g | u rows of the two tokens in flight, K8 16-bit entries each (arrive with the dZ row when K is a
-    // multiple of 8, i.e. when the rows are 16-byte multiples; plain loads otherwise)
-    const int K8 = (K + 7) & ~7;
-    uint16_t *saved0 = reinterpret_cast<uint16_t *>(entry + 2 * ((K + 1) & ~1));
-    const bool staged_saved = (K & 7) == 0;
-    uint64_t *bar_mem = reinterpret_cast<uint64_t *>(saved0 + 6 * K8);
-    const uint32_t bar0 = smem_u32(bar_mem);  // two mbarriers, 8 bytes apart
-    const uint32_t row_bytes = (uint32_t)ld * 2u, saved_bytes = (uint32_t)K * 2u;
-    const int64_t gw = (int64_t)blockIdx.x * wpc + team, nw = (int64_t)gridDim.x * wpc;
-
-    if (threadIdx.x == 0) s_abort = 0;
-    if (pl == 0) {
-        mbar_init(bar0, 1);
-        mbar_init(bar0 + 8u, 1);
-    }
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    __syncthreads();
-    uint32_t phases = 0;  // bit b: parity to wait for on barrier b
-    auto request = [&](int64_t tok, int buf) {  // lane 0: dZ row (+ saved rows) of a token into buffer `buf`
-        const uint32_t nbar = bar0 + 8u * (uint32_t)buf;
-        mbar_expect_tx(nbar, row_bytes + (staged_saved ? 3u * saved_bytes : 0u));
-        bulk_copy_g2s(smem_u32(zbuf0 + (size_t)buf * ld), dz_z + tok * (int64_t)ld, row_bytes, nbar);
-        if (staged_saved) {
-            uint16_t *sv = saved0 + (size_t)buf * 3 * K8;
-            bulk_copy_g2s(smem_u32(sv), idx + tok * K, saved_bytes, nbar);
-            bulk_copy_g2s(smem_u32(sv + K8), gval + tok * K, saved_bytes, nbar);
-            bulk_copy_g2s(smem_u32(sv + 2 * K8), uval + tok * K, saved_bytes, nbar);
-        }
-    };
-    if (pl == 0 && gw < T) request(gw, 0);
-    int b = 0;
-    for (int64_t t = gw; t < T; t += nw, b ^= 1) {
-        // a wait that gave up ends the team: the warps exchange their verdicts so that all of them leave together
-        const bool ok = __all_sync(0xffffffffu, mbar_wait(bar0 + 8u * (uint32_t)b, (phases >> b) & 1u, &s_abort, status));
-        if (W > 1) {
-            uint32_t *verdict = reinterpret_cast<uint32_t *>(bar_mem + 2);
-            if (lane == 0) verdict[wib % W] = ok ? 1u : 0u;
-            team_sync();
-            bool all_ok = true;
-#pragma unroll
-            for (int i = 0; i < W; ++i) all_ok = all_ok && verdict[i] != 0u;
-            if (!all_ok) break;
-        } else if (!ok) {
-            break;
-        }
-        phases ^= 1u << b;
-        __nv_bfloat16 *zr = zbuf0 + (size_t)b * ld;
-        const uint16_t *sv = saved0 + (size_t)b * 3 * K8;
-        for (int k0 = 0; k0 < K; k0 += 8 * TT) {
-            // eight saved entries per lane, their loads issued together
-            int jv[8];
-            __nv_bfloat16 gb[8], ub[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int k = k0 + i * TT + pl;
-                jv[i] = -1;
-                if (k < K) {
-                    if (staged_saved) {
-                        jv[i] = (int16_t)sv[k];
-                        gb[i] = *reinterpret_cast<const __nv_bfloat16 *>(sv + K8 + k);
-                        ub[i] = *reinterpret_cast<const __nv_bfloat16 *>(sv + 2 * K8 + k);
-                    } else {
-                        jv[i] = idx[t * K + k];
-                        gb[i] = gval[t * K + k];
-                        ub[i] = uval[t * K + k];
-                    }
-                }
-            }
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int k = k0 + i * TT + pl;
-                if (k >= K) continue;
-                const int j = jv[i];
-                uint32_t w0 = 0xffffu, w1 = 0;  // j = 0xffff marks a skipped entry
-                if (j >= 0 && j < F) {
-                    const float dz = __bfloat162float(zr[j]);
-                    const float g = __bfloat162float(gb[i]);
-                    const float u = __bfloat162float(ub[i]);
-                    const float s = silu_f(g);
-                    const __nv_bfloat16 zb = __float2bfloat16_rn(s * u);
-                    w0 = (uint32_t)j | ((uint32_t)(*reinterpret_cast<const uint16_t *>(&zb)) << 16);
-                    w1 = pack_bf16(s * dz, u * dz * dsilu_f(g));
-                } else {
-                    raise_status(status, MOC_ERR_BAD_INDEX);
-                }
-                entry[2 * k] = w0;
-                entry[2 * k + 1] = w1;
-            }
-        }
-        // by now the stores of the previous token have read their rows: the other dZ buffer (next token's row goes
-        // there) and the dU / dG rows are free
-        team_sync();  // every thread has sampled the dZ row
-        if (pl == 0) {
-            bulk_store_wait_read<0>();
-            fence_async_smem();
-            if (t + nw < T) request(t + nw, b ^ 1);
-        }
-        team_sync();
-        {
-            uint4 *z16 = reinterpret_cast<uint4 *>(zr), *u16 = reinterpret_cast<uint4 *>(ubuf),
-                  *g16 = reinterpret_cast<uint4 *>(gbuf);
-            const uint4 zero = make_uint4(0, 0, 0, 0);
-            for (int v = pl; v < (ld >> 3); v += TT) {
-                z16[v] = zero;
-                u16[v] = zero;
-                g16[v] = zero;
-            }
-        }
-        team_sync();
-        for (int k = pl; k < K; k += TT) {
-            const uint32_t w0 = entry[2 * k], w1 = entry[2 * k + 1];
-            const uint32_t j = w0 & 0xffffu;
-            if (j == 0xffffu) continue;
-            const uint16_t zb = (uint16_t)(w0 >> 16), ub = (uint16_t)(w1 & 0xffffu), gb = (uint16_t)(w1 >> 16);
-            zr[j] = *reinterpret_cast<const __nv_bfloat16 *>(&zb);
-            ubuf[j] = *reinterpret_cast<const __nv_bfloat16 *>(&ub);
-            gbuf[j] = *reinterpret_cast<const __nv_bfloat16 *>(&gb);
-        }
-        fence_async_smem();
-        team_sync();
-        if (pl == 0) {
-            bulk_copy_s2g(dz_z + t * (int64_t)ld, smem_u32(zr), row_bytes);
-            bulk_copy_s2g(du + t * (int64_t)ld, smem_u32(ubuf), row_bytes);
-            bulk_copy_s2g(dg + t * (int64_t)ld, smem_u32(gbuf), row_bytes);
-        }
-    }
-    if (pl == 0) bulk_store_wait_all();
-}
-
-// ------------------------------------------------------------------------------------------------
 struct TcForwardLayout {
     int64_t chunk;  // tokens per gate/up pass
     int ldf;        // leading dimension of the dense [*, F] arrays (multiple of 8)
