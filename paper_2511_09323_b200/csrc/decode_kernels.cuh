@@ -23,6 +23,7 @@
 #pragma once
 
 #include "moc_common.cuh"
+#include "row_select.cuh"
 #include "tc_gemm.cuh"  // mbarrier helpers
 #include "topk_select.cuh"
 
@@ -33,7 +34,7 @@ namespace dec {
 
 constexpr int kSelThreads = 1024;
 constexpr int kSelListCap = 4096;   // candidate list entries (two lists)
-constexpr int kSelCached = 12;      // keys per thread held in registers by the CTA selector (rows up to 12288 channels)
+constexpr int kSelCached = 12;      // keys per thread held in registers by the search over the whole range (up to 12288 channels)
 constexpr int kSliceCols = 512;     // down projection: columns per CTA (1 KiB of a bf16 row)
 constexpr int kMaxPart = 512;       // list entries per down CTA (bound of its shared arrays)
 
@@ -406,25 +407,89 @@ __device__ __forceinline__ bool cta_stage_rows(uint64_t *bar, int *abort_flag, i
 // tau must be left out (`ties_cut`; false: the set is exactly "key >= tau").
 // g == nullptr: keys[] already holds the row's fp32 values (staged by a bulk copy) and is converted in place.
 // lists0: two candidate lists of kSelListCap entries; sm: the full radix select's state (its arrays double as scratch).
-// kreg: the calling thread's keys when the row is short enough to be held in registers (F <= kSelCached * kSelThreads;
-// element i = channel tid + i * kSelThreads, 0 beyond the row), for callers that go over the row once more.
+// keys[j] of the calling thread's channels (j = tid modulo kSelThreads) may be read at once, the others behind a barrier.
+//
+// WINDOW: one histogram over a window around the expected threshold, which a sample of the row gives as in row_select.cuh,
+// then the few keys of the threshold's bin ranked by every warp for itself; the search over the whole range remains for
+// rows whose threshold lies outside.  Its loops stay rolled: a selection kernel runs this code once per launch, so every
+// instruction is also a fetch from L2 (unrolled twelve times with the keys in registers, a row of 2048 channels took as
+// long as one of 11008).  61 tokens at 4096 x 11008: 78.3 -> 74.8 us for the layer, 3 tokens at 1024 x 2731: 26.3 -> 24.8.
+// Inside the cooperative kernel (small_batch_fused.cuh) the selector waits for its row anyway and the instructions of a
+// second search delay it: 0.9 - 1.6 us slower with the window, so it takes the search over the whole range alone.
+template <bool WINDOW>
 __device__ __forceinline__ void cta_select_threshold(const float *__restrict__ g, int F, int K, uint32_t *keys,
                                                      uint32_t *lists0, SelectSmemT<kSelThreads / 32> &sm,
-                                                     uint32_t &tau_out, int &need_out, bool &ties_cut_out,
-                                                     uint32_t (&kreg)[kSelCached]) {
+                                                     uint32_t &tau_out, int &need_out, bool &ties_cut_out) {
     __shared__ uint32_t s_min[32], s_max[32], s_pick, s_above, s_inbin, s_n;
     uint32_t *lists[2] = {lists0, lists0 + kSelListCap};
     uint32_t *hist = sm.priv;  // 2048 entries
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     constexpr int NW = kSelThreads / 32;
-
-    // ---- keys, minimum and maximum.  Rows of up to kSelCached * kSelThreads channels also stay in registers (element
-    // i of a thread is channel tid + i * kSelThreads): the first level's passes then run without loads.
     uint32_t kmin = 0xffffffffu, kmax = 0u;
-    const bool cached = F <= kSelCached * kSelThreads;
-    if (cached) {
+    uint32_t kreg[WINDOW ? 1 : kSelCached];  // element i = channel tid + i * kSelThreads, 0 beyond the row
+    const bool cached = !WINDOW && F <= kSelCached * kSelThreads;
+    if constexpr (WINDOW) {
+        constexpr int kWindowBins = 512;
+        bool window = false;
+        float scale = 0.f, offset = 0.f;
+        if (F >= 128) {
+            const float *v = (g ? g : reinterpret_cast<const float *>(keys)) + ((uint32_t)lane * (uint32_t)(F >> 2) >> 5) * 4;
+            const float a = v[0], b = v[1], c = v[2], e = v[3];
+            const float mean = warp_sum(a + b + c + e) * (1.0f / 128.0f);
+            const float mad = warp_sum(fabsf(a - mean) + fabsf(b - mean) + fabsf(c - mean) + fabsf(e - mean)) * (1.0f / 128.0f);
+            window = mad > 1e-30f && mad < 1e30f && fabsf(mean) < 128.f * mad;
+            scale = window ? __fdividef(0.5f, rs::kWindowMad * mad) : 0.f;
+            offset = -fmaf(mad, 1.2533f * rs::normal_quantile_fast(F, K) - rs::kWindowMad, mean) * scale;
+        }
+        for (int i = tid; i < 2048; i += kSelThreads) hist[i] = 0;
+        if (tid == 0) s_n = 0;
+        __syncthreads();  // the sample is read before its values become keys
+#pragma unroll 1
+        for (int j = tid; j < F; j += kSelThreads) {
+            const uint32_t key = gate_key(g ? g[j] : __uint_as_float(keys[j]));
+            keys[j] = key;
+            kmin = min(kmin, key);
+            kmax = max(kmax, key);
+            if (window) atomicAdd(&hist[rs::bin4<kWindowBins>(key_to_float(key), scale, offset) >> 2], 1u);
+        }
+        if (window) {  // (the same for the whole CTA)
+            __syncthreads();
+            if (warp == 0) {
+                const rs::BinRank r = rs::scan_bins<kWindowBins>(hist, (uint32_t)K);
+                if (lane == 0) {
+                    s_pick = r.total >= (uint32_t)K ? r.bin : 0u;
+                    s_above = r.above;
+                    s_inbin = r.count;
+                }
+            }
+            __syncthreads();
+            const uint32_t bin = s_pick, m = (uint32_t)K - s_above, count = s_inbin;
+            if (bin >= 1u && bin < kWindowBins - 1u && count <= 32u) {
+#pragma unroll 1
+                for (int j = tid; j < F; j += kSelThreads) {
+                    const uint32_t key = keys[j];
+                    if (rs::bin4<kWindowBins>(key_to_float(key), scale, offset) >> 2 == bin) lists0[atomicAdd(&s_n, 1u)] = key;
+                }
+                __syncthreads();
+                const uint32_t mine = (uint32_t)lane < count ? lists0[lane] : 0u;
+                uint32_t gt = 0, eq = 0;
+#pragma unroll 1
+                for (uint32_t i = 0; i < count; ++i) {
+                    const uint32_t o = lists0[i];
+                    gt += o > mine ? 1u : 0u;
+                    eq += o == mine ? 1u : 0u;
+                }
+                const int src = __ffs(__ballot_sync(0xffffffffu, (uint32_t)lane < count && gt < m && m <= gt + eq)) - 1;
+                tau_out = __shfl_sync(0xffffffffu, mine, src);
+                need_out = (int)(m - __shfl_sync(0xffffffffu, gt, src));
+                ties_cut_out = need_out != (int)__shfl_sync(0xffffffffu, eq, src);
+                return;
+            }
+            for (int i = tid; i < 2048; i += kSelThreads) hist[i] = 0;
+        }
+    } else if (cached) {
 #pragma unroll
-        for (int i = 0; i < kSelCached; ++i) {
+        for (int i = 0; i < (int)(sizeof(kreg) / sizeof(kreg[0])); ++i) {
             const int j = tid + i * kSelThreads;
             kreg[i] = 0u;
             if (j < F) {
@@ -443,14 +508,17 @@ __device__ __forceinline__ void cta_select_threshold(const float *__restrict__ g
             kmax = max(kmax, key);
         }
     }
+    // ---- the whole range, by its minimum and maximum
     kmin = __reduce_min_sync(0xffffffffu, kmin);
     kmax = __reduce_max_sync(0xffffffffu, kmax);
     if (lane == 0) {
         s_min[warp] = kmin;
         s_max[warp] = kmax;
     }
-    for (int i = tid; i < 2048; i += kSelThreads) hist[i] = 0;
-    if (tid == 0) s_n = 0;
+    if constexpr (!WINDOW) {
+        for (int i = tid; i < 2048; i += kSelThreads) hist[i] = 0;
+        if (tid == 0) s_n = 0;
+    }
     __syncthreads();
     kmin = s_min[lane];
     kmax = s_max[lane];
@@ -522,7 +590,7 @@ __device__ __forceinline__ void cta_select_threshold(const float *__restrict__ g
         // histogram over the candidates (hist is zero on entry)
         if (src == keys && cached) {
 #pragma unroll
-            for (int i = 0; i < kSelCached; ++i)
+            for (int i = 0; i < (int)(sizeof(kreg) / sizeof(kreg[0])); ++i)
                 if (tid + i * kSelThreads < F) atomicAdd(&hist[bin_of(kreg[i])], 1u);
         } else {
             for (uint32_t i = tid; i < lv.count; i += kSelThreads) {
@@ -589,7 +657,7 @@ __device__ __forceinline__ void cta_select_threshold(const float *__restrict__ g
         };
         if (src == keys && cached) {
 #pragma unroll
-            for (int i = 0; i < kSelCached; ++i)
+            for (int i = 0; i < (int)(sizeof(kreg) / sizeof(kreg[0])); ++i)
                 if (tid + i * kSelThreads < F) keep(kreg[i]);
         } else {
             for (uint32_t i = tid; i < lv.count; i += kSelThreads) keep(src[i]);
@@ -632,8 +700,7 @@ __global__ void __launch_bounds__(kSelThreads) select_mask_kernel(Workspace ws, 
     uint32_t tau;
     int need;
     bool ties_cut;
-    uint32_t kreg[kSelCached];
-    cta_select_threshold(nullptr, F, K, dyn, dyn + Fp, sm, tau, need, ties_cut, kreg);
+    cta_select_threshold<true>(nullptr, F, K, dyn, dyn + Fp, sm, tau, need, ties_cut);
     uint32_t *my_bits = ws.sel_bits + (int64_t)t * ws.sel_words;
     const int nch = (F + kSelThreads - 1) / kSelThreads;
     if (!ties_cut) {
@@ -670,8 +737,7 @@ __global__ void __launch_bounds__(kSelThreads) cta_select_idx_kernel(const float
     uint32_t tau;
     int need;
     bool ties_cut;
-    uint32_t kreg[kSelCached];
-    cta_select_threshold(staged ? nullptr : g, n, k, dyn, dyn + np, sm, tau, need, ties_cut, kreg);
+    cta_select_threshold<true>(staged ? nullptr : g, n, k, dyn, dyn + np, sm, tau, need, ties_cut);
     int16_t *out = idx_out + (int64_t)blockIdx.x * k;
     block_ordered_emit<kSelThreads>(dyn, n, tau, need, sm, [&](int pos, int j) { out[pos] = (int16_t)j; });
 }

@@ -436,8 +436,7 @@ __global__ void __launch_bounds__(dec::kSelThreads) sb_select_kernel(const Selec
     uint32_t tau;
     int need;
     bool ties_cut;
-    uint32_t kreg[dec::kSelCached];
-    dec::cta_select_threshold(nullptr, p.F, p.K, keys, lists, sm, tau, need, ties_cut, kreg);
+    dec::cta_select_threshold<true>(nullptr, p.F, p.K, keys, lists, sm, tau, need, ties_cut);
     if (p.kept_bits) {
         uint32_t *my_bits = p.kept_bits + (int64_t)t * p.kept_words;
         const int lane = tid & 31, warp = tid >> 5;
@@ -488,42 +487,14 @@ __global__ void __launch_bounds__(dec::kSelThreads) sb_select_kernel(const Selec
         const float uv = save ? __bfloat162float(__float2bfloat16_rn(u_row[j])) : u_row[j];
         return __float2bfloat16_rn(silu_f(key_to_float(key)) * uv);
     };
-    if (p.F <= dec::kSelCached * dec::kSelThreads) {
-        // The thread's keys are still in registers: the row is zero-filled with 16-byte stores (into the padding up
-        // to ldz as well), then every thread drops the values of its own kept channels (one in eight) into place.
-        for (int q = tid; q * 8 < p.F; q += dec::kSelThreads) *reinterpret_cast<uint4 *>(z + q * 8) = make_uint4(0u, 0u, 0u, 0u);
-        __syncthreads();
-#pragma unroll
-        for (int i = 0; i < dec::kSelCached; ++i) {
-            const int j = tid + i * dec::kSelThreads;
-            if (j < p.F) {
-                const bool kept = by_bitmap ? ((bits[j >> 5] >> (j & 31)) & 1u) != 0u : kreg[i] >= tau;
-                if (kept) z[j] = z_of(kreg[i], j);
-            }
-        }
-    } else {
-        // long rows: eight channels (one 16-byte store) per thread and step
-        for (int q = tid; q * 8 < p.F; q += dec::kSelThreads) {
-            const int j0 = q * 8;
-            uint32_t kept = 0;
-            if (by_bitmap) {
-                kept = (bits[j0 >> 5] >> (j0 & 31)) & 0xffu;
-            } else {
-#pragma unroll
-                for (int e = 0; e < 8; ++e)
-                    if (j0 + e < p.F && keys[j0 + e] >= tau) kept |= 1u << e;
-            }
-            uint32_t w[4] = {0u, 0u, 0u, 0u};
-            while (kept) {
-                const int e = __ffs(kept) - 1;
-                kept &= kept - 1u;
-                const uint32_t hbits = (uint32_t)__bfloat16_as_ushort(z_of(keys[j0 + e], j0 + e)) << (16 * (e & 1));
-#pragma unroll
-                for (int q2 = 0; q2 < 4; ++q2)
-                    if ((e >> 1) == q2) w[q2] |= hbits;
-            }
-            *reinterpret_cast<uint4 *>(z + j0) = make_uint4(w[0], w[1], w[2], w[3]);
-        }
+    // The row is zero-filled with 16-byte stores (into the padding up to ldz as well), then every thread drops the values of
+    // its own kept channels (one in eight) into place.
+    for (int q = tid; q * 8 < p.F; q += dec::kSelThreads) *reinterpret_cast<uint4 *>(z + q * 8) = make_uint4(0u, 0u, 0u, 0u);
+    __syncthreads();
+#pragma unroll 1
+    for (int j = tid; j < p.F; j += dec::kSelThreads) {
+        const bool kept = by_bitmap ? ((bits[j >> 5] >> (j & 31)) & 1u) != 0u : keys[j] >= tau;
+        if (kept) z[j] = z_of(keys[j], j);
     }
 }
 

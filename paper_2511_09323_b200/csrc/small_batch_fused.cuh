@@ -205,8 +205,7 @@ __device__ __forceinline__ void selector_role(const FusedParams &p, uint32_t *dy
     uint32_t tau;
     int need;
     bool ties_cut;
-    uint32_t kreg[dec::kSelCached];
-    dec::cta_select_threshold(nullptr, p.F, p.K, keys, lists, sm, tau, need, ties_cut, kreg);
+    dec::cta_select_threshold<false>(nullptr, p.F, p.K, keys, lists, sm, tau, need, ties_cut);
     MOC_TL_CTA(3328);
     uint32_t *my_bits = p.kept_bits + (int64_t)t * p.kept_words;
     constexpr int NW = kBlock / 32;
