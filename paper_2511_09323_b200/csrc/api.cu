@@ -592,40 +592,58 @@ int sparse_gemm_pair(int64_t M, int N, int K, int segments, const __nv_bfloat16 
     return rc;
 }
 
-// out = bf16(a + b), 8 elements per thread (the two halves of a contraction that was split, see below)
-__global__ void __launch_bounds__(256) split_sum_kernel(const float *__restrict__ a, const float *__restrict__ b,
-                                                        __nv_bfloat16 *__restrict__ out, int64_t n8) {
+// out = bf16(sum of `parts` partial outputs, n8 groups of eight elements each), 8 elements per thread
+__global__ void __launch_bounds__(256) split_sum_kernel(const float *__restrict__ partial, int parts, __nv_bfloat16 *__restrict__ out,
+                                                        int64_t n8) {
     for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n8; i += (int64_t)gridDim.x * 256) {
-        const float4 a0 = __ldcs(reinterpret_cast<const float4 *>(a) + 2 * i), a1 = __ldcs(reinterpret_cast<const float4 *>(a) + 2 * i + 1);
-        const float4 b0 = __ldcs(reinterpret_cast<const float4 *>(b) + 2 * i), b1 = __ldcs(reinterpret_cast<const float4 *>(b) + 2 * i + 1);
-        reinterpret_cast<uint4 *>(out)[i] = make_uint4(tc::pack_bf16(a0.x + b0.x, a0.y + b0.y), tc::pack_bf16(a0.z + b0.z, a0.w + b0.w),
-                                                      tc::pack_bf16(a1.x + b1.x, a1.y + b1.y), tc::pack_bf16(a1.z + b1.z, a1.w + b1.w));
+        const float4 *a = reinterpret_cast<const float4 *>(partial) + 2 * i;
+        float4 v0 = __ldcs(a), v1 = __ldcs(a + 1);
+        for (int p = 1; p < parts; ++p) {
+            a += 2 * n8;
+            const float4 b0 = __ldcs(a), b1 = __ldcs(a + 1);
+            v0 = make_float4(v0.x + b0.x, v0.y + b0.y, v0.z + b0.z, v0.w + b0.w);
+            v1 = make_float4(v1.x + b1.x, v1.y + b1.y, v1.z + b1.z, v1.w + b1.w);
+        }
+        reinterpret_cast<uint4 *>(out)[i] = make_uint4(tc::pack_bf16(v0.x, v0.y), tc::pack_bf16(v0.z, v0.w), tc::pack_bf16(v1.x, v1.y),
+                                                       tc::pack_bf16(v1.z, v1.w));
     }
 }
 
-// (see tc::split_contraction_pays) -- here with the room the caller has for the partial outputs
-bool split_contraction(int64_t T, int n_cols, size_t scratch_floats) {
-    return tc::split_contraction_pays(T, n_cols) && (size_t)2 * T * n_cols <= scratch_floats;
-}
-
-int launch_split_sum(const float *partial, int64_t T, int n_cols, __nv_bfloat16 *out, cudaStream_t st) {
+int launch_split_sum(const float *partial, int parts, int64_t T, int n_cols, __nv_bfloat16 *out, cudaStream_t st) {
     const int64_t n8 = T * n_cols / 8;
     const unsigned grid = (unsigned)std::min<int64_t>((n8 + 255) / 256, (int64_t)tc::sm_count() * 8);
-    MOC_LAUNCH(KID_TC_SPLIT_SUM, st, (split_sum_kernel<<<grid, 256, 0, st>>>(partial, partial + T * n_cols, out, n8)));
+    MOC_LAUNCH(KID_TC_SPLIT_SUM, st, (split_sum_kernel<<<grid, 256, 0, st>>>(partial, parts, out, n8)));
     return launch_ok();
 }
 
 // D = Z' W_down over all tokens: A = Z' [T, F] (K-major), B = Wd [F, d] (its contiguous dimension is N).
-// scratch: fp32 words of dead workspace for the partial outputs of a split contraction (or none)
+// scratch: fp32 words of dead workspace for the partial outputs of a split contraction (plan.parts * T * d_model of them)
 int forward_tc_down(const moc_ffn_desc &d, const __nv_bfloat16 *Z, int ldz, const __nv_bfloat16 *wd, __nv_bfloat16 *out,
-                    int *status, cudaStream_t st, float *scratch = nullptr, size_t scratch_floats = 0) {
+                    int *status, cudaStream_t st, tc::DownPlan plan = {false, 1}, float *scratch = nullptr) {
     using namespace tc;
     const int F = d.d_ff, dm = d.d_model;
     const int64_t T = d.tokens;
     int rc = MOC_OK;
     Params q;
     init_params(q);
-    if (scratch && F >= 4 * BK && split_contraction(T, dm, scratch_floats)) {
+    q.status = status;
+    if (plan.swapped) {
+        if (!map_mn_major(&q.a_map[0], wd, F, dm, dm) || !map_b_k_major(q, 0, Z, T, F, ldz)) return MOC_ERR_CUDA;
+        q.k_blocks = ceil_div(ceil_div(F, BK), plan.parts);
+        q.M = dm;
+        q.N = (int)T;
+        q.m_tiles = ceil_div(dm, BM);
+        q.ldc[0] = dm;
+        if (plan.parts > 1) {
+            q.c[0] = scratch;
+            MOC_LAUNCH(KID_TC_DOWN_GEMM, st, (rc = launch_gemm<true, false, EPI_F32, true>(q, st, plan.parts, T * dm)));
+            return rc != MOC_OK ? rc : launch_split_sum(scratch, plan.parts, T, dm, out, st);
+        }
+        q.c[0] = out;
+        MOC_LAUNCH(KID_TC_DOWN_GEMM, st, (rc = launch_gemm<true, false, EPI_BF16, true>(q, st)));
+        return rc;
+    }
+    if (plan.parts > 1) {
         const int Kc = ceil_div(ceil_div(F, 2), BK) * BK;  // channels of the first half: whole 64-channel blocks
         for (int h = 0; h < 2; ++h) {
             const int k0 = h * Kc, kn = std::min(Kc, F - k0);
@@ -641,10 +659,9 @@ int forward_tc_down(const moc_ffn_desc &d, const __nv_bfloat16 *Z, int ldz, cons
         q.N = dm;
         q.m_tiles = ceil_div(T, BM);
         q.n_tiles = ceil_div(dm, BN);
-        q.status = status;
         MOC_LAUNCH(KID_TC_DOWN_GEMM, st, (rc = launch_gemm<false, true, EPI_F32>(q, st)));
         if (rc != MOC_OK) return rc;
-        return launch_split_sum(scratch, T, dm, out, st);
+        return launch_split_sum(scratch, 2, T, dm, out, st);
     }
     if (!map_k_major(&q.a_map[0], Z, T, F, ldz, BM) || !map_mn_major(&q.b_map[0], wd, F, dm, dm)) return MOC_ERR_CUDA;
     q.k_blocks = ceil_div(F, BK);
@@ -654,7 +671,6 @@ int forward_tc_down(const moc_ffn_desc &d, const __nv_bfloat16 *Z, int ldz, cons
     q.n_tiles = ceil_div(dm, BN);
     q.c[0] = out;
     q.ldc[0] = dm;
-    q.status = status;
     MOC_LAUNCH(KID_TC_DOWN_GEMM, st, (rc = launch_gemm<false, true, EPI_BF16>(q, st)));
     return rc;
 }
@@ -722,23 +738,33 @@ int forward_tc(const moc_ffn_desc &d, const __nv_bfloat16 *x, const __nv_bfloat1
     }
     Params p;
     init_params(p);
-    if (!map_b_k_major(p, 0, wg, F, dm, dm) || !map_b_k_major(p, 1, wu, F, dm, dm))
+    const bool swapped = swapped_gate_up_pays(std::min<int64_t>(L.chunk, T), F, dm);  // (equal chunks)
+    if (swapped ? !map_k_major(&p.a_map[0], wg, F, dm, dm, BM) || !map_k_major(&p.a_map[1], wu, F, dm, dm, BM)
+                : !map_b_k_major(p, 0, wg, F, dm, dm) || !map_b_k_major(p, 1, wu, F, dm, dm))
         return MOC_ERR_CUDA;
     p.status = status;
     p.num_problems = 2;
-    p.b_idx[1][0] = 1;
+    (swapped ? p.a_idx : p.b_idx)[1][0] = 1;
     p.k_blocks = ceil_div(dm, BK);
-    p.N = F;
-    p.n_tiles = f_tiles;
     p.ldc[0] = p.ldc[1] = L.ldf;
     for (int64_t t0 = 0; t0 < T; t0 += L.chunk) {
         const int64_t n = std::min<int64_t>(L.chunk, T - t0);
-        if (!map_k_major(&p.a_map[0], x + t0 * dm, n, dm, dm, BM)) return MOC_ERR_CUDA;
-        p.M = (int)n;
-        p.m_tiles = ceil_div(n, BM);
         p.c[0] = G;
         p.c[1] = U + t0 * L.ldf;
-        MOC_LAUNCH(KID_TC_GATE_UP_GEMM, st, (rc = launch_gemm<false, false, EPI_GATE_UP>(p, st)));
+        if (swapped) {
+            if (!map_b_k_major(p, 0, x + t0 * dm, n, dm, dm)) return MOC_ERR_CUDA;
+            p.M = F;
+            p.N = (int)n;
+            p.m_tiles = ceil_div(F, BM);
+            MOC_LAUNCH(KID_TC_GATE_UP_GEMM, st, (rc = launch_gemm<false, false, EPI_GATE_UP, true>(p, st)));
+        } else {
+            if (!map_k_major(&p.a_map[0], x + t0 * dm, n, dm, dm, BM)) return MOC_ERR_CUDA;
+            p.M = (int)n;
+            p.N = F;
+            p.m_tiles = ceil_div(n, BM);
+            p.n_tiles = f_tiles;
+            MOC_LAUNCH(KID_TC_GATE_UP_GEMM, st, (rc = launch_gemm<false, false, EPI_GATE_UP>(p, st)));
+        }
         if (rc != MOC_OK) return rc;
         if (t0 == 0 && sel.kind == TcSelect::kCtaPerRow) {
             MOC_LAUNCH(KID_TC_SELECT_HINT, st,
@@ -758,8 +784,7 @@ int forward_tc(const moc_ffn_desc &d, const __nv_bfloat16 *x, const __nv_bfloat1
         }
         if ((rc = launch_ok()) != MOC_OK) return rc;
     }
-    // (the fp32 gate values are dead by now: their buffer takes the partial outputs of a split contraction)
-    return forward_tc_down(d, U, L.ldf, wd, out, status, st, G, (size_t)std::min<int64_t>(L.chunk, T) * L.ldf);
+    return forward_tc_down(d, U, L.ldf, wd, out, status, st, L.down, G);
 }
 
 int small_batch_dx(const moc_ffn_desc &d, const __nv_bfloat16 *dG, const __nv_bfloat16 *dU, int ldf,
@@ -897,7 +922,7 @@ int backward_tc(const moc_ffn_desc &d, const __nv_bfloat16 *x, const __nv_bfloat
             p.ldc[0] = p.ldc[1] = dm;
             MOC_LAUNCH(KID_TC_DX_GEMM, st, (rc = launch_gemm<false, true, EPI_F32>(p, st)));
             if (rc != MOC_OK) return rc;
-            if ((rc = launch_split_sum(partial, T, dm, gx, st)) != MOC_OK) return rc;
+            if ((rc = launch_split_sum(partial, 2, T, dm, gx, st)) != MOC_OK) return rc;
         } else {
             p.k_segments = 2;
             p.a_idx[0][1] = 1;

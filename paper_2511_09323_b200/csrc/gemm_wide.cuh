@@ -30,21 +30,27 @@ constexpr uint32_t WIDE_B_BYTES = (BN / 2) * BK * 2;  // one accumulator's half 
 constexpr uint32_t WIDE_RING_BYTES = 192 * 1024;      // 4 stages of A | B | B, or 6 of A | B where no tile is wider than 256
 constexpr size_t WIDE_SMEM_BYTES = 1024 + WIDE_RING_BYTES + BAR_REGION_BYTES + WIDE_EPI_WARPS * EPI_BOX_BYTES;
 
-// How the output is cut.  Rows: 256-row blocks of all problems.  The first `t1` tiles are 512 columns wide, the others w2.
+// How the output is cut.  Rows: 256-row blocks of all problems.  The first `t1` tiles are w1 columns wide, the others w2.
 //   by_columns == 0: rows one after the other, their tiles from left to right; the first `split` rows have wide tiles
 //   by_columns == 1: column by column, all rows in turn (few rows and a large B: B is read once); the first `split` columns
 //                    have wide tiles
 struct TilePlan {
-    int rows, by_columns, split, nt1, w2, nt2, t1, total;
+    int rows, by_columns, split, w1, nt1, w2, nt2, t1, total;
+    double cycles;  // of the pair that finishes last, by the model below
 };
 
 struct WideParams {
     Params g;
     CUtensorMap b_rem[3];  // K-major B: boxes for the accumulator of fewer than 256 columns of the narrower tiles
+    CUtensorMap b_rem1;    // TRANSPOSED: the same for the first tiles (operand 0)
     TilePlan t;
     int m_blocks;          // 256-row blocks of one problem
     int stages;
     uint32_t stage_bytes;
+    // TRANSPOSED: the problems are `k_split` parts of one contraction (k_blocks blocks each; blocks past its end are zeros),
+    // their fp32 outputs c_step elements apart
+    int k_split;
+    int64_t c_step;
 };
 
 // one tile
@@ -58,7 +64,7 @@ __device__ __forceinline__ WideTile wide_tile(const WideParams &p, int tile) {
     int row, w;
     const bool first = tile < p.t.t1;
     const int i = first ? tile : tile - p.t.t1;
-    w = first ? WIDE_N : p.t.w2;
+    w = first ? p.t.w1 : p.t.w2;
     if (p.t.by_columns) {
         const int c = i / p.t.rows;
         row = i - c * p.t.rows;
@@ -82,6 +88,38 @@ __device__ __forceinline__ WideTile wide_tile(const WideParams &p, int tile) {
     t.box0 = (uint32_t)full0 / 2;
     t.box1 = (uint32_t)(w - full0) / 2;
     return t;
+}
+
+// The same for an output that is stored column by column (TRANSPOSED): the lanes are consecutive elements of a stored row, so
+// a column leaves as one contiguous store of the warp.
+template <int EPI>
+__device__ __forceinline__ void transposed_epilogue(const WideParams &w, int prob, int row0, int n0, int cols, int half, uint32_t taddr) {
+    const Params &p = w.g;
+    const int lane = threadIdx.x & 31, row = row0 + lane;
+    const bool f32_out = EPI == EPI_F32 || (EPI == EPI_GATE_UP && prob == 0);
+    const int out = w.k_split > 1 ? 0 : prob;
+    const int64_t ld = p.ldc[out], at = (int64_t)n0 * ld + row + (w.k_split > 1 ? prob * w.c_step : 0);
+    cols = min(cols, p.N - n0);
+    if (row0 >= p.M) return;
+#pragma unroll 1
+    for (int c0 = 32 * half; c0 < cols; c0 += 64) {
+        uint32_t r[32];
+        __syncwarp();
+        tmem_ld32(taddr + (uint32_t)c0, r);
+        tmem_ld_wait();
+        const int valid = row < p.M ? min(32, cols - c0) : 0;
+        if (f32_out) {
+            float *dst = static_cast<float *>(p.c[out]) + at + c0 * ld;
+#pragma unroll
+            for (int i = 0; i < 32; ++i, dst += ld)
+                if (i < valid) *dst = __uint_as_float(r[i]);
+        } else {
+            __nv_bfloat16 *dst = static_cast<__nv_bfloat16 *>(p.c[out]) + at + c0 * ld;
+#pragma unroll
+            for (int i = 0; i < 32; ++i, dst += ld)
+                if (i < valid) *dst = __float2bfloat16_rn(__uint_as_float(r[i]));
+        }
+    }
 }
 
 // One warp's share of an accumulator of `cols` columns: every other 128-byte chunk (`half` says which) of its 32 rows.
@@ -180,7 +218,8 @@ __device__ __forceinline__ void wide_epilogue(const Params &p, int prob, int row
     }
 }
 
-template <bool A_MN, bool B_MN, int EPI>
+// TRANSPOSED: the caller has exchanged the operands (see swapped_gemm_pays) and every output is stored as its transpose
+template <bool A_MN, bool B_MN, int EPI, bool TRANSPOSED = false>
 __global__ void __launch_bounds__(WIDE_THREADS, 1) gemm_wide_kernel(const __grid_constant__ WideParams p) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
@@ -246,12 +285,14 @@ __global__ void __launch_bounds__(WIDE_THREADS, 1) gemm_wide_kernel(const __grid
                                               : (t.box0 + (any1 ? t.box1 : 0u)) * (uint32_t)(BK * 2);
                 const uint32_t tx = 2 * (A_STAGE_BYTES + b_bytes);
                 for (int seg = 0; seg < p.g.k_segments && ok; ++seg) {
-                    const CUtensorMap *am = &p.g.a_map[p.g.a_idx[t.prob][seg]];
-                    const int bi = p.g.b_idx[t.prob][seg];
-                    const CUtensorMap *bm0 = !B_MN && t.box0 < BN / 2 ? &p.b_rem[bi] : &p.g.b_map[bi];
-                    const CUtensorMap *bm1 = !B_MN && t.box1 < BN / 2 ? &p.b_rem[bi] : &p.g.b_map[bi];
-                    const int k_end = p.g.k_blocks * BK;
-                    for (int kk = 0; kk < k_end; kk += BK) {
+                    const bool part = TRANSPOSED && p.k_split > 1;
+                    const CUtensorMap *am = &p.g.a_map[part ? 0 : p.g.a_idx[t.prob][seg]];
+                    const int bi = part ? 0 : p.g.b_idx[t.prob][seg];
+                    const CUtensorMap *rem = TRANSPOSED && tile < p.t.t1 ? &p.b_rem1 : &p.b_rem[bi];
+                    const CUtensorMap *bm0 = !B_MN && t.box0 < BN / 2 ? rem : &p.g.b_map[bi];
+                    const CUtensorMap *bm1 = !B_MN && t.box1 < BN / 2 ? rem : &p.g.b_map[bi];
+                    const int k_begin = part ? t.prob * p.g.k_blocks * BK : 0, k_end = k_begin + p.g.k_blocks * BK;
+                    for (int kk = k_begin; kk < k_end; kk += BK) {
                         if (!mbar_wait(bar_base + bar + 8u * WIDE_STAGES_MAX, phase ^ 1u, abort_flag, status)) {
                             ok = false;
                             break;
@@ -390,8 +431,12 @@ __global__ void __launch_bounds__(WIDE_THREADS, 1) gemm_wide_kernel(const __grid
                 ok = __all_sync(0xffffffffu, mbar_wait(tfull_bar(r), (used >> 1) & 1u, abort_flag, status));
                 if (!ok) break;
                 tc_fence_after();
-                wide_epilogue<EPI>(p.g, t.prob, t.m_blk * (2 * BM) + (int)rank * BM + quarter * 32, t.n0 + j * BN, j ? t.s1 : t.s0, half,
-                                   tmem_base + ((uint32_t)(quarter * 32) << 16) + r * BN, epi_base + (uint32_t)(warp - 2) * EPI_BOX_BYTES);
+                if constexpr (TRANSPOSED)
+                    transposed_epilogue<EPI>(p, t.prob, t.m_blk * (2 * BM) + (int)rank * BM + quarter * 32, t.n0 + j * BN, j ? t.s1 : t.s0,
+                                             half, tmem_base + ((uint32_t)(quarter * 32) << 16) + r * BN);
+                else
+                    wide_epilogue<EPI>(p.g, t.prob, t.m_blk * (2 * BM) + (int)rank * BM + quarter * 32, t.n0 + j * BN, j ? t.s1 : t.s0, half,
+                                       tmem_base + ((uint32_t)(quarter * 32) << 16) + r * BN, epi_base + (uint32_t)(warp - 2) * EPI_BOX_BYTES);
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive_cluster(map_to_cta(tempty_bar(r), 0));
@@ -425,7 +470,8 @@ constexpr int WIDE_DRAIN_BF16 = 2000, WIDE_DRAIN_F32 = 3500;
 // tokens, 40 tiles of 256 columns for 74 pairs, 36.8 us; 55 of 192.)  Remembered per problem size.
 // drain: cycles in which the epilogue moves an accumulator of 256 columns.  Of a tile with two accumulators the part of it
 // that the skew does not cover is lost; with one, the other is worked in meanwhile.
-inline TilePlan plan_tiles(int rows, int N, int kb, int pairs, bool by_columns, int drain) {
+// any_first: the first tiles may have any width, not 512 alone (few columns: one tile as wide as they are spans them).
+inline TilePlan plan_tiles(int rows, int N, int kb, int pairs, bool by_columns, int drain, bool any_first = false) {
     struct Key {
         int rows, n, kb, pairs, by_columns, drain;
         bool operator==(const Key &o) const {
@@ -441,55 +487,54 @@ inline TilePlan plan_tiles(int rows, int N, int kb, int pairs, bool by_columns, 
     };
     static std::mutex mu;
     static std::unordered_map<Key, TilePlan, Hash> known;
-    const Key key{rows, N, kb, pairs, by_columns ? 1 : 0, drain};
+    const Key key{rows, N, kb, pairs, (by_columns ? 1 : 0) + (any_first ? 2 : 0), drain};
     {
         std::lock_guard<std::mutex> lock(mu);
         auto it = known.find(key);
         if (it != known.end()) return it->second;
     }
-    const auto tile_cycles = [&](int w) {
+    const auto tile_cycles = [&](int w_of) {
+        const int w = std::min(w_of, (N + WIDE_STEP - 1) / WIDE_STEP * WIDE_STEP);
         const double mma = kb * wide_block_cycles(w) + 350.0;
         return w > BN ? mma + std::max(0, drain - WIDE_SKEW * 512) : std::max(mma, drain * w / 256.0);
     };
     const auto up = [](int64_t a, int64_t b) { return (int)((a + b - 1) / b); };
-    const int nt1 = up(N, WIDE_N);
     TilePlan best{};
-    double best_cycles = 0.0;
-    const auto consider = [&](int split, int w2) {
+    const auto consider = [&](int w1, int split, int w2) {
         TilePlan t{};
         t.rows = rows;
         t.by_columns = by_columns ? 1 : 0;
         t.split = split;
-        t.nt1 = nt1;
+        t.w1 = w1;
+        t.nt1 = up(N, w1);
         t.w2 = w2;
         if (by_columns) {
-            t.t1 = split / WIDE_N * rows;
+            t.t1 = split / w1 * rows;
             t.nt2 = split < N ? up(N - split, w2) : 0;
             t.total = t.t1 + t.nt2 * rows;
         } else {
-            t.t1 = split * nt1;
+            t.t1 = split * t.nt1;
             t.nt2 = up(N, w2);
             t.total = t.t1 + (rows - split) * t.nt2;
         }
         // tiles go round the pairs in turn: pair j has every pairs-th one from j on
-        double worst = 0.0;
         for (int j = 0; j < pairs; ++j) {
             const int n1 = t.t1 > j ? (t.t1 - 1 - j) / pairs + 1 : 0, n = t.total > j ? (t.total - 1 - j) / pairs + 1 : 0;
-            worst = std::max(worst, n1 * tile_cycles(WIDE_N) + (n - n1) * tile_cycles(w2));
+            t.cycles = std::max(t.cycles, n1 * tile_cycles(w1) + (n - n1) * tile_cycles(w2));
         }
-        if (best.total == 0 || worst < best_cycles) {
-            best = t;
-            best_cycles = worst;
-        }
+        if (best.total == 0 || t.cycles < best.cycles) best = t;
     };
-    const int units = by_columns ? N / WIDE_N : rows;              // what is split off as wide: columns' tiles or rows
-    const int per_unit = by_columns ? rows : nt1;                  // tiles of one
-    const int waves = (int)((int64_t)units * per_unit / pairs);
-    for (int w2 = WIDE_N; w2 >= WIDE_STEP; w2 -= WIDE_STEP) {
-        consider(0, w2);
-        for (int f = waves; f >= std::max(1, waves - 1); --f) {
-            const int u = std::min<int64_t>(units, (int64_t)f * pairs / per_unit);
-            for (int v = u; v >= std::max(1, u - 1); --v) consider(by_columns ? v * WIDE_N : v, w2);
+    const int most = any_first ? std::min(WIDE_N, up(N, WIDE_STEP) * WIDE_STEP) : WIDE_N;
+    for (int w1 = most; w1 >= (any_first ? WIDE_STEP : WIDE_N); w1 -= WIDE_STEP) {
+        const int units = by_columns ? N / w1 : rows;                  // what is split off as wide: columns' tiles or rows
+        const int per_unit = by_columns ? rows : up(N, w1);            // tiles of one
+        const int waves = (int)((int64_t)units * per_unit / pairs);
+        for (int w2 = most; w2 >= WIDE_STEP; w2 -= WIDE_STEP) {
+            if (w1 == most) consider(w1, 0, w2);
+            for (int f = waves; f >= std::max(1, waves - 1); --f) {
+                const int u = std::min<int64_t>(units, (int64_t)f * pairs / per_unit);
+                for (int v = u; v >= std::max(1, u - 1); --v) consider(w1, by_columns ? v * w1 : v, w2);
+            }
         }
     }
     std::lock_guard<std::mutex> lock(mu);

@@ -165,8 +165,16 @@ inline int resident_pairs(Kernel kern, int threads, size_t smem, int &cached) {
     return cached = n;
 }
 
-template <bool A_MN, bool B_MN, int EPI>
-inline int launch_gemm(const Params &p_in, cudaStream_t st) {
+// Few rows and a B that does not stay in L2: all rows of a column of tiles in turn, so that B is read once (2048 tokens, gate
+// and up projection of the 4096 x 11008 layer: 301 us row by row).
+inline bool walk_by_columns(int64_t M, int n_a, int64_t N, int n_b, int kb) {
+    const double block_bytes = (double)kb * BK * 2, b_bytes = block_bytes * N * n_b, a_bytes = block_bytes * M * n_a;
+    return b_bytes > 64e6 && a_bytes < 0.5 * b_bytes;
+}
+
+// k_split, c_step: see WideParams (TRANSPOSED only; the one problem of p_in is then split)
+template <bool A_MN, bool B_MN, int EPI, bool TRANSPOSED = false>
+inline int launch_gemm(const Params &p_in, cudaStream_t st, int k_split = 1, int64_t c_step = 0) {
     Params p = p_in;
     if (p.M <= 0 || p.N <= 0) return MOC_OK;
     p.direct_store = 0;
@@ -181,30 +189,33 @@ inline int launch_gemm(const Params &p_in, cudaStream_t st) {
         return launch_pairs(gemm_pair_kernel, p, std::min(((p.m_tiles + 1) / 2) * p.n_tiles, max_pairs), PAIR_THREADS, SMEM_BYTES, st);
     } else if (pair_mode()) {
         static int max_pairs = 0;
-        const auto kern = gemm_wide_kernel<A_MN, B_MN, EPI>;
+        const auto kern = gemm_wide_kernel<A_MN, B_MN, EPI, TRANSPOSED>;
         if (!resident_pairs(kern, WIDE_THREADS, WIDE_SMEM_BYTES, max_pairs)) return MOC_ERR_CUDA;
         WideParams w;
         memset(&w, 0, sizeof(w));
         w.g = p;
         w.m_blocks = (p.m_tiles + 1) / 2;
-        // Few rows and a B that does not stay in L2: all rows of a column of tiles in turn, so that B is read once (2048
-        // tokens, gate and up projection of the 4096 x 11008 layer: 301 us row by row).
         const int kb = p.k_blocks * p.k_segments;
         int n_b = 1, n_a = 1;
         for (int i = 1; i < p.num_problems; ++i) {
             n_b += p.b_idx[i][0] != p.b_idx[0][0] ? 1 : 0;
             n_a += p.a_idx[i][0] != p.a_idx[0][0] ? 1 : 0;
         }
-        const double block_bytes = (double)kb * BK * 2, b_bytes = block_bytes * p.N * n_b, a_bytes = block_bytes * p.M * n_a;
-        const bool by_columns = b_bytes > 64e6 && a_bytes < 0.5 * b_bytes;
-        w.t = plan_tiles(w.m_blocks * p.num_problems, p.N, kb, max_pairs, by_columns, EPI == EPI_BF16 ? WIDE_DRAIN_BF16 : WIDE_DRAIN_F32);
-        const int widest = w.t.t1 ? WIDE_N : w.t.w2;
+        w.k_split = k_split;
+        w.c_step = c_step;
+        if (k_split > 1) w.g.num_problems = k_split;
+        w.t = plan_tiles(w.m_blocks * w.g.num_problems, p.N, kb, max_pairs, !TRANSPOSED && walk_by_columns(p.M, n_a, p.N, n_b, kb),
+                         EPI == EPI_BF16 ? WIDE_DRAIN_BF16 : WIDE_DRAIN_F32, TRANSPOSED);
+        const int widest = w.t.t1 ? std::max(w.t.w1, w.t.total > w.t.t1 ? w.t.w2 : 0) : w.t.w2;
         w.stage_bytes = A_STAGE_BYTES + (widest > BN ? 2 : 1) * WIDE_B_BYTES;
         w.stages = (int)(WIDE_RING_BYTES / w.stage_bytes);
-        const int rem = w.t.w2 > BN ? w.t.w2 - BN : w.t.w2;  // columns of the narrower tiles' smaller accumulator
+        const auto remainder = [](int width) { return width > BN ? width - BN : width; };  // columns of the smaller accumulator
+        const int rem = remainder(w.t.w2), rem1 = remainder(w.t.w1);
         if (!B_MN && rem < BN && w.t.total > w.t.t1)
             for (int i = 0; i < 3; ++i)
                 if (p.b_op[i].ptr && !map_k_major(&w.b_rem[i], p.b_op[i].ptr, p.b_op[i].n, p.b_op[i].k, p.b_op[i].ld, rem / 2)) return MOC_ERR_CUDA;
+        if (TRANSPOSED && rem1 < BN && w.t.t1 > 0 && !map_k_major(&w.b_rem1, p.b_op[0].ptr, p.b_op[0].n, p.b_op[0].k, p.b_op[0].ld, rem1 / 2))
+            return MOC_ERR_CUDA;
         return launch_pairs(kern, w, std::min(w.t.total, max_pairs), WIDE_THREADS, WIDE_SMEM_BYTES, st);
     } else {
         const auto kern = gemm_kernel<A_MN, B_MN, EPI>;
@@ -218,6 +229,56 @@ inline int launch_gemm(const Params &p_in, cudaStream_t st) {
         kern<<<std::min(tiles, sm_count()), THREADS, SMEM_BYTES, st>>>(p);
         return cudaGetLastError() == cudaSuccess ? MOC_OK : MOC_ERR_CUDA;
     }
+}
+
+// ---- Exchanged operands.  A tile's rows come in blocks of 256, its columns in steps of 64: with a few hundred tokens the
+// weights are the better rows (307 tokens are 320 columns, but 512 rows), and their outputs are stored transposed.  The plan's
+// own cycles decide; the exchange has to save a twentieth of them.  (4096 x 11008, 307 tokens: gate + up 75.4 -> 64.7 us, down
+// in three parts 36.2 -> 30.4, the forward 145 -> 122; 600 tokens 207 -> 194; 2048 x 5504, 257 tokens: 61.1 -> 55.3.)
+inline bool swapped_gate_up_pays(int64_t T, int F, int dm) {
+    if (!pair_mode() || T > 4096) return false;
+    const int kb = (dm + BK - 1) / BK, pairs = sm_count() / 2;
+    const auto blocks = [](int64_t n) { return (int)((n + 255) / 256); };
+    const TilePlan plain = plan_tiles(2 * blocks(T), F, kb, pairs, walk_by_columns(T, 1, F, 2, kb), WIDE_DRAIN_F32);
+    const TilePlan swapped = plan_tiles(2 * blocks(F), (int)T, kb, pairs, false, WIDE_DRAIN_F32, true);
+    return swapped.cycles < 0.95 * plain.cycles;
+}
+
+// How the down projection [T, F] x [F, dm] runs: exchanged or not, in how many parts along its contraction (fp32 partial
+// outputs, which a kernel adds: launch, and the partial outputs written and read once through L2).
+struct DownPlan {
+    bool swapped;
+    int parts;
+};
+// MOC_FFN_SPLIT_K=0 in the environment switches every split off (comparisons).
+inline bool split_contraction_enabled() {
+    static const bool on = [] {
+        const char *e = getenv("MOC_FFN_SPLIT_K");
+        return !(e && atoi(e) == 0);
+    }();
+    return on;
+}
+inline bool split_contraction_pays(int64_t T, int n_cols);
+inline DownPlan plan_down(int64_t T, int F, int dm) {
+    const int kb = (F + BK - 1) / BK, pairs = sm_count() / 2;
+    const auto blocks = [](int64_t n) { return (int)((n + 255) / 256); };
+    const auto per_part = [&](int parts) { return (kb + parts - 1) / parts; };
+    const auto sum = [&](int parts) { return parts > 1 ? 5000.0 + (double)parts * T * dm * 8 / (30.0 * sm_count()) : 0.0; };
+    const auto drain = [](int parts) { return parts > 1 ? WIDE_DRAIN_F32 : WIDE_DRAIN_BF16; };
+    DownPlan best{false, F >= 4 * BK && split_contraction_pays(T, dm) ? 2 : 1};
+    if (!pair_mode() || T > 4096) return best;
+    double least = 0.95 * (plan_tiles(blocks(T) * best.parts, dm, per_part(best.parts), pairs, walk_by_columns(T, 1, dm, 1, kb),
+                                      drain(best.parts)).cycles + sum(best.parts));
+    // (where the plain form has too few tiles, so has the exchanged one)
+    for (int parts = best.parts; parts <= 4 && per_part(parts) >= 8; ++parts) {
+        if (parts > 1 && ((dm & 7) || !split_contraction_enabled())) break;
+        const double c = plan_tiles(blocks(dm) * parts, (int)T, per_part(parts), pairs, false, drain(parts), true).cycles + sum(parts);
+        if (c < least) {
+            least = c;
+            best = {true, parts};
+        }
+    }
+    return best;
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -819,7 +880,9 @@ __global__ void __launch_bounds__(256) backward_sample_rows_kernel(
 struct TcForwardLayout {
     int64_t chunk;  // tokens per gate/up pass
     int ldf;        // leading dimension of the dense [*, F] arrays (multiple of 8)
-    size_t off_g;   // fp32 G of one chunk [chunk, ldf]
+    size_t off_g;   // fp32 G of one chunk [chunk, ldf]; later the partial outputs of a split down projection
+    size_t g_floats;
+    DownPlan down;
     size_t off_u;   // bf16 U, rewritten in place into Z', for ALL tokens [T, ldf]
     size_t off_hint;  // bracket {center, width, tag}, statistics {sum, sum|dev|, rows}, CTA counter
     // MoC 2:8 on the sparse MMA: Z' in compressed form lives where U would (it is half as large), its metadata here
@@ -871,7 +934,10 @@ inline TcForwardLayout tc_forward_layout(const moc_ffn_desc &d) {
     L.chunk = best * BM;
     size_t off = 0;
     L.off_g = off;
-    off = align_up(off + (size_t)L.chunk * L.ldf * 4, 256);
+    L.down = plan_down(d.tokens, d.d_ff, d.d_model);
+    // (the gate values are dead when the down projection runs: its partial outputs take their buffer)
+    L.g_floats = std::max<size_t>((size_t)L.chunk * L.ldf, L.down.parts > 1 ? (size_t)L.down.parts * d.tokens * d.d_model : 0);
+    off = align_up(off + L.g_floats * 4, 256);
     L.off_u = off;
     off = align_up(off + (size_t)all_m * BM * L.ldf * 2, 256);
     L.off_hint = off;
@@ -887,13 +953,8 @@ inline TcForwardLayout tc_forward_layout(const moc_ffn_desc &d) {
 // A GEMM whose output has so few tiles that half of the CTA pairs would idle (a few hundred tokens: 32 tiles of
 // 256 x 256 for 512 tokens and d_model = 4096, each with the whole d_ffn to contract) is split in two along its
 // contraction: the halves run as two problems of one launch into fp32 partial outputs, which a small kernel adds.
-// MOC_FFN_SPLIT_K=0 in the environment switches the split off (comparisons).
 inline bool split_contraction_pays(int64_t T, int n_cols) {
-    static const bool on = [] {
-        const char *e = getenv("MOC_FFN_SPLIT_K");
-        return !(e && atoi(e) == 0);
-    }();
-    if (!on || !pair_mode() || (n_cols & 7)) return false;
+    if (!split_contraction_enabled() || !pair_mode() || (n_cols & 7)) return false;
     const int64_t tiles = ((T + BM - 1) / BM + 1) / 2 * ((n_cols + BN - 1) / BN);
     return 2 * tiles <= sm_count() / 2;
 }
