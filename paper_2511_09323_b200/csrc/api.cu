@@ -619,7 +619,7 @@ int launch_split_sum(const float *partial, int parts, int64_t T, int n_cols, __n
 // D = Z' W_down over all tokens: A = Z' [T, F] (K-major), B = Wd [F, d] (its contiguous dimension is N).
 // scratch: fp32 words of dead workspace for the partial outputs of a split contraction (plan.parts * T * d_model of them)
 int forward_tc_down(const moc_ffn_desc &d, const __nv_bfloat16 *Z, int ldz, const __nv_bfloat16 *wd, __nv_bfloat16 *out,
-                    int *status, cudaStream_t st, tc::DownPlan plan = {false, 1}, float *scratch = nullptr) {
+                    int *status, cudaStream_t st, tc::ContractionPlan plan = {false, 1}, float *scratch = nullptr) {
     using namespace tc;
     const int F = d.d_ff, dm = d.d_model;
     const int64_t T = d.tokens;
@@ -738,7 +738,7 @@ int forward_tc(const moc_ffn_desc &d, const __nv_bfloat16 *x, const __nv_bfloat1
     }
     Params p;
     init_params(p);
-    const bool swapped = swapped_gate_up_pays(std::min<int64_t>(L.chunk, T), F, dm);  // (equal chunks)
+    const bool swapped = swapped_projection_pays(std::min<int64_t>(L.chunk, T), F, ceil_div(dm, BK), 2, WIDE_DRAIN_F32);  // (equal chunks)
     if (swapped ? !map_k_major(&p.a_map[0], wg, F, dm, dm, BM) || !map_k_major(&p.a_map[1], wu, F, dm, dm, BM)
                 : !map_b_k_major(p, 0, wg, F, dm, dm) || !map_b_k_major(p, 1, wu, F, dm, dm))
         return MOC_ERR_CUDA;
@@ -812,17 +812,24 @@ int backward_tc(const moc_ffn_desc &d, const __nv_bfloat16 *x, const __nv_bfloat
     {
         Params p;
         init_params(p);
-        if (!map_k_major(&p.a_map[0], dout, T, dm, dm, BM) || !map_b_k_major(p, 0, wd, F, dm, dm))
-            return MOC_ERR_CUDA;
         p.k_blocks = ceil_div(dm, BK);
-        p.M = (int)T;
-        p.N = F;
-        p.m_tiles = ceil_div(T, BM);
-        p.n_tiles = ceil_div(F, BN);
         p.c[0] = Zp;
         p.ldc[0] = L.ldf;
         p.status = status;
-        MOC_LAUNCH(KID_TC_DZ_GEMM, st, (rc = launch_gemm<false, false, EPI_BF16>(p, st)));
+        if (swapped_projection_pays(T, F, p.k_blocks, 1, WIDE_DRAIN_BF16)) {
+            if (!map_k_major(&p.a_map[0], wd, F, dm, dm, BM) || !map_b_k_major(p, 0, dout, T, dm, dm)) return MOC_ERR_CUDA;
+            p.M = F;
+            p.N = (int)T;
+            p.m_tiles = ceil_div(F, BM);
+            MOC_LAUNCH(KID_TC_DZ_GEMM, st, (rc = launch_gemm<false, false, EPI_BF16, true>(p, st)));
+        } else {
+            if (!map_k_major(&p.a_map[0], dout, T, dm, dm, BM) || !map_b_k_major(p, 0, wd, F, dm, dm)) return MOC_ERR_CUDA;
+            p.M = (int)T;
+            p.N = F;
+            p.m_tiles = ceil_div(T, BM);
+            p.n_tiles = ceil_div(F, BN);
+            MOC_LAUNCH(KID_TC_DZ_GEMM, st, (rc = launch_gemm<false, false, EPI_BF16>(p, st)));
+        }
         if (rc != MOC_OK) return rc;
         // a team of warps per token with the token's rows staged in shared memory while two such tokens fit an SM; else one
         // CTA per token working in global memory
@@ -899,6 +906,29 @@ int backward_tc(const moc_ffn_desc &d, const __nv_bfloat16 *x, const __nv_bfloat
         // a small batch: the weight-streaming kernel of the small-batch plan (a 256-row tile of tokens would leave
         // most SMs without work: d_model / 256 tiles in all)
         if ((rc = small_batch_dx(d, dGp, dUp, L.ldf, wg, wu, gx, ws + L.off_small, st)) != MOC_OK) return rc;
+    } else if (gx && L.dx.swapped) {
+        Params p;
+        init_params(p);
+        if (!map_mn_major(&p.a_map[0], wg, F, dm, dm) || !map_mn_major(&p.a_map[1], wu, F, dm, dm) ||
+            !map_b_k_major(p, 0, dGp, T, F, L.ldf) || !map_b_k_major(p, 1, dUp, T, F, L.ldf))
+            return MOC_ERR_CUDA;
+        const int parts = L.dx.parts;
+        float *partial = reinterpret_cast<float *>(ws + L.off_split);
+        p.k_segments = 2;
+        p.a_idx[0][1] = p.b_idx[0][1] = 1;
+        p.k_blocks = parts > 1 ? ceil_div(ceil_div(F, BK), parts / 2) : ceil_div(F, BK);
+        p.M = dm;
+        p.N = (int)T;
+        p.m_tiles = ceil_div(dm, BM);
+        p.c[0] = parts > 1 ? static_cast<void *>(partial) : gx;
+        p.ldc[0] = dm;
+        p.status = status;
+        if (parts > 1) {
+            MOC_LAUNCH(KID_TC_DX_GEMM, st, (rc = launch_gemm<true, false, EPI_F32, true>(p, st, parts, T * dm)));
+            return rc != MOC_OK ? rc : launch_split_sum(partial, parts, T, dm, gx, st);
+        }
+        MOC_LAUNCH(KID_TC_DX_GEMM, st, (rc = launch_gemm<true, false, EPI_BF16, true>(p, st)));
+        if (rc != MOC_OK) return rc;
     } else if (gx) {
         Params p;
         init_params(p);

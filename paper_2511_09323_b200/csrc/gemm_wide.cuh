@@ -42,14 +42,14 @@ struct TilePlan {
 struct WideParams {
     Params g;
     CUtensorMap b_rem[3];  // K-major B: boxes for the accumulator of fewer than 256 columns of the narrower tiles
-    CUtensorMap b_rem1;    // TRANSPOSED: the same for the first tiles (operand 0)
+    CUtensorMap b_rem1[2]; // TRANSPOSED: the same for the first tiles
     TilePlan t;
     int m_blocks;          // 256-row blocks of one problem
     int stages;
     uint32_t stage_bytes;
-    // TRANSPOSED: the problems are `k_split` parts of one contraction (k_blocks blocks each; blocks past its end are zeros),
-    // their fp32 outputs c_step elements apart
-    int k_split;
+    // TRANSPOSED: the problems are `k_split` parts of one contraction, of its `k_operands` pairs of operands in turn (k_blocks
+    // blocks each; blocks past an operand's end are zeros), their fp32 outputs c_step elements apart
+    int k_split, k_operands;
     int64_t c_step;
 };
 
@@ -286,12 +286,13 @@ __global__ void __launch_bounds__(WIDE_THREADS, 1) gemm_wide_kernel(const __grid
                 const uint32_t tx = 2 * (A_STAGE_BYTES + b_bytes);
                 for (int seg = 0; seg < p.g.k_segments && ok; ++seg) {
                     const bool part = TRANSPOSED && p.k_split > 1;
-                    const CUtensorMap *am = &p.g.a_map[part ? 0 : p.g.a_idx[t.prob][seg]];
-                    const int bi = part ? 0 : p.g.b_idx[t.prob][seg];
-                    const CUtensorMap *rem = TRANSPOSED && tile < p.t.t1 ? &p.b_rem1 : &p.b_rem[bi];
+                    const int pair_of = part ? t.prob % p.k_operands : 0;
+                    const CUtensorMap *am = &p.g.a_map[part ? pair_of : p.g.a_idx[t.prob][seg]];
+                    const int bi = part ? pair_of : p.g.b_idx[t.prob][seg];
+                    const CUtensorMap *rem = TRANSPOSED && tile < p.t.t1 ? &p.b_rem1[bi] : &p.b_rem[bi];
                     const CUtensorMap *bm0 = !B_MN && t.box0 < BN / 2 ? rem : &p.g.b_map[bi];
                     const CUtensorMap *bm1 = !B_MN && t.box1 < BN / 2 ? rem : &p.g.b_map[bi];
-                    const int k_begin = part ? t.prob * p.g.k_blocks * BK : 0, k_end = k_begin + p.g.k_blocks * BK;
+                    const int k_begin = part ? t.prob / p.k_operands * p.g.k_blocks * BK : 0, k_end = k_begin + p.g.k_blocks * BK;
                     for (int kk = k_begin; kk < k_end; kk += BK) {
                         if (!mbar_wait(bar_base + bar + 8u * WIDE_STAGES_MAX, phase ^ 1u, abort_flag, status)) {
                             ok = false;

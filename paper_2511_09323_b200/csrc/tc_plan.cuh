@@ -172,7 +172,7 @@ inline bool walk_by_columns(int64_t M, int n_a, int64_t N, int n_b, int kb) {
     return b_bytes > 64e6 && a_bytes < 0.5 * b_bytes;
 }
 
-// k_split, c_step: see WideParams (TRANSPOSED only; the one problem of p_in is then split)
+// k_split, c_step: see WideParams (TRANSPOSED only; the one problem of p_in, with its segments' operands, is then split)
 template <bool A_MN, bool B_MN, int EPI, bool TRANSPOSED = false>
 inline int launch_gemm(const Params &p_in, cudaStream_t st, int k_split = 1, int64_t c_step = 0) {
     Params p = p_in;
@@ -195,7 +195,7 @@ inline int launch_gemm(const Params &p_in, cudaStream_t st, int k_split = 1, int
         memset(&w, 0, sizeof(w));
         w.g = p;
         w.m_blocks = (p.m_tiles + 1) / 2;
-        const int kb = p.k_blocks * p.k_segments;
+        const int kb = p.k_blocks * (k_split > 1 ? 1 : p.k_segments);
         int n_b = 1, n_a = 1;
         for (int i = 1; i < p.num_problems; ++i) {
             n_b += p.b_idx[i][0] != p.b_idx[0][0] ? 1 : 0;
@@ -203,7 +203,11 @@ inline int launch_gemm(const Params &p_in, cudaStream_t st, int k_split = 1, int
         }
         w.k_split = k_split;
         w.c_step = c_step;
-        if (k_split > 1) w.g.num_problems = k_split;
+        w.k_operands = p.k_segments;
+        if (k_split > 1) {
+            w.g.num_problems = k_split;
+            w.g.k_segments = 1;
+        }
         w.t = plan_tiles(w.m_blocks * w.g.num_problems, p.N, kb, max_pairs, !TRANSPOSED && walk_by_columns(p.M, n_a, p.N, n_b, kb),
                          EPI == EPI_BF16 ? WIDE_DRAIN_BF16 : WIDE_DRAIN_F32, TRANSPOSED);
         const int widest = w.t.t1 ? std::max(w.t.w1, w.t.total > w.t.t1 ? w.t.w2 : 0) : w.t.w2;
@@ -214,8 +218,9 @@ inline int launch_gemm(const Params &p_in, cudaStream_t st, int k_split = 1, int
         if (!B_MN && rem < BN && w.t.total > w.t.t1)
             for (int i = 0; i < 3; ++i)
                 if (p.b_op[i].ptr && !map_k_major(&w.b_rem[i], p.b_op[i].ptr, p.b_op[i].n, p.b_op[i].k, p.b_op[i].ld, rem / 2)) return MOC_ERR_CUDA;
-        if (TRANSPOSED && rem1 < BN && w.t.t1 > 0 && !map_k_major(&w.b_rem1, p.b_op[0].ptr, p.b_op[0].n, p.b_op[0].k, p.b_op[0].ld, rem1 / 2))
-            return MOC_ERR_CUDA;
+        if (TRANSPOSED && rem1 < BN && w.t.t1 > 0)
+            for (int i = 0; i < 2; ++i)
+                if (p.b_op[i].ptr && !map_k_major(&w.b_rem1[i], p.b_op[i].ptr, p.b_op[i].n, p.b_op[i].k, p.b_op[i].ld, rem1 / 2)) return MOC_ERR_CUDA;
         return launch_pairs(kern, w, std::min(w.t.total, max_pairs), WIDE_THREADS, WIDE_SMEM_BYTES, st);
     } else {
         const auto kern = gemm_kernel<A_MN, B_MN, EPI>;
@@ -234,19 +239,25 @@ inline int launch_gemm(const Params &p_in, cudaStream_t st, int k_split = 1, int
 // ---- Exchanged operands.  A tile's rows come in blocks of 256, its columns in steps of 64: with a few hundred tokens the
 // weights are the better rows (307 tokens are 320 columns, but 512 rows), and their outputs are stored transposed.  The plan's
 // own cycles decide; the exchange has to save a twentieth of them.  (4096 x 11008, 307 tokens: gate + up 75.4 -> 64.7 us, down
-// in three parts 36.2 -> 30.4, the forward 145 -> 122; 600 tokens 207 -> 194; 2048 x 5504, 257 tokens: 61.1 -> 55.3.)
-inline bool swapped_gate_up_pays(int64_t T, int F, int dm) {
-    if (!pair_mode() || T > 4096) return false;
-    const int kb = (dm + BK - 1) / BK, pairs = sm_count() / 2;
+// in three parts 36.2 -> 30.4, the forward 145 -> 122; 600 tokens 207 -> 194; 2048 x 5504, 257 tokens: 61.1 -> 55.3.
+// grad_x: 1111 tokens of 2048 x 5461 64.3 -> 50.6 us and 3.6 for the sum, 300 tokens of 4096 x 11008 67.3 -> 59.1.)
+// (with more the waste is small, and what the cycles promise for odd tile counts was not there: 16384 x 768 x 2048, down and
+// grad_x exchanged: step 519 -> 525 us; 3000 tokens 140 -> 141)
+constexpr int64_t SWAPPED_MAX_TOKENS = 2048;
+
+// `problems` products of x [T, ..] with weights of F rows each over kb blocks, outputs [T, F]
+inline bool swapped_projection_pays(int64_t T, int F, int kb, int problems, int drain) {
+    if (!pair_mode() || T > SWAPPED_MAX_TOKENS) return false;
+    const int pairs = sm_count() / 2;
     const auto blocks = [](int64_t n) { return (int)((n + 255) / 256); };
-    const TilePlan plain = plan_tiles(2 * blocks(T), F, kb, pairs, walk_by_columns(T, 1, F, 2, kb), WIDE_DRAIN_F32);
-    const TilePlan swapped = plan_tiles(2 * blocks(F), (int)T, kb, pairs, false, WIDE_DRAIN_F32, true);
+    const TilePlan plain = plan_tiles(problems * blocks(T), F, kb, pairs, walk_by_columns(T, 1, F, problems, kb), drain);
+    const TilePlan swapped = plan_tiles(problems * blocks(F), (int)T, kb, pairs, false, drain, true);
     return swapped.cycles < 0.95 * plain.cycles;
 }
 
-// How the down projection [T, F] x [F, dm] runs: exchanged or not, in how many parts along its contraction (fp32 partial
-// outputs, which a kernel adds: launch, and the partial outputs written and read once through L2).
-struct DownPlan {
+// How a contraction over the channels runs, [T, F] x [F, cols] summed over `segments` such pairs: exchanged or not, in how many
+// parts along it (fp32 partial outputs, which a kernel adds: its launch, and the partial outputs written and read through L2).
+struct ContractionPlan {
     bool swapped;
     int parts;
 };
@@ -259,20 +270,21 @@ inline bool split_contraction_enabled() {
     return on;
 }
 inline bool split_contraction_pays(int64_t T, int n_cols);
-inline DownPlan plan_down(int64_t T, int F, int dm) {
+inline ContractionPlan plan_contraction(int64_t T, int F, int cols, int segments) {
     const int kb = (F + BK - 1) / BK, pairs = sm_count() / 2;
     const auto blocks = [](int64_t n) { return (int)((n + 255) / 256); };
-    const auto per_part = [&](int parts) { return (kb + parts - 1) / parts; };
-    const auto sum = [&](int parts) { return parts > 1 ? 5000.0 + (double)parts * T * dm * 8 / (30.0 * sm_count()) : 0.0; };
+    // blocks of a part: of all segments, or of a share of one
+    const auto per_part = [&](int parts) { return parts == 1 ? kb * segments : (kb + parts / segments - 1) / (parts / segments); };
+    const auto sum = [&](int parts) { return parts > 1 ? 5000.0 + (double)parts * T * cols * 8 / (30.0 * sm_count()) : 0.0; };
     const auto drain = [](int parts) { return parts > 1 ? WIDE_DRAIN_F32 : WIDE_DRAIN_BF16; };
-    DownPlan best{false, F >= 4 * BK && split_contraction_pays(T, dm) ? 2 : 1};
-    if (!pair_mode() || T > 4096) return best;
-    double least = 0.95 * (plan_tiles(blocks(T) * best.parts, dm, per_part(best.parts), pairs, walk_by_columns(T, 1, dm, 1, kb),
-                                      drain(best.parts)).cycles + sum(best.parts));
+    ContractionPlan best{false, (segments > 1 || F >= 4 * BK) && split_contraction_pays(T, cols) ? 2 : 1};
+    if (!pair_mode() || T > SWAPPED_MAX_TOKENS) return best;
+    double least = 0.95 * (plan_tiles(blocks(T) * best.parts, cols, per_part(best.parts), pairs,
+                                      walk_by_columns(T, 1, cols, 1, per_part(best.parts)), drain(best.parts)).cycles + sum(best.parts));
     // (where the plain form has too few tiles, so has the exchanged one)
-    for (int parts = best.parts; parts <= 4 && per_part(parts) >= 8; ++parts) {
-        if (parts > 1 && ((dm & 7) || !split_contraction_enabled())) break;
-        const double c = plan_tiles(blocks(dm) * parts, (int)T, per_part(parts), pairs, false, drain(parts), true).cycles + sum(parts);
+    for (int parts = best.parts; parts <= 4; ++parts) {
+        if (parts > 1 && (parts % segments || per_part(parts) < 8 || (cols & 7) || !split_contraction_enabled())) continue;
+        const double c = plan_tiles(blocks(cols) * parts, (int)T, per_part(parts), pairs, false, drain(parts), true).cycles + sum(parts);
         if (c < least) {
             least = c;
             best = {true, parts};
@@ -882,7 +894,7 @@ struct TcForwardLayout {
     int ldf;        // leading dimension of the dense [*, F] arrays (multiple of 8)
     size_t off_g;   // fp32 G of one chunk [chunk, ldf]; later the partial outputs of a split down projection
     size_t g_floats;
-    DownPlan down;
+    ContractionPlan down;
     size_t off_u;   // bf16 U, rewritten in place into Z', for ALL tokens [T, ldf]
     size_t off_hint;  // bracket {center, width, tag}, statistics {sum, sum|dev|, rows}, CTA counter
     // MoC 2:8 on the sparse MMA: Z' in compressed form lives where U would (it is half as large), its metadata here
@@ -897,7 +909,8 @@ struct TcBackwardLayout {
     // MoC 2:8 with grad_x on the sparse MMA: dG' and dU' in compressed form [T, F / 2] with their metadata (sp_bytes == 0:
     // not used)
     size_t off_gc, off_uc, off_gmeta, off_umeta, sp_bytes;
-    size_t off_split, split_bytes;        // a few hundred tokens: two fp32 partial outputs [T, d] of the grad_x GEMM
+    size_t off_split, split_bytes;        // a few hundred tokens: fp32 partial outputs [T, d] of the grad_x GEMM
+    ContractionPlan dx;
 };
 
 inline int round_up8(int v) { return (v + 7) & ~7; }
@@ -934,7 +947,7 @@ inline TcForwardLayout tc_forward_layout(const moc_ffn_desc &d) {
     L.chunk = best * BM;
     size_t off = 0;
     L.off_g = off;
-    L.down = plan_down(d.tokens, d.d_ff, d.d_model);
+    L.down = plan_contraction(d.tokens, d.d_ff, d.d_model, 1);
     // (the gate values are dead when the down projection runs: its partial outputs take their buffer)
     L.g_floats = std::max<size_t>((size_t)L.chunk * L.ldf, L.down.parts > 1 ? (size_t)L.down.parts * d.tokens * d.d_model : 0);
     off = align_up(off + L.g_floats * 4, 256);
@@ -985,10 +998,11 @@ inline TcBackwardLayout tc_backward_layout(const moc_ffn_desc &d) {
         L.sp_bytes = 2 * comp + 2 * meta;
         off += L.sp_bytes;
     }
-    // fp32 partial outputs of the grad_x GEMM when its contraction is split (its two segments as two problems)
+    // fp32 partial outputs of the grad_x GEMM when its contraction is split
     L.off_split = off;
-    L.split_bytes = (!L.small_bytes && !L.sp_bytes && split_contraction_pays(d.tokens, d.d_model))
-                        ? align_up((size_t)2 * d.tokens * d.d_model * sizeof(float), 256) : 0;
+    L.dx = {false, 1};
+    if (!L.small_bytes && !L.sp_bytes) L.dx = plan_contraction(d.tokens, d.d_ff, d.d_model, 2);
+    L.split_bytes = L.dx.parts > 1 ? align_up((size_t)L.dx.parts * d.tokens * d.d_model * sizeof(float), 256) : 0;
     off += L.split_bytes;
     L.total = off;
     return L;

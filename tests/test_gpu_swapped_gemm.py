@@ -32,3 +32,26 @@ def test_forward_against_fp32(tokens, d, F, pad, K):
     ref = (torch.nn.functional.silu(G) * U * kept).bfloat16().float() @ wd[:F].float()
     assert (out.float() - ref).norm() <= 1e-2 * ref.norm()
     assert (out.float() - ref).abs().max() <= 0.05 * ref.abs().max()
+
+
+# one and two operand pairs per part; a part that ends inside a block; few and many tokens
+@pytest.mark.parametrize("tokens, d, F, K", ((257, 1032, 5460, 683), (300, 4096, 2048, 256), (513, 2048, 5504, 688), (1111, 2048, 5461, 683),
+                                             (1300, 520, 1000, 125), (2049, 768, 2048, 256)))
+def test_backward_against_fp32(tokens, d, F, K):
+    g = torch.Generator(device="cuda").manual_seed(tokens)
+    x, dD = (torch.randn(tokens, d, generator=g, device="cuda").bfloat16() for _ in range(2))
+    wg, wu, wd = ((torch.randn(F, d, generator=g, device="cuda") / d ** 0.5).bfloat16() for _ in range(3))
+    _, idx, tg, tu = B.moc_ffn_forward(x, wg, wu, wd, K)
+    got = B.moc_ffn_backward(x, wg, wu, wd, idx, tg, tu, dD)
+    assert B.moc_last_device_status() == B.MOC_OK
+    at, gv, uv = idx.long(), tg.float(), tu.float()
+    dz = (dD.float() @ wd.float().T).gather(1, at)
+    s = torch.sigmoid(gv)
+    dense = lambda v: torch.zeros(tokens, F, device="cuda").scatter_(1, at, v).bfloat16().float()  # noqa: E731
+    z, du, dg = dense(s * gv * uv), dense(dz * s * gv), dense(dz * uv * s * (1 + gv * (1 - s)))
+    want = {"grad_x": dg @ wg.float() + du @ wu.float(), "grad_w_down": z.T @ dD.float(), "grad_w_up": du.T @ x.float(),
+            "grad_w_gate": dg.T @ x.float()}
+    for name, w in want.items():
+        v = got[name].float()
+        assert (v - w).norm() <= 1e-2 * w.norm(), name
+        assert (v - w).abs().max() <= 0.05 * w.abs().max(), name
