@@ -84,8 +84,7 @@ enum KernelId {
     KID_FORWARD_TOKEN,
     KID_BACKWARD_TOKEN,
     KID_CSR_COUNT,
-    KID_CSR_SCAN_BLOCKS,
-    KID_CSR_SCAN_CHANNELS,
+    KID_CSR_SCAN,
     KID_CSR_FILL,
     KID_WGRAD_ROWS,
     KID_TOPK_SELECT,
@@ -118,7 +117,7 @@ enum KernelId {
 };
 static const char *const kKernelNames[KID_COUNT] = {
     "gate_gemm_alu", "select_rows",       "forward_token", "backward_token", "csr_count",
-    "csr_scan_blocks", "csr_scan_channels", "csr_fill",      "wgrad_rows",     "topk_select",
+    "csr_scan", "csr_fill",      "wgrad_rows",     "topk_select",
     "tc_gate_up_gemm", "tc_select_mask",  "tc_down_gemm",  "tc_bwd_sample",  "tc_dz_gemm",
     "tc_wgrad_gemm",   "tc_dx_gemm",      "tc_test_gemm",  "tc_select_hint", "dec_gate_gemv",
     "dec_select",      "dec_up",          "dec_down",      "sb_gate_up",     "sb_select",
@@ -217,7 +216,7 @@ ForwardPlan plan_forward(const moc_ffn_desc &d) {
 
 struct BackwardPlan {
     int tb, nb;  // tokens per block / number of token blocks of the channel-list build
-    size_t off_coef, off_counts, off_totals, off_rowstart, off_pairs, total;
+    size_t off_coef, off_counts, off_totals, off_rowstart, off_pairs, off_done, total;
 };
 
 BackwardPlan plan_backward(const moc_ffn_desc &d) {
@@ -236,6 +235,7 @@ BackwardPlan plan_backward(const moc_ffn_desc &d) {
     p.off_totals = c.take((size_t)d.d_ff * sizeof(uint32_t));
     p.off_rowstart = c.take(((size_t)d.d_ff + 1) * sizeof(uint32_t));
     p.off_pairs = c.take(TK * sizeof(uint32_t));
+    p.off_done = c.take(sizeof(unsigned int));
     p.total = c.off;
     return p;
 }
@@ -287,8 +287,17 @@ int forward_gather(const moc_ffn_desc &d, const T *x, const T *wg, const T *wu, 
 
     for (int64_t t0 = 0; t0 < d.tokens; t0 += p.chunk) {
         const int64_t n = std::min<int64_t>(p.chunk, d.tokens - t0);
-        dim3 grid((F + 63) / 64, (unsigned)((n + 63) / 64));
-        MOC_LAUNCH(KID_GATE_GEMM_ALU, st, (gemm_nt_alu_kernel<T><<<grid, 256, 0, st>>>(x + t0 * dm, wg, G, (int)n, F, dm, F)));
+        // tiles of 128 once they fill the SMs, of 64 once those do, else of 32
+        const auto tiles = [&](int side) { return dim3((unsigned)((F + side - 1) / side), (unsigned)((n + side - 1) / side)); };
+        const auto count = [&](int side) { return (int64_t)tiles(side).x * tiles(side).y; };
+        MOC_LAUNCH(KID_GATE_GEMM_ALU, st, {
+            if (count(128) >= tc::sm_count())
+                gemm_nt_alu_kernel<T, 128, 128, 8, 8, 16><<<tiles(128), 256, 0, st>>>(x + t0 * dm, wg, G, (int)n, F, dm, F);
+            else if (count(64) >= tc::sm_count())
+                gemm_nt_alu_kernel<T, 64, 64, 4, 4, 16><<<tiles(64), 256, 0, st>>>(x + t0 * dm, wg, G, (int)n, F, dm, F);
+            else
+                gemm_nt_alu_kernel<T, 32, 32, 4, 4, 32><<<tiles(32), 64, 0, st>>>(x + t0 * dm, wg, G, (int)n, F, dm, F);
+        });
         if ((rc = launch_ok()) != MOC_OK) return rc;
         if (d.flags & MOC_FLAG_SELECT_2_OF_8) {
             const unsigned grp_grid = (unsigned)std::min<int64_t>((n * (F / 8) + 255) / 256, 148 * 32);
@@ -344,12 +353,10 @@ int backward_gather(const moc_ffn_desc &d, const T *x, const T *wg, const T *wu,
     const size_t f_smem = (size_t)F * sizeof(uint32_t);
     if ((rc = set_smem(csr_count_kernel, f_smem)) != MOC_OK) return rc;
     if ((rc = set_smem(csr_fill_kernel, f_smem)) != MOC_OK) return rc;
-    MOC_LAUNCH(KID_CSR_COUNT, st, (csr_count_kernel<<<p.nb, 256, f_smem, st>>>(idx, d.tokens, K, F, p.tb, counts)));
+    unsigned int *done = reinterpret_cast<unsigned int *>(ws + p.off_done);
+    MOC_LAUNCH(KID_CSR_COUNT, st, (csr_count_kernel<<<p.nb, 256, f_smem, st>>>(idx, d.tokens, K, F, p.tb, counts, done)));
     if ((rc = launch_ok()) != MOC_OK) return rc;
-    MOC_LAUNCH(KID_CSR_SCAN_BLOCKS, st,
-               (csr_scan_blocks_kernel<<<(F + 255) / 256, 256, 0, st>>>(counts, p.nb, F, totals)));
-    if ((rc = launch_ok()) != MOC_OK) return rc;
-    MOC_LAUNCH(KID_CSR_SCAN_CHANNELS, st, (csr_scan_channels_kernel<<<1, 1024, 0, st>>>(totals, F, row_start)));
+    MOC_LAUNCH(KID_CSR_SCAN, st, (csr_scan_kernel<<<(F + 31) / 32, 1024, 0, st>>>(counts, p.nb, F, totals, row_start, done)));
     if ((rc = launch_ok()) != MOC_OK) return rc;
     MOC_LAUNCH(KID_CSR_FILL, st,
                (csr_fill_kernel<<<p.nb, 256, f_smem, st>>>(idx, d.tokens, K, F, p.tb, counts, row_start, pairs)));

@@ -15,56 +15,106 @@ namespace moc {
 constexpr int kTokenThreads = 256;
 
 // ------------------------------------------------------------------------------------------------
-// Dense gate projection on the ALUs:  C[M,N] (fp32) = A[M,Kd] * B[N,Kd]^T, both operands K-major.
-// 64x64 tile, 256 threads, 4x4 outputs per thread.  (Eq. (Moc-1), G = X W_gate.)
+// Dense gate projection on the ALUs:  C[M,N] (fp32) = A[M,Kd] * B[N,Kd]^T, both operands K-major, Kd a multiple of 8.
+// (Eq. (Moc-1), G = X W_gate.)  (BM / TM) x (BN / TN) threads, TM x TN outputs per thread.
+//
+// Large problems are bound by the FMA pipe if the operands come out of shared memory fast enough: 8 x 8 outputs read 64 bytes
+// per 64 FMAs (with 4 x 4: 32 per 16).  The next slab is loaded to registers while one is multiplied and goes into the other
+// buffer: one barrier per slab.  Small ones are bound by the chain of slabs, so they take small tiles (more CTAs) of long slabs.
+// 4096 x 2048 x 768: one buffer, 4 x 4 outputs and scalar loads took 541 us (24 TFLOP/s), now 341 (38); 256 x 512 x 128
+// 11.2 -> 5.3.
+// Every output is one chain of FMAs in ascending k, whatever the tile.
 template <typename T>
-__global__ void __launch_bounds__(256) gemm_nt_alu_kernel(const T *__restrict__ A, const T *__restrict__ B,
-                                                          float *__restrict__ C, int M, int N, int Kd, int ldc) {
-    constexpr int BM = 64, BN = 64, BK = 16;
-    __shared__ float As[BK][BM + 4];
-    __shared__ float Bs[BK][BN + 4];
-    const int tid = threadIdx.x;
-    const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-    const int tx = tid % 16, ty = tid / 16;
-    float acc[4][4] = {};
-    // each thread stages 4 A and 4 B elements per k-step: row = tid / 4, cols (tid % 4) * 4 .. +3
-    const int lr = tid / 4, lc = (tid % 4) * 4;
-    for (int k0 = 0; k0 < Kd; k0 += BK) {
+__device__ __forceinline__ float4 load4_f32(const T *p);
+template <>
+__device__ __forceinline__ float4 load4_f32<float>(const float *p) { return *reinterpret_cast<const float4 *>(p); }
+template <>
+__device__ __forceinline__ float4 load4_f32<__nv_bfloat16>(const __nv_bfloat16 *p) {
+    const uint2 w = *reinterpret_cast<const uint2 *>(p);
+    return make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xffff0000u), __uint_as_float(w.y << 16),
+                       __uint_as_float(w.y & 0xffff0000u));
+}
+
+template <typename T, int BM, int BN, int TM, int TN, int BK>
+__global__ void __launch_bounds__((BM / TM) * (BN / TN), 2) gemm_nt_alu_kernel(const T *__restrict__ A, const T *__restrict__ B,
+                                                                           float *__restrict__ C, int M, int N, int Kd, int ldc) {
+    constexpr int THREADS = (BM / TM) * (BN / TN), Q = BK / 4;  // Q: 4-element pieces of a row's slab
+    constexpr int NA = BM * Q / THREADS, NB = BN * Q / THREADS;
+    static_assert(BM * Q % THREADS == 0 && BN * Q % THREADS == 0 && TM % 4 == 0 && TN % 4 == 0, "tile");
+    __shared__ __align__(16) float As[2][BK][BM + 4], Bs[2][BK][BN + 4];
+    const int tid = threadIdx.x, m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
+    // a thread's outputs: groups of four rows (columns) BM / (TM / 4) apart, so that a warp's reads do not collide
+    constexpr int GM = BM / (TM / 4), GN = BN / (TN / 4);
+    const int tx = tid % (BN / TN), ty = tid / (BN / TN);
+    float acc[TM][TN] = {};
+    float4 ra[NA], rb[NB];
+    const auto load = [&](int k0) {
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const int kk = k0 + lc + c;
-            float a = 0.f, b = 0.f;
-            if (kk < Kd) {
-                if (m0 + lr < M) a = to_f32<T>(A[(int64_t)(m0 + lr) * Kd + kk]);
-                if (n0 + lr < N) b = to_f32<T>(B[(int64_t)(n0 + lr) * Kd + kk]);
-            }
-            As[lc + c][lr] = a;
-            Bs[lc + c][lr] = b;
+        for (int i = 0; i < NA; ++i) {
+            const int e = tid + i * THREADS, row = m0 + e / Q, k = k0 + e % Q * 4;
+            ra[i] = row < M && k < Kd ? load4_f32<T>(A + (int64_t)row * Kd + k) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
-        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < NB; ++i) {
+            const int e = tid + i * THREADS, row = n0 + e / Q, k = k0 + e % Q * 4;
+            rb[i] = row < N && k < Kd ? load4_f32<T>(B + (int64_t)row * Kd + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    };
+    const auto put = [&](int buf) {
+#pragma unroll
+        for (int i = 0; i < NA; ++i) {
+            const int e = tid + i * THREADS, row = e / Q, k = e % Q * 4;
+            As[buf][k][row] = ra[i].x;
+            As[buf][k + 1][row] = ra[i].y;
+            As[buf][k + 2][row] = ra[i].z;
+            As[buf][k + 3][row] = ra[i].w;
+        }
+#pragma unroll
+        for (int i = 0; i < NB; ++i) {
+            const int e = tid + i * THREADS, row = e / Q, k = e % Q * 4;
+            Bs[buf][k][row] = rb[i].x;
+            Bs[buf][k + 1][row] = rb[i].y;
+            Bs[buf][k + 2][row] = rb[i].z;
+            Bs[buf][k + 3][row] = rb[i].w;
+        }
+    };
+    load(0);
+    put(0);
+    __syncthreads();
+    for (int k0 = 0, buf = 0; k0 < Kd; k0 += BK, buf ^= 1) {
+        const bool more = k0 + BK < Kd;
+        if (more) load(k0 + BK);
 #pragma unroll
         for (int kk = 0; kk < BK; ++kk) {
-            float a[4], b[4];
+            float a[TM], b[TN];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                a[i] = As[kk][ty * 4 + i];
-                b[i] = Bs[kk][tx * 4 + i];
-            }
+            for (int i = 0; i < TM; i += 4) *reinterpret_cast<float4 *>(&a[i]) = *reinterpret_cast<const float4 *>(&As[buf][kk][i / 4 * GM + ty * 4]);
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int j = 0; j < TN; j += 4) *reinterpret_cast<float4 *>(&b[j]) = *reinterpret_cast<const float4 *>(&Bs[buf][kk][j / 4 * GN + tx * 4]);
 #pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+            for (int i = 0; i < TM; ++i)
+#pragma unroll
+                for (int j = 0; j < TN; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
         }
+        if (more) put(buf ^ 1);
         __syncthreads();
     }
+    const bool vec = (ldc & 3) == 0;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int m = m0 + ty * 4 + i;
+    for (int i = 0; i < TM; ++i) {
+        const int m = m0 + i / 4 * GM + ty * 4 + i % 4;
         if (m >= M) continue;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int n = n0 + tx * 4 + j;
-            if (n < N) C[(int64_t)m * ldc + n] = acc[i][j];
+        for (int j = 0; j < TN; j += 4) {
+            const int n = n0 + j / 4 * GN + tx * 4;
+            float *c = C + (int64_t)m * ldc + n;
+            if (vec && n + 4 <= N) {
+                *reinterpret_cast<float4 *>(c) = make_float4(acc[i][j], acc[i][j + 1], acc[i][j + 2], acc[i][j + 3]);
+            } else {
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    if (n + e < N) c[e] = acc[i][j + e];
+            }
         }
     }
 }
@@ -114,16 +164,29 @@ __device__ __forceinline__ void token_row_combine(int d, int K, const int *rowid
     for (int v = vl; v < nvec; v += lanes_v) {
         float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
         if (g < G) {
-            for (int k = g; k < K; k += G) {
-                const int j = rowidx[k];
-                if (j < 0) continue;  // invalid saved index: skipped (status already raised)
+            // four rows' loads are in flight together (an L2 round trip per row otherwise); the sum stays in the order of k
+            constexpr int ROWS = 4 / NSRC;
+            for (int k0 = g; k0 < K; k0 += ROWS * G) {
+                float w[ROWS][NSRC][8];
+                int j[ROWS];
 #pragma unroll
-                for (int s = 0; s < NSRC; ++s) {
-                    float w[8];
-                    Vec8<T>::load(roww(s) + (int64_t)j * d + 8 * v, w);
-                    const float c = coef(s, k);
+                for (int i = 0; i < ROWS; ++i) {
+                    const int k = k0 + i * G;
+                    j[i] = k < K ? rowidx[k] : -1;  // (negative: an invalid saved index, status already raised)
+                    if (j[i] >= 0) {
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) acc[e] = fmaf(c, w[e], acc[e]);
+                        for (int s = 0; s < NSRC; ++s) Vec8<T>::load(roww(s) + (int64_t)j[i] * d + 8 * v, w[i][s]);
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < ROWS; ++i) {
+                    if (j[i] < 0) continue;
+#pragma unroll
+                    for (int s = 0; s < NSRC; ++s) {
+                        const float c = coef(s, k0 + i * G);
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) acc[e] = fmaf(c, w[i][s][e], acc[e]);
+                    }
                 }
             }
         }
@@ -145,6 +208,36 @@ __device__ __forceinline__ void token_row_combine(int d, int K, const int *rowid
             __syncthreads();
         }
     }
+}
+
+// A warp's dot products of the vector in shared memory with DOT_ROWS rows k0, k0 + step, ... of W (negative index: none), their
+// loads in flight together; the product of row i comes back in lane i.
+// (100 tokens of 512 x 1365: step 168 -> 119 us with this, the rows taken together below and the gate projection; many tokens
+// are bound by L2, 4096 of 768 x 2048 read 6.4 GB in 597 us.)
+constexpr int DOT_ROWS = 4;
+template <typename T>
+__device__ __forceinline__ float warp_row_dots(const float *xs, const T *__restrict__ W, const int (&j)[DOT_ROWS], int d) {
+    const int lane = threadIdx.x & 31;
+    float acc[DOT_ROWS] = {};
+    for (int v = lane; v < (d >> 3); v += 32) {
+        float w[DOT_ROWS][8];
+#pragma unroll
+        for (int i = 0; i < DOT_ROWS; ++i)
+            if (j[i] >= 0) Vec8<T>::load(W + (int64_t)j[i] * d + 8 * v, w[i]);
+#pragma unroll
+        for (int i = 0; i < DOT_ROWS; ++i)
+            if (j[i] >= 0) {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) acc[i] = fmaf(xs[8 * v + e], w[i][e], acc[i]);
+            }
+    }
+    float mine = 0.f;
+#pragma unroll
+    for (int i = 0; i < DOT_ROWS; ++i) {
+        const float s = warp_sum(acc[i]);
+        if (lane == i) mine = s;
+    }
+    return mine;
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -177,21 +270,18 @@ __global__ void __launch_bounds__(kTokenThreads) forward_token_kernel(
     for (int k = tid; k < K; k += kTokenThreads) js[k] = idx[t * K + k];
     __syncthreads();
     const float *gt = G + t * (int64_t)ldg;
-    for (int k = warp; k < K; k += kTokenThreads / 32) {
-        const int j = js[k];
-        const T *wr = w_up + (int64_t)j * d;
-        float acc = 0.f;
-        for (int v = lane; v < (d >> 3); v += 32) {
-            float w[8];
-            Vec8<T>::load(wr + 8 * v, w);
+    constexpr int NW = kTokenThreads / 32;
+    for (int k0 = warp; k0 < K; k0 += DOT_ROWS * NW) {
+        int j[DOT_ROWS];
 #pragma unroll
-            for (int e = 0; e < 8; ++e) acc = fmaf(xs[8 * v + e], w[e], acc);
-        }
-        acc = warp_sum(acc);
-        if (lane == 0) {
-            const float g = gt[j];
-            zs[k] = silu_f(g) * acc;
-            if (topk_up) topk_up[t * K + k] = from_f32<T>(acc);
+        for (int i = 0; i < DOT_ROWS; ++i) j[i] = k0 + i * NW < K ? js[k0 + i * NW] : -1;
+        const int k = k0 + lane * NW;
+        const bool mine = lane < DOT_ROWS && k < K;
+        const float g = mine ? gt[js[k]] : 0.f;  // (its load is in flight beside the rows')
+        const float u = warp_row_dots<T>(xs, w_up, j, d);
+        if (mine) {
+            zs[k] = silu_f(g) * u;
+            if (topk_up) topk_up[t * K + k] = from_f32<T>(u);
         }
     }
     __syncthreads();
@@ -234,27 +324,23 @@ __global__ void __launch_bounds__(kTokenThreads) backward_token_kernel(
         js[k] = j;
     }
     __syncthreads();
-    for (int k = warp; k < K; k += kTokenThreads / 32) {
-        const int j = js[k];
-        float z = 0.f, dU = 0.f, dG = 0.f;
-        if (j >= 0) {
-            const T *wr = w_down + (int64_t)j * d;
-            float acc = 0.f;
-            for (int v = lane; v < (d >> 3); v += 32) {
-                float w[8];
-                Vec8<T>::load(wr + 8 * v, w);
+    constexpr int NW = kTokenThreads / 32;
+    for (int k0 = warp; k0 < K; k0 += DOT_ROWS * NW) {
+        int j[DOT_ROWS];
 #pragma unroll
-                for (int e = 0; e < 8; ++e) acc = fmaf(ds[8 * v + e], w[e], acc);
+        for (int i = 0; i < DOT_ROWS; ++i) j[i] = k0 + i * NW < K ? js[k0 + i * NW] : -1;
+        const int k = k0 + lane * NW;
+        const bool mine = lane < DOT_ROWS && k < K;
+        const float g = mine ? to_f32<T>(topk_gate[t * K + k]) : 0.f, u = mine ? to_f32<T>(topk_up[t * K + k]) : 0.f;
+        const float dz = warp_row_dots<T>(ds, w_down, j, d);
+        if (mine) {
+            float z = 0.f, dU = 0.f, dG = 0.f;
+            if (js[k] >= 0) {
+                const float s = silu_f(g);
+                z = s * u;
+                dU = s * dz;
+                dG = u * dz * dsilu_f(g);
             }
-            const float dz = warp_sum(acc);
-            const float g = to_f32<T>(topk_gate[t * K + k]);
-            const float u = to_f32<T>(topk_up[t * K + k]);
-            const float s = silu_f(g);
-            z = s * u;
-            dU = s * dz;
-            dG = u * dz * dsilu_f(g);
-        }
-        if (lane == 0) {
             dgs[k] = dG;
             dus[k] = dU;
             if (coef) {
@@ -280,8 +366,9 @@ __global__ void __launch_bounds__(kTokenThreads) backward_token_kernel(
 //   pairs [T*K]     : pair id p = t*K + k, grouped by channel, tokens ascending
 // Token block b covers tokens [b*tb, min(T,(b+1)*tb)).
 __global__ void __launch_bounds__(256) csr_count_kernel(const int16_t *__restrict__ idx, int64_t T, int K, int F,
-                                                        int tb, uint32_t *__restrict__ counts) {
+                                                        int tb, uint32_t *__restrict__ counts, unsigned int *done) {
     extern __shared__ __align__(16) uint32_t cnt[];
+    if (blockIdx.x == 0 && threadIdx.x == 0) *done = 0;
     for (int j = threadIdx.x; j < F; j += 256) cnt[j] = 0;
     __syncthreads();
     const int64_t t0 = (int64_t)blockIdx.x * tb;
@@ -296,31 +383,54 @@ __global__ void __launch_bounds__(256) csr_count_kernel(const int16_t *__restric
     for (int j = threadIdx.x; j < F; j += 256) o[j] = cnt[j];
 }
 
-// thread per channel: exclusive prefix over the token blocks; totals[j] = list length
-__global__ void __launch_bounds__(256) csr_scan_blocks_kernel(uint32_t *__restrict__ counts, int nb, int F,
-                                                              uint32_t *__restrict__ totals) {
-    const int j = blockIdx.x * 256 + threadIdx.x;
-    if (j >= F) return;
-    uint32_t run = 0;
-    for (int b = 0; b < nb; ++b) {
-        const uint32_t c = counts[(int64_t)b * F + j];
-        counts[(int64_t)b * F + j] = run;
-        run += c;
-    }
-    totals[j] = run;
-}
-
-// single CTA: exclusive scan of totals[F] -> row_start[F+1]
-__global__ void __launch_bounds__(1024) csr_scan_channels_kernel(const uint32_t *__restrict__ totals, int F,
-                                                                 uint32_t *__restrict__ row_start) {
+// A CTA for 32 channels: exclusive prefix over the token blocks, a warp for each 32nd of them (the loads of a channel's counts
+// one after the other took 66 us for 512 blocks); totals[j] = list length.  The last CTA to finish scans the totals:
+// row_start[F + 1].  done: zeroed by csr_count_kernel.
+__global__ void __launch_bounds__(1024) csr_scan_kernel(uint32_t *__restrict__ counts, int nb, int F, uint32_t *totals,
+                                                        uint32_t *__restrict__ row_start, unsigned int *done) {
+    __shared__ uint32_t part[32][33];
     __shared__ uint32_t wtot[32];
     __shared__ uint32_t carry;
+    __shared__ unsigned int s_last;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (tid == 0) carry = 0;
+    const int j0 = blockIdx.x * 32 + lane, per = (nb + 31) / 32;
+    const int b0 = min(warp * per, nb), b1 = min(b0 + per, nb);
+    uint32_t sum = 0;
+    if (j0 < F) {
+        const uint32_t *c = counts + j0;
+#pragma unroll 8
+        for (int b = b0; b < b1; ++b) sum += c[(int64_t)b * F];
+    }
+    part[warp][lane] = sum;
     __syncthreads();
+    uint32_t run = 0;
+    for (int w = 0; w < warp; ++w) run += part[w][lane];
+    if (j0 < F) {
+        uint32_t *c = counts + j0;
+        for (int b = b0; b < b1; b += 8) {
+            uint32_t v[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) v[i] = b + i < b1 ? c[(int64_t)(b + i) * F] : 0u;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                if (b + i < b1) c[(int64_t)(b + i) * F] = run;
+                run += v[i];
+            }
+        }
+        if (warp == 31) __stcg(&totals[j0], run);
+    }
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) {
+        s_last = atomicAdd(done, 1u) == gridDim.x - 1 ? 1u : 0u;
+        carry = 0;
+    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
     for (int base = 0; base < F; base += 1024) {
         const int j = base + tid;
-        const uint32_t v = j < F ? totals[j] : 0u;
+        const uint32_t v = j < F ? __ldcg(&totals[j]) : 0u;
         uint32_t s = v;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
