@@ -346,6 +346,18 @@ int backward_gather(const moc_ffn_desc &d, const T *x, const T *wg, const T *wu,
         return MOC_OK;
     }
 
+    const size_t red = token_red_floats(dm) * 3 * sizeof(float);
+    const int accumulate = (d.flags & MOC_FLAG_ACCUMULATE_WGRAD) ? 1 : 0;
+    if (list_scans_pay(d.tokens, K, d.d_ff_ld)) {
+        const size_t smem = red + (size_t)d.tokens * (sizeof(uint32_t) + sizeof(int16_t));
+        if ((rc = set_smem(wgrad_rows_kernel<T, true>, smem)) != MOC_OK) return rc;
+        MOC_LAUNCH(KID_WGRAD_ROWS, st,
+                   (wgrad_rows_kernel<T, true><<<d.d_ff_ld, kTokenThreads, smem, st>>>(
+                       x, dout, coef, TK, nullptr, nullptr, idx, (int)d.tokens, dm, F, K, gwg, gwu, gwd, accumulate)));
+        if ((rc = launch_ok()) != MOC_OK) return rc;
+        if (wgrad_done && cudaEventRecord(wgrad_done, st) != cudaSuccess) return MOC_ERR_CUDA;
+        return MOC_OK;
+    }
     uint32_t *counts = reinterpret_cast<uint32_t *>(ws + p.off_counts);
     uint32_t *totals = reinterpret_cast<uint32_t *>(ws + p.off_totals);
     uint32_t *row_start = reinterpret_cast<uint32_t *>(ws + p.off_rowstart);
@@ -362,12 +374,10 @@ int backward_gather(const moc_ffn_desc &d, const T *x, const T *wg, const T *wu,
                (csr_fill_kernel<<<p.nb, 256, f_smem, st>>>(idx, d.tokens, K, F, p.tb, counts, row_start, pairs)));
     if ((rc = launch_ok()) != MOC_OK) return rc;
 
-    const size_t red = token_red_floats(dm) * 3 * sizeof(float);
-    if ((rc = set_smem(wgrad_rows_kernel<T>, red)) != MOC_OK) return rc;
+    if ((rc = set_smem(wgrad_rows_kernel<T, false>, red)) != MOC_OK) return rc;
     MOC_LAUNCH(KID_WGRAD_ROWS, st,
-               (wgrad_rows_kernel<T><<<d.d_ff_ld, kTokenThreads, red, st>>>(
-                   x, dout, coef, TK, row_start, pairs, dm, F, K, gwg, gwu, gwd,
-                   (d.flags & MOC_FLAG_ACCUMULATE_WGRAD) ? 1 : 0)));
+               (wgrad_rows_kernel<T, false><<<d.d_ff_ld, kTokenThreads, red, st>>>(
+                   x, dout, coef, TK, row_start, pairs, idx, (int)d.tokens, dm, F, K, gwg, gwu, gwd, accumulate)));
     if ((rc = launch_ok()) != MOC_OK) return rc;
     if (wgrad_done && cudaEventRecord(wgrad_done, st) != cudaSuccess) return MOC_ERR_CUDA;
     return MOC_OK;

@@ -478,12 +478,62 @@ __global__ void __launch_bounds__(256) csr_fill_kernel(const int16_t *__restrict
 //   grad_w_up  [j,:] = sum_p dU_p * x[t_p,:]
 //   grad_w_gate[j,:] = sum_p dG_p * x[t_p,:]          p over the channel's (token, slot) pairs
 // Rows no token selected (and padding rows) are written as exact zeros.
-template <typename T>
+//
+// FIND: every CTA finds its channel's pairs in idx itself (list_scans_pay: while all CTAs together read little), and no lists are
+// built.  256 tokens, K = 64, 512 channels: 512 x 32 KiB out of L2, and three launches fewer in front of 11 us of work
+// (step 95.8 -> 88; 100 tokens of 512 x 1365: 116 -> 108).
+constexpr int kFindTokens = 4096;
+constexpr int64_t kFindBytes = 64 << 20;  // some 8 us of L2 reads, against the 16 or more of the kernels that build the lists
+inline bool list_scans_pay(int64_t tokens, int K, int rows) {
+    return tokens <= kFindTokens && tokens * K * 2 * rows <= kFindBytes;
+}
+// list[0..n) = the pairs of channel j, tokens ascending; slot: scratch, one entry per token.  Returns n.
+__device__ __forceinline__ int find_pairs(const int16_t *__restrict__ idx, int tokens, int K, int j, int16_t *slot, uint32_t *list) {
+    __shared__ int s_warp[kTokenThreads / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, TK = tokens * K;
+    for (int t = tid; t < tokens; t += kTokenThreads) slot[t] = -1;
+    __syncthreads();
+    // (channels of one token are distinct: at most one match each)
+    const auto check = [&](int e, int v) {
+        if (v == j) slot[e / K] = (int16_t)(e % K);
+    };
+    const int whole = (reinterpret_cast<uintptr_t>(idx) & 15u) == 0 ? TK / 8 : 0;
+#pragma unroll 4
+    for (int q = tid; q < whole; q += kTokenThreads) {
+        const uint4 v = reinterpret_cast<const uint4 *>(idx)[q];
+        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            check(8 * q + 2 * i, (int)(int16_t)(w[i] & 0xffffu));
+            check(8 * q + 2 * i + 1, (int)(int16_t)(w[i] >> 16));
+        }
+    }
+#pragma unroll 4
+    for (int e = 8 * whole + tid; e < TK; e += kTokenThreads) check(e, idx[e]);
+    __syncthreads();
+    int n = 0;
+    for (int base = 0; base < tokens; base += kTokenThreads) {
+        const int t = base + tid, k = t < tokens ? slot[t] : -1;
+        const uint32_t hits = __ballot_sync(0xffffffffu, k >= 0);
+        if (lane == 0) s_warp[warp] = __popc(hits);
+        __syncthreads();
+        int at = n;
+        for (int w = 0; w < kTokenThreads / 32; ++w) {
+            if (w < warp) at += s_warp[w];
+            n += s_warp[w];
+        }
+        if (k >= 0) list[at + __popc(hits & ((1u << lane) - 1u))] = (uint32_t)(t * K + k);
+        __syncthreads();
+    }
+    return n;
+}
+
+template <typename T, bool FIND>
 __global__ void __launch_bounds__(kTokenThreads) wgrad_rows_kernel(
     const T *__restrict__ x, const T *__restrict__ grad_out, const float *__restrict__ coef, int64_t TK,
-    const uint32_t *__restrict__ row_start, const uint32_t *__restrict__ pairs, int d, int F, int K,
-    T *__restrict__ gw_gate, T *__restrict__ gw_up, T *__restrict__ gw_down, int accumulate) {
-    extern __shared__ __align__(16) float red[];  // [G][3][d] when G > 1
+    const uint32_t *__restrict__ row_start, const uint32_t *__restrict__ pairs, const int16_t *__restrict__ idx, int tokens, int d,
+    int F, int K, T *__restrict__ gw_gate, T *__restrict__ gw_up, T *__restrict__ gw_down, int accumulate) {
+    extern __shared__ __align__(16) float red[];  // [G][3][d] when G > 1; FIND: the list and the slots behind it
     const int j = blockIdx.x;
     const int tid = threadIdx.x;
     const int nvec = d >> 3;
@@ -491,7 +541,11 @@ __global__ void __launch_bounds__(kTokenThreads) wgrad_rows_kernel(
     const int G = kTokenThreads / lanes_v;
     const int g = tid / lanes_v, vl = tid % lanes_v;
     uint32_t p0 = 0, p1 = 0;
-    if (j < F) {
+    if constexpr (FIND) {
+        uint32_t *list = reinterpret_cast<uint32_t *>(red + (G > 1 ? 3 * G * d : 0));
+        if (j < F) p1 = (uint32_t)find_pairs(idx, tokens, K, j, reinterpret_cast<int16_t *>(list + tokens), list);
+        pairs = list;
+    } else if (j < F) {
         p0 = row_start[j];
         p1 = row_start[j + 1];
     }

@@ -8,9 +8,9 @@ pytestmark = pytest.mark.gpu
 
 
 # tiles of 32, 64 and 128 with rows, columns and contraction off their sizes; K off the rows taken at once; one token, few
-# and many token blocks of the channel lists
-@pytest.mark.parametrize("tokens, d, F, K", ((1, 8, 9, 5), (33, 40, 31, 31), (256, 128, 512, 64), (770, 24, 833, 7), (1665, 136, 1501, 33),
-                                             (4100, 16, 600, 3)))
+# and many token blocks of the channel lists, and the channels' pairs found without lists (up to 4096 tokens)
+@pytest.mark.parametrize("tokens, d, F, K", ((1, 8, 9, 5), (33, 40, 31, 31), (256, 128, 512, 64), (257, 24, 1000, 127), (4096, 8, 64, 8),
+                                             (4097, 8, 64, 8), (770, 24, 833, 7), (1665, 136, 1501, 33), (4100, 16, 600, 3)))
 def test_f32_against_fp64(tokens, d, F, K):
     g = torch.Generator(device="cuda").manual_seed(tokens)
     x, dD = (torch.randn(tokens, d, generator=g, device="cuda") for _ in range(2))
