@@ -99,6 +99,18 @@ void *stream_of(PyObject *stream) {
 // ---- the autograd node ----------------------------------------------------------------------------------------
 // Between forward and backward only the compact Top-K activations live (Section 4, Table 1, column "MoC+GCP"), plus x.
 // recompute_up drops the up values as well; backward forms them again from x, w_up and the indices.
+// They share one allocation, and what backward has to know about the call is one list: with few tokens the step takes as long
+// as its host work (256 tokens of 128 x 512 in fp32: 88 us, of which an allocation is about one).
+struct Kept {
+    int64_t gate, up, total;  // byte offsets behind the indices
+    explicit Kept(const moc_ffn_desc &d, bool with_up) {
+        const int64_t n = d.tokens * d.k, e = d.dtype == MOC_BF16 ? 2 : 4;
+        const auto aligned = [](int64_t v) { return (v + 255) / 256 * 256; };
+        gate = aligned(2 * n);
+        up = aligned(gate + e * n);
+        total = with_up ? up + e * n : up;
+    }
+};
 struct MocFfnNode : public torch::autograd::Function<MocFfnNode> {
     static Tensor forward(torch::autograd::AutogradContext *ctx, const Tensor &x, const Tensor &w_gate, const Tensor &w_up,
                           const Tensor &w_down, int64_t k, int64_t d_ff, int64_t flags, bool recompute_up) {
@@ -106,62 +118,67 @@ struct MocFfnNode : public torch::autograd::Function<MocFfnNode> {
         const Tensor x2 = x.dim() == 2 && x.is_contiguous() ? x : x.reshape({-1, x.size(-1)}).contiguous();
         check_all(x2, w_gate, w_up, w_down);
         const moc_ffn_desc d = make_desc(x2, w_gate, k, d_ff, (uint32_t)flags);
-        Tensor out = at::empty_like(x2), idx, tg, tu;
+        Tensor out = at::empty_like(x2), kept;
+        char *idx = nullptr, *tg = nullptr, *tu = nullptr;
         if (save) {
-            idx = at::empty({d.tokens, d.k}, x2.options().dtype(at::kShort));
-            tg = at::empty({d.tokens, d.k}, x2.options());
-            tu = at::empty({d.tokens, d.k}, x2.options());
+            const Kept at(d, !recompute_up);
+            kept = at::empty({at.total}, x2.options().dtype(at::kByte));
+            idx = static_cast<char *>(outp(kept));
+            tg = idx + at.gate;
+            tu = idx + at.up;
+        }
+        Tensor dropped;  // the up values of a call that forms them again later
+        if (save && recompute_up) {
+            dropped = at::empty({d.tokens, d.k}, x2.options());
+            tu = static_cast<char *>(outp(dropped));
         }
         const Tensor ws = workspace_for(d, MOC_OP_FORWARD, x2);
-        const int rc = moc_ffn_forward(&d, in(x2), in(w_gate), in(w_up), in(w_down), outp(out), static_cast<int16_t *>(outp(idx)),
-                                       outp(tg), outp(tu), outp(ws), (size_t)ws.numel(), c10::cuda::getCurrentCUDAStream().stream());
+        const int rc = moc_ffn_forward(&d, in(x2), in(w_gate), in(w_up), in(w_down), outp(out), reinterpret_cast<int16_t *>(idx), tg, tu,
+                                       outp(ws), (size_t)ws.numel(), c10::cuda::getCurrentCUDAStream().stream());
         if (rc != MOC_OK) raise_moc(rc, "moc_ffn_forward");
         if (save) {
-            ctx->save_for_backward(recompute_up ? torch::autograd::variable_list{x2, w_gate, w_up, w_down, idx, tg}
-                                                : torch::autograd::variable_list{x2, w_gate, w_up, w_down, idx, tg, tu});
-            ctx->saved_data["d_ff"] = d_ff;
+            ctx->save_for_backward({x2, w_gate, w_up, w_down, kept});
             // the Top-K after the activation changes the choice of channels only: backward takes the mask as saved
-            ctx->saved_data["flags"] = flags & (int64_t)MOC_FLAG_SELECT_2_OF_8;
-            ctx->saved_data["shape"] = x.sizes();
+            std::vector<int64_t> call{d.k, d_ff, flags & (int64_t)MOC_FLAG_SELECT_2_OF_8, recompute_up ? 1 : 0};
+            if (x.dim() != 2) call.insert(call.end(), x.sizes().begin(), x.sizes().end());
+            ctx->saved_data["call"] = std::move(call);
         }
         return x.dim() == 2 ? out : out.reshape(x.sizes());
     }
 
     static torch::autograd::variable_list backward(torch::autograd::AutogradContext *ctx, torch::autograd::variable_list grads) {
         const auto saved = ctx->get_saved_variables();
-        const Tensor &x = saved[0], &w_gate = saved[1], &w_up = saved[2], &w_down = saved[3], &idx = saved[4], &tg = saved[5];
-        const int64_t d_ff = ctx->saved_data["d_ff"].toInt();
-        const uint32_t flags = (uint32_t)ctx->saved_data["flags"].toInt();
+        const Tensor &x = saved[0], &w_gate = saved[1], &w_up = saved[2], &w_down = saved[3], &kept = saved[4];
+        const std::vector<int64_t> call = ctx->saved_data["call"].toIntVector();  // k, d_ff, flags, recompute_up, x's shape unless 2-D
         torch::autograd::variable_list res(8);
         if (!grads[0].defined()) return res;
         const Tensor &g0 = grads[0];
         const Tensor go = g0.dim() == 2 && g0.is_contiguous() ? g0 : g0.reshape({-1, g0.size(-1)}).contiguous();
         check_dev(go);
-        moc_ffn_desc d = make_desc(x, w_gate, idx.size(1), d_ff, flags);
+        moc_ffn_desc d = make_desc(x, w_gate, call[0], call[1], (uint32_t)call[2]);
         void *stream = c10::cuda::getCurrentCUDAStream().stream();
         const Tensor ws = workspace_for(d, MOC_OP_BACKWARD, x);
-        Tensor tu;
-        if (saved.size() > 6) {
-            tu = saved[6];
-        } else {
-            tu = at::empty(tg.sizes(), tg.options());
+        const Kept at(d, call[3] == 0);
+        const char *base = static_cast<const char *>(in(kept));
+        const int16_t *idx = reinterpret_cast<const int16_t *>(base);
+        const void *tg = base + at.gate, *tu = base + at.up;
+        Tensor again;
+        if (call[3]) {
+            again = at::empty({d.tokens, d.k}, x.options());
+            tu = outp(again);
             moc_ffn_desc plain = d;
             plain.flags = 0;
-            const int rc = moc_ffn_recompute_up(&plain, in(x), in(w_up), static_cast<const int16_t *>(in(idx)), outp(tu), outp(ws),
-                                                (size_t)ws.numel(), stream);
+            const int rc = moc_ffn_recompute_up(&plain, in(x), in(w_up), idx, outp(again), outp(ws), (size_t)ws.numel(), stream);
             if (rc != MOC_OK) raise_moc(rc, "moc_ffn_recompute_up");
         }
         const Tensor *like[4] = {&x, &w_gate, &w_up, &w_down};
         for (int i = 0; i < 4; ++i)
             if (ctx->needs_input_grad(i)) res[i] = at::empty_like(*like[i]);
-        const int rc = moc_ffn_backward(&d, in(x), in(w_gate), in(w_up), in(w_down), static_cast<const int16_t *>(in(idx)), in(tg),
-                                        in(tu), in(go), outp(res[0]), outp(res[1]), outp(res[2]), outp(res[3]), outp(ws),
+        const int rc = moc_ffn_backward(&d, in(x), in(w_gate), in(w_up), in(w_down), idx, tg, tu, in(go),
+                                        outp(res[0]), outp(res[1]), outp(res[2]), outp(res[3]), outp(ws),
                                         (size_t)ws.numel(), stream);
         if (rc != MOC_OK) raise_moc(rc, "moc_ffn_backward");
-        if (res[0].defined()) {
-            const auto shape = ctx->saved_data["shape"].toIntVector();
-            if (shape.size() != 2) res[0] = res[0].reshape(shape);
-        }
+        if (res[0].defined() && call.size() > 4) res[0] = res[0].reshape(at::IntArrayRef(call).slice(4));
         return res;
     }
 };
