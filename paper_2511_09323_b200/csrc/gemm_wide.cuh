@@ -9,35 +9,22 @@
 // the second's last blocks and its next tile starts while the second is being drained.
 //
 // The tiles need not have one width.  With few tiles, or a last wave that few of them fill, the remaining rows (or columns)
-// are cut into narrower ones, in steps of 64 columns, so that all pairs finish together: plan_tiles() below chooses.
+// are cut into narrower ones, in steps of 64 columns, so that all pairs finish together: plan_tiles() (tile_plan.h) chooses.
 //
 // Roles: warp 0 TMA loads, warp 1 MMAs (leading CTA) and the TMEM allocation, warps 2..9 epilogue, two per TMEM lane quarter.
 // Barriers as in the pair kernel of tc_gemm.cuh.
 #pragma once
 
-#include <algorithm>
-#include <mutex>
-#include <unordered_map>
-
 #include "tc_gemm.cuh"
+#include "tile_plan.h"
 
 namespace moc {
 namespace tc {
 
-constexpr int WIDE_N = 512, WIDE_STEP = 64, WIDE_SKEW = 2;
 constexpr int WIDE_THREADS = 320, WIDE_EPI_WARPS = 8, WIDE_STAGES_MAX = 6;
 constexpr uint32_t WIDE_B_BYTES = (BN / 2) * BK * 2;  // one accumulator's half of B in a stage, at most
 constexpr uint32_t WIDE_RING_BYTES = 192 * 1024;      // 4 stages of A | B | B, or 6 of A | B where no tile is wider than 256
 constexpr size_t WIDE_SMEM_BYTES = 1024 + WIDE_RING_BYTES + BAR_REGION_BYTES + WIDE_EPI_WARPS * EPI_BOX_BYTES;
-
-// How the output is cut.  Rows: 256-row blocks of all problems.  The first `t1` tiles are w1 columns wide, the others w2.
-//   by_columns == 0: rows one after the other, their tiles from left to right; the first `split` rows have wide tiles
-//   by_columns == 1: column by column, all rows in turn (few rows and a large B: B is read once); the first `split` columns
-//                    have wide tiles
-struct TilePlan {
-    int rows, by_columns, split, w1, nt1, w2, nt2, t1, total;
-    double cycles;  // of the pair that finishes last, by the model below
-};
 
 struct WideParams {
     Params g;
@@ -458,90 +445,6 @@ __global__ void __launch_bounds__(WIDE_THREADS, 1) gemm_wide_kernel(const __grid
         tc_fence_after();
         tmem_dealloc_pair(tmem_base, TMEM_COLS);
     }
-}
-
-// SM cycles a pair needs for one contraction block of a tile of w columns: its MMAs, or the loads at what an SM gets from L2
-inline double wide_block_cycles(int w) { return std::max(2.06 * w, (16384.0 + 64.0 * w) / 58.0); }
-
-// Cycles in which the epilogue moves an accumulator of 256 columns (bf16, fp32 outputs).
-constexpr int WIDE_DRAIN_BF16 = 2000, WIDE_DRAIN_F32 = 3500;
-
-// Tiles of `rows` x N for `pairs` CTA pairs: wide ones for as many whole waves as there are (or one fewer), the rest in the
-// one width that finishes first; or that width throughout.  (Measured at d_model 2048, d_ff 5504: down projection of 1111
-// tokens, 40 tiles of 256 columns for 74 pairs, 36.8 us; 55 of 192.)  Remembered per problem size.
-// drain: cycles in which the epilogue moves an accumulator of 256 columns.  Of a tile with two accumulators the part of it
-// that the skew does not cover is lost; with one, the other is worked in meanwhile.
-// any_first: the first tiles may have any width, not 512 alone (few columns: one tile as wide as they are spans them).
-inline TilePlan plan_tiles(int rows, int N, int kb, int pairs, bool by_columns, int drain, bool any_first = false) {
-    struct Key {
-        int rows, n, kb, pairs, by_columns, drain;
-        bool operator==(const Key &o) const {
-            return rows == o.rows && n == o.n && kb == o.kb && pairs == o.pairs && by_columns == o.by_columns && drain == o.drain;
-        }
-    };
-    struct Hash {
-        size_t operator()(const Key &k) const {
-            uint64_t h = 0x9e3779b97f4a7c15ull;
-            for (const int v : {k.rows, k.n, k.kb, k.pairs, k.by_columns, k.drain}) h = (h ^ (uint64_t)(uint32_t)v) * 0xff51afd7ed558ccdull;
-            return (size_t)(h ^ (h >> 32));
-        }
-    };
-    static std::mutex mu;
-    static std::unordered_map<Key, TilePlan, Hash> known;
-    const Key key{rows, N, kb, pairs, (by_columns ? 1 : 0) + (any_first ? 2 : 0), drain};
-    {
-        std::lock_guard<std::mutex> lock(mu);
-        auto it = known.find(key);
-        if (it != known.end()) return it->second;
-    }
-    const auto tile_cycles = [&](int w_of) {
-        const int w = std::min(w_of, (N + WIDE_STEP - 1) / WIDE_STEP * WIDE_STEP);
-        const double mma = kb * wide_block_cycles(w) + 350.0;
-        return w > BN ? mma + std::max(0, drain - WIDE_SKEW * 512) : std::max(mma, drain * w / 256.0);
-    };
-    const auto up = [](int64_t a, int64_t b) { return (int)((a + b - 1) / b); };
-    TilePlan best{};
-    const auto consider = [&](int w1, int split, int w2) {
-        TilePlan t{};
-        t.rows = rows;
-        t.by_columns = by_columns ? 1 : 0;
-        t.split = split;
-        t.w1 = w1;
-        t.nt1 = up(N, w1);
-        t.w2 = w2;
-        if (by_columns) {
-            t.t1 = split / w1 * rows;
-            t.nt2 = split < N ? up(N - split, w2) : 0;
-            t.total = t.t1 + t.nt2 * rows;
-        } else {
-            t.t1 = split * t.nt1;
-            t.nt2 = up(N, w2);
-            t.total = t.t1 + (rows - split) * t.nt2;
-        }
-        // tiles go round the pairs in turn: pair j has every pairs-th one from j on
-        for (int j = 0; j < pairs; ++j) {
-            const int n1 = t.t1 > j ? (t.t1 - 1 - j) / pairs + 1 : 0, n = t.total > j ? (t.total - 1 - j) / pairs + 1 : 0;
-            t.cycles = std::max(t.cycles, n1 * tile_cycles(w1) + (n - n1) * tile_cycles(w2));
-        }
-        if (best.total == 0 || t.cycles < best.cycles) best = t;
-    };
-    const int most = any_first ? std::min(WIDE_N, up(N, WIDE_STEP) * WIDE_STEP) : WIDE_N;
-    for (int w1 = most; w1 >= (any_first ? WIDE_STEP : WIDE_N); w1 -= WIDE_STEP) {
-        const int units = by_columns ? N / w1 : rows;                  // what is split off as wide: columns' tiles or rows
-        const int per_unit = by_columns ? rows : up(N, w1);            // tiles of one
-        const int waves = (int)((int64_t)units * per_unit / pairs);
-        for (int w2 = most; w2 >= WIDE_STEP; w2 -= WIDE_STEP) {
-            if (w1 == most) consider(w1, 0, w2);
-            for (int f = waves; f >= std::max(1, waves - 1); --f) {
-                const int u = std::min<int64_t>(units, (int64_t)f * pairs / per_unit);
-                for (int v = u; v >= std::max(1, u - 1); --v) consider(w1, by_columns ? v * w1 : v, w2);
-            }
-        }
-    }
-    std::lock_guard<std::mutex> lock(mu);
-    if (known.size() > 512) known.clear();
-    known[key] = best;
-    return best;
 }
 
 }  // namespace tc

@@ -10,6 +10,7 @@
 #pragma once
 
 #include <cuda.h>
+#include <algorithm>
 #include <cstdlib>
 #include <cstring>
 #include <cuda_runtime.h>
@@ -250,9 +251,9 @@ inline bool swapped_projection_pays(int64_t T, int F, int kb, int problems, int 
     if (!pair_mode() || T > SWAPPED_MAX_TOKENS) return false;
     const int pairs = sm_count() / 2;
     const auto blocks = [](int64_t n) { return (int)((n + 255) / 256); };
-    const TilePlan plain = plan_tiles(problems * blocks(T), F, kb, pairs, walk_by_columns(T, 1, F, problems, kb), drain);
-    const TilePlan swapped = plan_tiles(problems * blocks(F), (int)T, kb, pairs, false, drain, true);
-    return swapped.cycles < 0.95 * plain.cycles;
+    const double most = 0.95 * plan_tiles(problems * blocks(T), F, kb, pairs, walk_by_columns(T, 1, F, problems, kb), drain).cycles;
+    return plan_cycles_at_least(problems * blocks(F), T, kb, pairs) < most &&
+           plan_tiles(problems * blocks(F), (int)T, kb, pairs, false, drain, true).cycles < most;
 }
 
 // How a contraction over the channels runs, [T, F] x [F, cols] summed over `segments` such pairs: exchanged or not, in how many
@@ -284,6 +285,7 @@ inline ContractionPlan plan_contraction(int64_t T, int F, int cols, int segments
     // (where the plain form has too few tiles, so has the exchanged one)
     for (int parts = best.parts; parts <= 4; ++parts) {
         if (parts > 1 && (parts % segments || per_part(parts) < 8 || (cols & 7) || !split_contraction_enabled())) continue;
+        if (plan_cycles_at_least(blocks(cols) * parts, T, per_part(parts), pairs) + sum(parts) >= least) continue;
         const double c = plan_tiles(blocks(cols) * parts, (int)T, per_part(parts), pairs, false, drain(parts), true).cycles + sum(parts);
         if (c < least) {
             least = c;

@@ -1,0 +1,135 @@
+"""The wide GEMM's tile search (csrc/tile_plan.h): the plans of an exhaustive search, found in microseconds, in a bounded memory."""
+import os
+import subprocess
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2511_09323_b200", "csrc")
+
+PROGRAM = r"""
+#include <chrono>
+#include <cstdio>
+#include <random>
+#include <vector>
+#include "tile_plan.h"
+using namespace moc::tc;
+
+// every candidate, every pair of CTAs, by the tile model written out again
+static TilePlan every(int rows, int N, int kb, int pairs, bool by_columns, int drain, bool any_first) {
+    const auto up = [](long a, long b) { return (int)((a + b - 1) / b); };
+    const auto cost = [&](int w_of) {
+        const int w = std::min(w_of, up(N, 64) * 64);
+        const double mma = kb * std::max(2.06 * w, (16384.0 + 64.0 * w) / 58.0) + 350.0;
+        return w > 256 ? mma + std::max(0, drain - 1024) : std::max(mma, drain * w / 256.0);
+    };
+    TilePlan best{};
+    const auto consider = [&](int w1, int split, int w2) {
+        TilePlan t{rows, by_columns, split, w1, up(N, w1), w2, 0, 0, 0, 0.0};
+        t.t1 = by_columns ? split / w1 * rows : split * t.nt1;
+        t.nt2 = by_columns ? (split < N ? up(N - split, w2) : 0) : up(N, w2);
+        t.total = t.t1 + (by_columns ? t.nt2 * rows : (rows - split) * t.nt2);
+        std::vector<double> load(pairs);
+        for (int j = 0; j < pairs; ++j) {
+            const int n1 = t.t1 > j ? (t.t1 - 1 - j) / pairs + 1 : 0, n = t.total > j ? (t.total - 1 - j) / pairs + 1 : 0;
+            t.cycles = std::max(t.cycles, n1 * cost(w1) + (n - n1) * cost(w2));
+        }
+        if (best.total == 0 || t.cycles < best.cycles) best = t;
+    };
+    const int most = any_first ? std::min(512, up(N, 64) * 64) : 512;
+    for (int w1 = most; w1 >= (any_first ? 64 : 512); w1 -= 64) {
+        const int units = by_columns ? N / w1 : rows, per_unit = by_columns ? rows : up(N, w1);
+        const int waves = (int)((long)units * per_unit / pairs);
+        for (int w2 = most; w2 >= 64; w2 -= 64) {
+            if (w1 == most) consider(w1, 0, w2);
+            for (int f = waves; f >= std::max(1, waves - 1); --f) {
+                const int u = (int)std::min<long>(units, (long)f * pairs / per_unit);
+                for (int v = u; v >= std::max(1, u - 1); --v) consider(w1, by_columns ? v * w1 : v, w2);
+            }
+        }
+    }
+    return best;
+}
+static bool same(const TilePlan &a, const TilePlan &b) {
+    return a.rows == b.rows && a.by_columns == b.by_columns && a.split == b.split && a.w1 == b.w1 && a.nt1 == b.nt1 && a.w2 == b.w2 &&
+           a.nt2 == b.nt2 && a.t1 == b.t1 && a.total == b.total && a.cycles == b.cycles;
+}
+
+struct Problem {
+    int rows, n, kb;
+    bool any_first;
+    int drain;
+};
+// what a forward and a backward of T tokens ask for at d x F
+static std::vector<Problem> asked(int T, int d, int F) {
+    const auto b = [](int n) { return (n + 255) / 256; };
+    const int kd = (d + 63) / 64, kf = (F + 63) / 64;
+    std::vector<Problem> p;
+    for (const int problems : {2, 1}) {
+        p.push_back({problems * b(T), F, kd, false, problems == 2 ? WIDE_DRAIN_F32 : WIDE_DRAIN_BF16});
+        p.push_back({problems * b(F), T, kd, true, problems == 2 ? WIDE_DRAIN_F32 : WIDE_DRAIN_BF16});
+    }
+    for (const int parts : {1, 2, 3, 4}) p.push_back({b(d) * parts, T, (kf + parts - 1) / parts, true, parts > 1 ? WIDE_DRAIN_F32 : WIDE_DRAIN_BF16});
+    p.push_back({b(T), d, kf, false, WIDE_DRAIN_BF16});
+    p.push_back({3 * b(F), d, (T + 63) / 64, false, WIDE_DRAIN_BF16});
+    return p;
+}
+
+int main() {
+    int wrong = 0;
+    std::mt19937 rng(7);
+    const auto pick = [&](int lo, int hi) { return std::uniform_int_distribution<int>(lo, hi)(rng); };
+    for (int i = 0; i < 4000; ++i) {
+        const bool any_first = pick(0, 1), by_columns = !any_first && pick(0, 1);
+        const int rows = i % 50 ? pick(1, 300) : pick(1, 6), n = pick(1, 40) == 1 ? pick(1, 200) : pick(1, 2100) * (any_first ? 1 : 6);
+        const int kb = pick(1, 200), pairs = pick(0, 3) ? 74 : pick(1, 80), drain = pick(0, 1) ? WIDE_DRAIN_BF16 : WIDE_DRAIN_F32;
+        const TilePlan want = every(rows, n, kb, pairs, by_columns, drain, any_first), got = search_tiles(rows, n, kb, pairs, by_columns, drain, any_first);
+        wrong += !same(want, got);
+        wrong += want.cycles < plan_cycles_at_least(rows, n, kb, pairs);
+    }
+    for (const int T : {257, 307, 512, 513, 777, 1111, 2000, 2048})
+        for (const Problem &p : asked(T, 2048, 5461)) wrong += !same(every(p.rows, p.n, p.kb, 74, false, p.drain, p.any_first), search_tiles(p.rows, p.n, p.kb, 74, false, p.drain, p.any_first));
+    // the memory: many more sizes than it holds, in two sweeps, with one that is asked for again and again
+    for (int sweep = 0; sweep < 2; ++sweep)
+        for (int n = 1; n <= 3000; ++n) {
+            wrong += !same(plan_tiles(8, n, 32, 74, false, WIDE_DRAIN_BF16), search_tiles(8, n, 32, 74, false, WIDE_DRAIN_BF16, false));
+            wrong += !same(plan_tiles(5, 2048, 32, 74, true, WIDE_DRAIN_F32), search_tiles(5, 2048, 32, 74, true, WIDE_DRAIN_F32, false));
+        }
+    // the plans of one token count, searched anew: the fastest of nine times, the slowest of 64 counts, in microseconds
+    const auto worst = [&](int d, int F, auto search) {
+        double slowest = 0;
+        for (int i = 0; i < 64; ++i) {
+            double fastest = 1e9;
+            for (int rep = 0; rep < 9; ++rep) {
+                const auto t0 = std::chrono::steady_clock::now();
+                double sum = 0;
+                for (const Problem &p : asked(257 + 28 * i, d, F)) sum += search(p.rows, p.n, p.kb, 74, false, p.drain, p.any_first).cycles;
+                const double us = std::chrono::duration<double, std::micro>(std::chrono::steady_clock::now() - t0).count();
+                if (sum > 0) fastest = std::min(fastest, us);
+            }
+            slowest = std::max(slowest, fastest);
+        }
+        return slowest;
+    };
+    std::printf("%d %.2f %.2f %.2f\n", wrong, worst(4096, 11008, search_tiles), worst(2048, 5461, search_tiles), worst(4096, 11008, every));
+    return 0;
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def result(tmp_path_factory):
+    where = tmp_path_factory.mktemp("tile_plan")
+    source, program = where / "plan.cpp", where / "plan"
+    source.write_text(PROGRAM)
+    subprocess.run([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-Wall", f"-I{CSRC}", str(source), "-o", str(program), "-lpthread"],
+                   check=True)
+    return [float(v) for v in subprocess.run([str(program)], check=True, capture_output=True, text=True).stdout.split()]
+
+
+def test_plans_are_those_of_the_exhaustive_search(result):
+    assert result[0] == 0
+
+
+def test_a_new_token_count_costs_microseconds(result):
+    # all ten plans that a forward and a backward can ask for; searching every pair of CTAs takes hundreds of microseconds
+    assert max(result[1:3]) < 50, result
