@@ -405,7 +405,7 @@ inline int ceil_div(int64_t a, int64_t b) { return (int)((a + b - 1) / b); }
 struct TcSelect {
     enum Kind { kRegisters, kSharedRow, kCtaPerRow } kind;
     int nv;             // 128-channel groups of a row
-    int team, vpl;      // warps per token; values per lane (kRegisters)
+    int team, vpl, bins;  // warps per token; values per lane and bins of the histogram (kRegisters)
     int tokens_per_cta, ctas_per_sm;
     size_t smem;        // dynamic shared memory of the launch
     int variant;        // MOC_SELECT_VARIANT_* (what a test hook reports)
@@ -418,27 +418,32 @@ enum {
     MOC_SELECT_VARIANT_TEAM4_SHARED = 3,  // teams of four, one shared-memory buffer for both rows
 };
 
-// (warps per token, values per lane), each for up to 32 * W * VPL channels.  The fewest warps that leave a lane at most 64
+// (warps per token, values per lane, bins), each for up to 32 * W * VPL channels and for the K that need so many bins
+// (rs::bins_for; the counts that no K needs at a form's lengths are left out).  The fewest warps that leave a lane at most 64
 // values: every warp of a team repeats the scan of the histogram and the ranking (16384 rows of 2048 channels: 71 us with
 // one or two warps, 119 us with four).
-#define MOC_ROW_SELECT_FORMS(DO) DO(1, 16) DO(1, 32) DO(2, 32) DO(2, 48) DO(4, 32) DO(4, 44) DO(4, 64) DO(8, 44) DO(8, 56)
+#define MOC_ROW_SELECT_FORMS(DO)                                                                                       \
+    DO(1, 16, 256) DO(1, 32, 256) DO(2, 32, 256) DO(2, 48, 256) DO(4, 32, 256) DO(4, 44, 256) DO(4, 44, 512)           \
+    DO(4, 64, 256) DO(4, 64, 512) DO(8, 44, 256) DO(8, 44, 512) DO(8, 44, 1024) DO(8, 56, 256) DO(8, 56, 512) DO(8, 56, 1024)
 
 TcSelect tc_select_config(int F, int K) {
     using namespace tc;
     TcSelect c{};
     c.nv = ceil_div(F, 128);
-#define MOC_DO_PICK(W, VPL)                      \
-    if (c.team == 0 && F <= 32 * W * VPL) {      \
-        c.team = W;                              \
-        c.vpl = VPL;                             \
-        c.ctas_per_sm = rs::ctas_per_sm(W, VPL); \
+    const int bins = rs::bins_for(F, K);
+#define MOC_DO_PICK(W, VPL, BINS)                               \
+    if (c.team == 0 && F <= 32 * W * VPL && bins <= BINS) {     \
+        c.team = W;                                             \
+        c.vpl = VPL;                                            \
+        c.bins = BINS;                                          \
+        c.ctas_per_sm = rs::ctas_per_sm(W, VPL);                \
     }
     MOC_ROW_SELECT_FORMS(MOC_DO_PICK)
 #undef MOC_DO_PICK
     if (c.team) {
         c.kind = TcSelect::kRegisters;
         c.tokens_per_cta = 1;
-        c.smem = rs::layout(c.team, c.nv * 128, K).total;  // (rows may be padded up to whole groups)
+        c.smem = rs::layout(c.team, c.bins, c.nv * 128, K).total;  // (rows may be padded up to whole groups)
         c.ctas_per_sm = std::max(1, std::min(c.ctas_per_sm, (int)((size_t)kMaxDynSmem / (c.smem + 1024))));
         c.variant = c.team <= 2 ? MOC_SELECT_VARIANT_TEAM2 : MOC_SELECT_VARIANT_TEAM4;
         return c;
@@ -465,8 +470,8 @@ TcSelect tc_select_config(int F, int K) {
 
 int tc_select_prepare(const TcSelect &c, int F, int K) {
     if (c.kind == TcSelect::kRegisters) {
-#define MOC_DO_SET(W, VPL) \
-    if (c.team == W && c.vpl == VPL) return set_smem(rs::select_rows_reg_kernel<W, VPL>, c.smem, 1024);
+#define MOC_DO_SET(W, VPL, BINS)                           \
+    if (c.team == W && c.vpl == VPL && c.bins == BINS) return set_smem(rs::select_rows_reg_kernel<W, VPL, BINS>, c.smem, 1024);
         MOC_ROW_SELECT_FORMS(MOC_DO_SET)
 #undef MOC_DO_SET
     }
@@ -487,12 +492,11 @@ void tc_select_launch(const TcSelect &c, const float *G, int ldg, __nv_bfloat16 
     const unsigned grid = (unsigned)std::min<int64_t>((n + c.tokens_per_cta - 1) / c.tokens_per_cta,
                                                       (int64_t)sm_count() * c.ctas_per_sm);
     if (c.kind == TcSelect::kRegisters) {
-#define MOC_DO_LAUNCH(W, VPL)                                                                                                   \
-    if (c.team == W && c.vpl == VPL)                                                                                            \
-        MOC_LAUNCH(KID_TC_SELECT_MASK, st,                                                                                      \
-                   (rs::select_rows_reg_kernel<W, VPL><<<grid, 32 * W, c.smem, st>>>(G, ldg, U, ldu, n, F, K,                   \
-                                                                                     rs::normal_quantile(F, K), o_idx, o_g, o_u, \
-                                                                                     status)));
+#define MOC_DO_LAUNCH(W, VPL, BINS)                                                                                              \
+    if (c.team == W && c.vpl == VPL && c.bins == BINS)                                                                           \
+        MOC_LAUNCH(KID_TC_SELECT_MASK, st,                                                                                       \
+                   (rs::select_rows_reg_kernel<W, VPL, BINS><<<grid, 32 * W, c.smem, st>>>(                                      \
+                       G, ldg, U, ldu, n, F, K, rs::normal_quantile(F, K), o_idx, o_g, o_u, status)));
         MOC_ROW_SELECT_FORMS(MOC_DO_LAUNCH)
 #undef MOC_DO_LAUNCH
     } else if (c.kind == TcSelect::kSharedRow) {

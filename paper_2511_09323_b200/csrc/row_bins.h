@@ -1,0 +1,44 @@
+// The row selector's histogram (row_select.cuh): where its window lies and how many bins it has.  Host code only, free of CUDA.
+#pragma once
+
+#include <algorithm>
+#include <cmath>
+
+namespace moc {
+namespace rs {
+
+constexpr float kWindowMad = 0.95f;  // half width of the window in mean absolute deviations (0.76 sigma of normal values)
+constexpr float kMadOfNormal = 0.797885f;  // mean absolute deviation of normal values, in standard deviations
+
+// Where the K-th largest of F normal values lies, in standard deviations above the mean (Abramowitz and Stegun 26.2.23,
+// absolute error below 4.5e-4).
+inline float normal_quantile(int F, int K) {
+    double p = ((double)K - 0.5) / F;
+    const double s = p > 0.5 ? -1.0 : 1.0;
+    p = std::min(p, 1.0 - p);
+    const double t = std::sqrt(-2.0 * std::log(p));
+    return (float)(s * (t - (2.515517 + t * (0.802853 + t * 0.010328)) / (1.0 + t * (1.432788 + t * (0.189269 + t * 0.001308)))));
+}
+
+// Values of a normal row that fall into the bin of its K-th largest, on average.
+inline float values_in_bin(int F, int K, int bins) {
+    const float z = normal_quantile(F, K);
+    return F * 0.398942f * std::exp(-0.5f * z * z) * (2.f * kWindowMad * kMadOfNormal) / bins;
+}
+
+// The fewest bins that leave at most eleven values in the threshold's.  The selector ranks 28 of them at once and searches a
+// row with more over the whole range, 30 us: with an average of 11 that is one row in 10^5, with 15 one in 400, with 19 one
+// in 25, and then nearly every launch of thousands of rows ends with some.  More bins than needed cost the clearing and the
+// scan (5504 channels, K = F/4, 10.4 values in one of 256 bins: 230 us, with 512 bins 238).
+// 16384 rows, with the count that the length alone gave before and with this rule, us: 8192 channels, F/4 520 -> 363, F/2
+// 1045 -> 574; 5504, F/2 369 -> 314; 11008, F/16 350 -> 330, F/2 742 -> 656; 14336, F/2 1500 -> 1293.
+constexpr float kBinValues = 11.f;
+constexpr int kMinBins = 256, kMaxBins = 1024;
+inline int bins_for(int F, int K) {
+    int bins = kMinBins;
+    while (bins < kMaxBins && values_in_bin(F, K, bins) > kBinValues) bins *= 2;
+    return bins;
+}
+
+}  // namespace rs
+}  // namespace moc

@@ -9,7 +9,7 @@
 // What bounds it: 8 bytes per channel have to move (G, U in, Z' out), and the instructions of the search have to stay
 // below what the SM issues meanwhile.  A row is therefore read once, into registers, and walked three times in straight
 // lines of predicated instructions (as branches, which is what plain code compiles to, each walk costs twice as much):
-//   1. histogram: every value is mapped to one of 256 equal bins (512 for teams of eight) of a window around the expected
+//   1. histogram: every value is mapped to one of 256, 512 or 1024 equal bins (row_bins.h: as many as K needs) of a window around the expected
 //      threshold (multiply-add with saturation, so that what lies outside falls into the end bins) and counted with one
 //      shared-memory atomic;
 //   2. every warp scans the counts: bin b of the K-th largest value.  Everything from (just below) bin b on is a candidate
@@ -24,38 +24,21 @@
 // values).  The team meets at five barriers a row and shares nothing with other teams.
 #pragma once
 
-#include <algorithm>
-#include <cmath>
-
+#include "row_bins.h"
 #include "tc_gemm.cuh"
 #include "topk_select.cuh"
 
 namespace moc {
 namespace rs {
 
-constexpr int kMaxBins = 512;
-// Bins of the histogram: some 7 values in the threshold's bin (2048 channels: 3, 5504: 7, 11008: 7).  More would go over
-// what one lane each can rank for a row in a few hundred, and a row searched over the whole range takes 30 us.
-constexpr int bins(int W) { return W >= 8 ? 512 : 256; }
 constexpr uint32_t kMaxRanked = 32;     // candidates ranked by one lane each
-constexpr float kWindowMad = 0.95f;     // half width of the window in mean absolute deviations (0.76 sigma of normal values)
 
 // CTAs (= teams) of W warps that an SM should hold: registers for VPL values per lane plus some 60.  More warps with fewer
 // registers spill the values that are on their way, which stalls the walk they should overlap (16384 rows of 5504
 // channels: 178 us with 128 registers, 251 with 96).
 constexpr int ctas_per_sm(int W, int VPL) { return (VPL > 32 ? 16 : 20) / W; }
 
-// Where the K-th largest of F normal values lies, in standard deviations above the mean (Abramowitz and Stegun 26.2.23,
-// absolute error below 4.5e-4).
-inline float normal_quantile(int F, int K) {
-    double p = ((double)K - 0.5) / F;
-    const double s = p > 0.5 ? -1.0 : 1.0;
-    p = std::min(p, 1.0 - p);
-    const double t = std::sqrt(-2.0 * std::log(p));
-    return (float)(s * (t - (2.515517 + t * (0.802853 + t * 0.010328)) / (1.0 + t * (1.432788 + t * (0.189269 + t * 0.001308)))));
-}
-
-// the same on the device, with the fast functions (it only places a window)
+// normal_quantile on the device, with the fast functions (it only places a window)
 __device__ __forceinline__ float normal_quantile_fast(int F, int K) {
     const float q = ((float)K - 0.5f) / (float)F, p = fminf(q, 1.0f - q), t = sqrtf(-2.0f * __logf(fmaxf(p, 1e-6f)));
     const float z = t - (2.515517f + t * (0.802853f + t * 0.010328f)) / (1.0f + t * (1.432788f + t * (0.189269f + t * 0.001308f)));
@@ -65,7 +48,7 @@ __device__ __forceinline__ float normal_quantile_fast(int F, int K) {
 struct Layout {
     uint32_t z, kept, hist, xch, bar, total;  // byte offsets (the up row is at 0)
 };
-__host__ __device__ inline Layout layout(int W, int ldu, int K) {
+__host__ __device__ inline Layout layout(int W, int bins, int ldu, int K) {
     Layout L{};
     uint32_t o = (uint32_t)ldu * 2u;
     L.z = o;
@@ -73,7 +56,7 @@ __host__ __device__ inline Layout layout(int W, int ldu, int K) {
     L.kept = o;  // {gate value, channel} in ascending channel order
     o += (((uint32_t)K + kMaxRanked) * 8u + 15u) & ~15u;
     L.hist = o;
-    o += kMaxBins * 4u;
+    o += (uint32_t)bins * 4u;
     L.xch = o;  // number of ranked entries, pad[3] | ranked entries {value, list index} | two words per warp
     o += (4u + 2u * kMaxRanked + 2u * (uint32_t)W) * 4u;
     L.bar = (o + 7u) & ~7u;
@@ -92,7 +75,7 @@ __device__ __forceinline__ void keep_if_ge(float x, float tau, int ch, uint32_t 
 // four times the bin of a value: non-decreasing in x, NaN and everything below the window in bin 0, above it in the last
 template <int BINS>
 __device__ __forceinline__ uint32_t bin4(float x, float scale, float offset) {
-    constexpr int bits = BINS == 512 ? 9 : 8;
+    constexpr int bits = BINS == 1024 ? 10 : BINS == 512 ? 9 : 8;
     const float q = __saturatef(fmaf(x, scale, offset));
     return (__float_as_uint(fmaf(q, 1.0f - 0.5f / BINS, 1.0f)) >> (23 - bits - 2)) & (4u * BINS - 4u);
 }
@@ -108,37 +91,63 @@ template <int BINS>
 __device__ __forceinline__ BinRank scan_bins(const uint32_t *hist, uint32_t want) {
     constexpr int N = BINS / 32;  // bins of a lane
     const int lane = threadIdx.x & 31;
-    uint32_t h[N], tot = 0;
+    // values counted by this lane and by those above it
+    const auto from_lane_up = [&](uint32_t v) {
 #pragma unroll
-    for (int i = 0; i < N / 4; ++i) {
-        const uint4 q = reinterpret_cast<const uint4 *>(hist)[N / 4 * lane + i];
-        h[4 * i] = q.x;
-        h[4 * i + 1] = q.y;
-        h[4 * i + 2] = q.z;
-        h[4 * i + 3] = q.w;
-    }
-#pragma unroll
-    for (int i = 0; i < N; ++i) tot += h[i];
-    uint32_t suf = tot;  // values in this lane's bins and those of higher lanes
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t nb = __shfl_down_sync(0xffffffffu, suf, o);
-        if (lane + o < 32) suf += nb;
-    }
-    BinRank r;
-    r.total = __shfl_sync(0xffffffffu, suf, 0);
-    uint32_t gt = suf - tot, bin = 0, above = 0, cnt = 0;
-    const bool here = gt < want && want <= suf;
-#pragma unroll
-    for (int i = N - 1; i >= 0; --i) {
-        if (gt < want && want <= gt + h[i]) {
-            bin = (uint32_t)(lane * N + i);
-            above = gt;
-            cnt = h[i];
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t nb = __shfl_down_sync(0xffffffffu, v, o);
+            if (lane + o < 32) v += nb;
         }
-        gt += h[i];
+        return v;
+    };
+    BinRank r;
+    uint32_t tot = 0, bin = 0, above = 0, cnt = 0;
+    int src;
+    if constexpr (N <= 8) {
+        uint32_t h[N];
+#pragma unroll
+        for (int i = 0; i < N / 4; ++i) {
+            const uint4 q = reinterpret_cast<const uint4 *>(hist)[N / 4 * lane + i];
+            h[4 * i] = q.x;
+            h[4 * i + 1] = q.y;
+            h[4 * i + 2] = q.z;
+            h[4 * i + 3] = q.w;
+        }
+#pragma unroll
+        for (int i = 0; i < N; ++i) tot += h[i];
+        const uint32_t suf = from_lane_up(tot);
+        r.total = __shfl_sync(0xffffffffu, suf, 0);
+        uint32_t gt = suf - tot;
+        const bool here = gt < want && want <= suf;
+#pragma unroll
+        for (int i = N - 1; i >= 0; --i) {
+            if (gt < want && want <= gt + h[i]) {
+                bin = (uint32_t)(lane * N + i);
+                above = gt;
+                cnt = h[i];
+            }
+            gt += h[i];
+        }
+        src = max(0, __ffs(__ballot_sync(0xffffffffu, here)) - 1);
+    } else {
+        // Many bins beside a row that fills the registers: a lane's sum first (its 16-byte pieces in an order that keeps the
+        // lanes off each other's banks), then the bins of the lane that holds the one looked for, one to a lane.
+#pragma unroll
+        for (int i = 0; i < N / 4; ++i) {
+            const uint4 q = reinterpret_cast<const uint4 *>(hist)[N / 4 * lane + ((i + lane * N / 32) & (N / 4 - 1))];
+            tot += q.x + q.y + q.z + q.w;
+        }
+        uint32_t suf = from_lane_up(tot);
+        r.total = __shfl_sync(0xffffffffu, suf, 0);
+        above = suf - tot;
+        src = max(0, __ffs(__ballot_sync(0xffffffffu, above < want && want <= suf)) - 1);
+        const uint32_t over = __shfl_sync(0xffffffffu, above, src);
+        bin = (uint32_t)(N * src + lane);
+        cnt = lane < N ? hist[bin] : 0u;
+        suf = from_lane_up(cnt) + over;
+        above = suf - cnt;
+        src = max(0, __ffs(__ballot_sync(0xffffffffu, above < want && want <= suf)) - 1);
     }
-    const int src = max(0, __ffs(__ballot_sync(0xffffffffu, here)) - 1);
     r.bin = __shfl_sync(0xffffffffu, bin, src);
     r.above = __shfl_sync(0xffffffffu, above, src);
     r.count = __shfl_sync(0xffffffffu, cnt, src);
@@ -148,7 +157,7 @@ __device__ __forceinline__ BinRank scan_bins(const uint32_t *hist, uint32_t want
 // A row whose threshold the window missed (or whose bin holds too many values): 8 bits of the threshold's key per pass over
 // the row in global memory, then the kept channels in order.  The whole team; leaves the list complete behind a barrier of
 // its own.  (A function: in line, its registers and its branches cost the common path a quarter.)
-template <int W>
+template <int W, int BINS>
 __device__ __noinline__ void search_whole_range(const float *g, int F, int K, uint32_t *hist, uint2 *kept, volatile uint32_t *xw) {
     constexpr int TT = 32 * W;
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -208,21 +217,20 @@ __device__ __noinline__ void search_whole_range(const float *g, int F, int K, ui
         eq += (uint32_t)__popc(be);
     }
     sync();
-    for (int i = tid; i < bins(W); i += TT) hist[i] = 0u;
+    for (int i = tid; i < BINS; i += TT) hist[i] = 0u;
     sync();
 }
 
-template <int W, int VPL>
+template <int W, int VPL, int BINS>
 __global__ void __launch_bounds__(32 * W, ctas_per_sm(W, VPL)) select_rows_reg_kernel(
     const float *__restrict__ G, int ldg, __nv_bfloat16 *__restrict__ U, int ldu, int64_t rows, int F, int K, float quantile,
     int16_t *__restrict__ idx_out, __nv_bfloat16 *__restrict__ g_out, __nv_bfloat16 *__restrict__ u_out, int *status) {
     using namespace tc;
     extern __shared__ __align__(16) uint8_t smem[];
     constexpr int TT = 32 * W;         // threads of the team (= of the CTA)
-    constexpr int BINS = bins(W);
     constexpr int GPW = VPL / 4;       // 128-channel groups per warp: lane l of a group holds channels 4 l .. 4 l + 3
     constexpr int NP = (GPW + 3) / 4;  // words of packed per-group counts
-    const Layout L = layout(W, ldu, K);
+    const Layout L = layout(W, BINS, ldu, K);
     const __nv_bfloat16 *su = reinterpret_cast<const __nv_bfloat16 *>(smem);
     __nv_bfloat16 *sz = reinterpret_cast<__nv_bfloat16 *>(smem + L.z);
     uint2 *kept = reinterpret_cast<uint2 *>(smem + L.kept);
@@ -369,7 +377,7 @@ __global__ void __launch_bounds__(32 * W, ctas_per_sm(W, VPL)) select_rows_reg_k
             }
         }
         if (!fast) {
-            search_whole_range<W>(G + r * (int64_t)ldg, F, K, hist, kept, xw);
+            search_whole_range<W, BINS>(G + r * (int64_t)ldg, F, K, hist, kept, xw);
             n_list = (uint32_t)K;
         }
         for (int i = tid; i < (ldu >> 3); i += TT) reinterpret_cast<uint4 *>(sz)[i] = make_uint4(0, 0, 0, 0);
@@ -409,7 +417,7 @@ __global__ void __launch_bounds__(32 * W, ctas_per_sm(W, VPL)) select_rows_reg_k
                 }
                 __syncwarp();
             } else {  // too many values at the bin's edges
-                search_whole_range<W>(G + r * (int64_t)ldg, F, K, hist, kept, xw);
+                search_whole_range<W, BINS>(G + r * (int64_t)ldg, F, K, hist, kept, xw);
                 n_list = (uint32_t)K;
             }
         }

@@ -1,0 +1,51 @@
+"""Bins of the row selector's histogram (csrc/row_bins.h): few enough values in the threshold's bin at every length and K, and
+exact results on both sides of each switch."""
+import os
+import subprocess
+
+import numpy as np
+import pytest
+import torch
+from scipy.stats import norm
+
+from oracle import moc_oracle as orc
+from paper_2511_09323_b200 import binding as B
+from test_gpu_selector_plans import _adversarial_rows
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2511_09323_b200", "csrc")
+LONGEST = 14336   # channels of the longest row held in registers
+
+
+def test_the_threshold_bin_holds_few_values(tmp_path):
+    source, program = tmp_path / "bins.cpp", tmp_path / "bins"
+    source.write_text('#include <cstdio>\n#include "row_bins.h"\nint main() { int f, k; while (std::scanf("%d %d", &f, &k) == 2) '
+                      'std::printf("%d\\n", moc::rs::bins_for(f, k)); }')
+    subprocess.run([os.environ.get("CXX", "g++"), "-O1", "-std=c++17", f"-I{CSRC}", str(source), "-o", str(program)], check=True)
+    sizes = [(f, k) for f in (128, 1000, 2048, 4096, 4300, 5461, 5504, 5632, 5633, 6144, 8192, 8193, 11008, 11264, 12288, LONGEST)
+             for k in sorted({1, f // 64, f // 16, f // 8, f // 4, f // 3, f // 2, 3 * f // 4, f})]
+    out = subprocess.run([str(program)], input="\n".join(f"{f} {k}" for f, k in sizes), check=True, capture_output=True, text=True).stdout
+    for (f, k), bins in zip(sizes, map(int, out.split()), strict=True):
+        # a bin is 2 * 0.95 mean absolute deviations (0.798 sigma) over the bins; the K-th value is in it, the others by chance
+        average = f * norm.pdf(norm.isf((k - 0.5) / f)) * 2 * 0.95 * 0.797885 / bins
+        assert average <= 11.1, (f, k, bins, average)
+        assert bins == 256 or 2 * average > 10.9, (f, k, bins, average)   # and no more bins than that takes
+
+
+# both sides of each switch of 256 / 512 / 1024 bins, by length at K = n / 2 and by K at one length
+@pytest.mark.gpu
+@pytest.mark.parametrize("n, k", ((4230, 2115), (4236, 2118), (5632, 1000), (5632, 1400), (5632, 2816), (8192, 900), (8192, 1100), (8192, 4096),
+                                  (8462, 4231), (8472, 4236), (11008, 688), (11008, 1000), (11008, 2700), (11008, 3400), (11008, 5504),
+                                  (14336, 500), (14336, 900), (14336, 1792), (14336, 2500), (14336, 7168)))
+def test_exact_on_both_sides_of_the_switches(n, k):
+    rng = np.random.default_rng(n + k)
+    tau = norm.isf((k - 0.5) / n)
+    packed = rng.standard_normal((6, n))
+    packed[:, rng.permutation(n)[: n // 3]] = tau + 1e-4 * rng.standard_normal((6, n // 3))
+    steps = np.round(rng.standard_normal((6, n)) * 600) / 600          # values that repeat, at the bins' own spacing
+    g = np.concatenate([_adversarial_rows(n), rng.standard_normal((60, n)), packed, steps, 100.0 + rng.standard_normal((6, n)),
+                        rng.exponential(size=(6, n)) ** 3]).astype(np.float32)
+    pad = np.full((g.shape[0], (n + 7) // 8 * 8), 1e9, np.float32)
+    pad[:, :n] = g
+    idx, _ = B.moc_topk_select_tc(torch.from_numpy(pad).cuda(), k, n=n)
+    np.testing.assert_array_equal(idx.cpu().numpy().astype(np.int32), orc.topk(g, k))
+    assert B.moc_last_device_status() == B.MOC_OK
