@@ -35,15 +35,7 @@ constexpr int kMaxD = 4096;          // a thread owns 8 output columns
 constexpr int kConsumerWarps = 16;
 constexpr int kThreads = (kConsumerWarps + 1) * 32;  // + one producer warp
 constexpr int kMaxRows = 256;        // channels per CTA
-// Bins of the order-preserving keys: every octave of 2^-6 <= g < 2^6, where a gate's threshold usually lies, in 128 bins of
-// equal key steps (some 20 keys of 11008 share one); one bin per octave for everything else.
-constexpr int kBins = 2048;
-constexpr uint32_t kFineFrom = 0xbc800000u, kFineTo = 0xc2800000u;  // keys of 2^-6 and 2^6
-constexpr uint32_t kFineBase = kFineFrom >> 23, kFineEnd = kFineBase + ((kFineTo - kFineFrom) >> 16);
-static_assert(kFineEnd + ((0xffffffffu - kFineTo) >> 23) < (uint32_t)kBins, "the bins cover every key");
-__device__ __forceinline__ uint32_t key_bin(uint32_t key) {
-    return key < kFineFrom ? key >> 23 : key < kFineTo ? kFineBase + ((key - kFineFrom) >> 16) : kFineEnd + ((key - kFineTo) >> 23);
-}
+constexpr int kBins = 2048;          // top 11 bits of the key
 constexpr int kMaxStages = 32;         // a multiple of kConsumerWarps
 constexpr int kFirstRows = 8;  // gate rows requested before x is staged and the shared arrays are cleared (16 or 32 of them
                                // made that start-up 0.9 us longer and the call 1 us slower: they compete with it for the path from L2)
@@ -238,7 +230,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_coop_kernel(const Params p
     if (!p.grouped) {
         for (int i = tid; i < T * rows; i += kThreads) {
             const int t = i / rows, r = i - t * rows;
-            atomicAdd(&p.hist[t * kBins + key_bin(gate_key(sg[t * kMaxRows + r]))], 1u);
+            atomicAdd(&p.hist[t * kBins + (gate_key(sg[t * kMaxRows + r]) >> 21)], 1u);
         }
         grid.sync();  // #1 (the barrier's release / acquire pair orders the CTAs' writes before the others' reads): every CTA's keys are in the histogram
         MOC_TL_CTA(1024);
@@ -278,7 +270,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_coop_kernel(const Params p
         for (int i = tid; i < T * rows; i += kThreads) {
             const int t = i / rows, r = i - t * rows;
             const uint32_t key = gate_key(sg[t * kMaxRows + r]);
-            if (key_bin(key) == s_bin[t]) {
+            if ((key >> 21) == s_bin[t]) {
                 const uint32_t pos = atomicAdd(&p.cand_n[t], 1u);
                 p.cand[(int64_t)t * F + pos] = make_uint2(key, (uint32_t)(c0 + r));
             }
@@ -306,7 +298,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_coop_kernel(const Params p
         for (int i = warp; i < T * rows; i += kConsumerWarps + 1) {
             const int t = i / rows, r = i - t * rows;
             const uint32_t key = gate_key(sg[t * kMaxRows + r]);
-            const uint32_t bin = key_bin(key);
+            const uint32_t bin = key >> 21;
             bool kept = bin > s_bin[t];
             if (bin == s_bin[t]) {
                 uint32_t nt = 0, ot = 0;
