@@ -30,6 +30,32 @@ def moc_ffn(x: torch.Tensor, w_gate: torch.Tensor, w_up: torch.Tensor, w_down: t
     return (B._front or B.front()).ffn(x, w_gate, w_up, w_down, k, d_ff, B._flags(grouped, post_silu), recompute_up)
 
 
+class _TracedFunction(torch.autograd.Function):
+    """`moc_ffn` while `torch.jit.trace` records: the same calls as the C++ node's, as one step of the trace."""
+
+    @staticmethod
+    def forward(ctx, x, w_gate, w_up, w_down, k, d_ff, flags, recompute_up):
+        ctx.x_shape, ctx.d_ff, ctx.grouped = x.shape, d_ff, bool(flags & B.MOC_FLAG_SELECT_2_OF_8)
+        x2 = x.reshape(-1, x.shape[-1]).contiguous()
+        save = any(ctx.needs_input_grad[:4])
+        out, idx, gate, up = B.moc_ffn_forward(x2, w_gate, w_up, w_down, k, d_ff=d_ff, save=save, grouped=ctx.grouped,
+                                               post_silu=bool(flags & B.MOC_FLAG_SELECT_POST_SILU))
+        if save:
+            ctx.save_for_backward(x2, w_gate, w_up, w_down, idx, gate, *(() if recompute_up else (up,)))
+        return out.reshape(x.shape)
+
+    @staticmethod
+    def backward(ctx, grad_out):
+        x, w_gate, w_up, w_down, idx, gate, *up = ctx.saved_tensors
+        up = up[0] if up else B.moc_ffn_recompute_up(x, w_up, idx, d_ff=ctx.d_ff)
+        want = [n for n, need in zip(("x", "w_gate", "w_up", "w_down"), ctx.needs_input_grad) if need]
+        grads = B.moc_ffn_backward(x, w_gate, w_up, w_down, idx, gate, up, grad_out.reshape(x.shape).contiguous(), d_ff=ctx.d_ff,
+                                   want=want, grouped=ctx.grouped)
+        gx = grads["grad_x"]
+        return (None if gx is None else gx.reshape(ctx.x_shape), grads["grad_w_gate"], grads["grad_w_up"], grads["grad_w_down"],
+                None, None, None, None)
+
+
 class MoCFFN(torch.nn.Module):
     """SwiGLU feed-forward block with Top-K channel selection on the gate (Section 3.2)."""
 

@@ -148,7 +148,9 @@ def front():
             from . import _front as module
         except ImportError as exc:
             raise RuntimeError(f"_front.so cannot be loaded ({exc}): build it with `python -m paper_2511_09323_b200.build`") from exc
+        from .autograd import _TracedFunction
         module.set_error(MocError)
+        module.set_traced_ffn(_TracedFunction.apply)
         _front = module
     return _front
 

@@ -15,6 +15,7 @@
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/custom_function.h>
 #include <torch/csrc/autograd/python_variable.h>
+#include <torch/csrc/jit/frontend/tracer.h>
 
 #include "../../include/moc_ffn.h"
 
@@ -23,6 +24,7 @@ namespace {
 using at::Tensor;
 
 PyObject *g_moc_error = nullptr;  // binding.MocError(status, where)
+PyObject *g_traced_ffn = nullptr;  // autograd._TracedFunction.apply, with ffn's arguments
 
 // Raises binding.MocError as a C++ exception that the interpreter, or the autograd engine's thread, turns back into it.
 [[noreturn]] void raise_moc(int status, const char *where) {
@@ -222,6 +224,9 @@ void need_args(Py_ssize_t have, Py_ssize_t want) {
 PyObject *py_ffn(PyObject *, PyObject *const *a, Py_ssize_t n) {
     HANDLE_TH_ERRORS
     need_args(n, 8);
+    // torch.jit.trace sees the torch calls of the C++ node (empty tensors) and not what the library writes into them; a Python
+    // function is recorded as one opaque step
+    if (torch::jit::tracer::isTracing()) return PyObject_Vectorcall(g_traced_ffn, a, (size_t)n, nullptr);
     const Tensor x = tensor_arg(a[0], "x", false), wg = tensor_arg(a[1], "w_gate", false), wu = tensor_arg(a[2], "w_up", false),
                  wd = tensor_arg(a[3], "w_down", false);
     const int64_t k = int_arg(a[4]), d_ff = int_arg(a[5]), flags = int_arg(a[6]);
@@ -309,11 +314,12 @@ PyObject *py_decode(PyObject *, PyObject *const *a, Py_ssize_t n) {
     END_HANDLE_TH_ERRORS
 }
 
-// set_error(class): the exception raised for a negative moc_status
-PyObject *py_set_error(PyObject *, PyObject *cls) {
-    Py_INCREF(cls);
-    Py_XDECREF(g_moc_error);
-    g_moc_error = cls;
+// set_error(class): the exception raised for a negative moc_status; set_traced_ffn(function): what ffn is while tracing
+template <PyObject *&KEPT>
+PyObject *py_set(PyObject *, PyObject *o) {
+    Py_INCREF(o);
+    Py_XDECREF(KEPT);
+    KEPT = o;
     Py_RETURN_NONE;
 }
 
@@ -323,7 +329,8 @@ PyMethodDef kMethods[] = {
     {"forward", MOC_FAST(py_forward), METH_FASTCALL, nullptr},
     {"decode", MOC_FAST(py_decode<false>), METH_FASTCALL, nullptr},
     {"decode_block", MOC_FAST(py_decode<true>), METH_FASTCALL, nullptr},
-    {"set_error", py_set_error, METH_O, nullptr},
+    {"set_error", py_set<g_moc_error>, METH_O, nullptr},
+    {"set_traced_ffn", py_set<g_traced_ffn>, METH_O, nullptr},
     {nullptr, nullptr, 0, nullptr},
 };
 PyModuleDef kModule = {PyModuleDef_HEAD_INIT, "_front", nullptr, -1, kMethods, nullptr, nullptr, nullptr, nullptr};
