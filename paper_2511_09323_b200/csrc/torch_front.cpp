@@ -58,17 +58,21 @@ int dtype_code(const Tensor &t) {
     TORCH_CHECK_TYPE(false, "unsupported storage dtype torch.", c10::toString(t.scalar_type()));
 }
 
-// d_ff < 0: all rows of the weights are channels; k < 0: not given (the 2-of-8 mask implies it)
+// None in the place of a whole number
+constexpr int64_t kNotGiven = INT64_MIN;
+
+// d_ff not given: all rows of the weights are channels; k not given: the 2-of-8 mask implies it
 moc_ffn_desc make_desc(const Tensor &x, const Tensor &w, int64_t k, int64_t d_ff, uint32_t flags) {
     TORCH_CHECK_VALUE(x.dim() == 2, "expected a [tokens, d_model] tensor");
     moc_ffn_desc d{};
     const int64_t rows = w.size(0);
-    if (d_ff < 0) d_ff = rows;
+    if (d_ff == kNotGiven) d_ff = rows;
     if (flags & MOC_FLAG_SELECT_2_OF_8) {
         TORCH_CHECK_VALUE(d_ff % 8 == 0, "the 2-of-8 mask needs d_ff to be a multiple of 8");
-        TORCH_CHECK_VALUE(k < 0 || k == d_ff / 4, "the 2-of-8 mask keeps d_ff / 4 channels");
+        TORCH_CHECK_VALUE(k == kNotGiven || k == d_ff / 4, "the 2-of-8 mask keeps d_ff / 4 channels");
         k = d_ff / 4;
     }
+    TORCH_CHECK_TYPE(k != kNotGiven, "k must be a whole number, not None");
     d.tokens = x.size(0);
     d.d_model = (int32_t)x.size(1);
     d.d_ff = (int32_t)d_ff;
@@ -194,9 +198,9 @@ Tensor tensor_arg(PyObject *o, const char *name, bool optional) {
     }
     return THPVariable_Unpack(o);
 }
-// a whole number, or -1 for None
+// a whole number, or kNotGiven for None
 int64_t int_arg(PyObject *o) {
-    if (o == Py_None) return -1;
+    if (o == Py_None) return kNotGiven;
     const long long v = PyLong_AsLongLong(o);
     if (v != -1 || !PyErr_Occurred()) return v;
     // (numbers that int() takes, as before: numpy integers, 0-d tensors, floats)

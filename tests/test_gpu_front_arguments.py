@@ -1,0 +1,29 @@
+"""Sizes that the entry points refuse: -1 is a number like any other and not the same as leaving an argument out."""
+import pytest
+import torch
+
+from paper_2511_09323_b200 import binding as B
+from paper_2511_09323_b200.autograd import moc_ffn
+
+pytestmark = pytest.mark.gpu
+CALLS = {"ffn": moc_ffn, "forward": lambda *a, **o: B.moc_ffn_forward(*a, **o, save=False)[0], "decode": B.moc_ffn_decode,
+         "decode_block": lambda x, *a, **o: B.moc_ffn_decode_block(x, torch.ones_like(x[0]), 1e-5, *a, **o)}
+
+
+@pytest.mark.parametrize("call", CALLS)
+def test_minus_one_and_none(call):
+    x, *w = (torch.randn(n, 64, device="cuda").bfloat16() for n in (4, 96, 96, 96))
+    run = CALLS[call]
+    for k in (-1, 0, 25):
+        with pytest.raises(ValueError, match="d_ff / 4"):
+            run(x, *w, k, grouped=True)
+    for k, d_ff in ((8, -1), (8, 0), (-1, None), (-1, 64)):
+        with pytest.raises(B.MocError) as e:
+            run(x, *w, k, d_ff=d_ff)
+        assert e.value.status == B.MOC_ERR_INVALID_ARG
+    with pytest.raises(ValueError, match="multiple of 8"):
+        run(x, *w, None, d_ff=-1, grouped=True)
+    with pytest.raises(TypeError):
+        run(x, *w, None)
+    assert torch.equal(run(x, *w, None, grouped=True), run(x, *w, 24, grouped=True))
+    torch.testing.assert_close(run(x, *w, 8, d_ff=None), run(x, *w, 8, d_ff=96), rtol=2e-2, atol=2e-2)
