@@ -160,11 +160,12 @@ struct MocFfnNode : public torch::autograd::Function<MocFfnNode> {
         if (!grads[0].defined()) return res;
         const Tensor &g0 = grads[0];
         const Tensor go = g0.dim() == 2 && g0.is_contiguous() ? g0 : g0.reshape({-1, g0.size(-1)}).contiguous();
-        check_dev(go);
+        check_all(x, w_gate, w_up, w_down, kept, go);  // (saved-tensor hooks hand back what they like)
         moc_ffn_desc d = make_desc(x, w_gate, call[0], call[1], (uint32_t)call[2]);
         void *stream = c10::cuda::getCurrentCUDAStream().stream();
         const Tensor ws = workspace_for(d, MOC_OP_BACKWARD, x);
         const Kept at(d, call[3] == 0);
+        TORCH_CHECK_VALUE(kept.scalar_type() == at::kByte && kept.numel() == at.total, "the saved activations came back in another form");
         const char *base = static_cast<const char *>(in(kept));
         const int16_t *idx = reinterpret_cast<const int16_t *>(base);
         const void *tg = base + at.gate, *tu = base + at.up;
