@@ -182,6 +182,12 @@ def _stream_ptr(stream=None):
     return ctypes.c_void_p(s.cuda_stream)
 
 
+def _used_on(stream, workspace):
+    """A workspace allocated for one call on `stream`: not to be handed out again before that stream has passed the call."""
+    if stream is not None and stream.cuda_stream != torch.cuda.current_stream().cuda_stream:
+        workspace.record_stream(stream if isinstance(stream, torch.Stream) else torch.cuda.ExternalStream(stream.cuda_stream))
+
+
 def _check_dev(*tensors):
     for t in tensors:
         if t is None:
@@ -256,6 +262,7 @@ def moc_ffn_backward(x, w_gate, w_up, w_down, topk_idx, topk_gate, topk_up, grad
     _check_dev(*res.values())
     if workspace is None:
         workspace = alloc_workspace(desc, MOC_OP_BACKWARD, x.device)
+        _used_on(stream, workspace)
     args = (ctypes.byref(desc), _ptr(x), _ptr(w_gate), _ptr(w_up), _ptr(w_down), _ptr(topk_idx), _ptr(topk_gate),
             _ptr(topk_up), _ptr(grad_out), _ptr(res["grad_x"]), _ptr(res["grad_w_gate"]), _ptr(res["grad_w_up"]),
             _ptr(res["grad_w_down"]), _ptr(workspace), workspace.numel(), _stream_ptr(stream))
@@ -282,6 +289,7 @@ def moc_ffn_recompute_up(x, w_up, topk_idx, d_ff=None, out=None, workspace=None,
         out = torch.empty((T, k), dtype=x.dtype, device=x.device)
     if workspace is None:
         workspace = alloc_workspace(desc, MOC_OP_BACKWARD, x.device)
+        _used_on(stream, workspace)
     rc = load().moc_ffn_recompute_up(ctypes.byref(desc), _ptr(x), _ptr(w_up), _ptr(topk_idx), _ptr(out),
                                      _ptr(workspace), workspace.numel(), _stream_ptr(stream))
     if rc != MOC_OK:
@@ -349,6 +357,7 @@ def moc_topk_select_tc(gate: torch.Tensor, k: int, n: int | None = None, bracket
     if need == 0:
         raise MocError(MOC_ERR_UNSUPPORTED, "moc_topk_select_tc")
     ws = torch.empty(need, dtype=torch.uint8, device=gate.device)
+    _used_on(stream, ws)
     idx = torch.empty((rows, k), dtype=torch.int16, device=gate.device)
     variant = ctypes.c_int(-1)
     br = None if bracket is None else (ctypes.c_float * 2)(float(bracket[0]), float(bracket[1]))
@@ -374,6 +383,7 @@ def moc_ffn_decode_probe(x, w_gate, w_up, w_down, k, d_ff=None, stream=None, gro
     if need == 0:
         raise MocError(MOC_ERR_UNSUPPORTED, "moc_ffn_decode_probe")
     ws = torch.empty(need, dtype=torch.uint8, device=x.device)
+    _used_on(stream, ws)
     rc = load().moc_ffn_decode_probe(ctypes.byref(desc), _ptr(x), _ptr(w_gate), _ptr(w_up), _ptr(w_down), _ptr(out),
                                      _ptr(kept), _ptr(ws), ws.numel(), _stream_ptr(stream))
     if rc != MOC_OK:
@@ -407,6 +417,7 @@ def moc_tc_gemm_sp_dense_bf16(a: torch.Tensor, b: torch.Tensor, out=None, accumu
     if need == 0:
         raise MocError(MOC_ERR_INVALID_ARG, "moc_tc_gemm_sp_dense_bf16")
     ws = torch.empty(need, dtype=torch.uint8, device=a.device)
+    _used_on(stream, ws)
     if out is None:
         out = torch.empty((m, n), dtype=torch.bfloat16, device=a.device)
     left_out = ctypes.c_int64(-1)
@@ -442,6 +453,7 @@ def moc_test_small_batch_stall(x, w_gate, w_up, w_down, k, limit_cycles: int, d_
         out = torch.empty_like(x)
     if workspace is None:
         workspace = alloc_workspace(desc, MOC_OP_DECODE, x.device)
+        _used_on(stream, workspace)
     rc = load().moc_test_small_batch_stall(ctypes.byref(desc), _ptr(x), _ptr(w_gate), _ptr(w_up), _ptr(w_down), _ptr(out),
                                            _ptr(workspace), workspace.numel(), int(limit_cycles), _stream_ptr(stream))
     if rc != MOC_OK:

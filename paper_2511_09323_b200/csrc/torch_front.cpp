@@ -10,6 +10,7 @@
 #include <Python.h>
 
 #include <ATen/ATen.h>
+#include <c10/cuda/CUDACachingAllocator.h>
 #include <c10/cuda/CUDAGuard.h>
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/Exceptions.h>
@@ -100,6 +101,14 @@ void *stream_of(PyObject *stream) {
     Py_DECREF(v);
     if (!p && PyErr_Occurred()) throw python_error();
     return p;
+}
+
+// A workspace allocated here for a call on another stream than the current one: free again when the call returns, and not to be
+// handed out before that stream has passed the call.
+void used_on(void *stream, const Tensor &own) {
+    if (!own.defined() || c10::cuda::getCurrentCUDAStream().stream() == stream) return;
+    c10::cuda::CUDACachingAllocator::recordStream(
+        own.storage().data_ptr(), c10::cuda::getStreamFromExternal(static_cast<cudaStream_t>(stream), own.device().index()));
 }
 
 // ---- the autograd node ----------------------------------------------------------------------------------------
@@ -265,14 +274,16 @@ PyObject *py_forward(PyObject *, PyObject *const *a, Py_ssize_t n) {
     } else {
         idx = tg = tu = Tensor();
     }
-    if (!ws.defined()) ws = workspace_for(d, MOC_OP_FORWARD, x);
     void *stream = stream_of(a[13]);
+    Tensor own;
+    if (!ws.defined()) own = ws = workspace_for(d, MOC_OP_FORWARD, x);
     int rc;
     {
         pybind11::gil_scoped_release no_gil;
         rc = moc_ffn_forward(&d, in(x), in(wg), in(wu), in(wd), outp(out), static_cast<int16_t *>(outp(idx)), outp(tg), outp(tu),
                              outp(ws), (size_t)ws.numel(), stream);
     }
+    used_on(stream, own);
     if (rc != MOC_OK) raise_moc(rc, "moc_ffn_forward");
     PyObject *t = PyTuple_New(4);
     if (!t) throw python_error();
@@ -305,8 +316,9 @@ PyObject *py_decode(PyObject *, PyObject *const *a, Py_ssize_t n) {
                          "rms_weight must be a [d_model] tensor of the activations' dtype");
     const moc_ffn_desc d = make_desc(x, wg, int_arg(a[4]), int_arg(a[5]), (uint32_t)int_arg(a[6]));
     if (!out.defined()) out = at::empty_like(x);
-    if (!ws.defined()) ws = workspace_for(d, BLOCK ? MOC_OP_DECODE_BLOCK : MOC_OP_DECODE, x);
     void *stream = stream_of(a[9]);
+    Tensor own;
+    if (!ws.defined()) own = ws = workspace_for(d, BLOCK ? MOC_OP_DECODE_BLOCK : MOC_OP_DECODE, x);
     int rc;
     {
         pybind11::gil_scoped_release no_gil;
@@ -314,6 +326,7 @@ PyObject *py_decode(PyObject *, PyObject *const *a, Py_ssize_t n) {
                                           (size_t)ws.numel(), stream)
                    : moc_ffn_decode(&d, in(x), in(wg), in(wu), in(wd), outp(out), outp(ws), (size_t)ws.numel(), stream);
     }
+    used_on(stream, own);
     if (rc != MOC_OK) raise_moc(rc, BLOCK ? "moc_ffn_decode_block" : "moc_ffn_decode");
     return THPVariable_Wrap(out);
     END_HANDLE_TH_ERRORS

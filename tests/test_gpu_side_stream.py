@@ -1,0 +1,36 @@
+"""Calls on another stream than the current one that allocate their own workspace: nobody else gets its memory while they run."""
+import pytest
+import torch
+
+from paper_2511_09323_b200 import binding as B
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("call", ("forward", "backward", "recompute_up", "decode", "decode_block"))
+def test_workspace_outlives_the_call(call):
+    T, d, F, K = 300 if call in ("forward", "backward", "recompute_up") else 20, 512, 2048, 256
+    g = torch.Generator(device="cuda").manual_seed(3)
+    x, *w = (torch.randn(n, d, generator=g, device="cuda").bfloat16() for n in (T, F, F, F))
+    out, idx, gate, up = B.moc_ffn_forward(x, *w, K)
+    run = {"forward": lambda s: B.moc_ffn_forward(x, *w, K, save=False, out=out, stream=s),
+           "backward": lambda s: B.moc_ffn_backward(x, *w, idx, gate, up, x, want=("x",), grads={"grad_x": out}, stream=s),
+           "recompute_up": lambda s: B.moc_ffn_recompute_up(x, w[1], idx, out=up, stream=s),
+           "decode": lambda s: B.moc_ffn_decode(x, *w, K, out=out, stream=s),
+           "decode_block": lambda s: B.moc_ffn_decode_block(x, w[0][0], 1e-5, *w, K, out=out, stream=s)}[call]
+    op = {"forward": B.MOC_OP_FORWARD, "decode": B.MOC_OP_DECODE, "decode_block": B.MOC_OP_DECODE_BLOCK}.get(call, B.MOC_OP_BACKWARD)
+    size = B.moc_ffn_workspace_bytes(B.make_desc(T, d, F, K, x.dtype), op)
+    run(None)
+    torch.zeros(1, dtype=torch.uint8, device="cuda").any()   # (the kernels used below are loaded)
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(side):
+        torch.cuda._sleep(200_000_000)   # some hundred milliseconds, in which the call waits
+    run(side)
+    others = [torch.zeros(size, dtype=torch.uint8, device="cuda") for _ in range(2)]   # would be the workspace's memory
+    torch.cuda.current_stream().synchronize()
+    busy = not side.query()
+    torch.cuda.synchronize()
+    assert busy                          # (else the call was over before the memory could be taken)
+    assert not any(o.any() for o in others)
+    assert B.moc_last_device_status() == B.MOC_OK
