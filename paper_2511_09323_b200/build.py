@@ -25,9 +25,20 @@ def _nvcc() -> str:
     return "nvcc"
 
 
+def front_built_for() -> str:
+    """The interpreter and torch that a _front.so built now belongs to (it uses torch's C++ interface, which has no stable ABI)."""
+    import sysconfig
+
+    import torch
+    return f"{sysconfig.get_config_var('SOABI')}, torch {torch.__version__}"
+
+
 def _front_is_current() -> bool:
     if not os.path.exists(FRONT):
         return False
+    with open(FRONT, "rb") as fh:
+        if f"[{front_built_for()}]".encode() not in fh.read():
+            return False
     have = os.path.getmtime(FRONT)
     include = os.path.join(os.path.dirname(HERE), "include")
     sources = [os.path.join(CSRC, FRONT_SOURCE)] + [os.path.join(include, n) for n in os.listdir(include)]
@@ -43,7 +54,7 @@ def build_front() -> str:
     tmp = FRONT + ".tmp.%d" % os.getpid()
     libs = cpp_extension.library_paths(device_type="cuda")
     cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", "-Wall",
-           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"]
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", f'-DMOC_FRONT_BUILT_FOR="[{front_built_for()}]"']
     cmd += ["-isystem" + p for p in cpp_extension.include_paths(device_type="cuda") + [sysconfig.get_paths()["include"]]]
     cmd += [os.path.join(CSRC, FRONT_SOURCE), "-o", tmp, "-L" + HERE, "-l:" + os.path.basename(LIB), "-Wl,-rpath,$ORIGIN"]
     cmd += ["-L" + p for p in libs] + ["-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda"]

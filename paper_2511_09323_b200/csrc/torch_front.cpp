@@ -351,6 +351,8 @@ PyMethodDef kMethods[] = {
     {"set_traced_ffn", py_set<g_traced_ffn>, METH_O, nullptr},
     {nullptr, nullptr, 0, nullptr},
 };
+// (build.py looks for it in the file: a module built for another torch is built again)
+__attribute__((used)) const char kBuiltFor[] = MOC_FRONT_BUILT_FOR;
 PyModuleDef kModule = {PyModuleDef_HEAD_INIT, "_front", nullptr, -1, kMethods, nullptr, nullptr, nullptr, nullptr};
 
 }  // namespace
