@@ -223,6 +223,8 @@ inline int launch_gemm(const Params &p_in, cudaStream_t st, int k_split = 1, int
             for (int i = 0; i < 2; ++i)
                 if (p.b_op[i].ptr && !map_k_major(&w.b_rem1[i], p.b_op[i].ptr, p.b_op[i].n, p.b_op[i].k, p.b_op[i].ld, rem1 / 2)) return MOC_ERR_CUDA;
         return launch_pairs(kern, w, std::min(w.t.total, max_pairs), WIDE_THREADS, WIDE_SMEM_BYTES, st);
+    } else if constexpr (TRANSPOSED) {
+        return MOC_ERR_UNSUPPORTED;  // (operands are exchanged for CTA pairs alone)
     } else {
         const auto kern = gemm_kernel<A_MN, B_MN, EPI>;
         static bool configured = false;
