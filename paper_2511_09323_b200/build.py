@@ -87,7 +87,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
 
 def _build_library(verbose: bool) -> None:
     tmp = LIB + ".tmp.%d" % os.getpid()
-    extra = os.environ.get("MOC_FFN_NVCC_FLAGS", "").split()   # e.g. -DMOC_TIMELINE for a development build
+    extra = os.environ.get("MOC_FFN_NVCC_FLAGS", "").split()   # further compiler flags
     cmd = [_nvcc()] + NVCC_FLAGS + extra + (["-Xptxas", "-v"] if verbose else []) + \
         [os.path.join(CSRC, s) for s in SOURCES] + ["-o", tmp]
     proc = subprocess.run(cmd, capture_output=True, text=True)

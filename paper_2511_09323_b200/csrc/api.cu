@@ -2291,169 +2291,6 @@ int moc_last_device_status(void *cuda_stream) {
     return v;
 }
 
-#ifdef MOC_TIMELINE
-extern "C" __attribute__((visibility("default"))) int moc_debug_timeline(unsigned long long *out, int n) {
-    if (cudaDeviceSynchronize() != cudaSuccess) return MOC_ERR_CUDA;
-    return cudaMemcpyFromSymbol(out, g_timeline, sizeof(unsigned long long) * (size_t)std::min(n, 4096)) == cudaSuccess
-               ? MOC_OK : MOC_ERR_CUDA;
-}
-
-// development probe: W [rows_total, cols] bf16 is read once in TMA boxes of rows_per_cta rows x 64 columns, `boxes`
-// adjacent boxes per stage through a ring of `stages` stages, nothing computed
-namespace moc { namespace {
-struct BoxProbe {
-    CUtensorMap map;
-    int rows, cols, boxes, stages;
-    uint32_t pitch;
-    int *status;
-};
-__global__ void __launch_bounds__(64, 1) box_probe_kernel(const __grid_constant__ BoxProbe p) {
-    extern __shared__ uint8_t smem_raw[];
-    __shared__ uint64_t bars[64];
-    __shared__ int s_abort;
-    const uint32_t base = (tc::smem_u32(smem_raw) + 1023u) & ~1023u;
-    auto full_bar = [&](int s) { return tc::smem_u32(&bars[s]); };
-    auto empty_bar = [&](int s) { return tc::smem_u32(&bars[32 + s]); };
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < p.stages; ++s) {
-            tc::mbar_init(full_bar(s), 1);
-            tc::mbar_init(empty_bar(s), 1);
-        }
-        s_abort = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    }
-    __syncthreads();
-    const int n = (p.cols / 64 + p.boxes - 1) / p.boxes;
-    const int row0 = (int)blockIdx.x * p.rows;
-    if (threadIdx.x == 0) {
-        int stage = 0;
-        uint32_t phase = 0;
-        for (int i = 0; i < n; ++i) {
-            if (!tc::mbar_wait(empty_bar(stage), phase ^ 1u, &s_abort, p.status)) return;
-            tc::mbar_expect_tx(full_bar(stage), (uint32_t)p.boxes * (uint32_t)p.rows * 128u);
-            for (int b = 0; b < p.boxes; ++b)
-                tc::tma_load_2d(base + (uint32_t)stage * p.boxes * p.pitch + (uint32_t)b * p.pitch, &p.map, full_bar(stage),
-                                (i * p.boxes + b) * 64, row0);
-            if (++stage == p.stages) {
-                stage = 0;
-                phase ^= 1u;
-            }
-        }
-    } else if (threadIdx.x == 32) {
-        int stage = 0;
-        uint32_t phase = 0;
-        for (int i = 0; i < n; ++i) {
-            if (!tc::mbar_wait(full_bar(stage), phase, &s_abort, p.status)) return;
-            tc::mbar_arrive(empty_bar(stage));
-            if (++stage == p.stages) {
-                stage = 0;
-                phase ^= 1u;
-            }
-        }
-    }
-}
-} }
-extern "C" MOC_API int moc_debug_stream_boxes(const void *w, int rows_total, int cols, int rows_per_cta, int boxes, int stages,
-                                              void *cuda_stream) {
-    BoxProbe p;
-    memset(&p, 0, sizeof(p));
-    if (stages > 32 || rows_per_cta > 256) return MOC_ERR_INVALID_ARG;
-    if (!tc::make_map(&p.map, static_cast<const __nv_bfloat16 *>(w), rows_total, cols, cols, 64, rows_per_cta)) return MOC_ERR_CUDA;
-    p.rows = rows_per_cta;
-    p.cols = cols;
-    p.boxes = boxes;
-    p.stages = stages;
-    p.pitch = ((uint32_t)rows_per_cta * 128u + 1023u) & ~1023u;
-    p.status = device_status_ptr();
-    const size_t smem = 1024 + (size_t)stages * boxes * p.pitch;
-    int rc = set_smem(box_probe_kernel, smem, 1024);
-    if (rc != MOC_OK) return rc;
-    box_probe_kernel<<<(rows_total + rows_per_cta - 1) / rows_per_cta, 64, smem, static_cast<cudaStream_t>(cuda_stream)>>>(p);
-    return launch_ok();
-}
-
-// development probe: cycles per MMA, seen by the issuing thread, of `count` MMAs of shape M x N x 16 (bf16, operands in
-// shared memory, K-major, all zero) issued back to back with a tcgen05.commit after every `per_commit` of them.
-// mode bit 0: the thread waits for every commit's barrier (else only for the last); bit 1: a second thread issues the same
-// sequence at the same time into its own TMEM columns and barriers (the figure is still the first thread's).
-namespace moc { namespace {
-__global__ void __launch_bounds__(128, 1) mma_probe_kernel(int m, int n, int count, int per_commit, int mode, long long *cycles, int *status) {
-    extern __shared__ uint8_t smem_raw[];
-    __shared__ uint64_t bars4[4];
-    __shared__ uint32_t holder;
-    __shared__ int s_abort;
-    const uint32_t base = (tc::smem_u32(smem_raw) + 1023u) & ~1023u;
-    for (int i = threadIdx.x; i < 96 * 1024 / 4; i += 128) reinterpret_cast<uint32_t *>(smem_raw + (base - tc::smem_u32(smem_raw)))[i] = 0u;
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < 4; ++i) tc::mbar_init(tc::smem_u32(&bars4[i]), 1);
-        s_abort = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    }
-    if (threadIdx.x < 32) {
-        tc::tmem_alloc(tc::smem_u32(&holder), 512);
-        tc::tmem_relinquish();
-    }
-    tc::tc_fence_before();
-    __syncthreads();
-    tc::tc_fence_after();
-    const uint32_t who = threadIdx.x >> 5;
-    const uint32_t tmem = holder + who * 256;
-    const uint32_t bar = tc::smem_u32(&bars4[2 * who]), bar_unwaited = tc::smem_u32(&bars4[2 * who + 1]);
-    if (threadIdx.x == 0 || ((mode & 2) && threadIdx.x == 32)) {
-        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
-        uint32_t parity = 0;
-        // eight descriptor pairs held in registers: A walks over three 11 KiB regions, so that the loop is nothing but MMAs
-        const uint64_t ad0 = tc::make_smem_desc(base, 16, 1024), bd0 = tc::make_smem_desc(base + 49152, 16, 1024);
-        uint64_t ad[8], bd[8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            ad[e] = ad0 + (uint64_t)((e & 3) * 2 + (e >> 2) * 704);
-            bd[e] = bd0 + (uint64_t)((e & 3) * 2);
-        }
-        const long long t0 = clock64();
-        for (int i = 0; i < count; i += per_commit) {
-            for (int j = 0; j < per_commit; j += 8) {
-#pragma unroll
-                for (int e = 0; e < 8; ++e)
-                    asm volatile(
-                        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, 1, 0;\n\t"
-                        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem), "l"(ad[e]), "l"(bd[e]), "r"(idesc)
-                        : "memory");
-            }
-            if (!(mode & 1) && i + per_commit < count) {
-                tc::umma_commit(bar_unwaited);  // nobody waits for this one
-                continue;
-            }
-            tc::umma_commit(bar);
-            if (!tc::mbar_wait(bar, parity, &s_abort, status)) break;
-            parity ^= 1u;
-        }
-        if (blockIdx.x == 0 && threadIdx.x == 0) *cycles = clock64() - t0;
-    }
-    tc::tc_fence_before();
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        tc::tc_fence_after();
-        tc::tmem_dealloc(holder, 512);
-    }
-}
-} }
-extern "C" MOC_API long long moc_debug_mma_cycles(int m, int n, int count, int per_commit, int mode) {
-    if (m != 64 && m != 128) return -4;
-    if (n < 16 || n > 256 || n % 16 || count < 8 || per_commit < 8 || per_commit % 8 || count % per_commit) return -4;
-    long long *dev = nullptr, host = -1;
-    if (cudaMalloc(&dev, sizeof(long long)) != cudaSuccess) return -1;
-    const size_t smem = 100 * 1024;  // A within the first 48 KiB, B (up to 256 rows of 128 bytes) behind it
-    if (set_smem(mma_probe_kernel, smem, 1024) != MOC_OK) return -2;
-    mma_probe_kernel<<<tc::sm_count(), 128, smem>>>(m, n, count, per_commit, mode, dev, device_status_ptr());
-    if (cudaMemcpy(&host, dev, sizeof(host), cudaMemcpyDeviceToHost) != cudaSuccess) host = -3;
-    cudaFree(dev);
-    return host;
-}
-#endif
-
 int moc_profile_stream_read(const void *a, size_t a_bytes, const void *b, size_t b_bytes, const void *c, size_t c_bytes,
                             void *cuda_stream) {
     const void *ptr[3] = {a, b, c};

@@ -142,8 +142,6 @@ __global__ void __launch_bounds__(kThreads, 1) sb_gate_up_kernel(const __grid_co
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_holder + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     tc::pdl_launch_dependents();
-    MOC_TL(p.mask_mode ? 32 : 0);
-    MOC_TL_CTA(p.mask_mode ? 1536 : 256);
 
     const int prob = p.prob0 + (int)blockIdx.x / p.ctas_per_matrix;
     const int ch0 = ((int)blockIdx.x % p.ctas_per_matrix) * p.rows;
@@ -233,14 +231,11 @@ __global__ void __launch_bounds__(kThreads, 1) sb_gate_up_kernel(const __grid_co
                 }
             }
             if (ok) tc::umma_commit(ring.tfull());
-            MOC_TL_IF(p.mask_mode ? 34 : 2, blockIdx.x == 0);
-            MOC_TL_CTA_ANY(p.mask_mode ? 1792 : 512);
         }
     } else {
         // ---- epilogue: lane = channel, columns = tokens; a warp's store of one token is 128 contiguous bytes
         const int quarter = warp & 3;
         tc::pdl_wait();  // the workspace may still be read by the previous call's kernels
-        MOC_TL_IF(p.mask_mode ? 35 : 3, blockIdx.x == 0 && threadIdx.x == 64);
         if (blockIdx.x == 0)
             for (int i = (int)threadIdx.x - 64; i < p.n_counters; i += kEpiThreads) p.counters[i] = 0;
         const int valid = min(p.rows, p.F - ch0);  // channels of this CTA inside the matrix
@@ -368,8 +363,6 @@ __global__ void __launch_bounds__(kThreads, 1) sb_gate_up_kernel(const __grid_co
     }
     tc::tc_fence_before();
     __syncthreads();
-    MOC_TL(p.mask_mode ? 36 : 4);
-    MOC_TL_CTA(p.mask_mode ? 2048 : 768);
     if (warp == 1) {
         tc::tc_fence_after();
         tc::tmem_dealloc(tmem_base, (uint32_t)p.tmem_cols);
@@ -415,14 +408,11 @@ __global__ void __launch_bounds__(dec::kSelThreads) sb_select_kernel(const Selec
     uint32_t *bits = lists;  // bitmap of the kept channels once the search is over
     const float *u_row = p.stage_u ? reinterpret_cast<const float *>(lists + 2 * dec::kSelListCap)
                                    : p.U + (int64_t)t * p.ldf;
-    MOC_TL(16);
     if (p.kept_bits) {
         // the up kernel behind this one streams its weights while the selection runs; it may start only now that the
         // gate kernel has completed (it reads x without a wait of its own)
         tc::pdl_wait();
         tc::pdl_launch_dependents();
-        MOC_TL(17);
-        MOC_TL_CTA(1024);
     } else {
         tc::pdl_launch_dependents();
         tc::pdl_wait();
@@ -458,8 +448,6 @@ __global__ void __launch_bounds__(dec::kSelThreads) sb_select_kernel(const Selec
             __syncthreads();
             for (int i = tid; i < p.kept_words; i += dec::kSelThreads) my_bits[i] = bits[i];
         }
-        MOC_TL(18);
-        MOC_TL_CTA(1280);
         return;
     }
     const bool save = p.idx_out != nullptr;
@@ -566,8 +554,6 @@ __global__ void __launch_bounds__(kThreads, 1) sb_down_kernel(const __grid_const
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_holder + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     tc::pdl_launch_dependents();
-    MOC_TL(48);
-    MOC_TL_CTA(2304);
 
     const int m_blk = (int)blockIdx.x / p.splits, split = (int)blockIdx.x - m_blk * p.splits;
     const int kb_all = p.k_blocks * p.segments;
@@ -615,8 +601,6 @@ __global__ void __launch_bounds__(kThreads, 1) sb_down_kernel(const __grid_const
     if (warp == 0) {
         if (lane == 0) {
             tc::pdl_wait();  // Z' comes from the select kernel
-            MOC_TL_IF(49, blockIdx.x == 0);
-            MOC_TL_CTA_ANY(2560);
             for (int i = 0; i < ahead; ++i) load_z(i, kb0 + i);
             int stage = 0;
             uint32_t phase = 1;
@@ -659,7 +643,6 @@ __global__ void __launch_bounds__(kThreads, 1) sb_down_kernel(const __grid_const
                 }
             }
             if (ok) tc::umma_commit(ring.tfull());
-            MOC_TL_CTA_ANY(2816);
         }
     } else {
         // ---- epilogue: lane = output column, TMEM columns = tokens
@@ -782,8 +765,6 @@ __global__ void __launch_bounds__(kThreads, 1) sb_down_kernel(const __grid_const
     }
     tc::tc_fence_before();
     __syncthreads();
-    MOC_TL(52);
-    MOC_TL_CTA(3072);
     if (warp == 1) {
         tc::tc_fence_after();
         tc::tmem_dealloc(tmem_base, (uint32_t)p.tmem_cols);

@@ -199,14 +199,11 @@ __device__ __forceinline__ void selector_role(const FusedParams &p, uint32_t *dy
     }
     __syncthreads();
     if (s_abort) return;
-    MOC_TL_CTA(1280);
     if (!dec::cta_stage_rows(&s_bar, &s_abort, p.status, keys, p.G + (int64_t)t * p.ldf, (uint32_t)Fp * 4u)) return;
-    MOC_TL_CTA(3072);
     uint32_t tau;
     int need;
     bool ties_cut;
     dec::cta_select_threshold<false>(nullptr, p.F, p.K, keys, lists, sm, tau, need, ties_cut);
-    MOC_TL_CTA(3328);
     uint32_t *my_bits = p.kept_bits + (int64_t)t * p.kept_words;
     constexpr int NW = kBlock / 32;
     if (!ties_cut) {
@@ -229,10 +226,8 @@ __device__ __forceinline__ void selector_role(const FusedParams &p, uint32_t *dy
     __syncthreads();
     if (tid == 0) {
         atomicAdd(p.flags + 1, 1u);
-        MOC_TL_CTA_ANY(3840);
         cta_finished(p);
     }
-    MOC_TL_CTA(1536);
 }
 
 // ------------------------------------------------------------------------------------------------ the kernel
@@ -249,15 +244,6 @@ __global__ void __launch_bounds__(kBlock, 1) sb_fused_kernel(const __grid_consta
         const CUtensorMap *m = lane == 0 ? &p.wg_map : lane == 1 ? &p.x_map : lane == 2 ? &p.wu_map : lane == 3 ? &p.wd_map : &p.z_map;
         asm volatile("prefetch.tensormap [%0];" ::"l"(m) : "memory");
     }
-    MOC_TL_CTA(256);
-#ifdef MOC_TIMELINE
-    if (blockIdx.x == 0 && threadIdx.x == 0) {  // the starts of the last 64 calls
-        const unsigned long long n = atomicAdd(&g_timeline[4095], 1ull);
-        unsigned long long t;
-        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-        g_timeline[3584 + (int)(n & 63ull)] = t;
-    }
-#endif
 
     // ---- the streamer's shared memory and work (a selector CTA computes the same numbers and uses none of them)
     const uint32_t raw = tc::smem_u32(smem_raw);
@@ -363,7 +349,6 @@ __global__ void __launch_bounds__(kBlock, 1) sb_fused_kernel(const __grid_consta
         cg::this_grid().sync();  // the flags and counters are zero for everyone
     }
     tc::tc_fence_after();
-    MOC_TL_CTA(512);
 
     if (!streamer) {
         selector_role(p, reinterpret_cast<uint32_t *>(smem_raw));
@@ -411,7 +396,6 @@ __global__ void __launch_bounds__(kBlock, 1) sb_fused_kernel(const __grid_consta
             if (ok && n_d > 0) {
                 ok = flag_wait(p.flags + 2, (unsigned int)p.n_gu, abort_flag, p.status, p.wait_limit);  // every streamer's part of Z' is written
                 asm volatile("fence.proxy.async;" ::: "memory");                           // ... by ordinary stores; TMA reads it
-                MOC_TL_CTA_ANY(2304);
                 int st = first_stage;
                 for (int i = 0; i < issued && ok; ++i) {
                     tc::tma_load_2d(slot(st) + d_w_bytes, &p.z_map, full_bar(st), (kb0 + i) * kBK, 0);
@@ -470,7 +454,6 @@ __global__ void __launch_bounds__(kBlock, 1) sb_fused_kernel(const __grid_consta
                     next();
                 }
                 if (ok && n_gu > 0) tc::umma_commit(m == 0 ? tfull_g : tfull_u);
-                MOC_TL_IF((m == 0 ? 768 : 1792) + (int)blockIdx.x, w == 1u);
             }
             const uint32_t accd = tmem_base + 256u + 64u * w;
             uint32_t accum = 0u;
@@ -493,7 +476,6 @@ __global__ void __launch_bounds__(kBlock, 1) sb_fused_kernel(const __grid_consta
                 next();
             }
             if (ok && n_d > 0) tc::umma_commit(tfull_d);
-            MOC_TL_IF(2560 + (int)blockIdx.x, w == 1u);
         }
     } else if (warp < 3 + kEpiWarps) {
         // ------------------------------------------------------------------ epilogue warps 3..10
@@ -569,7 +551,6 @@ __global__ void __launch_bounds__(kBlock, 1) sb_fused_kernel(const __grid_consta
                 if (etid == 0 && !*abort_flag) atomicAdd(p.flags, 1u);  // (a CTA that gave up is never counted: those that
                                                                           //  wait for it give up in turn, nothing half-done is read)
             }
-            MOC_TL_IF(1024 + (int)blockIdx.x, etid == 0);
             // ---- Z' = SiLU(g) u on the kept channels.  The products are formed for every channel as soon as the up
             // projection is complete; the bitmaps, which usually arrive last, then only decide which of them are stored.
             ok = ok && __all_sync(0xffffffffu, tc::mbar_wait(tfull_u, 0u, abort_flag, p.status, p.wait_limit));
@@ -640,7 +621,6 @@ __global__ void __launch_bounds__(kBlock, 1) sb_fused_kernel(const __grid_consta
             __threadfence();
             asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory");
             if (etid == 0 && !*abort_flag) atomicAdd(p.flags + 2, 1u);
-            MOC_TL_IF(2048 + (int)blockIdx.x, etid == 0);
         }
         // ---- D: partial sums into the fp32 accumulator, the last CTA of the column block rounds
         if (has_d) {
@@ -718,7 +698,6 @@ __global__ void __launch_bounds__(kBlock, 1) sb_fused_kernel(const __grid_consta
     }
     tc::tc_fence_before();
     __syncthreads();
-    MOC_TL_CTA(2816);
     if (threadIdx.x == 0 && !*abort_flag) cta_finished(p);
     if (warp == 1) {
         tc::tc_fence_after();
