@@ -314,6 +314,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_coop_kernel(const Params p
             }
             if (kept && lane == 0) atomicOr(reinterpret_cast<unsigned int *>(s_mask) + (r >> 2), (1u << t) << (8 * (r & 3)));
         }
+        tc::fence_async_smem();  // (the list was written with ordinary stores, bulk copies write there next)
         __syncthreads();  // the ring is the producer's again
     } else {
         // MoC 2:8 (Section 4): the CTA's range is made of whole groups of eight channels; the mask is local
