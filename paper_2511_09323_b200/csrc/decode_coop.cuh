@@ -5,7 +5,7 @@
 // share of the CHANNELS for the whole call, so that nothing but a few words per token has to cross between SMs:
 //
 //   phase 1   the CTA streams its channels' rows of W_gate and keeps their gate values g[t][j] in shared memory
-//             (Eq. (Moc-1)); it adds them to a global 2048-bin histogram of the order-preserving keys
+//             (Eq. (Moc-1)); it adds them to a global histogram of the order-preserving keys
 //   select    grid barrier; every CTA scans the histogram for the bin that holds the K-th largest key, appends its
 //             own keys of that bin (with their channels) to a global list; grid barrier; every CTA ranks its own
 //             candidates against the list: a channel is kept when fewer than K channels precede it in
@@ -35,7 +35,22 @@ constexpr int kMaxD = 4096;          // a thread owns 8 output columns
 constexpr int kConsumerWarps = 16;
 constexpr int kThreads = (kConsumerWarps + 1) * 32;  // + one producer warp
 constexpr int kMaxRows = 256;        // channels per CTA
-constexpr int kBins = 2048;          // top 11 bits of the key
+// Bins of the order-preserving keys: 128 to an octave of 2^-5 <= g < 2^4, where a threshold usually lies, 4 to an octave of every
+// other 2^-24 <= |g| < 2^14, one to an octave beyond.  The keys of the threshold's bin go through one counter and are ranked
+// against one another: of 11008 gate values of deviation 1.3 some 480 share a bin of 4 to an octave and 20 one of 128
+// (two tokens, K = F / 8: 2048 x 8192 40.4 -> 39.6, 4096 x 11008 54.2 -> 53.0 us).  With one bin to an octave from 2^-6 down
+// gates of deviation 0.013 took 46.0 us against 40.1 at one token and 66.2 against 54 at two; with 4096 bins, of which none is
+// wider than a quarter of an octave, one token takes 0.3 us more to clear and scan them.
+constexpr int kBins = 2048;
+__host__ __device__ constexpr uint32_t bins_below(uint32_t key, uint32_t from, uint32_t to, int shift) {
+    return ((key < from ? from : key < to ? key : to) - from) >> shift;
+}
+__host__ __device__ constexpr uint32_t key_bin(uint32_t key) {
+    return (key >> 23) + bins_below(key, 0x39800000u, 0x4c800000u, 21) +  // -2^14 < g <= -2^-24
+           bins_below(key, 0xb3800000u, 0xc6800000u, 21) +                // 2^-24 <= g < 2^14
+           bins_below(key, 0xbd000000u, 0xc1800000u, 16);                 // 2^-5 <= g < 2^4
+}
+static_assert(key_bin(0xffffffffu) < (uint32_t)kBins, "the bins cover every key");
 constexpr int kMaxStages = 32;         // a multiple of kConsumerWarps
 constexpr int kFirstRows = 8;  // gate rows requested before x is staged and the shared arrays are cleared (16 or 32 of them
                                // made that start-up 0.9 us longer and the call 1 us slower: they compete with it for the path from L2)
@@ -227,17 +242,21 @@ __global__ void __launch_bounds__(kThreads, 1) decode_coop_kernel(const Params p
     if (!p.grouped) {
         for (int i = tid; i < T * rows; i += kThreads) {
             const int t = i / rows, r = i - t * rows;
-            atomicAdd(&p.hist[t * kBins + (gate_key(sg[t * kMaxRows + r]) >> 21)], 1u);
+            atomicAdd(&p.hist[t * kBins + key_bin(gate_key(sg[t * kMaxRows + r]))], 1u);
         }
         grid.sync();  // #1 (the barrier's release / acquire pair orders the CTAs' writes before the others' reads): every CTA's keys are in the histogram
-        // the bin of the K-th largest key and the number of keys above that bin, per token (suffix sums over 2048 bins:
-        // four bins per consumer thread)
+        // the bin of the K-th largest key and the number of keys above that bin, per token (suffix sums over the bins:
+        // four per consumer thread)
         for (int t = 0; t < T; ++t) {
-            uint32_t h[4] = {0u, 0u, 0u, 0u}, s = 0u;
+            constexpr int N = kBins / (kConsumerWarps * 32);
+            static_assert(N == 4, "one 16-byte load per thread");
+            uint32_t h[N] = {}, s = 0u, own = 0u;
             if (!producer) {
+                const uint4 q = __ldcg(reinterpret_cast<const uint4 *>(p.hist + t * kBins) + tid);
+                h[0] = q.x, h[1] = q.y, h[2] = q.z, h[3] = q.w;
 #pragma unroll
-                for (int i = 0; i < 4; ++i) h[i] = __ldcg(&p.hist[t * kBins + 4 * tid + i]);
-                s = h[0] + h[1] + h[2] + h[3];
+                for (int i = 0; i < N; ++i) s += h[i];
+                own = s;
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) {
                     const uint32_t v = __shfl_down_sync(0xffffffffu, s, o);
@@ -250,11 +269,11 @@ __global__ void __launch_bounds__(kThreads, 1) decode_coop_kernel(const Params p
                 uint32_t after = 0u;
                 for (int w = warp + 1; w < kConsumerWarps; ++w) after += s_scan[w];
                 s += after;  // keys in this thread's bins and all higher ones
-                uint32_t above = s - (h[0] + h[1] + h[2] + h[3]);  // keys in strictly higher bins than this thread's
+                uint32_t above = s - own;  // keys in strictly higher bins than this thread's
 #pragma unroll
-                for (int i = 3; i >= 0; --i) {
+                for (int i = N - 1; i >= 0; --i) {
                     if (above < (uint32_t)p.K && above + h[i] >= (uint32_t)p.K) {
-                        s_bin[t] = (uint32_t)(4 * tid + i);
+                        s_bin[t] = (uint32_t)(N * tid + i);
                         s_above[t] = above;
                     }
                     above += h[i];
@@ -266,7 +285,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_coop_kernel(const Params p
         for (int i = tid; i < T * rows; i += kThreads) {
             const int t = i / rows, r = i - t * rows;
             const uint32_t key = gate_key(sg[t * kMaxRows + r]);
-            if ((key >> 21) == s_bin[t]) {
+            if (key_bin(key) == s_bin[t]) {
                 const uint32_t pos = atomicAdd(&p.cand_n[t], 1u);
                 p.cand[(int64_t)t * F + pos] = make_uint2(key, (uint32_t)(c0 + r));
             }
@@ -293,7 +312,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_coop_kernel(const Params p
         for (int i = warp; i < T * rows; i += kConsumerWarps + 1) {
             const int t = i / rows, r = i - t * rows;
             const uint32_t key = gate_key(sg[t * kMaxRows + r]);
-            const uint32_t bin = key >> 21;
+            const uint32_t bin = key_bin(key);
             bool kept = bin > s_bin[t];
             if (bin == s_bin[t]) {
                 uint32_t nt = 0, ot = 0;

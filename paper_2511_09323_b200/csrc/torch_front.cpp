@@ -5,8 +5,9 @@
 // What bounds it: a small call is over on the GPU in some tens of microseconds, and the same work written in Python
 // (tensor checks, ctypes marshalling, a Python autograd.Function, whose backward has to take the interpreter lock on
 // the autograd thread) took longer than that: 256 fp32 tokens of a 128 x 512 layer, forward and backward, 191 us of which
-// the GPU worked for 62; now 99.  The host's part of a one-token decode call: 15.5 us, now 6.1.  binding.py and autograd.py keep the public signatures and pass their
-// arguments on by position; one call here crosses the language border once, through the vectorcall convention.
+// the GPU worked for 62; now some 90.  The host's part of a one-token decode call: 15.5 us, now 6.1.  binding.py and autograd.py
+// keep the public signatures and pass their arguments on by position; one call here crosses the language border once, through
+// the vectorcall convention.
 #include <Python.h>
 
 #include <ATen/ATen.h>
@@ -115,7 +116,7 @@ void used_on(void *stream, const Tensor &own) {
 // Between forward and backward only the compact Top-K activations live (Section 4, Table 1, column "MoC+GCP"), plus x.
 // recompute_up drops the up values as well; backward forms them again from x, w_up and the indices.
 // They share one allocation, and what backward has to know about the call is one list: with few tokens the step takes as long
-// as its host work (256 tokens of 128 x 512 in fp32: 88 us, of which an allocation is about one).
+// as its host work (256 tokens of 128 x 512 in fp32: some 90 us, of which an allocation is about one).
 struct Kept {
     int64_t gate, up, total;  // byte offsets behind the indices
     explicit Kept(const moc_ffn_desc &d, bool with_up) {
