@@ -40,15 +40,15 @@ FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustain
 # thousand tokens on the device (the full batch is too large to capture); two token counts give the two coefficients,
 # and `roofline.traffic` is their value at the benchmarked token count.
 NCU_DRAM_BYTES = {
-    # weight-gradient GEMM on the LLaMA-1B shape: 524.4 MB at 8192 tokens, 1144.8 MB at 16384 (read + write); the L2
+    # weight-gradient GEMM on the LLaMA-1B shape: 503.0 MB at 8192 tokens, 1106.8 MB at 16384 (read + write); the L2
     # holds a larger share of the operands at the smaller size, hence the negative constant
-    ("C5", "tc_wgrad_gemm"): (-96.1e6, 75735.0),
-    ("C3", "tc_wgrad_gemm"): (-96.1e6, 75735.0),
+    ("C5", "tc_wgrad_gemm"): (-100.8e6, 73706.0),
+    ("C3", "tc_wgrad_gemm"): (-100.8e6, 73706.0),
 }
 # the same for the LLaMA-130M workload, measured at its full size (one launch of each kernel per step)
 NCU_DRAM_BYTES_C2 = {
-    "tc_gate_up_gemm": 173.5e6, "tc_select_mask": 255.1e6, "tc_down_gemm": 75.0e6, "tc_bwd_sample": 235.6e6,
-    "tc_dz_gemm": 43.4e6, "tc_wgrad_gemm": 256.7e6, "tc_dx_gemm": 158.6e6,
+    "tc_gate_up_gemm": 172.0e6, "tc_select_mask": 232.1e6, "tc_down_gemm": 70.8e6, "tc_bwd_sample": 232.2e6,
+    "tc_dz_gemm": 37.8e6, "tc_wgrad_gemm": 252.1e6, "tc_dx_gemm": 151.6e6,
 }
 
 
