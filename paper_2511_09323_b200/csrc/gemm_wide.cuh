@@ -34,6 +34,7 @@ struct WideParams {
     int m_blocks;          // 256-row blocks of one problem
     int stages;
     uint32_t stage_bytes;
+    uint32_t f32_outputs;  // bit i: problem i's output is fp32, not bf16
     // TRANSPOSED: the problems are `k_split` parts of one contraction, of its `k_operands` pairs of operands in turn (k_blocks
     // blocks each; blocks past an operand's end are zeros), their fp32 outputs c_step elements apart
     int k_split, k_operands;
@@ -77,132 +78,233 @@ __device__ __forceinline__ WideTile wide_tile(const WideParams &p, int tile) {
     return t;
 }
 
-// The same for an output that is stored column by column (TRANSPOSED): the lanes are consecutive elements of a stored row, so
+// The epilogues read an accumulator into registers and hand it back to the MMAs (release) before they store it: what the
+// stores take is then hidden behind the next tile's MMAs.  (Released after its last store, by an arrival that also waited for
+// the stores to arrive, an accumulator was held for 4000 cycles (bf16) to 7000 (fp32) and the MMAs stood still for a
+// quarter of gate + up and a fifth of dZ; held for 570 and 2600, 65536 x 2048 x 5504, thousands of SM cycles: gate + up 2 x
+// 1602 -> 2 x 1422, dZ 1508 -> 1320, down 1314 -> 1250, grad_x 2531 -> 2469; 16384 x 768 x 2048, dZ 67.3 -> 56.1.)
+
+// An output that is stored column by column (TRANSPOSED): the lanes are consecutive elements of a stored row, so
 // a column leaves as one contiguous store of the warp.
-template <int EPI>
-__device__ __forceinline__ void transposed_epilogue(const WideParams &w, int prob, int row0, int n0, int cols, int half, uint32_t taddr) {
+template <int EPI, class Release>
+__device__ __forceinline__ void transposed_epilogue(const WideParams &w, int prob, int row0, int n0, int cols, int half, uint32_t taddr,
+                                                    Release release) {
     const Params &p = w.g;
     const int lane = threadIdx.x & 31, row = row0 + lane;
     const bool f32_out = EPI == EPI_F32 || (EPI == EPI_GATE_UP && prob == 0);
     const int out = w.k_split > 1 ? 0 : prob;
     const int64_t ld = p.ldc[out], at = (int64_t)n0 * ld + row + (w.k_split > 1 ? prob * w.c_step : 0);
     cols = min(cols, p.N - n0);
-    if (row0 >= p.M) return;
+    if (row0 >= p.M) cols = 0;
+    uint32_t r[4][32];
+    const auto column = [&](int i) { return 32 * half + 64 * i; };
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        if (column(i) < cols) tmem_ld32(taddr + (uint32_t)column(i), r[i]);
+    tmem_ld_wait();
+    release();
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int c0 = column(j);
+        if (c0 >= cols) break;
+        const int valid = row < p.M ? min(32, cols - c0) : 0;
+        if (f32_out) {
+            float *dst = static_cast<float *>(p.c[out]) + at + c0 * ld;
+#pragma unroll
+            for (int i = 0; i < 32; ++i, dst += ld)
+                if (i < valid) *dst = __uint_as_float(r[j][i]);
+        } else {
+            __nv_bfloat16 *dst = static_cast<__nv_bfloat16 *>(p.c[out]) + at + c0 * ld;
+#pragma unroll
+            for (int i = 0; i < 32; ++i, dst += ld)
+                if (i < valid) *dst = __float2bfloat16_rn(__uint_as_float(r[j][i]));
+        }
+    }
+}
+
+// Every thread stores its own row (outputs without 16-byte rows, accumulation).
+template <int EPI, class Release>
+__device__ __forceinline__ void direct_epilogue(const Params &p, int prob, int row0, int n0, int cols, int half, uint32_t taddr,
+                                                Release release) {
+    const int row = row0 + (int)(threadIdx.x & 31);
+    const bool f32_out = EPI == EPI_F32 || (EPI == EPI_GATE_UP && prob == 0);
+    cols = row0 < p.M ? min(cols, p.N - n0) : 0;
 #pragma unroll 1
     for (int c0 = 32 * half; c0 < cols; c0 += 64) {
         uint32_t r[32];
         __syncwarp();
         tmem_ld32(taddr + (uint32_t)c0, r);
         tmem_ld_wait();
-        const int valid = row < p.M ? min(32, cols - c0) : 0;
+        const int valid = cols - c0;
+        if (row >= p.M) continue;
         if (f32_out) {
-            float *dst = static_cast<float *>(p.c[out]) + at + c0 * ld;
-#pragma unroll
-            for (int i = 0; i < 32; ++i, dst += ld)
-                if (i < valid) *dst = __uint_as_float(r[i]);
+            store_row_f32(static_cast<float *>(p.c[prob]) + (int64_t)row * p.ldc[prob] + n0 + c0, r, valid);
         } else {
-            __nv_bfloat16 *dst = static_cast<__nv_bfloat16 *>(p.c[out]) + at + c0 * ld;
+            __nv_bfloat16 *dst = static_cast<__nv_bfloat16 *>(p.c[prob]) + (int64_t)row * p.ldc[prob] + n0 + c0;
+            float v[32];
 #pragma unroll
-            for (int i = 0; i < 32; ++i, dst += ld)
-                if (i < valid) *dst = __float2bfloat16_rn(__uint_as_float(r[i]));
+            for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+            if (EPI == EPI_BF16 && p.accumulate) {
+#pragma unroll
+                for (int i = 0; i < 32; ++i)
+                    if (i < valid) v[i] += __bfloat162float(dst[i]);
+            }
+            store_row_bf16(dst, v, valid);
         }
     }
+    release();
 }
 
-// One warp's share of an accumulator of `cols` columns: every other 128-byte chunk (`half` says which) of its 32 rows.
-template <int EPI>
-__device__ __forceinline__ void wide_epilogue(const Params &p, int prob, int row0, int n0, int cols, int half, uint32_t taddr,
-                                              uint32_t box) {
-    const int lane = threadIdx.x & 31, row = row0 + lane;
-    const bool f32_out = EPI == EPI_F32 || (EPI == EPI_GATE_UP && prob == 0);
-    cols = min(cols, p.N - n0);
-    if (row0 >= p.M) return;
-    if (p.direct_store != 0 || (EPI == EPI_BF16 && p.accumulate)) {
-        // every thread stores its own row (outputs a tensor map cannot describe, accumulation)
-#pragma unroll 1
-        for (int c0 = 32 * half; c0 < cols; c0 += 64) {
-            uint32_t r[32];
-            __syncwarp();
-            tmem_ld32(taddr + (uint32_t)c0, r);
-            tmem_ld_wait();
-            const int valid = cols - c0;
-            if (row >= p.M) continue;
-            if (f32_out) {
-                store_row_f32(static_cast<float *>(p.c[prob]) + (int64_t)row * p.ldc[prob] + n0 + c0, r, valid);
-            } else {
-                __nv_bfloat16 *dst = static_cast<__nv_bfloat16 *>(p.c[prob]) + (int64_t)row * p.ldc[prob] + n0 + c0;
-                float v[32];
+// Where a warp's 32 rows of the output go.  A chunk of 32 rows x 128 bytes passes through the warp's box in shared memory (16-byte
+// pieces XOR-swizzled, free of bank conflicts both ways) and leaves as stores of whole 128-byte lines, eight lanes to a row.
+// (Bulk tensor stores queue behind the loads in flight: some 3000 cycles until such a store has read its box.  Every thread
+// storing 32-byte sectors of its own row, without the box: gate + up at 65536 x 2048 x 11008 1.24 -> 1.37 ms a chunk.)
+struct RowChunks {
+    uint8_t *out;     // first of this lane's pieces
+    int64_t pitch4;   // bytes from a row to the fourth after it
+    int rows_left;    // rows from this lane's first on
+    bool whole;       // all 32 rows exist
+    uint32_t box;
+
+    __device__ __forceinline__ void store(int byte, int bytes, const uint32_t (&w)[32]) const {  // `bytes` of each row exist from `byte` on
+        const uint32_t lane = threadIdx.x & 31, r_sub = lane >> 3, piece = lane & 7;
+        uint8_t *dst = out + byte;
+        const uint32_t my_row = box + lane * 128u;
 #pragma unroll
-                for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
-                if (EPI == EPI_BF16 && p.accumulate) {
-#pragma unroll
-                    for (int i = 0; i < 32; ++i)
-                        if (i < valid) v[i] += __bfloat162float(dst[i]);
-                }
-                store_row_bf16(dst, v, valid);
-            }
-        }
-        return;
-    }
-    // A chunk of 32 rows x 128 bytes goes through the warp's box in shared memory (16-byte pieces XOR-swizzled, free of bank
-    // conflicts both ways) and leaves as ordinary 16-byte stores, eight lanes to a row.  (Bulk tensor stores queue behind the
-    // loads in flight: some 3000 cycles until such a store has read its box, which the accumulator waits for.)
-    const uint32_t sw = (uint32_t)(lane & 7), my_row = box + (uint32_t)lane * 128u;
-    const int step = f32_out ? 32 : 64, esz = f32_out ? 4 : 2, per_piece = 16 / esz;
-    const int r_sub = lane >> 3, piece = lane & 7;
-    uint8_t *const out0 = static_cast<uint8_t *>(p.c[prob]) + ((int64_t)(row0 + r_sub) * p.ldc[prob] + n0 + piece * per_piece) * esz;
-    const int64_t pitch4 = (int64_t)p.ldc[prob] * esz * 4;
-    const int rows_left = p.M - row0 - r_sub;
-#pragma unroll 1
-    for (int c0 = step * half; c0 < cols; c0 += 2 * step) {
-        uint32_t r[32];
+        for (int i = 0; i < 8; ++i) st_shared_v4(my_row + (((uint32_t)i ^ piece) << 4), w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
         __syncwarp();
-        tmem_ld32(taddr + (uint32_t)c0, r);
-        if (f32_out) {
-            tmem_ld_wait();
+        const auto staged = [&](int i) {
+            const uint32_t rr = (uint32_t)(4 * i) + r_sub;
+            return ld_shared_v4(box + rr * 128u + ((piece ^ (rr & 7u)) << 4));
+        };
+        if (whole && bytes >= 128) {
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
-                st_shared_v4(my_row + (((uint32_t)i ^ sw) << 4), r[4 * i], r[4 * i + 1], r[4 * i + 2], r[4 * i + 3]);
+            for (int h = 0; h < 8; h += 4) {
+                uint4 v[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) v[i] = staged(h + i);
+#pragma unroll
+                for (int i = 0; i < 4; ++i, dst += pitch4) *reinterpret_cast<uint4 *>(dst) = v[i];
+            }
         } else {
-            uint32_t q[32];
-            tmem_ld32(taddr + (uint32_t)c0 + 32u, q);
-            tmem_ld_wait();
+            const int left = bytes - 16 * (int)piece;  // from this lane's piece on
+#pragma unroll 1
+            for (int i = 0; i < 8; ++i, dst += pitch4) {
+                const uint4 v = staged(i);
+                if (4 * i >= rows_left) continue;
+                if (left >= 16) {
+                    *reinterpret_cast<uint4 *>(dst) = v;
+                } else {
+                    const uint32_t x[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                st_shared_v4(my_row + (((uint32_t)i ^ sw) << 4), pack_bf16(__uint_as_float(r[8 * i]), __uint_as_float(r[8 * i + 1])),
-                             pack_bf16(__uint_as_float(r[8 * i + 2]), __uint_as_float(r[8 * i + 3])),
-                             pack_bf16(__uint_as_float(r[8 * i + 4]), __uint_as_float(r[8 * i + 5])),
-                             pack_bf16(__uint_as_float(r[8 * i + 6]), __uint_as_float(r[8 * i + 7])));
-                st_shared_v4(my_row + (((uint32_t)(i + 4) ^ sw) << 4), pack_bf16(__uint_as_float(q[8 * i]), __uint_as_float(q[8 * i + 1])),
-                             pack_bf16(__uint_as_float(q[8 * i + 2]), __uint_as_float(q[8 * i + 3])),
-                             pack_bf16(__uint_as_float(q[8 * i + 4]), __uint_as_float(q[8 * i + 5])),
-                             pack_bf16(__uint_as_float(q[8 * i + 6]), __uint_as_float(q[8 * i + 7])));
-            }
-        }
-        __syncwarp();
-        const int left = cols - c0 - piece * per_piece;  // columns from this lane's piece on
-        uint8_t *dst = out0 + (int64_t)c0 * esz;
-#pragma unroll
-        for (int i = 0; i < 8; ++i, dst += pitch4) {
-            const uint32_t rr = (uint32_t)(4 * i + r_sub);
-            const uint4 v = ld_shared_v4(box + rr * 128u + (((uint32_t)piece ^ (rr & 7u)) << 4));
-            if (4 * i >= rows_left) continue;
-            if (left >= per_piece) {
-                *reinterpret_cast<uint4 *>(dst) = v;
-            } else if (left > 0) {
-                const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                    if (e >= left) break;
-                    if (f32_out) {
-                        if (e < 4) reinterpret_cast<uint32_t *>(dst)[e] = w[e];
-                    } else {
-                        reinterpret_cast<uint16_t *>(dst)[e] = (uint16_t)(w[e >> 1] >> (16 * (e & 1)));
-                    }
+                    for (int e = 0; e < 8; ++e)
+                        if (2 * e < left) reinterpret_cast<uint16_t *>(dst)[e] = (uint16_t)(x[e >> 1] >> (16 * (e & 1)));
                 }
             }
         }
+        __syncwarp();
     }
+};
+
+// A tile's one or two accumulators, as the epilogue sees them: address in tensor memory, barriers that say "complete" and (in the
+// leading CTA) "read".
+struct TileAccumulators {
+    uint32_t taddr, full, empty;  // of the accumulators in the order of tensor memory
+    uint32_t used;                // accumulators handed out before this tile: they alternate
+    int cols0, cols1;             // that exist in the output; 0: none
+    bool two;
+    volatile int *abort_flag;
+    int *status;
+
+    __device__ __forceinline__ uint32_t slot(int j) const { return (used + (uint32_t)j) & 1u; }
+    __device__ __forceinline__ uint32_t at(int j) const { return taddr + slot(j) * BN; }
+    __device__ __forceinline__ int cols(int j) const { return j ? cols1 : cols0; }
+    __device__ __forceinline__ bool wait(int j) const {
+        const bool ok = __all_sync(0xffffffffu, mbar_wait(full + 8u * slot(j), ((used + (uint32_t)j) >> 1) & 1u, abort_flag, status));
+        tc_fence_after();
+        return ok;
+    }
+    __device__ __forceinline__ void release(int j) const {  // (nothing but the reads of tensor memory is ordered by this arrival)
+        tc_fence_before();
+        __syncwarp();
+        if ((threadIdx.x & 31) == 0) mbar_arrive_cluster_relaxed(empty + 8u * slot(j));
+    }
+};
+
+// A warp's share of a tile: every other 128-byte chunk (`half` says which) of its 32 rows, in registers as it will be stored: 32 fp32
+// columns a chunk, or 64 rounded to bf16.  Three chunks are held at a time, so that an accumulator is read ahead of the
+// stores as far as the registers go.  (All four of an fp32 accumulator: the registers spill, into an L1 that shared memory has
+// left no room: gate + up 1620 thousand cycles again.)  The second accumulator of a tile is complete a thousand cycles after the first.
+// (One sequence for both element types, not one each: side by side in a kernel that has both, the two spilled as well.)
+__device__ __forceinline__ bool wide_epilogue(const TileAccumulators &acc, const RowChunks &rows, bool f32, int half) {
+    uint32_t v0[32], v1[32], v2[32];
+    const int width = f32 ? 32 : 64, shift = f32 ? 2 : 1;  // columns of a chunk; bytes of an element, as a power of two
+    const auto column = [&](int i) { return width * (half + 2 * i); };
+    const auto read = [&](int j, int i, uint32_t (&h)[32]) __attribute__((always_inline)) {
+        if (column(i) >= acc.cols(j)) return;
+        if (f32) {
+            tmem_ld32(acc.at(j) + (uint32_t)column(i), h);
+        } else {
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                uint32_t r[2][16];
+                tmem_ld16(acc.at(j) + (uint32_t)(column(i) + 32 * c), r[0]);
+                tmem_ld16(acc.at(j) + (uint32_t)(column(i) + 32 * c + 16), r[1]);
+                tmem_ld_wait();
+#pragma unroll
+                for (int q = 0; q < 16; ++q)
+                    h[16 * c + q] = pack_bf16(__uint_as_float(r[q >> 3][2 * (q & 7)]), __uint_as_float(r[q >> 3][2 * (q & 7) + 1]));
+            }
+        }
+    };
+    const auto done = [&](int j) __attribute__((always_inline)) {
+        tmem_ld_wait();
+        acc.release(j);
+    };
+    const auto store = [&](int j, int i, const uint32_t (&h)[32]) __attribute__((always_inline)) {
+        if (column(i) < acc.cols(j)) rows.store((j * BN + column(i)) << shift, (acc.cols(j) - column(i)) << shift, h);
+    };
+    if (!acc.wait(0)) return false;
+    read(0, 0, v0);
+    read(0, 1, v1);
+    if (f32) {
+        read(0, 2, v2);
+        tmem_ld_wait();
+        store(0, 0, v0);
+        read(0, 3, v0);
+        done(0);
+        store(0, 1, v1);
+        if (acc.two) {
+            if (!acc.wait(1)) return false;
+            read(1, 0, v1);
+        }
+        store(0, 2, v2);
+        if (acc.two) read(1, 1, v2);
+        store(0, 3, v0);
+        if (!acc.two) return true;
+        read(1, 2, v0);
+        tmem_ld_wait();
+        store(1, 0, v1);
+        read(1, 3, v1);
+        done(1);
+        store(1, 2, v0);
+        store(1, 3, v1);
+        store(1, 1, v2);
+    } else {
+        done(0);
+        store(0, 0, v0);
+        if (acc.two) {
+            if (!acc.wait(1)) return false;
+            read(1, 0, v2);
+            read(1, 1, v0);
+            done(1);
+        }
+        store(0, 1, v1);
+        if (!acc.two) return true;
+        store(1, 0, v2);
+        store(1, 1, v0);
+    }
+    return true;
 }
 
 // TRANSPOSED: the caller has exchanged the operands (see swapped_gemm_pays) and every output is stored as its transpose
@@ -213,7 +315,6 @@ __global__ void __launch_bounds__(WIDE_THREADS, 1) gemm_wide_kernel(const __grid
     const uint32_t base = (raw + 1023u) & ~1023u;  // 128-byte swizzle atoms need 1024-byte alignment
     uint8_t *smem = smem_raw + (base - raw);
     const uint32_t bar_base = base + WIDE_RING_BYTES;
-    const uint32_t epi_base = bar_base + BAR_REGION_BYTES;
     auto full_bar = [&](int s) { return bar_base + 8u * s; };
     auto empty_bar = [&](int s) { return bar_base + 8u * (WIDE_STAGES_MAX + s); };
     auto tfull_bar = [&](uint32_t a) { return bar_base + 8u * (2 * WIDE_STAGES_MAX + a); };
@@ -413,21 +514,39 @@ __global__ void __launch_bounds__(WIDE_THREADS, 1) gemm_wide_kernel(const __grid
         bool ok = true;
         for (int tile = pair; tile < p.t.total && ok; tile += num_pairs) {
             const WideTile t = wide_tile(p, tile);
+            const int row0 = t.m_blk * (2 * BM) + (int)rank * BM + quarter * 32;
+            TileAccumulators acc;
+            acc.taddr = tmem_base + ((uint32_t)(quarter * 32) << 16);
+            acc.full = tfull_bar(0);
+            acc.empty = map_to_cta(tempty_bar(0), 0);
+            acc.used = used;
+            acc.cols0 = row0 < p.g.M ? min(t.s0, p.g.N - t.n0) : 0;
+            acc.cols1 = row0 < p.g.M ? min(t.s1, p.g.N - t.n0 - BN) : 0;
+            acc.two = t.s1 > 0;
+            acc.abort_flag = abort_flag;
+            acc.status = status;
+            used += acc.two ? 2u : 1u;
+            if (TRANSPOSED || p.g.direct_store != 0 || (EPI == EPI_BF16 && p.g.accumulate)) {
 #pragma unroll 1
-            for (int j = 0; j < (t.s1 ? 2 : 1); ++j, ++used) {
-                const uint32_t r = used & 1u;
-                ok = __all_sync(0xffffffffu, mbar_wait(tfull_bar(r), (used >> 1) & 1u, abort_flag, status));
-                if (!ok) break;
-                tc_fence_after();
-                if constexpr (TRANSPOSED)
-                    transposed_epilogue<EPI>(p, t.prob, t.m_blk * (2 * BM) + (int)rank * BM + quarter * 32, t.n0 + j * BN, j ? t.s1 : t.s0,
-                                             half, tmem_base + ((uint32_t)(quarter * 32) << 16) + r * BN);
-                else
-                    wide_epilogue<EPI>(p.g, t.prob, t.m_blk * (2 * BM) + (int)rank * BM + quarter * 32, t.n0 + j * BN, j ? t.s1 : t.s0, half,
-                                       tmem_base + ((uint32_t)(quarter * 32) << 16) + r * BN, epi_base + (uint32_t)(warp - 2) * EPI_BOX_BYTES);
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive_cluster(map_to_cta(tempty_bar(r), 0));
+                for (int j = 0; j < (acc.two ? 2 : 1); ++j) {
+                    if (!(ok = acc.wait(j))) break;
+                    const auto done = [&]() { acc.release(j); };
+                    if constexpr (TRANSPOSED)
+                        transposed_epilogue<EPI>(p, t.prob, row0, t.n0 + j * BN, j ? t.s1 : t.s0, half, acc.at(j), done);
+                    else
+                        direct_epilogue<EPI>(p.g, t.prob, row0, t.n0 + j * BN, j ? t.s1 : t.s0, half, acc.at(j), done);
+                }
+            } else {
+                const bool f32_out = (p.f32_outputs >> t.prob) & 1u;  // (not from EPI: as a constant it leaves a register allocation that spills)
+                const int esz = f32_out ? 4 : 2, r_sub = lane >> 3;
+                const int64_t pitch = (int64_t)p.g.ldc[t.prob] * esz;
+                RowChunks rows;
+                rows.out = static_cast<uint8_t *>(p.g.c[t.prob]) + (row0 + r_sub) * pitch + t.n0 * esz + (lane & 7) * 16;
+                rows.pitch4 = 4 * pitch;
+                rows.rows_left = p.g.M - row0 - r_sub;
+                rows.whole = row0 + 32 <= p.g.M;
+                rows.box = bar_base + BAR_REGION_BYTES + (uint32_t)(warp - 2) * EPI_BOX_BYTES;
+                ok = wide_epilogue(acc, rows, f32_out, half);
             }
         }
     }

@@ -125,24 +125,15 @@ __device__ __forceinline__ bool flag_wait(const unsigned int *flag, unsigned int
     return true;
 }
 
-// 16 consecutive fp32 columns of this thread's TMEM lane
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]),
-          "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
-}
 // sum of the two issuers' accumulators: 16 columns at `taddr` and at `taddr` + 64 (when the second issuer had work)
 __device__ __forceinline__ void tmem_ld16_sum(uint32_t taddr, bool two, float (&v)[16]) {
     uint32_t a[16];
-    tmem_ld16(taddr, a);
+    tc::tmem_ld16(taddr, a);
     tc::tmem_ld_wait();
 #pragma unroll
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(a[i]);
     if (two) {  // (warp-uniform)
-        tmem_ld16(taddr + 64u, a);
+        tc::tmem_ld16(taddr + 64u, a);
         tc::tmem_ld_wait();
 #pragma unroll
         for (int i = 0; i < 16; ++i) v[i] += __uint_as_float(a[i]);

@@ -202,6 +202,7 @@ inline int launch_gemm(const Params &p_in, cudaStream_t st, int k_split = 1, int
             n_b += p.b_idx[i][0] != p.b_idx[0][0] ? 1 : 0;
             n_a += p.a_idx[i][0] != p.a_idx[0][0] ? 1 : 0;
         }
+        w.f32_outputs = EPI == EPI_F32 ? 7u : EPI == EPI_GATE_UP ? 1u : 0u;
         w.k_split = k_split;
         w.c_step = c_step;
         w.k_operands = p.k_segments;

@@ -29,8 +29,12 @@ struct TilePlan {
 constexpr double WIDE_MMA_CYCLES = 2.06;  // per column
 inline double wide_block_cycles(int w) { return std::max(WIDE_MMA_CYCLES * w, (16384.0 + 64.0 * w) / 58.0); }
 
-// Cycles in which the epilogue moves an accumulator of 256 columns (bf16, fp32 outputs).
-constexpr int WIDE_DRAIN_BF16 = 2000, WIDE_DRAIN_F32 = 3500;
+// Cycles for which the epilogue keeps an accumulator of 256 columns from the MMAs (bf16 outputs; fp32 ones among them).  Of a
+// tile with two accumulators the skew covers a bf16 one's (34.0 thousand cycles a tile of 32 blocks, 33.75 of them MMAs); with fp32
+// gate values every other tile is measured 2700 cycles longer.  That figure less what a 256-column tile loses to its stores,
+// which share the loads' way to L2 (634 and 742 cycles a block for gate + up of 32 and 12 blocks, against 565 of the loads):
+// 16384 x 768 x 2048, gate + up on tiles of 256 columns 123 thousand cycles, of 512 119.
+constexpr int WIDE_DRAIN_BF16 = 1024, WIDE_DRAIN_F32 = 2000;
 
 // No plan of `rows` x N over kb blocks is shorter: its MMAs spread evenly.
 inline double plan_cycles_at_least(int rows, int64_t N, int kb, int pairs) { return WIDE_MMA_CYCLES * rows * (double)N * kb / pairs; }
@@ -38,8 +42,8 @@ inline double plan_cycles_at_least(int rows, int64_t N, int kb, int pairs) { ret
 // Tiles of `rows` x N for `pairs` CTA pairs: wide ones for as many whole waves as there are (or one fewer), the rest in the
 // one width that finishes first; or that width throughout.  (Measured at d_model 2048, d_ff 5504: down projection of 1111
 // tokens, 40 tiles of 256 columns for 74 pairs, 36.8 us; 55 of 192.)
-// drain: cycles in which the epilogue moves an accumulator of 256 columns.  Of a tile with two accumulators the part of it
-// that the skew does not cover is lost; with one, the other is worked in meanwhile.
+// drain: one of the two above.  Of a tile with two accumulators the part of it that the skew does not cover is lost; with
+// one, the other is worked in meanwhile.
 // any_first: the first tiles may have any width, not 512 alone (few columns: one tile as wide as they are spans them).
 inline TilePlan search_tiles(int rows, int N, int kb, int pairs, bool by_columns, int drain, bool any_first) {
     constexpr int kWidths = WIDE_N / WIDE_STEP;
