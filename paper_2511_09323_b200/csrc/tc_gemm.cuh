@@ -224,11 +224,8 @@ __device__ __forceinline__ uint32_t map_to_cta(uint32_t smem_addr, uint32_t rank
 __device__ __forceinline__ void cluster_sync_all() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
-}
-// The same without memory ordering: a release at cluster scope waits for the thread's global stores in flight (1500 cycles
-// behind an epilogue's).  Enough where only accesses to tensor memory are handed over, between the two tcgen05 fences.
+// Arrival on a barrier of another CTA, without memory ordering: a release at cluster scope waits for the thread's global stores in
+// flight (1500 cycles behind an epilogue's).  Enough where only accesses to tensor memory are handed over, between the two tcgen05 fences.
 __device__ __forceinline__ void mbar_arrive_cluster_relaxed(uint32_t cluster_addr) {
     asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
@@ -957,7 +954,7 @@ __global__ void __launch_bounds__(PAIR_THREADS, 1) gemm_pair_kernel(const __grid
                                epi_base + (uint32_t)(warp - 2) * EPI_BOX_BYTES);
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive_cluster(map_to_cta(tempty_bar(acc), 0));
+            if (lane == 0) mbar_arrive_cluster_relaxed(map_to_cta(tempty_bar(acc), 0));
             if (++acc == ACC_STAGES) {
                 acc = 0;
                 acc_phase ^= 1u;

@@ -470,7 +470,7 @@ __global__ void __launch_bounds__(PTHREADS, 1) gemm_sp_pair_kernel(const __grid_
             tmem_ld_wait();
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive_cluster(map_to_cta(tempty_bar, 0));  // the accumulator may be overwritten
+            if (lane == 0) mbar_arrive_cluster_relaxed(map_to_cta(tempty_bar, 0));  // the accumulator may be overwritten
             const int row = m_blk * (2 * SBM) + (int)rank * SBM + quarter * 32 + lane;
             const int n0 = n_blk * PBN + half * 128;
             if (row < p.M) {
