@@ -11,6 +11,7 @@
 #include <unordered_map>
 #include <vector>
 
+#include "decode_cluster.cuh"
 #include "decode_coop.cuh"
 #include "decode_kernels.cuh"
 #include "gather_kernels.cuh"
@@ -113,6 +114,7 @@ enum KernelId {
     KID_STREAM_PROBE,
     KID_SB_FUSED,
     KID_TC_SPLIT_SUM,
+    KID_DEC_CLUSTER,
     KID_COUNT
 };
 static const char *const kKernelNames[KID_COUNT] = {
@@ -123,7 +125,7 @@ static const char *const kKernelNames[KID_COUNT] = {
     "dec_select",      "dec_up",          "dec_down",      "sb_gate_up",     "sb_select",
     "sb_down",         "recompute_up",    "dec_coop",      "dec_rmsnorm",    "tc_compress_2of4",
     "tc_sp_down_gemm", "tc_sp_dx_gemm", "stream_probe",    "sb_fused",
-    "tc_split_sum",
+    "tc_split_sum",    "dec_cluster",
 };
 
 struct Profiler {
@@ -1151,6 +1153,133 @@ int decode_coop(const moc_ffn_desc &d, const CoopLayout &L, const __nv_bfloat16 
     }
 }
 
+// ---- decode on small layers: clusters of 16 CTAs, a token or two each ---------------------------------------
+struct ClusterForm {
+    int T, unit, stages;  // tokens per cluster; as in dcl::Params
+    int most;             // clusters that can run at a time
+    size_t smem;
+};
+
+void cluster_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute (&attr)[2], unsigned clusters, size_t smem, cudaStream_t st) {
+    cfg = {};
+    cfg.gridDim = dim3(clusters * dcl::kCluster);
+    cfg.blockDim = dim3(dcl::kThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = dcl::kCluster;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+}
+
+// Clusters of this size that the device holds at a time (0: none, or an error); asked once per form and shared-memory size.
+template <int T>
+int clusters_resident(size_t smem) {
+    const auto kern = dcl::decode_cluster_kernel<T>;
+    static std::mutex mu;
+    static std::unordered_map<size_t, int> known;
+    std::lock_guard<std::mutex> lock(mu);
+    const auto it = known.find(smem);
+    if (it != known.end()) return it->second;
+    int n = 0;
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[2];
+    cluster_config(cfg, attr, 1, smem, nullptr);
+    cfg.numAttrs = 1;
+    if (set_smem(kern, smem, 8 * 1024) != MOC_OK ||
+        cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) {
+        (void)cudaGetLastError();
+        n = 0;
+    }
+    return known[smem] = n;
+}
+
+template <int T>
+bool cluster_fits(const moc_ffn_desc &d, ClusterForm &f) {
+    const int groups = ceil_div(dcl::rows_of(d.d_ff, f.unit), 16);
+    for (int stages = std::min(dcl::kMaxStages, std::max(2, groups)); stages >= 2; --stages) {
+        const size_t smem = dcl::layout(T, d.d_model, d.d_ff, f.unit, stages).total;
+        if (smem > (size_t)218 * 1024) continue;
+        f.T = T;
+        f.stages = stages;
+        f.smem = smem;
+        f.most = clusters_resident<T>(smem);
+        return f.most > 0;
+    }
+    return false;
+}
+
+// Where the cluster form is the faster one, `most` clusters running at a time (7 on a B200).  It takes the calls of the decode
+// plan.  us, this form | the one it replaces: a token to a cluster, 384 x 1024, 1, 2, 4, 6 tokens 9.4 9.5 10.7 11.5 | 18.1 20.6 22.9
+// 25.0; 768 x 2048 13.2 13.3 15.3 16.7 | 19.2 22.9 25.7 29.4; 1024 x 2736 18.2 18.4 19.7 20.8 | 21.6 26.0 24.9 32.9; 1536 x 4096 31.1
+// 31.8 33.3 34.0 | 24.7 29.6 28.8 32.9.  Two to a cluster, 8 tokens: 768 x 2048 19.0 | 29.8, and from 16 tokens on it is slower.
+bool cluster_pays(const moc_ffn_desc &d, int most) {
+    const double weights = (double)d.d_model * d.d_ff;
+    return d.tokens <= most ? weights <= 3.5e6 : d.tokens <= 2 * most && weights <= 1.6e6;
+}
+
+// false: another form serves the call
+bool cluster_form(const moc_ffn_desc &d, ClusterForm &f) {
+    static const bool off = [] {  // MOC_FFN_DECODE: "chain" and "grid" keep to the forms on all SMs (comparisons, tests)
+        const char *e = getenv("MOC_FFN_DECODE");
+        return e && (strcmp(e, "chain") == 0 || strcmp(e, "grid") == 0);
+    }();
+    if (off || !use_decode_plan(d) || d.d_model > dcl::kMaxD || d.d_ff > dcl::kCluster * (dcl::kMaxRows - 8)) return false;
+    f.unit = d.d_ff % 8 == 0 ? 8 : 1;
+    if (!cluster_pays(d, 1 << 20)) return false;
+    return (cluster_fits<1>(d, f) && d.tokens <= f.most && cluster_pays(d, f.most)) ||
+           (cluster_fits<2>(d, f) && d.tokens <= 2 * f.most && cluster_pays(d, f.most));
+}
+
+template <int T>
+int launch_cluster(const dcl::Params &prm, const ClusterForm &f, cudaStream_t st) {
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[2];
+    cluster_config(cfg, attr, (unsigned)ceil_div(prm.tokens, T), f.smem, st);
+    cudaError_t err = cudaSuccess;
+    MOC_LAUNCH(KID_DEC_CLUSTER, st, err = cudaLaunchKernelEx(&cfg, dcl::decode_cluster_kernel<T>, prm));
+    if (err != cudaSuccess) {  // refused: nothing ran, another form serves the call
+        (void)cudaGetLastError();
+        return MOC_ERR_UNSUPPORTED;
+    }
+    return launch_ok();
+}
+
+// rms_w != nullptr: the block form (x is the residual stream h)
+int decode_cluster(const moc_ffn_desc &d, const ClusterForm &f, const __nv_bfloat16 *x, const __nv_bfloat16 *wg, const __nv_bfloat16 *wu,
+                   const __nv_bfloat16 *wd, __nv_bfloat16 *out, cudaStream_t st, const __nv_bfloat16 *rms_w = nullptr, float rms_eps = 0.f) {
+    int *status = device_status_ptr();
+    if (!status) return MOC_ERR_CUDA;
+    dcl::Params prm{};
+    prm.x = x;
+    prm.wg = wg;
+    prm.wu = wu;
+    prm.wd = wd;
+    prm.out = out;
+    prm.tokens = (int)d.tokens;
+    prm.d = d.d_model;
+    prm.F = d.d_ff;
+    prm.K = d.k;
+    prm.grouped = (d.flags & MOC_FLAG_SELECT_2_OF_8) ? 1 : 0;
+    prm.unit = f.unit;
+    prm.stages = f.stages;
+    prm.rp = dcl::rows_of(d.d_ff, f.unit);
+    prm.own_vecs = dcl::slice_vecs(d.d_model);
+    prm.at = dcl::layout(f.T, d.d_model, d.d_ff, f.unit, f.stages);
+    prm.status = status;
+    prm.rms_w = rms_w;
+    prm.rms_eps = rms_eps;
+    switch (f.T) {
+        case 1: return launch_cluster<1>(prm, f, st);
+        default: return launch_cluster<2>(prm, f, st);
+    }
+}
+
 // resid != nullptr: added to the layer's output before the rounding (the block form)
 int decode_bf16(const moc_ffn_desc &d, const __nv_bfloat16 *x, const __nv_bfloat16 *wg, const __nv_bfloat16 *wu,
                 const __nv_bfloat16 *wd, __nv_bfloat16 *out, char *wsp, cudaStream_t st,
@@ -1848,6 +1977,14 @@ int moc_ffn_decode(const moc_ffn_desc *desc, const void *x, const void *w_gate, 
     if (!good_ptr(workspace) || workspace_bytes < need) return MOC_ERR_WORKSPACE;
     using T = __nv_bfloat16;
     {
+        ClusterForm f{};
+        if (cluster_form(*desc, f)) {
+            const int rc2 = decode_cluster(*desc, f, (const T *)x, (const T *)w_gate, (const T *)w_up, (const T *)w_down, (T *)out,
+                                           static_cast<cudaStream_t>(cuda_stream));
+            if (rc2 != MOC_ERR_UNSUPPORTED) return rc2;
+        }
+    }
+    {
         // a handful of tokens: one cooperative kernel; where the device or the problem does not admit it, or its
         // launch is refused, the four-kernel plan
         bool coop = false;
@@ -1877,6 +2014,14 @@ int moc_ffn_decode_block(const moc_ffn_desc *desc, const void *h, const void *rm
     using T = __nv_bfloat16;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     char *wsp = static_cast<char *>(workspace);
+    {
+        ClusterForm f{};
+        if (cluster_form(*desc, f)) {
+            const int rc2 = decode_cluster(*desc, f, (const T *)h, (const T *)w_gate, (const T *)w_up, (const T *)w_down, (T *)out, st,
+                                           (const T *)rms_weight, rms_eps);
+            if (rc2 != MOC_ERR_UNSUPPORTED) return rc2;
+        }
+    }
     if (use_decode_plan(*desc)) {
         // one or two tokens: the cooperative kernel normalises its staged rows and adds h itself
         bool coop = false;

@@ -1,0 +1,147 @@
+"""Decode on small layers (csrc/decode_cluster.cuh): clusters of 16 CTAs, one or two tokens each."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import moc_oracle as orc
+from oracle import parity
+from paper_2511_09323_b200 import binding as B
+from paper_2511_09323_b200 import synthetic as syn
+
+pytestmark = pytest.mark.gpu
+
+
+def _run(call):
+    B.moc_profile_enable(True)
+    out = call()
+    names = {k for k, (n, _) in B.moc_profile_collect().items() if n}
+    B.moc_profile_enable(False)
+    assert names == {"dec_cluster"}, names
+    assert B.moc_last_device_status() == B.MOC_OK
+    return out
+
+
+def _rows(F):
+    """Gate rows that bf16 holds exactly: ties at the threshold, one value throughout, runs, many magnitudes, NaN and -inf."""
+    rng = np.random.default_rng(5)
+    rows = [rng.normal(size=F), rng.integers(-3, 4, F) * 0.5, np.full(F, 1.25), np.linspace(2, -2, F), np.linspace(-2, 2, F),
+            rng.normal(size=F) * 2.0 ** rng.integers(-20, 3, F), np.where(np.arange(F) % 3 == 0, 1.0, 0.5), -np.abs(rng.normal(size=F))]
+    special = rng.normal(size=F)
+    special[::7], special[3::11] = np.nan, -np.inf
+    return torch.tensor(np.stack(rows + [special]), dtype=torch.float32).bfloat16().float().numpy()
+
+
+@pytest.mark.parametrize("F,K", [(1000, 1), (1000, 62), (1000, 125), (997, 41), (17, 1), (24, 2), (8, 1)])
+@pytest.mark.parametrize("tokens", [1, 2, 7, 9])
+def test_the_channels_that_are_kept(F, K, tokens):
+    # x is one-hot on the column of W_gate that holds the row, u is one, channel j goes to output j
+    if 1 - (1 - K / F) ** tokens >= 0.45:
+        pytest.skip("another form's share of the channels")
+    rows, d = _rows(F), max(64, (F + 7) // 8 * 8)
+    wg, wu, wd = torch.zeros(F, d), torch.zeros(F, d), torch.zeros(F, d)
+    wg[:, :len(rows)] = torch.from_numpy(rows.T)
+    wu[:, :len(rows)] = 1
+    wd[torch.arange(F), torch.arange(F)] = 1
+    want = np.zeros(rows.shape, bool)
+    np.put_along_axis(want, orc.topk(rows, K).astype(np.int64), True, axis=1)
+    weights = [w.bfloat16().cuda() for w in (wg, wu, wd)]
+    for first in range(0, len(rows) if tokens == 1 else 2):
+        # (0 * NaN would leak the special row's values into other tokens' gate values: it is looked at alone)
+        order = [first] if tokens == 1 else [(first + 3 * t) % (len(rows) - 1) for t in range(tokens)]
+        case = [w.clone() for w in weights]
+        if tokens > 1 or first != len(rows) - 1:
+            case[0][:, len(rows) - 1] = 0
+        x = torch.zeros(tokens, d)
+        x[torch.arange(tokens), order] = 1
+        out = _run(lambda: B.moc_ffn_decode(x.bfloat16().cuda(), *case, K)).float().cpu().numpy()[:, :F]
+        for t, i in enumerate(order):
+            told = np.abs(rows[i]) > 1e-6   # (SiLU of less is not told from zero)
+            told &= np.isfinite(rows[i]) & (rows[i] > -50)
+            np.testing.assert_array_equal((out[t] != 0)[told], want[i][told], err_msg=f"row {i}")
+
+
+@pytest.mark.parametrize("T,d,F,F_ld,K", [
+    (1, 768, 2048, 2048, 256),
+    (2, 64, 96, 96, 12),
+    (1, 8, 40, 40, 17),          # one piece of columns, CTAs without channels
+    (3, 264, 333, 336, 41),      # channels dealt one by one, padding rows, no whole block of the contraction
+    (4, 384, 1024, 1024, 128),
+    (7, 1024, 2736, 2752, 171),  # stages used more than once; the largest layer
+    (1, 408, 8064, 8064, 1008),  # the most channels a CTA can have, kept rows in several batches
+    (1, 1744, 2000, 2000, 880),  # few stages, more kept rows than half of them hold
+    (9, 768, 2048, 2048, 128),   # two tokens a cluster, the last one alone
+    (8, 200, 1000, 1000, 60),
+])
+def test_against_the_oracle(T, d, F, F_ld, K):
+    w = syn.Workload(f"dcl-{T}-{d}-{F}", "bf16", T, d, F, F_ld, K, seed=900 + T)
+    wg, wu, wd = syn.make_weights(w)
+    x = syn.make_x(w)
+    dev = [t.cuda() for t in (x, wg, wu, wd)]
+    gamma = (0.5 + torch.rand(d, generator=torch.Generator().manual_seed(3))).bfloat16()
+    outs = [_run(lambda: B.moc_ffn_decode(*dev, K, d_ff=F)) for _ in range(2)]
+    assert torch.equal(*outs)   # the sums are in a fixed order
+    block = dev[0].clone()
+    _run(lambda: B.moc_ffn_decode_block(block, gamma.cuda(), 1e-5, *dev[1:], K, d_ff=F, out=block))
+    x64, g64, *w64 = (syn.to_f64(t) for t in (x, gamma, wg[:F], wu[:F], wd[:F]))
+    store = lambda a: torch.from_numpy(np.ascontiguousarray(a)).bfloat16().double().numpy()
+    full = orc.forward(x64, *w64, K, want_g=True)
+    ref, xn, full_block = orc.decode_block(x64, g64, 1e-5, *w64, K, store=store)
+    for got, want, g, xin, add in ((outs[0], full["out"], full["g"], x64, 0 * x64), (block, ref, full_block["g"], xn, x64)):
+        tol, got = parity.REL_TOL["bf16"] * np.abs(want).max(), syn.to_f64(got)
+        for t in range(T):
+            if np.abs(got[t] - want[t]).max() <= tol:
+                continue
+            # the K-th and the next gate value nearly tie: the swapped pick
+            order = np.lexsort((np.arange(F), -g[t]))
+            assert K < F and g[t][order[K - 1]] - g[t][order[K]] <= 1e-3, f"token {t}"
+            alt = np.sort(np.concatenate([order[: K - 1], order[K: K + 1]])).astype(np.int32)[None]
+            assert np.abs(got[t] - add[t] - orc.forward_given_idx(xin[t: t + 1], *w64, alt)["out"][0]).max() <= tol, f"token {t}"
+
+
+@pytest.mark.parametrize("T,d,F", [(1, 768, 2048), (2, 264, 1000)])
+def test_the_2_of_8_mask(T, d, F):
+    w = syn.Workload(f"dcl-2of8-{T}-{d}-{F}", "bf16", T, d, F, F, F // 4, seed=70 + T)
+    wg, wu, wd = syn.make_weights(w)
+    wg[1::2] = wg[0::2]    # equal values inside every group: the lower channels
+    x = syn.make_x(w)
+    out = _run(lambda: B.moc_ffn_decode(x.cuda(), wg.cuda(), wu.cuda(), wd.cuda(), None, grouped=True))
+    x64, *w64 = (syn.to_f64(t) for t in (x, wg, wu, wd))
+    parity.assert_close(syn.to_f64(out), orc.forward_grouped(x64, *w64)["out"], "bf16", "decode, 2 of 8")
+
+
+def test_infinite_weight():
+    """An infinite weight of a kept row gives an infinite output in its column, and nothing but it."""
+    gen = torch.Generator().manual_seed(1)
+    x = torch.randn(1, 64, generator=gen).bfloat16()
+    wg, wu, wd = (torch.randn(64, 64, generator=gen).bfloat16() for _ in range(3))
+    j = int(orc.topk((syn.to_f64(x) @ syn.to_f64(wg).T).astype(np.float32), 8)[0, 0])
+    wd[j, 5] = float("inf")
+    out = _run(lambda: B.moc_ffn_decode(x.cuda(), wg.cuda(), wu.cuda(), wd.cuda(), 8)).float().cpu()[0]
+    assert out[5].isinf() and out[torch.arange(64) != 5].isfinite().all()
+
+
+def test_calls_in_a_row_and_in_a_graph():
+    """A launch begins before the one in front has ended: every call reads what the one before it wrote."""
+    w = syn.Workload("dcl-row", "bf16", 2, 384, 1024, 1024, 128, seed=8)
+    weights = [t.cuda() for t in syn.make_weights(w)]
+    gamma = torch.ones(384, dtype=torch.bfloat16, device="cuda")
+    h0 = syn.make_x(w).cuda()
+
+    def layers(h, sync):
+        for _ in range(12):
+            h = B.moc_ffn_decode_block(h, gamma, 1e-5, *weights, w.k)
+            if sync:
+                torch.cuda.synchronize()
+        return h
+
+    want = layers(h0, True)
+    assert torch.equal(layers(h0, False), want)
+    side, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(side):
+        with torch.cuda.graph(graph, stream=side):
+            out = layers(h0, False)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, want)
+    assert B.moc_last_device_status() == B.MOC_OK
