@@ -483,6 +483,23 @@ int tc_select_prepare(const TcSelect &c, int F, int K) {
     return set_smem(tc::select_hint_kernel, (size_t)F * sizeof(uint32_t));
 }
 
+// Launch with programmatic stream serialization allowed: the kernel may become resident while its predecessor in
+// the stream drains (every kernel launched this way calls pdl_wait before it touches global data).
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, unsigned block, size_t smem, cudaStream_t st, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, KArgs(args)...);
+}
+
 // Team selector with the row in shared memory: every launch works with one bracket kept in the workspace ({center, width,
 // tag} at hint[0..2]); it gathers the statistics of its thresholds (hint[4..6], CTA counter at hint[8]) and its last CTA
 // rewrites the bracket for the next launch.  The bracket is only a hint: a stale or garbage one costs time (rows take the
@@ -497,8 +514,8 @@ void tc_select_launch(const TcSelect &c, const float *G, int ldg, __nv_bfloat16 
 #define MOC_DO_LAUNCH(W, VPL, BINS)                                                                                              \
     if (c.team == W && c.vpl == VPL && c.bins == BINS)                                                                           \
         MOC_LAUNCH(KID_TC_SELECT_MASK, st,                                                                                       \
-                   (rs::select_rows_reg_kernel<W, VPL, BINS><<<grid, 32 * W, c.smem, st>>>(                                      \
-                       G, ldg, U, ldu, n, F, K, rs::normal_quantile(F, K), o_idx, o_g, o_u, status)));
+                   launch_pdl(rs::select_rows_reg_kernel<W, VPL, BINS>, dim3(grid), 32 * W, c.smem, st, G, ldg, U, ldu, n, F, K,  \
+                              rs::normal_quantile(F, K), o_idx, o_g, o_u, status));
         MOC_ROW_SELECT_FORMS(MOC_DO_LAUNCH)
 #undef MOC_DO_LAUNCH
     } else if (c.kind == TcSelect::kSharedRow) {
@@ -588,11 +605,13 @@ int sparse_gemm_pair(int64_t M, int N, int K, int segments, const __nv_bfloat16 
     p.status = status;
     static int max_pairs = 0;
     cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 2;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.blockDim = dim3(PTHREADS);
     cfg.dynamicSmemBytes = PSMEM_BYTES;
     cfg.stream = st;
@@ -610,14 +629,17 @@ int sparse_gemm_pair(int64_t M, int N, int K, int segments, const __nv_bfloat16 
     const int pairs = std::min(tiles, max_pairs);
     if (pairs <= 0) return MOC_OK;
     cfg.gridDim = dim3(2 * (unsigned)pairs);
+    cfg.numAttrs = 2;
     int rc = MOC_OK;
     MOC_LAUNCH(kid, st, (rc = cudaLaunchKernelEx(&cfg, gemm_sp_pair_kernel, p) == cudaSuccess ? MOC_OK : MOC_ERR_CUDA));
     return rc;
 }
 
 // out = bf16(sum of `parts` partial outputs, n8 groups of eight elements each), 8 elements per thread
-__global__ void __launch_bounds__(256) split_sum_kernel(const float *__restrict__ partial, int parts, __nv_bfloat16 *__restrict__ out,
+__global__ void __launch_bounds__(256) split_sum_kernel(const float *partial_in, int parts, __nv_bfloat16 *__restrict__ out,
                                                         int64_t n8) {
+    tc::pdl_wait();
+    const float *const partial = tc::after_pdl_wait(partial_in);
     for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n8; i += (int64_t)gridDim.x * 256) {
         const float4 *a = reinterpret_cast<const float4 *>(partial) + 2 * i;
         float4 v0 = __ldcs(a), v1 = __ldcs(a + 1);
@@ -635,7 +657,7 @@ __global__ void __launch_bounds__(256) split_sum_kernel(const float *__restrict_
 int launch_split_sum(const float *partial, int parts, int64_t T, int n_cols, __nv_bfloat16 *out, cudaStream_t st) {
     const int64_t n8 = T * n_cols / 8;
     const unsigned grid = (unsigned)std::min<int64_t>((n8 + 255) / 256, (int64_t)tc::sm_count() * 8);
-    MOC_LAUNCH(KID_TC_SPLIT_SUM, st, (split_sum_kernel<<<grid, 256, 0, st>>>(partial, parts, out, n8)));
+    MOC_LAUNCH(KID_TC_SPLIT_SUM, st, launch_pdl(split_sum_kernel, dim3(grid), 256, 0, st, partial, parts, out, n8));
     return launch_ok();
 }
 
@@ -864,7 +886,7 @@ int backward_tc(const moc_ffn_desc &d, const __nv_bfloat16 *x, const __nv_bfloat
             if ((rc = set_smem(kern, team_bytes, 1024)) != MOC_OK) return rc;
             const unsigned grid = (unsigned)std::min<int64_t>(T, (int64_t)sm_count() * per_sm);
             MOC_LAUNCH(KID_TC_BWD_SAMPLE, st,
-                       (kern<<<grid, 32 * w, team_bytes, st>>>(idx, tg, tu, T, K, F, L.ldf, Zp, dUp, dGp, status)));
+                       launch_pdl(kern, dim3(grid), 32 * w, team_bytes, st, idx, tg, tu, T, K, F, L.ldf, Zp, dUp, dGp, status));
         } else {
             const size_t smem = (size_t)K * 8;
             if ((rc = set_smem(backward_sample_rows_kernel, smem)) != MOC_OK) return rc;
@@ -1022,23 +1044,6 @@ bool small_batch_preferred(const moc_ffn_desc &d);
 bool use_decode_plan(const moc_ffn_desc &d) {
     return !(d.flags & MOC_FLAG_SELECT_POST_SILU) && d.dtype == MOC_BF16 && d.tokens >= 1 && d.tokens <= 16 && d.d_model <= 256 * dec::kSliceCols &&
            !(use_small_batch_plan(d) && small_batch_preferred(d));
-}
-
-// Launch with programmatic stream serialization allowed: the kernel may become resident while its predecessor in
-// the stream drains (every kernel launched this way calls pdl_wait before it touches global data).
-template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, unsigned block, size_t smem, cudaStream_t st, Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(block);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, KArgs(args)...);
 }
 
 // ---- cooperative decode (bf16, one or two tokens, d_model <= 4096): one kernel, every SM keeps its channels ----

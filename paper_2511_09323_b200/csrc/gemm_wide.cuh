@@ -351,6 +351,7 @@ __global__ void __launch_bounds__(WIDE_THREADS, 1) gemm_wide_kernel(const __grid
     cluster_sync_all();  // the partner's barriers exist before anything signals them
     tc_fence_after();
     const uint32_t tmem_base = *tmem_holder;
+    pdl_wait();  // (for the kernel in front)
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer (one per CTA).  One thread's
@@ -552,6 +553,12 @@ __global__ void __launch_bounds__(WIDE_THREADS, 1) gemm_wide_kernel(const __grid
     }
 
     // ---------------------------------------------------------------------- teardown
+    // The next kernel of the stream may be launched once every pair has come here; it does its set-up beside the last ones and waits
+    // for their outputs, as the selector, the element-wise kernel and the sum of partial outputs do.  Those give no such sign
+    // themselves, and this kernel not at its start: what is launched early takes its place on the first SMs that are free.  us,
+    // none | all at their start | this: forward of 307 tokens, 4096 x 11008, 117.6 | 120.6 | 110.2; step of 1111 tokens, 2048 x 5461,
+    // 265 | 253 | 247; of 16384, 768 x 2048, 524 | 515 | 510.
+    pdl_launch_dependents();
     __syncwarp();
     if (*abort_flag) {
         const long long t0 = clock64();

@@ -35,13 +35,16 @@ __host__ __device__ inline SampleLayout sample_layout(int ld, int K) {
 constexpr int sample_warps(int F) { return F <= 1024 ? 1 : F <= 3072 ? 2 : F <= 8192 ? 4 : 8; }
 
 template <int W>
-__global__ void __launch_bounds__(32 * W) sample_rows_kernel(const int16_t *__restrict__ idx, const __nv_bfloat16 *__restrict__ gval,
-                                                            const __nv_bfloat16 *__restrict__ uval, int64_t T, int K, int F, int ld,
+__global__ void __launch_bounds__(32 * W) sample_rows_kernel(const int16_t *idx_in, const __nv_bfloat16 *gval_in,
+                                                            const __nv_bfloat16 *uval_in, int64_t T, int K, int F, int ld,
                                                             __nv_bfloat16 *__restrict__ dz_z, __nv_bfloat16 *__restrict__ du,
                                                             __nv_bfloat16 *__restrict__ dg, int *__restrict__ status) {
     using namespace tc;
     extern __shared__ __align__(16) uint8_t smem[];
     __shared__ int s_abort;
+    pdl_wait();
+    const int16_t *const idx = after_pdl_wait(idx_in);
+    const __nv_bfloat16 *const gval = after_pdl_wait(gval_in), *const uval = after_pdl_wait(uval_in);
     constexpr int TT = 32 * W;
     const SampleLayout L = sample_layout(ld, K);
     const int tid = threadIdx.x, K8 = (K + 7) & ~7;

@@ -169,6 +169,12 @@ __device__ __forceinline__ void bulk_store_wait_all() { asm volatile("cp.async.b
 // run their set-up and then block in pdl_wait until this grid has completed and its writes are visible).
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// The pointer behind such a wait: no load through it can be moved ahead (as loads of what a kernel declares constant might be).
+template <class T>
+__device__ __forceinline__ T *after_pdl_wait(T *p) {
+    asm volatile("" : "+l"(p)::"memory");
+    return p;
+}
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
     asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
@@ -863,6 +869,7 @@ __global__ void __launch_bounds__(PAIR_THREADS, 1) gemm_pair_kernel(const __grid
     __syncthreads();
     cluster_sync_all();  // the partner's barriers exist before anything signals them
     tc_fence_after();
+    pdl_wait();
     const uint32_t tmem_base = *tmem_holder;
 
     auto decode_tile = [&](int tile, int &m_blk, int &n_blk) {

@@ -369,6 +369,7 @@ __global__ void __launch_bounds__(PTHREADS, 1) gemm_sp_pair_kernel(const __grid_
     tc_fence_before();
     __syncthreads();
     cluster_sync_all();
+    pdl_wait();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_holder;
 

@@ -132,17 +132,19 @@ inline bool make_out_map(CUtensorMap *m, void *ptr, int64_t rows, int64_t cols, 
 template <typename Kernel, typename Prm>
 inline int launch_pairs(Kernel kern, const Prm &p, int pairs, int threads, size_t smem, cudaStream_t st) {
     cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 2;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.blockDim = dim3((unsigned)threads);
     cfg.gridDim = dim3(2 * (unsigned)pairs);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     return cudaLaunchKernelEx(&cfg, kern, p) == cudaSuccess ? MOC_OK : MOC_ERR_CUDA;
 }
 // pairs that can be resident at once (0: none, or an error)
