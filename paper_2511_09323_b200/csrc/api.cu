@@ -514,8 +514,8 @@ void tc_select_launch(const TcSelect &c, const float *G, int ldg, __nv_bfloat16 
 #define MOC_DO_LAUNCH(W, VPL, BINS)                                                                                              \
     if (c.team == W && c.vpl == VPL && c.bins == BINS)                                                                           \
         MOC_LAUNCH(KID_TC_SELECT_MASK, st,                                                                                       \
-                   launch_pdl(rs::select_rows_reg_kernel<W, VPL, BINS>, dim3(grid), 32 * W, c.smem, st, G, ldg, U, ldu, n, F, K,  \
-                              rs::normal_quantile(F, K), o_idx, o_g, o_u, status));
+                   (rs::select_rows_reg_kernel<W, VPL, BINS><<<grid, 32 * W, c.smem, st>>>(                                      \
+                       G, ldg, U, ldu, n, F, K, rs::normal_quantile(F, K), o_idx, o_g, o_u, status)));
         MOC_ROW_SELECT_FORMS(MOC_DO_LAUNCH)
 #undef MOC_DO_LAUNCH
     } else if (c.kind == TcSelect::kSharedRow) {

@@ -223,12 +223,10 @@ __device__ __noinline__ void search_whole_range(const float *g, int F, int K, ui
 
 template <int W, int VPL, int BINS>
 __global__ void __launch_bounds__(32 * W, ctas_per_sm(W, VPL)) select_rows_reg_kernel(
-    const float *G_in, int ldg, __nv_bfloat16 *__restrict__ U, int ldu, int64_t rows, int F, int K, float quantile,
+    const float *__restrict__ G, int ldg, __nv_bfloat16 *__restrict__ U, int ldu, int64_t rows, int F, int K, float quantile,
     int16_t *__restrict__ idx_out, __nv_bfloat16 *__restrict__ g_out, __nv_bfloat16 *__restrict__ u_out, int *status) {
     using namespace tc;
     extern __shared__ __align__(16) uint8_t smem[];
-    pdl_wait();
-    const float *const G = after_pdl_wait(G_in);
     constexpr int TT = 32 * W;         // threads of the team (= of the CTA)
     constexpr int GPW = VPL / 4;       // 128-channel groups per warp: lane l of a group holds channels 4 l .. 4 l + 3
     constexpr int NP = (GPW + 3) / 4;  // words of packed per-group counts

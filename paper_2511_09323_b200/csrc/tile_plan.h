@@ -29,12 +29,13 @@ struct TilePlan {
 constexpr double WIDE_MMA_CYCLES = 2.06;  // per column
 inline double wide_block_cycles(int w) { return std::max(WIDE_MMA_CYCLES * w, (16384.0 + 64.0 * w) / 58.0); }
 
-// Cycles for which the epilogue keeps an accumulator of 256 columns from the MMAs (bf16 outputs; fp32 ones among them).  Of a
-// tile with two accumulators the skew covers a bf16 one's (34.0 thousand cycles a tile of 32 blocks, 33.75 of them MMAs); with fp32
-// gate values every other tile is measured 2700 cycles longer.  That figure less what a 256-column tile loses to its stores,
-// which share the loads' way to L2 (634 and 742 cycles a block for gate + up of 32 and 12 blocks, against 565 of the loads):
-// 16384 x 768 x 2048, gate + up on tiles of 256 columns 123 thousand cycles, of 512 119.
-constexpr int WIDE_DRAIN_BF16 = 1024, WIDE_DRAIN_F32 = 2000;
+// Cycles that an accumulator of 256 columns costs (bf16 outputs; fp32 ones among them): what the epilogue keeps it from the MMAs,
+// of which the skew covers a part, and what its stores take of the loads' way to L2.  Measured, a tile of two accumulators and 32
+// blocks is 250 cycles longer than its MMAs with bf16 outputs and 2700 with fp32 gate values in every other tile.  Larger than
+// that, because they also keep the search from tiles of 256 + 64 columns, whose MMAs of 64 columns take what 128 do (62 blocks: 890
+// cycles each instead of the 659 of wide_block_cycles): with 1024 and 2000, 16544 x 3960 x 10560 took such tiles throughout
+// and its gate + up 2.77 ms instead of 2.42.
+constexpr int WIDE_DRAIN_BF16 = 2000, WIDE_DRAIN_F32 = 3500;
 
 // No plan of `rows` x N over kb blocks is shorter: its MMAs spread evenly.
 inline double plan_cycles_at_least(int rows, int64_t N, int kb, int pairs) { return WIDE_MMA_CYCLES * rows * (double)N * kb / pairs; }
