@@ -358,7 +358,7 @@ __global__ void __launch_bounds__(WIDE_THREADS, 1) gemm_wide_kernel(const __grid
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer (one per CTA).  One thread's
         // instructions per block have to stay well below a block's MMAs: everything that a tile fixes is worked out ahead.
-        if (lane == 0) {
+        if (elect_one()) {
             for (int i = 0; i < 3; ++i) {
                 prefetch_tmap(&p.g.a_map[i]);
                 prefetch_tmap(&p.g.b_map[i]);
@@ -419,7 +419,7 @@ __global__ void __launch_bounds__(WIDE_THREADS, 1) gemm_wide_kernel(const __grid
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer (leading CTA only)
-        if (lane == 0 && rank == 0) {
+        if (rank == 0 && elect_one()) {
             // one instruction consumes 16 contraction elements: 32 bytes along a K-major row, or 16 rows of 128 bytes in
             // an MN-major box (descriptor addresses are in units of 16 bytes)
             constexpr uint32_t a_step = A_MN ? 128u : 2u, b_step = B_MN ? 128u : 2u;

@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(STHREADS, 1) gemm_sp_kernel(const __grid_const
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
-        if (lane == 0) {
+        if (elect_one()) {
             prefetch_tmap(&p.a_map);
             prefetch_tmap(&p.b_map);
             int stage = 0;
@@ -158,7 +158,7 @@ __global__ void __launch_bounds__(STHREADS, 1) gemm_sp_kernel(const __grid_const
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer
-        if (lane == 0) {
+        if (elect_one()) {
             constexpr uint32_t idesc0 = make_sp_idesc<B_MN>();
             int stage = 0, acc = 0;
             uint32_t phase = 0, acc_phase = 0;
@@ -375,7 +375,7 @@ __global__ void __launch_bounds__(PTHREADS, 1) gemm_sp_pair_kernel(const __grid_
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer (one per CTA)
-        if (lane == 0) {
+        if (elect_one()) {
             for (int i = 0; i < 2; ++i) {
                 prefetch_tmap(&p.a_map[i]);
                 prefetch_tmap(&p.b_map[i]);
@@ -415,7 +415,7 @@ __global__ void __launch_bounds__(PTHREADS, 1) gemm_sp_pair_kernel(const __grid_
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer (leading CTA only)
-        if (lane == 0 && rank == 0) {
+        if (rank == 0 && elect_one()) {
             constexpr uint32_t idesc0 = (1u << 2) | (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) |
                                         ((uint32_t)(PBN >> 3) << 17) | ((uint32_t)((2 * SBM) >> 4) << 24);
             int stage = 0;
