@@ -16,10 +16,11 @@
 //             Z' boxes once flags[2] says every CTA's Z' is written) -> partial sums, added to an fp32 accumulator; the
 //             last CTA of a column block rounds to bf16
 //
-// Two warps issue the MMAs, stage about: with 16 or 32 tokens an MMA is short (some 45 cycles), and the instruction that
-// hands a stage back once its MMAs have read it (tcgen05.commit) stalls the issuing thread for some 450 cycles -- as long
-// as a whole stage's MMAs.  The stall is the thread's, not the tensor core's: a second issuer fills it.  Each issuer
-// accumulates into its own tensor-memory columns.
+// One elected thread issues the MMAs (tc::elect_one says why elected).  Chosen as lane 0 it took 1100 cycles for a stage of twelve
+// short MMAs and their commit, more than HBM takes to bring the stage, so that two warps issued stage about; a fast one then
+// overtakes the other by a round of the ring, which a parity test cannot tell.  us per call, two of lane 0 | one elected: 4096 x
+// 11008, 16 tokens 64.7 | 63.0, block form 68.8 | 66.6, 32 tokens 69.3 | 67.4; 2048 x 5504, 20 tokens 38.9 | 36.9; 768 x 2048,
+// 12 tokens 30.6 | 26.6.  Its loops over boxes stay rolled: unrolled they cost the other roles 200 bytes of spills and 5 us.
 //
 // CTAs wait on one another, so the launch is cooperative: all CTAs are resident, or the launch fails.  Every wait is
 // bounded as everywhere else in the library.
@@ -43,7 +44,7 @@ using sb::kBK;
 using sb::kTile;
 
 constexpr int kBlock = dec::kSelThreads;  // the selector's block size; a streamer CTA uses its first eleven warps:
-                                          // warp 0 TMA, warps 1 and 2 MMA, warps 3..10 epilogue (two per TMEM lane quarter)
+                                          // warp 0 TMA, warp 1 MMA, warps 3..10 epilogue (two per TMEM lane quarter)
 constexpr int kEpiWarps = 8;
 constexpr int kEpiThreads = kEpiWarps * 32;
 constexpr int kMaxTokens = 32;            // one 32-token accumulator chunk
@@ -51,8 +52,8 @@ constexpr int kTn = 32;                   // columns of tensor memory per accumu
 constexpr int kStagesMax = 8;
 constexpr int kStateCounters = 112;        // counters of the column blocks; the flags follow them in the state block
 constexpr unsigned long long kCleanMark = 0x6d6f632d66757365ull;  // "the flags and counters of this workspace are zero"
-// Tensor memory: every MMA issuer has its own accumulators (the epilogue adds them).  32 columns per tile;
-// issuer w: gate tiles at 64 w (+32), up tiles at 128 + 64 w (+32), down accumulators at 256 + 64 w (+32).
+// Tensor memory: every tile has two accumulators, of the even and the odd stages (the epilogue adds them).  32 columns per tile;
+// w = 0, 1: gate tiles at 64 w (+32), up tiles at 128 + 64 w (+32), down accumulators at 256 + 64 w (+32).
 constexpr uint32_t kTmemCols = 512;
 
 struct FusedParams {
@@ -125,7 +126,7 @@ __device__ __forceinline__ bool flag_wait(const unsigned int *flag, unsigned int
     return true;
 }
 
-// sum of the two issuers' accumulators: 16 columns at `taddr` and at `taddr` + 64 (when the second issuer had work)
+// sum of a tile's two accumulators: 16 columns at `taddr` and at `taddr` + 64 (when the second one was written)
 __device__ __forceinline__ void tmem_ld16_sum(uint32_t taddr, bool two, float (&v)[16]) {
     uint32_t a[16];
     tc::tmem_ld16(taddr, a);
@@ -298,14 +299,14 @@ __global__ void __launch_bounds__(kBlock, 1) sb_fused_kernel(const __grid_consta
     const int ahead = min(p.stages, 2 * n_gu);  // stages requested before the grid barrier
 
     if (streamer) {
-        if (threadIdx.x == 0) {
+        if (warp == 0 && tc::elect_one()) {
             for (int s = 0; s < p.stages; ++s) {
                 tc::mbar_init(full_bar(s), 1);
                 tc::mbar_init(empty_bar(s), 1);
             }
-            tc::mbar_init(tfull_g, 2);  // one arrival per MMA issuer
-            tc::mbar_init(tfull_u, 2);
-            tc::mbar_init(tfull_d, 2);
+            tc::mbar_init(tfull_g, 1);
+            tc::mbar_init(tfull_u, 1);
+            tc::mbar_init(tfull_d, 1);
             *abort_flag = 0;
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -319,7 +320,7 @@ __global__ void __launch_bounds__(kBlock, 1) sb_fused_kernel(const __grid_consta
     }
     // everything below touches what earlier kernels in the stream may still read or write (x, the workspace, out)
     tc::pdl_wait();
-    if (streamer && threadIdx.x == 0 && !p.rms_w) {
+    if (streamer && warp == 0 && !p.rms_w && tc::elect_one()) {
         for (int i = 0; i < ahead; ++i) {
             issue_gu_x(i, i);
             pr_next();
@@ -349,7 +350,7 @@ __global__ void __launch_bounds__(kBlock, 1) sb_fused_kernel(const __grid_consta
 
     if (warp == 0) {
         // ------------------------------------------------------------------ producer
-        if (lane == 0) {
+        if (tc::elect_one()) {
             bool ok = true;
             if (p.rms_w) {  // the first ring's activation boxes: once the selector CTAs have normalised every token
                 ok = flag_wait(p.flags + 5, (unsigned int)p.T, abort_flag, p.status, p.wait_limit);
@@ -401,13 +402,10 @@ __global__ void __launch_bounds__(kBlock, 1) sb_fused_kernel(const __grid_consta
                 pr_next();
             }
         }
-    } else if (warp <= 2) {
-        // ------------------------------------------------------------------ MMA issuers: stages about.  Both walk the
-        // whole sequence of stages and wait for every one (a parity test only tells an odd from an even number of
-        // completed rounds, so a thread must see every round of a barrier it waits on); issuer w works on the stages
-        // whose number within their phase is w modulo 2.
-        if (lane == 0) {
-            const uint32_t w = (uint32_t)(warp - 1);
+    } else if (warp == 1) {
+        // ------------------------------------------------------------------ MMA issuer.  Stages go alternately to two sets
+        // of accumulators: each sums half of the contraction.
+        if (tc::elect_one()) {
             const uint32_t idesc_gu = sb::idesc_bf16(false, p.tn), idesc_d = sb::idesc_bf16(true, p.tn);
             const uint64_t dk = tc::make_smem_desc(0, 16, 1024), dm = tc::make_smem_desc(0, kBK * 128, 1024);
             const uint32_t hi = (uint32_t)(dk >> 32), lo_k = (uint32_t)dk, lo_m = (uint32_t)dm;  // (the high words agree)
@@ -422,53 +420,50 @@ __global__ void __launch_bounds__(kBlock, 1) sb_fused_kernel(const __grid_consta
             };
             const uint32_t xp = kXBox >> 4, wp = p.w_pitch >> 4;
             for (int m = 0; m < 2 && ok; ++m) {
-                const uint32_t acc0 = tmem_base + (uint32_t)(128 * m) + 64u * w;
-                uint32_t accum = 0u;
                 for (int s = 0; s < n_gu; ++s) {
                     if (!tc::mbar_wait(full_bar(stage), phase, abort_flag, p.status, p.wait_limit)) {
                         ok = false;
                         break;
                     }
-                    if (((uint32_t)s & 1u) == w) {
-                        tc::tc_fence_after();
-                        const uint32_t x_lo = lo_k + (slot(stage) >> 4), w_lo = x_lo + nb * xp;
-                        for (uint32_t b = 0; b < nb; ++b) {
+                    tc::tc_fence_after();
+                    const uint32_t acc = tmem_base + (uint32_t)(128 * m) + 64u * ((uint32_t)s & 1u);
+                    const uint32_t x_lo = lo_k + (slot(stage) >> 4), w_lo = x_lo + nb * xp;
+                    uint32_t accum = s < 2 ? 0u : 1u;
+#pragma unroll 1
+                    for (uint32_t b = 0; b < nb; ++b) {
 #pragma unroll
-                            for (uint32_t k = 0; k < kBK / 16; ++k) {
-                                umma_lohi(acc0, w_lo + b * wp + 2u * k, x_lo + b * xp + 2u * k, hi, idesc_gu, accum);
-                                if (extra) umma_lohi(acc0 + (uint32_t)kTn, w_lo + b * wp + 8u * (uint32_t)extra + 2u * k, x_lo + b * xp + 2u * k, hi, idesc_gu, accum);
-                                accum = 1u;
-                            }
+                        for (uint32_t k = 0; k < kBK / 16; ++k) {
+                            umma_lohi(acc, w_lo + b * wp + 2u * k, x_lo + b * xp + 2u * k, hi, idesc_gu, accum);
+                            if (extra) umma_lohi(acc + (uint32_t)kTn, w_lo + b * wp + 8u * (uint32_t)extra + 2u * k, x_lo + b * xp + 2u * k, hi, idesc_gu, accum);
+                            accum = 1u;
                         }
-                        tc::umma_commit(empty_bar(stage));
                     }
+                    tc::umma_commit(empty_bar(stage));
                     next();
                 }
                 if (ok && n_gu > 0) tc::umma_commit(m == 0 ? tfull_g : tfull_u);
             }
-            const uint32_t accd = tmem_base + 256u + 64u * w;
-            uint32_t accum = 0u;
             for (int i = 0; i < n_d && ok; ++i) {
                 if (!tc::mbar_wait(full_bar(stage), phase, abort_flag, p.status, p.wait_limit)) {
                     ok = false;
                     break;
                 }
-                if (((uint32_t)i & 1u) == w) {
-                    tc::tc_fence_after();
-                    const uint32_t a_lo = lo_m + (slot(stage) >> 4), z_lo = lo_k + ((slot(stage) + d_w_bytes) >> 4);
+                tc::tc_fence_after();
+                const uint32_t acc = tmem_base + 256u + 64u * ((uint32_t)i & 1u);
+                const uint32_t a_lo = lo_m + (slot(stage) >> 4), z_lo = lo_k + ((slot(stage) + d_w_bytes) >> 4);
+                uint32_t accum = i < 2 ? 0u : 1u;
 #pragma unroll
-                    for (uint32_t k = 0; k < kBK / 16; ++k) {
-                        for (uint32_t a = 0; a < (uint32_t)p.accs; ++a)
-                            umma_lohi(accd + a * (uint32_t)kTn, a_lo + a * 1024u + k * 128u, z_lo + 2u * k, hi, idesc_d, accum);
-                        accum = 1u;
-                    }
-                    tc::umma_commit(empty_bar(stage));
+                for (uint32_t k = 0; k < kBK / 16; ++k) {
+                    for (uint32_t a = 0; a < (uint32_t)p.accs; ++a)
+                        umma_lohi(acc + a * (uint32_t)kTn, a_lo + a * 1024u + k * 128u, z_lo + 2u * k, hi, idesc_d, accum);
+                    accum = 1u;
                 }
+                tc::umma_commit(empty_bar(stage));
                 next();
             }
             if (ok && n_d > 0) tc::umma_commit(tfull_d);
         }
-    } else if (warp < 3 + kEpiWarps) {
+    } else if (warp >= 3 && warp < 3 + kEpiWarps) {
         // ------------------------------------------------------------------ epilogue warps 3..10
         // Work items are (tile, 16-token chunk); the two warps of a TMEM lane quarter take alternate items.
         const int quarter = warp & 3, half = (warp - 3) >> 2, etid = (int)threadIdx.x - 96;
@@ -479,7 +474,7 @@ __global__ void __launch_bounds__(kBlock, 1) sb_fused_kernel(const __grid_consta
         bool ok = true;
         if (has_gu) {
             const int items = (extra ? 2 : 1) * chunks;
-            const bool two = n_gu >= 2;  // the second issuer had stages of its own
+            const bool two = n_gu >= 2;  // the second accumulator had stages of its own
             uint32_t kept0 = 0u;         // MoC 2:8: bit i = this lane's channel is kept by token i of the warp's first item
             // MoC 2:8: the kept bits of tokens t0 .. t0 + 15 for this lane's channel, from the gate values in shared memory.
             // The 8 channels of a group sit in 8 adjacent lanes: a channel is kept when fewer than two of its group come
