@@ -162,13 +162,17 @@ __global__ void __launch_bounds__(kThreads, 1) decode_cluster_kernel(const __gri
     __syncthreads();
     cluster_arrive();  // #0: the CTA's shared memory exists (waited for before the first store into another CTA's)
     tc::pdl_launch_dependents();
-    const auto request = [&](int g, int s) {  // (the producer warp) 16 rows, or what is left of them, to stage s
+    // (the producer warp) 16 rows, or what is left of them, to stage s; by one elected thread (a lane for each row: four tokens of
+    // 768 x 2048 15.2 us instead of 14.3)
+    const auto request = [&](int g, int s) {
         const int n = min(16, rows - g * 16);
         const uint32_t bar = tc::smem_u32(&full[s]);
-        if (lane == 0) tc::mbar_expect_tx(bar, (uint32_t)n * row_bytes);
+        if (tc::elect_one()) {
+            tc::mbar_expect_tx(bar, (uint32_t)n * row_bytes);
+            for (int i = 0; i < n; ++i)
+                tc::bulk_copy_g2s(smem + (uint32_t)s * stage_bytes + (uint32_t)i * pitch, p.wg + (int64_t)(c0 + g * 16 + i) * d, row_bytes, bar);
+        }
         __syncwarp();
-        if (lane < n)
-            tc::bulk_copy_g2s(smem + (uint32_t)s * stage_bytes + (uint32_t)lane * pitch, p.wg + (int64_t)(c0 + g * 16 + lane) * d, row_bytes, bar);
     };
     if (producer)
         for (int g = 0; g < min(groups, p.stages); ++g) request(g, g);
