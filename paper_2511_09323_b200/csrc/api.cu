@@ -1048,8 +1048,8 @@ bool use_decode_plan(const moc_ffn_desc &d) {
 
 // ---- cooperative decode (bf16, one or two tokens, d_model <= 4096): one kernel, every SM keeps its channels ----
 struct CoopLayout {
-    int grid, unit, stages;
-    size_t smem, off_hist, off_n, off_cand, off_acc, total;
+    int grid, unit, most_tokens, stages, of_stage, col_groups, rp, parts, part_shift;  // as in dc::Params; most_tokens: the kernel's T
+    size_t smem, off_hist, off_fine, off_n, off_cand, off_acc, total;
 };
 
 // ok == false: the problem or the device does not admit the cooperative kernel (the four-kernel plan runs then)
@@ -1069,24 +1069,42 @@ CoopLayout coop_layout(const moc_ffn_desc &d, bool &ok) {
     }();
     if (!coop_ok) return L;
     const int T = (int)d.tokens, dm = d.d_model, F = d.d_ff;
-    L.unit = (F % 8 == 0) ? 8 : 1;
-    if ((d.flags & MOC_FLAG_SELECT_2_OF_8) && L.unit != 8) return L;
+    const bool grouped = (d.flags & MOC_FLAG_SELECT_2_OF_8) != 0;
+    if (grouped && F % 8 != 0) return L;
+    L.unit = grouped ? 8 : 1;
     const int units = (F + L.unit - 1) / L.unit;
     L.grid = std::min(tc::sm_count(), units);
-    if (((units + L.grid - 1) / L.grid) * L.unit > dc::kMaxRows) return L;
-    const size_t fixed = (size_t)T * dm * 2 + (size_t)2 * T * dc::kMaxRows * 4;
-    const size_t budget = (size_t)216 * 1024;
-    if (fixed + (size_t)4 * dm * 2 > budget) return L;
-    // a multiple of the consumer warps: every stage is then always consumed by the same warp (see the kernel)
-    L.stages = (int)std::min<size_t>(dc::kMaxStages, (budget - fixed) / ((size_t)dm * 2)) / dc::kConsumerWarps * dc::kConsumerWarps;
-    if (L.stages < dc::kConsumerWarps) return L;
-    L.smem = dc::smem_bytes(T, dm, L.stages);
-    Carver c;
-    L.off_hist = c.take((size_t)T * dc::kBins * sizeof(uint32_t));
-    L.off_n = c.take((size_t)T * sizeof(uint32_t));
-    L.off_cand = c.take((size_t)T * F * sizeof(uint2));
-    L.off_acc = c.take((size_t)T * dm * sizeof(float));
-    L.total = c.off;
+    const int rows = ((units + L.grid - 1) / L.grid) * L.unit;  // of a CTA, at most
+    if (rows > dc::kMaxRows) return L;
+    L.rp = (rows + 7) & ~7;
+    L.most_tokens = T;
+    // a warp holds 4 / most_tokens vectors of 8 columns a lane
+    for (L.col_groups = 1; L.col_groups * 256 * (4 / L.most_tokens) < dm;) L.col_groups *= 2;
+    // stages of some 32 KiB
+    for (L.of_stage = 32; L.of_stage > 1 && (size_t)L.of_stage * dc::row_pitch(dm) > (size_t)34 * 1024;) L.of_stage /= 2;
+    const auto smem = [&](int stages) { return dc::smem_bytes(L.most_tokens, dm, L.rp, L.col_groups, L.of_stage, stages); };
+    constexpr size_t kBudget = (size_t)kMaxDynSmem - dc::kStaticReserve;
+    for (L.stages = dc::kMaxStages; L.stages > 2 && smem(L.stages) > kBudget;) --L.stages;
+    L.smem = smem(L.stages);
+    if (L.smem > kBudget) return L;
+    const auto carve = [&]() {
+        Carver c;
+        L.off_hist = c.take((size_t)T * dc::kBins * sizeof(uint32_t));
+        L.off_n = c.take((size_t)T * sizeof(uint32_t));
+        L.off_cand = c.take((size_t)T * F * sizeof(uint2));
+        L.off_acc = c.take((size_t)T * dm * sizeof(float));
+        L.off_fine = c.take((size_t)T * dc::kNarrowBins * L.parts / 2);
+        L.total = c.off;
+    };
+    carve();
+    // parts of the narrow bins: what the four-kernel plan's workspace, which every call has, leaves room for
+    if (!grouped)
+        for (L.parts = dc::kMostParts; L.parts > 0; L.parts = L.parts > 8 ? L.parts / 2 : 0) {
+            carve();
+            if (L.parts == 0 || L.total <= decode_layout(d).total) break;
+        }
+    carve();
+    for (L.part_shift = 16; (1 << (16 - L.part_shift)) < L.parts;) --L.part_shift;
     ok = true;
     return L;
 }
@@ -1095,7 +1113,7 @@ template <int T>
 int launch_coop(const dc::Params &prm, const CoopLayout &L, cudaStream_t st) {
     auto kern = dc::decode_coop_kernel<T>;
     int rc;
-    if ((rc = set_smem(kern, L.smem, 8 * 1024)) != MOC_OK) return rc;
+    if ((rc = set_smem(kern, L.smem, dc::kStaticReserve)) != MOC_OK) return rc;
     // all CTAs must be resident at once (the launch would be refused otherwise); asked once per shared-memory size
     static std::mutex mu;
     static std::unordered_map<size_t, int> per_sm_of;
@@ -1112,11 +1130,20 @@ int launch_coop(const dc::Params &prm, const CoopLayout &L, cudaStream_t st) {
         }
     }
     if (per_sm < 1 || L.grid > per_sm * tc::sm_count()) return MOC_ERR_UNSUPPORTED;
-    dc::Params local = prm;
-    void *args[] = {&local};
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = dim3((unsigned)L.grid);
+    cfg.blockDim = dim3(dc::kThreads);
+    cfg.dynamicSmemBytes = L.smem;
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
     cudaError_t err = cudaSuccess;
-    MOC_LAUNCH(KID_DEC_COOP, st,
-               err = cudaLaunchCooperativeKernel(reinterpret_cast<void *>(kern), dim3(L.grid), dim3(dc::kThreads), args, L.smem, st));
+    MOC_LAUNCH(KID_DEC_COOP, st, err = cudaLaunchKernelEx(&cfg, kern, prm));
     if (err != cudaSuccess) {  // refused: nothing ran, the four-kernel plan serves the call
         (void)cudaGetLastError();
         return MOC_ERR_UNSUPPORTED;
@@ -1136,25 +1163,30 @@ int decode_coop(const moc_ffn_desc &d, const CoopLayout &L, const __nv_bfloat16 
     prm.wu = wu;
     prm.wd = wd;
     prm.out = out;
-    prm.T = (int)d.tokens;
+    prm.tokens = (int)d.tokens;
     prm.d = d.d_model;
     prm.F = d.d_ff;
     prm.K = d.k;
     prm.grouped = (d.flags & MOC_FLAG_SELECT_2_OF_8) ? 1 : 0;
     prm.unit = L.unit;
     prm.stages = L.stages;
+    prm.of_stage = L.of_stage;
+    prm.col_groups = L.col_groups;
+    prm.parts = L.parts;
+    prm.part_shift = L.part_shift;
+    prm.rp = L.rp;
     prm.rms_w = rms_w;
     prm.rms_eps = rms_eps;
     prm.kept_out = kept_out;
     prm.hist = reinterpret_cast<uint32_t *>(wsp + L.off_hist);
+    prm.fine = reinterpret_cast<uint32_t *>(wsp + L.off_fine);
     prm.cand_n = reinterpret_cast<uint32_t *>(wsp + L.off_n);
     prm.cand = reinterpret_cast<uint2 *>(wsp + L.off_cand);
     prm.acc = reinterpret_cast<float *>(wsp + L.off_acc);
     prm.status = status;
-    switch (prm.T) {
+    switch (L.most_tokens) {
         case 1: return launch_coop<1>(prm, L, st);
-        case 2: return launch_coop<2>(prm, L, st);
-        default: return MOC_ERR_UNSUPPORTED;
+        default: return launch_coop<2>(prm, L, st);
     }
 }
 
