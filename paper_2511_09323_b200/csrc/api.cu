@@ -1141,9 +1141,17 @@ int launch_coop(const dc::Params &prm, const CoopLayout &L, cudaStream_t st) {
     cfg.dynamicSmemBytes = L.smem;
     cfg.stream = st;
     cfg.attrs = attr;
-    cfg.numAttrs = 2;
+    // (a driver that refuses the combination gets the plain cooperative launch from then on)
+    static std::atomic<int> pdl_ok{1};
+    cfg.numAttrs = pdl_ok.load(std::memory_order_relaxed) ? 2 : 1;
     cudaError_t err = cudaSuccess;
     MOC_LAUNCH(KID_DEC_COOP, st, err = cudaLaunchKernelEx(&cfg, kern, prm));
+    if (err != cudaSuccess && cfg.numAttrs == 2) {
+        (void)cudaGetLastError();
+        cfg.numAttrs = 1;
+        MOC_LAUNCH(KID_DEC_COOP, st, err = cudaLaunchKernelEx(&cfg, kern, prm));
+        if (err == cudaSuccess) pdl_ok.store(0, std::memory_order_relaxed);
+    }
     if (err != cudaSuccess) {  // refused: nothing ran, the four-kernel plan serves the call
         (void)cudaGetLastError();
         return MOC_ERR_UNSUPPORTED;
@@ -1464,12 +1472,44 @@ int small_batch_down(const moc_ffn_desc &d, const SmallBatchLayout &L, const sb:
 // masked hidden state Z' from its accumulators, the gate values and the selection bitmaps.  Four kernels:
 //   gate (all SMs) -> select (T CTAs, bitmaps only) || up + mask (SMs - ceil(T/2) CTAs) -> down.
 // MOC_FFN_SB_OVERLAP=0 in the environment keeps the three-kernel form everywhere (comparisons); =n: up to n tokens.
-bool small_batch_overlapped(const moc_ffn_desc &d, bool saving) {
+int overlap_limit_asked() {  // -1: not set
     static const int limit = [] {
         const char *e = getenv("MOC_FFN_SB_OVERLAP");
-        return e ? atoi(e) : 32;  // measured on the LLaMA-7B shape: 67 / 70 us against 70 / 72 us at 16 / 32 tokens, but 86 against 76 us at 64
+        return e ? atoi(e) : -1;
     }();
-    return !saving && !(d.flags & MOC_FLAG_SELECT_2_OF_8) && d.tokens <= limit && tc::sm_count() >= 32;
+    return limit;
+}
+
+// Which form of the small-batch plan a decode call takes (Top-K mask, no block form).  us per call over three sets of weights, three
+// kernels | four, overlapped | one: 6 and 32 tokens of 768 x 2048 18.3 20.0 | 20.3 22.4 | 26.7 28.7, of 2048 x 5504 30.4 33.3 | 31.4
+// 34.8 | 34.9 38.8, of 2560 x 6912 36.0 38.0 | 35.9 39.6 | 39.2 43.3; of 3072 x 8192 43.4 46.2 | 41.9 45.9 | 44.3 48.4, of 4096 x 11008
+// 62.9 66.3 | 58.5 61.5 | 59.9 66.0, of 4096 x 16384 83.9 88.0 | 74.7 83.3 | 83.9 89.1; 12 and 24 tokens of 5120 x 20480 142 144 | 111 114
+// | 110 122.  More than 32 tokens, three | four: 36 of 3072 x 8192 46.7 | 46.6 and 44 46.9 | 48.4, 44 of 4096 x 11008 68.1 | 66.1 and 52
+// 69.0 | 69.5, 48 of 4608 x 12288 79.7 | 78.5.  The overlapped form's last CTA takes channels one by one where they do not come in
+// fours: 24 tokens of 5120 x 13653 87.5 | 92.1 | 84.3, of 3584 x 9557 55.4 | 60.2 | 54.9.
+// (Layers of fewer weights than any that was measured stay with the one kernel, and so does moc_ffn_forward with nothing saved.)
+enum class SmallBatchForm { kOne, kThree, kOverlapped };
+SmallBatchForm decode_form(const moc_ffn_desc &d) {
+    const int64_t weights = (int64_t)d.d_model * d.d_ff;  // of one matrix
+    const bool fours = d.d_ff % 4 == 0;
+    if ((d.flags & MOC_FLAG_SELECT_2_OF_8) || weights < 300'000) return SmallBatchForm::kOne;
+    if (weights < (fours ? 18'000'000 : 25'000'000)) return SmallBatchForm::kThree;
+    if (fours && tc::sm_count() >= 96 && d.tokens <= (weights < 30'000'000 ? 32 : 44) && !(weights >= 90'000'000 && d.tokens <= 16))
+        return SmallBatchForm::kOverlapped;
+    return SmallBatchForm::kOne;  // (the three kernels beyond its 32 tokens)
+}
+
+// Three to five tokens for which the four-kernel decode plan reads fewer bytes (small_batch_preferred): these forms are faster all the same
+// below 40 million weights, or where 0.4 of the channels are in use.  Decode plan | form above, us: 2048 x 5504, three tokens, K = F / 8
+// 33.3 | 30.1, F / 16 31.4 | 30.0; 1440 x 3840 27.6 | 23.7; 3072 x 8192, F / 8 44.5 | 41.1, F / 16 41.7 | 41.1; 3072 x 12288 52.9 | 50.6; 4096 x
+// 11008, three 57.3 | 58.0, four 59.4 | 58.1, F / 16 55.2 | 57.8; 4608 x 12288, four 71.0 | 67.0; 5120 x 20480, three 151 | 107.
+bool small_batch_faster_than_gathering(const moc_ffn_desc &d, size_t workspace_bytes) {
+    static const bool asked = getenv("MOC_FFN_DECODE") != nullptr;  // for another form
+    if (asked || d.tokens < 3 || d.tokens > 5 || (d.flags & MOC_FLAG_SELECT_2_OF_8) || !use_small_batch_plan(d)) return false;
+    const int64_t weights = (int64_t)d.d_model * d.d_ff;
+    const double used = 1.0 - std::pow(1.0 - (double)d.k / (double)d.d_ff, (double)d.tokens);
+    return weights >= 300'000 && (weights < (d.d_ff % 4 == 0 ? 40'000'000 : 25'000'000) || used >= 0.4 || weights >= 90'000'000) &&
+           small_batch_layout(d).total <= workspace_bytes;
 }
 
 // channels per CTA when `ctas` CTAs share the F channels of one matrix: a multiple of 8, at most sb::kMaxRows
@@ -1727,7 +1767,7 @@ int forward_small_batch_fused(const moc_ffn_desc &d, const SmallBatchLayout &L, 
 int forward_small_batch(const moc_ffn_desc &d, const __nv_bfloat16 *x, const __nv_bfloat16 *wg,
                         const __nv_bfloat16 *wu, const __nv_bfloat16 *wd, __nv_bfloat16 *out, int16_t *idx,
                         __nv_bfloat16 *tg, __nv_bfloat16 *tu, char *wsp, cudaStream_t st,
-                        const __nv_bfloat16 *resid = nullptr) {
+                        const __nv_bfloat16 *resid = nullptr, SmallBatchForm form = SmallBatchForm::kOne) {
     const SmallBatchLayout L = small_batch_layout(d);
     const int T = (int)d.tokens, F = d.d_ff, dm = d.d_model;
     int *status = device_status_ptr();
@@ -1751,15 +1791,18 @@ int forward_small_batch(const moc_ffn_desc &d, const __nv_bfloat16 *x, const __n
     if ((rc = set_smem(sb::sb_down_kernel, ds.smem, 1024)) != MOC_OK) return rc;
     if ((rc = set_smem(sb::sb_select_kernel, sel_smem)) != MOC_OK) return rc;
 
-    {
+    const int asked = overlap_limit_asked();
+    if (form == SmallBatchForm::kOne) {
         bool fused_ok = false;
         const FusedLayout FL = fused_layout(d, idx != nullptr, fused_ok);
         if (fused_ok) {
             rc = forward_small_batch_fused(d, L, FL, x, wg, wu, wd, out, wsp, st, resid);
             if (rc != MOC_ERR_UNSUPPORTED) return rc;
         }
+        if (T <= 32) form = SmallBatchForm::kOverlapped;  // where that kernel is not admitted
     }
-    if (small_batch_overlapped(d, idx != nullptr))
+    if (asked >= 0) form = T <= asked ? SmallBatchForm::kOverlapped : SmallBatchForm::kThree;
+    if (form == SmallBatchForm::kOverlapped && idx == nullptr && !(d.flags & MOC_FLAG_SELECT_2_OF_8) && tc::sm_count() >= 32)
         return forward_small_batch_overlapped(d, L, x, wg, wu, wd, out, wsp, st, resid);
 
     sb::GateUpParams gp;
@@ -1924,9 +1967,9 @@ size_t moc_ffn_saved_bytes_per_token(const moc_ffn_desc *desc) {
     return (size_t)desc->k * (sizeof(int16_t) + 2 * esize(desc->dtype));
 }
 
-int moc_ffn_forward(const moc_ffn_desc *desc, const void *x, const void *w_gate, const void *w_up,
-                    const void *w_down, void *out, int16_t *topk_idx, void *topk_gate, void *topk_up,
-                    void *workspace, size_t workspace_bytes, void *cuda_stream) {
+static int forward_or_decode(const moc_ffn_desc *desc, const void *x, const void *w_gate, const void *w_up,
+                             const void *w_down, void *out, int16_t *topk_idx, void *topk_gate, void *topk_up,
+                             void *workspace, size_t workspace_bytes, void *cuda_stream, bool decode) {
     int rc = check_desc(desc);
     if (rc != MOC_OK) return rc;
     const bool save_all = topk_idx && topk_gate && topk_up;
@@ -1945,7 +1988,8 @@ int moc_ffn_forward(const moc_ffn_desc *desc, const void *x, const void *w_gate,
         using T = __nv_bfloat16;
         if (use_small_batch_plan(*desc))
             return forward_small_batch(*desc, (const T *)x, (const T *)w_gate, (const T *)w_up, (const T *)w_down,
-                                       (T *)out, topk_idx, (T *)topk_gate, (T *)topk_up, ws, st);
+                                       (T *)out, topk_idx, (T *)topk_gate, (T *)topk_up, ws, st, nullptr,
+                                       decode ? decode_form(*desc) : SmallBatchForm::kOne);
         if (use_tc_forward(*desc))
             return forward_tc(*desc, (const T *)x, (const T *)w_gate, (const T *)w_up, (const T *)w_down, (T *)out,
                               topk_idx, (T *)topk_gate, (T *)topk_up, ws, st);
@@ -1955,6 +1999,13 @@ int moc_ffn_forward(const moc_ffn_desc *desc, const void *x, const void *w_gate,
     return forward_gather<float>(*desc, (const float *)x, (const float *)w_gate, (const float *)w_up,
                                  (const float *)w_down, (float *)out, topk_idx, (float *)topk_gate,
                                  (float *)topk_up, ws, st);
+}
+
+int moc_ffn_forward(const moc_ffn_desc *desc, const void *x, const void *w_gate, const void *w_up,
+                    const void *w_down, void *out, int16_t *topk_idx, void *topk_gate, void *topk_up,
+                    void *workspace, size_t workspace_bytes, void *cuda_stream) {
+    return forward_or_decode(desc, x, w_gate, w_up, w_down, out, topk_idx, topk_gate, topk_up, workspace, workspace_bytes,
+                             cuda_stream, false);
 }
 
 int moc_ffn_backward(const moc_ffn_desc *desc, const void *x, const void *w_gate, const void *w_up,
@@ -2024,8 +2075,8 @@ int moc_ffn_decode(const moc_ffn_desc *desc, const void *x, const void *w_gate, 
     if (rc != MOC_OK) return rc;
     if (desc->tokens > sb::kMaxTokens) return MOC_ERR_UNSUPPORTED;
     if (!use_decode_plan(*desc))  // more than 16 tokens, or fp32 storage: the forward with nothing saved
-        return moc_ffn_forward(desc, x, w_gate, w_up, w_down, out, nullptr, nullptr, nullptr, workspace,
-                               workspace_bytes, cuda_stream);
+        return forward_or_decode(desc, x, w_gate, w_up, w_down, out, nullptr, nullptr, nullptr, workspace,
+                                 workspace_bytes, cuda_stream, true);
     if (!good_ptr(x) || !good_ptr(w_gate) || !good_ptr(w_up) || !good_ptr(w_down) || !good_ptr(out))
         return MOC_ERR_INVALID_ARG;
     const size_t need = moc_ffn_workspace_bytes(desc, MOC_OP_DECODE);
@@ -2049,6 +2100,12 @@ int moc_ffn_decode(const moc_ffn_desc *desc, const void *x, const void *w_gate, 
                                         (T *)out, static_cast<char *>(workspace), static_cast<cudaStream_t>(cuda_stream));
             if (rc2 != MOC_ERR_UNSUPPORTED) return rc2;
         }
+    }
+    if (small_batch_faster_than_gathering(*desc, need)) {
+        const int rc2 = forward_small_batch(*desc, (const T *)x, (const T *)w_gate, (const T *)w_up, (const T *)w_down, (T *)out, nullptr,
+                                            nullptr, nullptr, static_cast<char *>(workspace), static_cast<cudaStream_t>(cuda_stream),
+                                            nullptr, decode_form(*desc));
+        if (rc2 != MOC_ERR_UNSUPPORTED) return rc2;
     }
     return decode_bf16(*desc, (const T *)x, (const T *)w_gate, (const T *)w_up, (const T *)w_down, (T *)out,
                        static_cast<char *>(workspace), static_cast<cudaStream_t>(cuda_stream));
