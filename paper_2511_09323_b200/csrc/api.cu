@@ -1543,7 +1543,7 @@ int forward_small_batch_overlapped(const moc_ffn_desc &d, const SmallBatchLayout
     const size_t sel_smem = std::max(sb::select_smem(F, false), (size_t)116 * 1024);
     if ((rc = set_smem(sb::sb_gate_up_kernel, std::max(gg.smem, gu.smem), 1024)) != MOC_OK) return rc;
     if ((rc = set_smem(sb::sb_down_kernel, ds.smem, 1024)) != MOC_OK) return rc;
-    if ((rc = set_smem(sb::sb_select_kernel, sel_smem)) != MOC_OK) return rc;
+    if ((rc = set_smem(sb::sb_select_kernel<true>, sel_smem)) != MOC_OK) return rc;
 
     auto gate_up_params = [&](sb::GateUpParams &gp, const sb::GemmShape &gs, int rows, int ctas) {
         memset(&gp, 0, sizeof(gp));
@@ -1575,7 +1575,7 @@ int forward_small_batch_overlapped(const moc_ffn_desc &d, const SmallBatchLayout
     if ((rc = launch_ok()) != MOC_OK) return rc;
 
     sb::SelectParams sp{G, nullptr, L.ldf, F, d.k, dm, Z, L.ldz, acc, nullptr, nullptr, nullptr, 0, status, kept, kept_words};
-    MOC_LAUNCH(KID_SB_SELECT, st, launch_pdl(sb::sb_select_kernel, dim3(T), dec::kSelThreads, sel_smem, st, sp));
+    MOC_LAUNCH(KID_SB_SELECT, st, launch_pdl(sb::sb_select_kernel<true>, dim3(T), dec::kSelThreads, sel_smem, st, sp));
     if ((rc = launch_ok()) != MOC_OK) return rc;
 
     sb::GateUpParams up;
@@ -1789,7 +1789,7 @@ int forward_small_batch(const moc_ffn_desc &d, const __nv_bfloat16 *x, const __n
     const size_t sel_smem = std::max(sb::select_smem(F, L.stage_u), T <= tc::sm_count() ? kOnePerSm : 0);
     if ((rc = set_smem(sb::sb_gate_up_kernel, gs.smem, 1024)) != MOC_OK) return rc;
     if ((rc = set_smem(sb::sb_down_kernel, ds.smem, 1024)) != MOC_OK) return rc;
-    if ((rc = set_smem(sb::sb_select_kernel, sel_smem)) != MOC_OK) return rc;
+    if ((rc = set_smem(sb::sb_select_kernel<false>, sel_smem)) != MOC_OK) return rc;
 
     const int asked = overlap_limit_asked();
     if (form == SmallBatchForm::kOne) {
@@ -1837,7 +1837,7 @@ int forward_small_batch(const moc_ffn_desc &d, const __nv_bfloat16 *x, const __n
         MOC_LAUNCH(KID_SB_SELECT, st,
                    launch_pdl(sb::sb_select_grouped_kernel, dim3(T), dec::kSelThreads, 0, st, sp));
     } else {
-        MOC_LAUNCH(KID_SB_SELECT, st, launch_pdl(sb::sb_select_kernel, dim3(T), dec::kSelThreads, sel_smem, st, sp));
+        MOC_LAUNCH(KID_SB_SELECT, st, launch_pdl(sb::sb_select_kernel<false>, dim3(T), dec::kSelThreads, sel_smem, st, sp));
     }
     if ((rc = launch_ok()) != MOC_OK) return rc;
 

@@ -408,6 +408,7 @@ __device__ __forceinline__ bool cta_stage_rows(uint64_t *bar, int *abort_flag, i
 // g == nullptr: keys[] already holds the row's fp32 values (staged by a bulk copy) and is converted in place.
 // lists0: two candidate lists of kSelListCap entries; sm: the full radix select's state (its arrays double as scratch).
 // keys[j] of the calling thread's channels (j = tid modulo kSelThreads) may be read at once, the others behind a barrier.
+// With WINDOW keys[] has whole fours (the last ones need not be values).
 //
 // WINDOW: one histogram over a window around the expected threshold, which a sample of the row gives as in row_select.cuh,
 // then the few keys of the threshold's bin ranked by every warp for itself; the search over the whole range remains for
@@ -416,11 +417,13 @@ __device__ __forceinline__ bool cta_stage_rows(uint64_t *bar, int *abort_flag, i
 // long as one of 11008).  61 tokens at 4096 x 11008: 78.3 -> 74.8 us for the layer, 3 tokens at 1024 x 2731: 26.3 -> 24.8.
 // Inside the cooperative kernel (small_batch_fused.cuh) the selector waits for its row anyway and the instructions of a
 // second search delay it: 0.9 - 1.6 us slower with the window, so it takes the search over the whole range alone.
+// kept (WINDOW, optional, room for K): the pass that collects the bin's keys also lists the channels of the bins above it, in no
+// order, and the kept ones of the bin join them: returns true when `kept` then holds the set.
 template <bool WINDOW>
-__device__ __forceinline__ void cta_select_threshold(const float *__restrict__ g, int F, int K, uint32_t *keys,
+__device__ __forceinline__ bool cta_select_threshold(const float *__restrict__ g, int F, int K, uint32_t *keys,
                                                      uint32_t *lists0, SelectSmemT<kSelThreads / 32> &sm,
-                                                     uint32_t &tau_out, int &need_out, bool &ties_cut_out) {
-    __shared__ uint32_t s_min[32], s_max[32], s_pick, s_above, s_inbin, s_n;
+                                                     uint32_t &tau_out, int &need_out, bool &ties_cut_out, uint16_t *kept = nullptr) {
+    __shared__ uint32_t s_min[32], s_max[32], s_pick, s_above, s_inbin, s_n, s_kept;
     uint32_t *lists[2] = {lists0, lists0 + kSelListCap};
     uint32_t *hist = sm.priv;  // 2048 entries
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -432,8 +435,12 @@ __device__ __forceinline__ void cta_select_threshold(const float *__restrict__ g
         constexpr int kWindowBins = 512;
         bool window = false;
         float scale = 0.f, offset = 0.f;
+        if (g) {
+            for (int j = tid; j < F; j += kSelThreads) keys[j] = __float_as_uint(g[j]);
+            __syncthreads();
+        }
         if (F >= 128) {
-            const float *v = (g ? g : reinterpret_cast<const float *>(keys)) + ((uint32_t)lane * (uint32_t)(F >> 2) >> 5) * 4;
+            const float *v = reinterpret_cast<const float *>(keys) + ((uint32_t)lane * (uint32_t)(F >> 2) >> 5) * 4;
             const float a = v[0], b = v[1], c = v[2], e = v[3];
             const float mean = warp_sum(a + b + c + e) * (1.0f / 128.0f);
             const float mad = warp_sum(fabsf(a - mean) + fabsf(b - mean) + fabsf(c - mean) + fabsf(e - mean)) * (1.0f / 128.0f);
@@ -442,15 +449,20 @@ __device__ __forceinline__ void cta_select_threshold(const float *__restrict__ g
             offset = -fmaf(mad, 1.2533f * rs::normal_quantile_fast(F, K) - rs::kWindowMad, mean) * scale;
         }
         for (int i = tid; i < 2048; i += kSelThreads) hist[i] = 0;
-        if (tid == 0) s_n = 0;
+        if (tid == 0) s_n = s_kept = 0;
         __syncthreads();  // the sample is read before its values become keys
 #pragma unroll 1
-        for (int j = tid; j < F; j += kSelThreads) {
-            const uint32_t key = gate_key(g ? g[j] : __uint_as_float(keys[j]));
-            keys[j] = key;
-            kmin = min(kmin, key);
-            kmax = max(kmax, key);
-            if (window) atomicAdd(&hist[rs::bin4<kWindowBins>(key_to_float(key), scale, offset) >> 2], 1u);
+        for (int j = 4 * tid; j < F; j += 4 * kSelThreads) {  // (the arrays have whole fours)
+            const uint4 q = *reinterpret_cast<const uint4 *>(keys + j);
+            const uint32_t k4[4] = {gate_key(__uint_as_float(q.x)), gate_key(__uint_as_float(q.y)), gate_key(__uint_as_float(q.z)), gate_key(__uint_as_float(q.w))};
+            *reinterpret_cast<uint4 *>(keys + j) = make_uint4(k4[0], k4[1], k4[2], k4[3]);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                if (j + e >= F) break;
+                kmin = min(kmin, k4[e]);
+                kmax = max(kmax, k4[e]);
+                if (window) atomicAdd(&hist[rs::bin4<kWindowBins>(key_to_float(k4[e]), scale, offset) >> 2], 1u);
+            }
         }
         if (window) {  // (the same for the whole CTA)
             __syncthreads();
@@ -465,10 +477,29 @@ __device__ __forceinline__ void cta_select_threshold(const float *__restrict__ g
             __syncthreads();
             const uint32_t bin = s_pick, m = (uint32_t)K - s_above, count = s_inbin;
             if (bin >= 1u && bin < kWindowBins - 1u && count <= 32u) {
+                uint32_t *const channels = lists0 + 32;  // of the bin's keys
 #pragma unroll 1
-                for (int j = tid; j < F; j += kSelThreads) {
-                    const uint32_t key = keys[j];
-                    if (rs::bin4<kWindowBins>(key_to_float(key), scale, offset) >> 2 == bin) lists0[atomicAdd(&s_n, 1u)] = key;
+                for (int j0 = 0; j0 < F; j0 += 4 * kSelThreads) {
+                    const int j = j0 + 4 * tid;
+                    const uint4 q = j < F ? *reinterpret_cast<const uint4 *>(keys + j) : make_uint4(0u, 0u, 0u, 0u);
+                    const uint32_t k4[4] = {q.x, q.y, q.z, q.w};
+                    uint32_t b[4], mine = 0;
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        b[e] = j + e < F ? rs::bin4<kWindowBins>(key_to_float(k4[e]), scale, offset) >> 2 : 0u;
+                        mine += b[e] > bin ? 1u : 0u;
+                        if (b[e] == bin) {
+                            const uint32_t at = atomicAdd(&s_n, 1u);
+                            lists0[at] = k4[e];
+                            channels[at] = (uint32_t)(j + e);
+                        }
+                    }
+                    if (kept && mine) {
+                        uint32_t at = atomicAdd(&s_kept, mine);
+#pragma unroll
+                        for (int e = 0; e < 4; ++e)
+                            if (b[e] > bin) kept[at++] = (uint16_t)(j + e);
+                    }
                 }
                 __syncthreads();
                 const uint32_t mine = (uint32_t)lane < count ? lists0[lane] : 0u;
@@ -483,7 +514,13 @@ __device__ __forceinline__ void cta_select_threshold(const float *__restrict__ g
                 tau_out = __shfl_sync(0xffffffffu, mine, src);
                 need_out = (int)(m - __shfl_sync(0xffffffffu, gt, src));
                 ties_cut_out = need_out != (int)__shfl_sync(0xffffffffu, eq, src);
-                return;
+                if (kept == nullptr || ties_cut_out) return false;
+                if (warp == 0) {  // (all warps have read the count of the others: the barrier above)
+                    const uint32_t in = __ballot_sync(0xffffffffu, (uint32_t)lane < count && mine >= tau_out);
+                    if ((in >> lane) & 1u) kept[s_above + (uint32_t)__popc(in & ((1u << lane) - 1u))] = (uint16_t)channels[lane];
+                }
+                __syncthreads();
+                return true;
             }
             for (int i = tid; i < 2048; i += kSelThreads) hist[i] = 0;
         }
@@ -679,6 +716,7 @@ __device__ __forceinline__ void cta_select_threshold(const float *__restrict__ g
     tau_out = tau;
     need_out = need;
     ties_cut_out = ties_cut;
+    return false;
 }
 
 __global__ void __launch_bounds__(kSelThreads) select_mask_kernel(Workspace ws, int F, int K, int *arrivals,
