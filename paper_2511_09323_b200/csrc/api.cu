@@ -1486,7 +1486,8 @@ int overlap_limit_asked() {  // -1: not set
 // 62.9 66.3 | 58.5 61.5 | 59.9 66.0, of 4096 x 16384 83.9 88.0 | 74.7 83.3 | 83.9 89.1; 12 and 24 tokens of 5120 x 20480 142 144 | 111 114
 // | 110 122.  More than 32 tokens, three | four: 36 of 3072 x 8192 46.7 | 46.6 and 44 46.9 | 48.4, 44 of 4096 x 11008 68.1 | 66.1 and 52
 // 69.0 | 69.5, 48 of 4608 x 12288 79.7 | 78.5.  The overlapped form's last CTA takes channels one by one where they do not come in
-// fours: 24 tokens of 5120 x 13653 87.5 | 92.1 | 84.3, of 3584 x 9557 55.4 | 60.2 | 54.9.
+// fours: 24 tokens of 5120 x 13653 87.5 | 92.1 | 84.3, of 3584 x 9557 55.4 | 60.2 | 54.9.  Up to 16 tokens the one kernel is ahead of it on
+// wide layers: four | one, 14 tokens of 4328 x 11520 69.1 | 66.1, 12 of 4776 x 12736 79.8 | 75.7; of 3728 x 14912 69.6 | 70.4.
 // (Layers of fewer weights than any that was measured stay with the one kernel, and so does moc_ffn_forward with nothing saved.)
 enum class SmallBatchForm { kOne, kThree, kOverlapped };
 SmallBatchForm decode_form(const moc_ffn_desc &d) {
@@ -1494,21 +1495,23 @@ SmallBatchForm decode_form(const moc_ffn_desc &d) {
     const bool fours = d.d_ff % 4 == 0;
     if ((d.flags & MOC_FLAG_SELECT_2_OF_8) || weights < 300'000) return SmallBatchForm::kOne;
     if (weights < (fours ? 18'000'000 : 25'000'000)) return SmallBatchForm::kThree;
-    if (fours && tc::sm_count() >= 96 && d.tokens <= (weights < 30'000'000 ? 32 : 44) && !(weights >= 90'000'000 && d.tokens <= 16))
+    if (fours && tc::sm_count() >= 96 && d.tokens <= (weights < 30'000'000 ? 32 : 44) && (d.d_model <= 4224 || d.tokens > 16))
         return SmallBatchForm::kOverlapped;
     return SmallBatchForm::kOne;  // (the three kernels beyond its 32 tokens)
 }
 
 // Three to five tokens for which the four-kernel decode plan reads fewer bytes (small_batch_preferred): these forms are faster all the same
-// below 40 million weights, or where 0.4 of the channels are in use.  Decode plan | form above, us: 2048 x 5504, three tokens, K = F / 8
-// 33.3 | 30.1, F / 16 31.4 | 30.0; 1440 x 3840 27.6 | 23.7; 3072 x 8192, F / 8 44.5 | 41.1, F / 16 41.7 | 41.1; 3072 x 12288 52.9 | 50.6; 4096 x
-// 11008, three 57.3 | 58.0, four 59.4 | 58.1, F / 16 55.2 | 57.8; 4608 x 12288, four 71.0 | 67.0; 5120 x 20480, three 151 | 107.
+// below 30 million weights, below 40 million with 0.3 of the channels in use, and where that plan's list of rows is longest.  Decode plan |
+// form above, us: 2048 x 5504, three tokens, K = F / 8 33.3 | 30.1, F / 16 31.4 | 30.0; 1440 x 3840 27.6 | 23.7; 3072 x 8192, F / 8 44.5 | 41.1,
+// F / 16 41.7 | 41.1; 3072 x 12288, F / 8 52.9 | 50.6; 2984 x 11936, F / 16 49.2 | 52.0; 4096 x 11008, three 57.3 | 58.0, four 59.4 | 58.1 but
+// 75 | 80 the first time on new buffers (tensor maps to encode), F / 16 55.2 | 57.8; 5120 x 20480, three 151 | 107.
 bool small_batch_faster_than_gathering(const moc_ffn_desc &d, size_t workspace_bytes) {
     static const bool asked = getenv("MOC_FFN_DECODE") != nullptr;  // for another form
     if (asked || d.tokens < 3 || d.tokens > 5 || (d.flags & MOC_FLAG_SELECT_2_OF_8) || !use_small_batch_plan(d)) return false;
     const int64_t weights = (int64_t)d.d_model * d.d_ff;
     const double used = 1.0 - std::pow(1.0 - (double)d.k / (double)d.d_ff, (double)d.tokens);
-    return weights >= 300'000 && (weights < (d.d_ff % 4 == 0 ? 40'000'000 : 25'000'000) || used >= 0.4 || weights >= 90'000'000) &&
+    const bool fours = d.d_ff % 4 == 0;
+    return weights >= 300'000 && (weights < (fours ? 30'000'000 : 25'000'000) || (fours && weights < 40'000'000 && used >= 0.3) || weights >= 90'000'000) &&
            small_batch_layout(d).total <= workspace_bytes;
 }
 

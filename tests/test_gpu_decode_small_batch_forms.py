@@ -27,8 +27,10 @@ def _form(launches):
     (16, 2560, 9765, 1220, THREE), (16, 2560, 9767, 1221, ONE), (16, 2560, 9764, 1220, OVERLAPPED),   # 25 million, channels not in fours
     (32, 2560, 7032, 879, OVERLAPPED), (33, 2560, 7032, 879, THREE),
     (44, 2560, 11720, 1465, OVERLAPPED), (45, 2560, 11720, 1465, THREE),                     # 30 million
-    (3, 1440, 3840, 480, THREE), (4, 2560, 7032, 440, OVERLAPPED), (4, 4096, 9768, 1221, OVERLAPPED),  # three to five tokens: four tenths in use,
-    (3, 4096, 9768, 1221, CHAIN), (4, 2560, 9767, 610, CHAIN),                               # 40 million, or 25 not in fours
+    (16, 4232, 7032, 879, ONE), (17, 4232, 7032, 879, OVERLAPPED),                           # wide layers
+    (3, 1440, 3840, 480, THREE), (4, 2560, 7032, 440, OVERLAPPED), (3, 2560, 11716, 732, OVERLAPPED),   # three to five tokens: below 30 million
+    (3, 2560, 11720, 732, CHAIN), (3, 2560, 11720, 1465, OVERLAPPED), (3, 4096, 9768, 1221, CHAIN),     # or 40 with 0.3 in use
+    (4, 2560, 9767, 610, CHAIN),                                                             # 25 million not in fours
 ])
 def test_form_and_result(tokens, d, F, k, form):
     g = torch.Generator(device="cuda").manual_seed(tokens + F)
