@@ -185,7 +185,6 @@ __global__ void __launch_bounds__(kThreads, 1) decode_coop_kernel(const __grid_c
     const int c0 = u0 * p.unit, c1 = min(F, u1 * p.unit);
     const int rows = max(0, c1 - c0);  // <= kMaxRows (the host checks)
 
-    tc::pdl_launch_dependents();
     if (tid == 0) {
         for (int s = 0; s < p.stages; ++s) {
             tc::mbar_init(full_bar(s), 1);
@@ -308,6 +307,9 @@ __global__ void __launch_bounds__(kThreads, 1) decode_coop_kernel(const __grid_c
     //      arrays that all CTAs share
     const int first = min(min(p.stages, kFirstStages) * p.of_stage, rows);  // (the producer joins the barrier below: it must not be late)
     tc::pdl_wait();  // (weights, too, may come from the kernel in front; requested ahead of this they are not there any earlier)
+    // Released behind that wait: the next kernel may fetch weights ahead of its own wait, and what wrote them may be the kernel in front
+    // of this one.  (Nothing is lost: the CTAs hold their SM for some 30 us yet.)
+    tc::pdl_launch_dependents();
     if (producer && tc::elect_one()) request(p.wg, nullptr, 0, first);
     {
         if (p.rms_w) {
