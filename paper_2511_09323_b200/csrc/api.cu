@@ -13,6 +13,7 @@
 
 #include "decode_cluster.cuh"
 #include "decode_coop.cuh"
+#include "decode_form.h"
 #include "decode_kernels.cuh"
 #include "gather_kernels.cuh"
 #include "grouped_select.cuh"
@@ -1024,8 +1025,9 @@ DecodeLayout decode_layout(const moc_ffn_desc &d) {
     // about two CTAs per SM in the down kernel; a CTA's share of the list is bounded by its shared arrays
     const int sms = tc::sm_count();
     L.parts = std::max(std::max(1, 2 * sms / L.slices), (d.d_ff + dec::kMaxPart - 1) / dec::kMaxPart);
-    // GEMV kernels: two CTAs per SM, never more than 64 rows per CTA
-    L.gemv_grid = std::max(std::max(1, std::min(2 * sms, (d.d_ff + 7) / 8)), (d.d_ff + 63) / 64);
+    // GEMV kernels: two CTAs per SM, never more than kGateRows rows per CTA
+    static_assert(kGateRows == dec::kGemvMaxRows, "what a CTA's arrays hold");
+    L.gemv_grid = std::max(std::max(1, std::min(2 * sms, (d.d_ff + 7) / 8)), (d.d_ff + kGateRows - 1) / kGateRows);
     Carver c;
     L.off_g = c.take((size_t)d.tokens * L.ldf * sizeof(float));
     L.off_zb = c.take((size_t)((d.d_ff + 15) / 16) * 256 * sizeof(__nv_bfloat16));
@@ -1500,19 +1502,11 @@ SmallBatchForm decode_form(const moc_ffn_desc &d) {
     return SmallBatchForm::kOne;  // (the three kernels beyond its 32 tokens)
 }
 
-// Three to five tokens for which the four-kernel decode plan reads fewer bytes (small_batch_preferred): these forms are faster all the same
-// below 30 million weights, below 40 million with 0.3 of the channels in use, and where that plan's list of rows is longest.  Decode plan |
-// form above, us: 2048 x 5504, three tokens, K = F / 8 33.3 | 30.1, F / 16 31.4 | 30.0; 1440 x 3840 27.6 | 23.7; 3072 x 8192, F / 8 44.5 | 41.1,
-// F / 16 41.7 | 41.1; 3072 x 12288, F / 8 52.9 | 50.6; 2984 x 11936, F / 16 49.2 | 52.0; 4096 x 11008, three 57.3 | 58.0, four 59.4 | 58.1 but
-// 75 | 80 the first time on new buffers (tensor maps to encode), F / 16 55.2 | 57.8; 5120 x 20480, three 151 | 107.
+// Three to five tokens for which small_batch_preferred chooses the gathering plan (decode_form.h).
 bool small_batch_faster_than_gathering(const moc_ffn_desc &d, size_t workspace_bytes) {
     static const bool asked = getenv("MOC_FFN_DECODE") != nullptr;  // for another form
     if (asked || d.tokens < 3 || d.tokens > 5 || (d.flags & MOC_FLAG_SELECT_2_OF_8) || !use_small_batch_plan(d)) return false;
-    const int64_t weights = (int64_t)d.d_model * d.d_ff;
-    const double used = 1.0 - std::pow(1.0 - (double)d.k / (double)d.d_ff, (double)d.tokens);
-    const bool fours = d.d_ff % 4 == 0;
-    return weights >= 300'000 && (weights < (fours ? 30'000'000 : 25'000'000) || (fours && weights < 40'000'000 && used >= 0.3) || weights >= 90'000'000) &&
-           small_batch_layout(d).total <= workspace_bytes;
+    return streaming_beats_gathering((int)d.tokens, d.d_model, d.d_ff, d.k, tc::sm_count()) && small_batch_layout(d).total <= workspace_bytes;
 }
 
 // channels per CTA when `ctas` CTAs share the F channels of one matrix: a multiple of 8, at most sb::kMaxRows
