@@ -22,6 +22,8 @@
 //                    fixed, so the last bit of `out` may vary from run to run).
 #pragma once
 
+#include <cstddef>
+
 #include "moc_common.cuh"
 #include "row_select.cuh"
 #include "tc_gemm.cuh"  // mbarrier helpers
@@ -425,7 +427,8 @@ __device__ __forceinline__ bool cta_select_threshold(const float *__restrict__ g
                                                      uint32_t &tau_out, int &need_out, bool &ties_cut_out, uint16_t *kept = nullptr) {
     __shared__ uint32_t s_min[32], s_max[32], s_pick, s_above, s_inbin, s_n, s_kept;
     uint32_t *lists[2] = {lists0, lists0 + kSelListCap};
-    uint32_t *hist = sm.priv;  // 2048 entries
+    uint32_t *hist = sm.priv;  // 2048 entries, read sixteen bytes at a time
+    static_assert(alignof(SelectSmemT<kSelThreads / 32>) % 16 == 0 && offsetof(SelectSmemT<kSelThreads / 32>, priv) % 16 == 0);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     constexpr int NW = kSelThreads / 32;
     uint32_t kmin = 0xffffffffu, kmax = 0u;

@@ -29,8 +29,10 @@ constexpr int kSelectTable = kSelectMaxN / 256 * 8;     // (chunk, warp) slots: 
 
 constexpr int kPrivStride = 257;  // per-warp histogram stride: equal bins of different warps hit different banks
 
+// (aligned for 16-byte reads of priv, which the CTA-per-row selector uses as one histogram: among a kernel's other shared variables its
+// words alone would ask for 4 bytes)
 template <int NW>
-struct SelectSmemT {
+struct alignas(16) SelectSmemT {
     uint32_t hist[256];
     uint32_t warp_tot[32];
     uint32_t cand[kSelectCandCap];
