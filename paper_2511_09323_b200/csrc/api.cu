@@ -1440,6 +1440,14 @@ SmallBatchLayout small_batch_layout(const moc_ffn_desc &d) {
     return L;
 }
 
+int small_batch_least_tokens_asked() {  // 0: not set
+    static const int forced = [] {
+        const char *e = getenv("MOC_FFN_SB_MIN_TOKENS");
+        return e ? std::max(0, atoi(e)) : 0;
+    }();
+    return forced;
+}
+
 // Which of the two small-batch forms reads fewer bytes: the decode plan reads W_gate and the rows of W_up / W_down
 // that some token selected, (1 + 2 u) F d elements with u = 1 - (1 - K/F)^T the expected share of used channels; the
 // small-batch plan reads all 3 F d but is one kernel without gathers.  Measured on the LLaMA-7B shape the two cross
@@ -1447,10 +1455,7 @@ SmallBatchLayout small_batch_layout(const moc_ffn_desc &d) {
 // passes 0.45; from 17 tokens on only the small-batch plan exists.
 // MOC_FFN_SB_MIN_TOKENS=n in the environment moves the boundary to n tokens (measurements only).
 bool small_batch_preferred(const moc_ffn_desc &d) {
-    static const int forced = [] {
-        const char *e = getenv("MOC_FFN_SB_MIN_TOKENS");
-        return e ? atoi(e) : 0;
-    }();
+    const int forced = small_batch_least_tokens_asked();
     if (forced >= 1) return d.tokens >= forced;
     if (d.tokens > 16) return true;
     const double unused = std::pow(1.0 - (double)d.k / (double)d.d_ff, (double)d.tokens);
@@ -1504,7 +1509,7 @@ SmallBatchForm decode_form(const moc_ffn_desc &d) {
 
 // Three to five tokens for which small_batch_preferred chooses the gathering plan (decode_form.h).
 bool small_batch_faster_than_gathering(const moc_ffn_desc &d, size_t workspace_bytes) {
-    static const bool asked = getenv("MOC_FFN_DECODE") != nullptr;  // for another form
+    static const bool asked = getenv("MOC_FFN_DECODE") != nullptr || small_batch_least_tokens_asked() >= 1;  // for another form
     if (asked || d.tokens < 3 || d.tokens > 5 || (d.flags & MOC_FLAG_SELECT_2_OF_8) || !use_small_batch_plan(d)) return false;
     return streaming_beats_gathering((int)d.tokens, d.d_model, d.d_ff, d.k, tc::sm_count()) && small_batch_layout(d).total <= workspace_bytes;
 }
