@@ -1050,7 +1050,7 @@ bool use_decode_plan(const moc_ffn_desc &d) {
 
 // ---- cooperative decode (bf16, one or two tokens, d_model <= 4096): one kernel, every SM keeps its channels ----
 struct CoopLayout {
-    int grid, unit, most_tokens, stages, of_stage, col_groups, rp, parts, part_shift;  // as in dc::Params; most_tokens: the kernel's T
+    int grid, unit, stages, of_stage, col_groups, rp, parts, part_shift;  // as in dc::Params
     size_t smem, off_hist, off_fine, off_n, off_cand, off_acc, total;
 };
 
@@ -1079,12 +1079,11 @@ CoopLayout coop_layout(const moc_ffn_desc &d, bool &ok) {
     const int rows = ((units + L.grid - 1) / L.grid) * L.unit;  // of a CTA, at most
     if (rows > dc::kMaxRows) return L;
     L.rp = (rows + 7) & ~7;
-    L.most_tokens = T;
-    // a warp holds 4 / most_tokens vectors of 8 columns a lane
-    for (L.col_groups = 1; L.col_groups * 256 * (4 / L.most_tokens) < dm;) L.col_groups *= 2;
+    // a warp holds 4 / T vectors of 8 columns a lane
+    for (L.col_groups = 1; L.col_groups * 256 * (4 / T) < dm;) L.col_groups *= 2;
     // stages of some 32 KiB
     for (L.of_stage = 32; L.of_stage > 1 && (size_t)L.of_stage * dc::row_pitch(dm) > (size_t)34 * 1024;) L.of_stage /= 2;
-    const auto smem = [&](int stages) { return dc::smem_bytes(L.most_tokens, dm, L.rp, L.col_groups, L.of_stage, stages); };
+    const auto smem = [&](int stages) { return dc::smem_bytes(T, dm, L.rp, L.col_groups, L.of_stage, stages); };
     constexpr size_t kBudget = (size_t)kMaxDynSmem - dc::kStaticReserve;
     for (L.stages = dc::kMaxStages; L.stages > 2 && smem(L.stages) > kBudget;) --L.stages;
     L.smem = smem(L.stages);
@@ -1103,7 +1102,7 @@ CoopLayout coop_layout(const moc_ffn_desc &d, bool &ok) {
     if (!grouped)
         for (L.parts = dc::kMostParts; L.parts > 0; L.parts = L.parts > 8 ? L.parts / 2 : 0) {
             carve();
-            if (L.parts == 0 || L.total <= decode_layout(d).total) break;
+            if (L.total <= decode_layout(d).total) break;
         }
     carve();
     for (L.part_shift = 16; (1 << (16 - L.part_shift)) < L.parts;) --L.part_shift;
@@ -1173,7 +1172,6 @@ int decode_coop(const moc_ffn_desc &d, const CoopLayout &L, const __nv_bfloat16 
     prm.wu = wu;
     prm.wd = wd;
     prm.out = out;
-    prm.tokens = (int)d.tokens;
     prm.d = d.d_model;
     prm.F = d.d_ff;
     prm.K = d.k;
@@ -1194,10 +1192,7 @@ int decode_coop(const moc_ffn_desc &d, const CoopLayout &L, const __nv_bfloat16 
     prm.cand = reinterpret_cast<uint2 *>(wsp + L.off_cand);
     prm.acc = reinterpret_cast<float *>(wsp + L.off_acc);
     prm.status = status;
-    switch (L.most_tokens) {
-        case 1: return launch_coop<1>(prm, L, st);
-        default: return launch_coop<2>(prm, L, st);
-    }
+    return d.tokens == 1 ? launch_coop<1>(prm, L, st) : launch_coop<2>(prm, L, st);
 }
 
 // ---- decode on small layers: clusters of 16 CTAs, a token or two each ---------------------------------------

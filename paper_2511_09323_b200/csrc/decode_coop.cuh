@@ -60,7 +60,7 @@ __host__ __device__ constexpr uint32_t key_bin(uint32_t key) {
 }
 static_assert(key_bin(0xffffffffu) < (uint32_t)kBins, "the bins cover every key");
 // Counters of equal parts of each of the narrow bins, of 2^-5 <= g < 2^4: as many parts as the workspace has room for (256 at one
-// token of 11008 channels, 64 at four), four bits each, eight to a word.  Where the part that holds the K-th largest key holds no more
+// token of 11008 channels, 128 at two), four bits each, eight to a word.  Where the part that holds the K-th largest key holds no more
 // keys than are kept of it, it decides alone, and the exchange of the bin's keys, a barrier of the grid and 3 us in all, does not
 // take place.  A counter that overflows lowers the sum of its bin's counters, which then differs from the bin's own.
 constexpr uint32_t kFineFrom = 0xbd000000u, kFineTo = 0xc1800000u;  // keys
@@ -83,24 +83,24 @@ constexpr int kFirstStages = 2;  // requested before the shared arrays are clear
 struct Params {
     const __nv_bfloat16 *x, *wg, *wu, *wd;
     __nv_bfloat16 *out;
-    int tokens, d, F, K, grouped;
+    int d, F, K, grouped;
     int unit;            // channels are dealt to the CTAs in units of this many (8 with the 2-of-8 mask, else 1)
     int stages, of_stage;  // ring stages of `of_stage` weight rows each
     int col_groups;        // parts of the columns that the consumer warps share out (a power of two)
     int rp;              // channels of a CTA, at most, rounded up to 8
     int parts, part_shift;  // of a narrow bin (a power of two, at least 8; or 0: none), and log2 of the keys in one
     // workspace
-    uint32_t *hist;      // [tokens][kBins]
-    uint32_t *fine;      // [tokens][kNarrowBins][parts / 8]
-    uint32_t *cand_n;    // [tokens]
-    uint2 *cand;         // [tokens][F]  (key, channel)
-    float *acc;          // [tokens][d]
+    uint32_t *hist;      // [T][kBins]
+    uint32_t *fine;      // [T][kNarrowBins][parts / 8]
+    uint32_t *cand_n;    // [T]
+    uint2 *cand;         // [T][F]  (key, channel)
+    float *acc;          // [T][d]
     int *status;
     // the block form (Section 2, "LLM structure"): x holds the residual stream h, the layer reads RMSNorm(h) with
     // weight rms_w and adds h to its output; rms_w == nullptr: the plain layer on x
     const __nv_bfloat16 *rms_w;
     float rms_eps;
-    // test hook: when not null, [tokens][F] bytes that receive 1 for every channel a token keeps and 0 for the others
+    // test hook: when not null, [T][F] bytes that receive 1 for every channel a token keeps and 0 for the others
     uint8_t *kept_out;
 };
 
@@ -168,7 +168,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_coop_kernel(const __grid_c
     // on it: its warp is the last one here and streams nothing.
     const int lane = threadIdx.x & 31, warp = threadIdx.x < 32 ? kThreads / 32 - 1 : (int)threadIdx.x / 32 - 1, tid = 32 * warp + lane;
     const bool producer = warp == kConsumerWarps, consumer = warp < kConsumerWarps;
-    const int d = p.d, F = p.F, nt = p.tokens, rp = p.rp;
+    const int d = p.d, F = p.F, rp = p.rp;
     const uint32_t pitch = row_pitch(d), stage_bytes = (uint32_t)p.of_stage * pitch;
     uint8_t *const ring = dsm;
     float *const part = reinterpret_cast<float *>(ring + (size_t)p.stages * stage_bytes);  // [col_groups][T][rp]
@@ -246,7 +246,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_coop_kernel(const __grid_c
             for (int t = 0; t < T; ++t) {
                 const int v = v0 + 32 * j;
                 uint4 q = make_uint4(0, 0, 0, 0);
-                if (v < v1 && t < nt) {
+                if (v < v1) {
                     q = reinterpret_cast<const uint4 *>(p.x + (int64_t)t * d)[v];
                     if (p.rms_w) {  // y = h / sqrt(mean(h^2) + eps) . weight, rounded to bf16 as the layer's input
                         float h8[8], w8[8];
@@ -320,7 +320,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_coop_kernel(const __grid_c
 #pragma unroll
             for (int t = 0; t < T; ++t) {
                 float ss = 0.f;
-                if (t < nt && tid * 8 < d) {
+                if (tid * 8 < d) {
                     float h8[8];
                     Vec8<__nv_bfloat16>::load(p.x + (int64_t)t * d + tid * 8, h8);
 #pragma unroll
@@ -341,11 +341,15 @@ __global__ void __launch_bounds__(kThreads, 1) decode_coop_kernel(const __grid_c
         for (int i = tid; i < kMaxRows; i += kThreads) s_mask[i] = 0;
         const int nthr = (int)gridDim.x * kThreads, gtid = (int)blockIdx.x * kThreads + tid;
         if (!p.grouped) {
-            for (int i = gtid; i < nt * kBins; i += nthr) p.hist[i] = 0u;
-            for (int i = gtid; i < nt * kNarrowBins * p.parts / 32; i += nthr) reinterpret_cast<uint4 *>(p.fine)[i] = make_uint4(0, 0, 0, 0);
-            for (int i = gtid; i < nt; i += nthr) p.cand_n[i] = 0u;
+#pragma unroll 1
+            for (int i = gtid; i < T * kBins; i += nthr) p.hist[i] = 0u;
+#pragma unroll 1
+            for (int i = gtid; i < T * kNarrowBins * p.parts / 32; i += nthr) reinterpret_cast<uint4 *>(p.fine)[i] = make_uint4(0, 0, 0, 0);
+#pragma unroll 1
+            for (int i = gtid; i < T; i += nthr) p.cand_n[i] = 0u;
         }
-        for (int i = gtid; i < nt * d; i += nthr) p.acc[i] = 0.f;
+#pragma unroll 1
+        for (int i = gtid; i < T * d; i += nthr) p.acc[i] = 0.f;
     }
     // #0, split: the CTA announces that its slices are clear now and waits for the others only when it is about to
     // touch the shared arrays, after phase 1 (the arrival is a block-wide barrier too)
@@ -358,7 +362,8 @@ __global__ void __launch_bounds__(kThreads, 1) decode_coop_kernel(const __grid_c
         consume_dots(rows);
     }
     __syncthreads();
-    for (int i = tid; i < nt * rows; i += kThreads) {
+#pragma unroll 1
+    for (int i = tid; i < T * rows; i += kThreads) {
         const int t = i / rows, r = i - t * rows;
         sg[t * rp + r] = dot(t, r);
     }
@@ -367,7 +372,8 @@ __global__ void __launch_bounds__(kThreads, 1) decode_coop_kernel(const __grid_c
 
     // ---- selection
     if (!p.grouped) {
-        for (int i = tid; i < nt * rows; i += kThreads) {
+#pragma unroll 1
+        for (int i = tid; i < T * rows; i += kThreads) {
             const int t = i / rows, r = i - t * rows;
             const uint32_t key = gate_key(sg[t * rp + r]);
             atomicAdd(&p.hist[t * kBins + key_bin(key)], 1u);
@@ -383,9 +389,8 @@ __global__ void __launch_bounds__(kThreads, 1) decode_coop_kernel(const __grid_c
             constexpr int kWarpsOf = kConsumerWarps / T, N = kBins / (kWarpsOf * 32);
             static_assert(N % 4 == 0, "16-byte loads");
             const int t = warp / kWarpsOf, j = tid - t * kWarpsOf * 32;
-            const bool mine = consumer && t < nt;
             uint32_t h[N] = {}, s = 0u, own = 0u;
-            if (mine) {
+            if (consumer) {
 #pragma unroll
                 for (int i = 0; i < N / 4; ++i) {
                     const uint4 q = __ldcg(reinterpret_cast<const uint4 *>(p.hist + t * kBins) + j * (N / 4) + i);
@@ -402,7 +407,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_coop_kernel(const __grid_c
                 if (lane == 0) s_scan[warp] = s;
             }
             __syncthreads();
-            if (mine) {
+            if (consumer) {
                 uint32_t after = 0u;
                 for (int w = warp + 1; w < (t + 1) * kWarpsOf; ++w) after += s_scan[w];
                 uint32_t above = s + after - own;  // keys in strictly higher bins than this thread's
@@ -419,7 +424,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_coop_kernel(const __grid_c
             __syncthreads();
         }
         // its parts, by a warp for each token
-        if (warp < nt) {
+        if (warp < T) {
             constexpr uint32_t kFirst = key_bin(kFineFrom), kLast = key_bin(kFineTo - 1u);
             const uint32_t bin = s_bin[warp], need = (uint32_t)p.K - s_above[warp];
             uint32_t least = 0u;
@@ -452,9 +457,10 @@ __global__ void __launch_bounds__(kThreads, 1) decode_coop_kernel(const __grid_c
         __syncthreads();
         bool open = false;  // (the same in every CTA: all have read the same counts)
 #pragma unroll
-        for (int t = 0; t < T; ++t) open = open || (t < nt && s_least[t] == 0u);
+        for (int t = 0; t < T; ++t) open = open || s_least[t] == 0u;
         const auto keep = [&](int t, int r) { atomicOr(reinterpret_cast<unsigned int *>(s_mask) + (r >> 2), (1u << t) << (8 * (r & 3))); };
-        for (int i = tid; i < nt * rows; i += kThreads) {
+#pragma unroll 1
+        for (int i = tid; i < T * rows; i += kThreads) {
             const int t = i / rows, r = i - t * rows;
             const uint32_t key = gate_key(sg[t * rp + r]), bin = key_bin(key);
             if (s_least[t] != 0u ? key >= s_least[t] : bin > s_bin[t]) keep(t, r);
@@ -472,7 +478,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_coop_kernel(const __grid_c
             uint32_t n_of[T], off_of[T], total = 0;
 #pragma unroll
             for (int t = 0; t < T; ++t) {
-                n_of[t] = t < nt ? min(__ldcg(&p.cand_n[t]), (uint32_t)F) : 0u;
+                n_of[t] = min(__ldcg(&p.cand_n[t]), (uint32_t)F);
                 off_of[t] = total;
                 total += n_of[t];
             }
@@ -484,7 +490,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_coop_kernel(const __grid_c
                     for (uint32_t j = tid; j < n_of[t]; j += kThreads) scand[off_of[t] + j] = __ldcg(&p.cand[(int64_t)t * F + j]);
             }
             __syncthreads();
-            for (int i = warp; i < nt * rows; i += kThreads / 32) {
+            for (int i = warp; i < T * rows; i += kThreads / 32) {
                 const int t = i / rows, r = i - t * rows;
                 const uint32_t key = gate_key(sg[t * rp + r]);
                 if (s_least[t] == 0u && key_bin(key) == s_bin[t]) {
@@ -509,7 +515,8 @@ __global__ void __launch_bounds__(kThreads, 1) decode_coop_kernel(const __grid_c
         }
     } else {
         // MoC 2:8 (Section 4): the CTA's range is made of whole groups of eight channels; the mask is local
-        for (int i = tid; i < nt * (rows >> 3); i += kThreads) {
+#pragma unroll 1
+        for (int i = tid; i < T * (rows >> 3); i += kThreads) {
             const int t = i / (rows >> 3), q = i - t * (rows >> 3);
             uint32_t key[8];
 #pragma unroll
@@ -522,7 +529,8 @@ __global__ void __launch_bounds__(kThreads, 1) decode_coop_kernel(const __grid_c
     }
     __syncthreads();  // (and the ring is the producer's again)
     if (p.kept_out)
-        for (int i = tid; i < nt * rows; i += kThreads) {
+#pragma unroll 1
+        for (int i = tid; i < T * rows; i += kThreads) {
             const int t = i / rows, r = i - t * rows;
             p.kept_out[(int64_t)t * F + c0 + r] = (uint8_t)((s_mask[r] >> t) & 1);
         }
@@ -579,7 +587,6 @@ __global__ void __launch_bounds__(kThreads, 1) decode_coop_kernel(const __grid_c
         if (col < d && nsel > 0) {
 #pragma unroll
             for (int t = 0; t < T; ++t) {
-                if (t >= nt) break;
                 float *dst = p.acc + (int64_t)t * d + col;
 #pragma unroll
                 for (int h = 0; h < 2; ++h)
@@ -594,7 +601,8 @@ __global__ void __launch_bounds__(kThreads, 1) decode_coop_kernel(const __grid_c
 
     // ---- out = bf16(accumulator), a slice per CTA
     {
-        const int vecs = nt * d / 8;
+        const int vecs = T * d / 8;
+#pragma unroll 1
         for (int v = (int)blockIdx.x * kThreads + tid; v < vecs; v += (int)gridDim.x * kThreads) {
             float4 a = __ldcg(reinterpret_cast<const float4 *>(p.acc) + 2 * v);
             float4 b = __ldcg(reinterpret_cast<const float4 *>(p.acc) + 2 * v + 1);
