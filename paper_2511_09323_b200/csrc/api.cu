@@ -1482,24 +1482,9 @@ int overlap_limit_asked() {  // -1: not set
     return limit;
 }
 
-// Which form of the small-batch plan a decode call takes (Top-K mask, no block form).  us per call over three sets of weights, three
-// kernels | four, overlapped | one: 6 and 32 tokens of 768 x 2048 18.3 20.0 | 20.3 22.4 | 26.7 28.7, of 2048 x 5504 30.4 33.3 | 31.4
-// 34.8 | 34.9 38.8, of 2560 x 6912 36.0 38.0 | 35.9 39.6 | 39.2 43.3; of 3072 x 8192 43.4 46.2 | 41.9 45.9 | 44.3 48.4, of 4096 x 11008
-// 62.9 66.3 | 58.5 61.5 | 59.9 66.0, of 4096 x 16384 83.9 88.0 | 74.7 83.3 | 83.9 89.1; 12 and 24 tokens of 5120 x 20480 142 144 | 111 114
-// | 110 122.  More than 32 tokens, three | four: 36 of 3072 x 8192 46.7 | 46.6 and 44 46.9 | 48.4, 44 of 4096 x 11008 68.1 | 66.1 and 52
-// 69.0 | 69.5, 48 of 4608 x 12288 79.7 | 78.5.  The overlapped form's last CTA takes channels one by one where they do not come in
-// fours: 24 tokens of 5120 x 13653 87.5 | 92.1 | 84.3, of 3584 x 9557 55.4 | 60.2 | 54.9.  Up to 16 tokens the one kernel is ahead of it on
-// wide layers: four | one, 14 tokens of 4328 x 11520 69.1 | 66.1, 12 of 4776 x 12736 79.8 | 75.7; of 3728 x 14912 69.6 | 70.4.
-// (Layers of fewer weights than any that was measured stay with the one kernel, and so does moc_ffn_forward with nothing saved.)
-enum class SmallBatchForm { kOne, kThree, kOverlapped };
+// (the 2-of-8 mask keeps the one kernel, and so do the block form and moc_ffn_forward with nothing saved)
 SmallBatchForm decode_form(const moc_ffn_desc &d) {
-    const int64_t weights = (int64_t)d.d_model * d.d_ff;  // of one matrix
-    const bool fours = d.d_ff % 4 == 0;
-    if ((d.flags & MOC_FLAG_SELECT_2_OF_8) || weights < 300'000) return SmallBatchForm::kOne;
-    if (weights < (fours ? 18'000'000 : 25'000'000)) return SmallBatchForm::kThree;
-    if (fours && tc::sm_count() >= 96 && d.tokens <= (weights < 30'000'000 ? 32 : 44) && (d.d_model <= 4224 || d.tokens > 16))
-        return SmallBatchForm::kOverlapped;
-    return SmallBatchForm::kOne;  // (the three kernels beyond its 32 tokens)
+    return (d.flags & MOC_FLAG_SELECT_2_OF_8) ? SmallBatchForm::kOne : small_batch_form((int)d.tokens, d.d_model, d.d_ff, tc::sm_count());
 }
 
 // Three to five tokens for which small_batch_preferred chooses the gathering plan (decode_form.h).
@@ -2081,7 +2066,7 @@ int moc_ffn_decode(const moc_ffn_desc *desc, const void *x, const void *w_gate, 
     int rc = check_desc(desc);
     if (rc != MOC_OK) return rc;
     if (desc->tokens > sb::kMaxTokens) return MOC_ERR_UNSUPPORTED;
-    if (!use_decode_plan(*desc))  // more than 16 tokens, or fp32 storage: the forward with nothing saved
+    if (!use_decode_plan(*desc))  // more than 16 tokens, half of the channels in use, or fp32 storage: the forward's plans with nothing saved
         return forward_or_decode(desc, x, w_gate, w_up, w_down, out, nullptr, nullptr, nullptr, workspace,
                                  workspace_bytes, cuda_stream, true);
     if (!good_ptr(x) || !good_ptr(w_gate) || !good_ptr(w_up) || !good_ptr(w_down) || !good_ptr(out))
