@@ -49,10 +49,11 @@
  * Non-finite A token keeps its own channels, but its sums may run over others with a factor of zero (of neighbours in a
  *            small batch, of all channels on the tensor cores): an infinite or NaN weight can reach tokens that do not
  *            keep its row.
- * Co-op      Two kernels are launched cooperatively (cudaLaunchCooperativeKernel: their CTAs wait on one another, so
- *            all must be resident): the one-kernel forms of moc_ffn_decode / moc_ffn_forward for one or two tokens
- *            and for up to 32 tokens that keep nothing.  On a device or in a context that cannot launch them
- *            (no cooperative launch, SMs partly reserved) the multi-kernel forms run instead.  Small layers have a third
+ * Co-op      Two kernels are launched cooperatively (their CTAs wait on one another, so all must be resident): the
+ *            one-kernel form of moc_ffn_decode for one or two tokens, and that of the calls of up to 32 tokens that keep
+ *            nothing (moc_ffn_forward without the triple, moc_ffn_decode_block, the 2-of-8 mask; of plain decode calls
+ *            some up to 16 tokens).  On a device or in a context that cannot launch them (no cooperative launch, SMs
+ *            partly reserved) the multi-kernel forms run instead.  Small layers have a third
  *            one-kernel form of moc_ffn_decode, a cluster of 16 CTAs for each token or two, launched the ordinary way;
  *            it uses neither the workspace nor those counters.
  */
@@ -187,12 +188,12 @@ MOC_API int moc_ffn_recompute_up(const moc_ffn_desc *desc, const void *x, const 
 
 /*
  * Small-batch inference (Section 5): the same forward with nothing saved, for tokens <= 256
- * (more: MOC_ERR_UNSUPPORTED; use moc_ffn_forward).  Up to 16 tokens it is organised so that only the
- * gate matrix and the selected rows of w_up / w_down are read from HBM (d d_ffn + 2 K d weight
- * elements per token instead of 3 d d_ffn).  From 17 tokens on the union of the tokens' channel sets
- * covers nearly every channel (from 5 tokens on nearly half of them at K = d_ff / 8), and all three matrices are
- * streamed once through tensor-core kernels whose tiles are shaped for a few dozen tokens;
- * moc_ffn_forward takes the same path for such batches.
+ * (more: MOC_ERR_UNSUPPORTED; use moc_ffn_forward).  One or two tokens read the gate matrix and the selected rows of
+ * w_up / w_down alone (d d_ffn + 2 K d weight elements per token instead of 3 d d_ffn), and so do up to 16 while fewer
+ * than 0.45 of the channels are selected by some token (4 tokens at K = d_ff / 8) -- but three to five on layers where
+ * streaming is the faster way all the same (below 25 to 40 million weights of a matrix, by the share in use, and where
+ * d_ff is beyond what the gate kernel takes in one go, 18944).  All others stream the three matrices once, through
+ * tensor-core kernels whose tiles are shaped for a few dozen tokens; moc_ffn_forward takes the same path for such batches.
  * In both forms the partial sums of the down projection meet in an fp32 accumulator in an order that
  * is not fixed, so the last bit of `out` can differ from run to run.  On small layers a few tokens take a third form, one
  * cluster of CTAs for each token or two, whose order is fixed.
@@ -207,7 +208,7 @@ MOC_API int moc_ffn_decode(const moc_ffn_desc *desc, const void *x, const void *
  * RMSNorm(h) = h / sqrt(mean(h^2) + rms_eps) . rms_weight per token, rounded to bf16 as the layer's input, and the
  * sum h + D is formed in fp32 from the layer's unrounded output and rounded once.  The normalisation and the
  * residual addition ride on the decode kernels instead of being two more launches around them: the one-kernel forms (one
- * or two tokens, some 5 to 32, a few tokens of small layers) do both themselves; otherwise a one-CTA-per-token kernel
+ * or two tokens, some 5 to 32 with the Top-K mask, a few tokens of small layers) do both themselves; otherwise a one-CTA-per-token kernel
  * chained in front writes the normalised rows and the last step of the down projection adds h.
  *
  *   h           [tokens, d_model] bf16, device: the residual stream

@@ -16,7 +16,7 @@
 //             and its partial output, adds it to a global fp32 accumulator; grid barrier; the CTAs round slices of
 //             the accumulator to bf16.
 //
-// What bounds it (one token of 4096 x 11008, us from the first CTA's start, medians): the gate rows have passed at 16.7 (90 MB at
+// What bounds it (one token of 4096 x 11008, us from the first CTA's start, medians, stamps of a measuring build): the gate rows have passed at 16.7 (90 MB at
 // 7.2 TB/s from 4 on), the histogram is complete at 19.2, the kept channels are known at 21.6, W_up's rows have passed at 24.8,
 // W_down's at 26.2, those of the CTA with the most kept channels (15 against 9 on average) at 27.8, the last barrier at 29.9; 4.5 more
 // until the next call's start.  us per call, a row to a warp, its products by one FMA each with x read from shared memory for every

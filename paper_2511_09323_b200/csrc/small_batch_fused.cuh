@@ -21,7 +21,8 @@
 // overtakes the other by a round of the ring, which a parity test cannot tell.  us per call, two of lane 0 | one elected: 4096 x
 // 11008, 16 tokens 64.7 | 63.0, block form 68.8 | 66.6, 32 tokens 69.3 | 67.4; 2048 x 5504, 20 tokens 38.9 | 36.9; 768 x 2048,
 // 12 tokens 30.6 | 26.6.  (Two elected ones, each giving back every stage, gain 0.5 % on layers wider than 4100 and lose as much at 4096: not
-// taken.)  Its loops over boxes stay rolled: unrolled they cost the other roles 200 bytes of spills and 5 us.
+// taken.)  Its loops over boxes stay rolled: unrolled they cost the other roles 200 bytes of spills and
+// 5 us.  (Rolled, the Top-K instance spills 12 bytes and the 2-of-8 one 8.)
 //
 // CTAs wait on one another, so the launch is cooperative: all CTAs are resident, or the launch fails.  Every wait is
 // bounded as everywhere else in the library.

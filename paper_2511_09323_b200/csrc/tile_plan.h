@@ -26,9 +26,11 @@ struct TilePlan {
 };
 
 // SM cycles of one contraction block in a tile of w columns, operands in L2.  Measured (74 tiles at a time, the difference of
-// contractions of 8, 16 and 32 blocks, sm__cycles_elapsed): 64 to 256 columns, one accumulator, 540 to 570, whatever they are:
-// the thread that issues the MMAs spends 480 of them on a block's four and its commit; 320 columns 770 to 820 and 384 780 to 800
-// (MMAs of 64 columns take what those of 128 do), 448 985, 512 1100.
+// contractions of 8, 16 and 32 blocks, sm__cycles_elapsed) when lane 0 issued the MMAs, 480 cycles for a block's four and its commit: 64 to
+// 256 columns, one accumulator, 540 to 570, whatever they are; 320 columns 770 to 820 and 384 780 to 800 (MMAs of 64 columns take
+// what those of 128 do), 448 985, 512 1100.  The constants are older than the kernel: issued by an elected thread a block of 64 or 128
+// columns takes 350, 256 610.  They stay because a fit to those (335 up to 128 columns, 560 at 256, 70 bytes a cycle) made 1111
+// tokens of 2048 x 5461 246 -> 240 us, but 33736 of 1696 x 6784 6104 -> 6368 and 615 of 2184 x 5824 195 -> 206.
 constexpr double WIDE_MMA_CYCLES = 2.06;  // per column
 inline double wide_block_cycles(int w) { return w <= WIDE_N / 2 ? 528.0 + w / 8.0 : WIDE_MMA_CYCLES * std::max(w, 3 * WIDE_N / 4); }
 
