@@ -1610,21 +1610,22 @@ FusedLayout fused_layout(const moc_ffn_desc &d, bool saving, bool &ok) {
     if (L.m_tiles > L.n_stream) return L;
     // a stage of phases G and U holds as many 64-element blocks as make it about the size of a stage of phase D (the
     // ring's slots have one size): few large stages keep more bytes in flight than many small ones that leave slots half used.
-    // At most two blocks, though, where the rows of x and of the weights are not whole 128-byte lines and a CTA has 24 channels or more,
-    // and two instead of three up to eight tokens; with the 2-of-8 mask where the rows are not whole 32-byte sectors, a CTA has 80 channels
-    // or more and would get three.  us per call, moc_ffn_forward, as many as fit | two: 4104 x 10944, 8 tokens 62.5 | 57.3, 12 64.5 |
-    // 60.4; 4328 x 11520, 16 69.4 | 65.5; 3592 x 9560, 12 57.4 | 53.4; 2056 x 5488, 12 36.2 | 34.9, 32 39.7 | 39.0; 4128 x 11008, 12 62.8 |
-    // 61.6; 1032 x 2752 (20 channels), 12 29.6 | 30.2; whole lines: 4672 x 12456, 4 69.8 | 66.1; 3584 x 9560, 8 53.0 | 49.3; 4096 x 11008, 8
-    // 60.9 | 59.8 and 12 61.9 | 62.4.  Block form, 16 tokens of 4328 x 11520 73.2 | 70.2, of 4096 x 11008 66.5 | 66.8.  2-of-8 mask: 4104 x
-    // 10944, 6 tokens 60.7 | 57.7, 32 66.3 | 63.2; 4328 x 11520, 16 66.0 | 65.0; 3592 x 9560 (72 channels), 32 54.9 | 55.4; 4112 x 11008, 16 58.5
-    // | 59.1; 3336 x 8896 (64 channels), 16 46.0 | 47.1.
+    // At most two blocks, though, where the rows of x and of the weights are not whole 128-byte lines and a CTA has 32 channels or more,
+    // and two instead of three up to eight tokens; with the 2-of-8 mask where the rows are not whole 32-byte sectors, a CTA has 80
+    // channels or more and would get three.  us per call, moc_ffn_forward, as many as fit | two: 4104 x 10944, 8 tokens 62.5 | 57.3, 12
+    // 64.5 | 60.4; 4328 x 11520, 16 69.4 | 65.5; 3592 x 9560, 12 57.4 | 53.4; 2056 x 5488, 12 36.2 | 34.9, 32 39.7 | 39.0; 4128 x 11008,
+    // 12 62.8 | 61.6; 1032 x 2752 (21 channels), 12 29.6 | 30.2; 1432 x 3816 (29), 12 31.9 | 31.4, as the block 16 34.3 | 34.8; whole
+    // lines: 4672 x 12456, 4 69.8 | 66.1; 3584 x 9560, 8 53.0 | 49.3; 4096 x 11008, 8 60.9 | 59.8 and 12 61.9 | 62.4.  Block form, 16
+    // tokens of 4328 x 11520 73.2 | 70.2, of 4096 x 11008 66.5 | 66.8.  2-of-8 mask: 4104 x 10944, 6 tokens 60.7 | 57.7, 32 66.3 | 63.2;
+    // 4328 x 11520, 16 66.0 | 65.0; 3592 x 9560 (72 channels), 32 54.9 | 55.4; 4112 x 11008, 16 58.5 | 59.1; 3336 x 8896 (64 channels), 16
+    // 46.0 | 47.1.
     const uint32_t d_slot = (uint32_t)L.accs * 16384u + xbox, gu_box = xbox + L.w_pitch;
     static const int forced_boxes = [] {
         const char *e = getenv("MOC_FFN_SB_FUSED_BOXES");
         return e ? atoi(e) : 0;
     }();
     int boxes = std::max(1, std::min(8, (int)((d_slot + gu_box / 2) / gu_box)));
-    if (grouped ? dm % 16 != 0 && boxes == 3 && L.rows >= 80 : (dm % 64 != 0 && L.rows >= 24) || (T <= 8 && boxes == 3)) boxes = std::min(boxes, 2);
+    if (grouped ? dm % 16 != 0 && boxes == 3 && L.rows >= 80 : (dm % 64 != 0 && L.rows >= 32) || (T <= 8 && boxes == 3)) boxes = std::min(boxes, 2);
     L.gu_boxes = forced_boxes > 0 ? forced_boxes : boxes;
     L.gu_stages = (dm + L.gu_boxes * sb::kBK - 1) / (L.gu_boxes * sb::kBK);
     const uint32_t gu_slot = (uint32_t)L.gu_boxes * gu_box;

@@ -1,5 +1,5 @@
 """The one-kernel form of the small-batch plan (csrc/small_batch_fused.cuh) on both sides of the rule for the contraction blocks of a stage
-(csrc/api.cu: fused_layout): rows that are whole 128-byte lines, whole sectors or neither, 23 and 24 channels to a CTA, eight and nine tokens."""
+(csrc/api.cu: fused_layout): rows that are whole 128-byte lines, whole sectors or neither, 31 and 32 channels to a CTA, eight and nine tokens."""
 import pytest
 import torch
 
@@ -9,7 +9,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("tokens,d,F", [
-    (8, 1032, 3220), (12, 1032, 3128), (12, 1032, 3131), (32, 1040, 2784), (12, 4104, 3400), (12, 4160, 3400), (8, 2560, 8448), (9, 2560, 8448),
+    (8, 1032, 4340), (12, 1032, 4216), (12, 1032, 4219), (32, 1040, 3712), (12, 4104, 3400), (12, 4160, 3400), (8, 2560, 8448), (9, 2560, 8448),
     (3, 3592, 9557), (12, 2056, 16000),
 ])
 def test_top_k(tokens, d, F):
